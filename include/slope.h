@@ -122,14 +122,11 @@ slope_status_t slope_linear_fwd(const void* X, int b, const void* Wc_vals, const
  * The same sums as slope_adapter_fwd_bwd(phase 0) followed by slope_linear_fwd: T bit for bit; Y up
  * to the order of fp32 partial sums (a fused pair may split the reduction differently), and
  * deterministic like every other call.
- * T is caller-owned scratch that holds X L afterwards.  At inference sizes (decode, and prefill
- * up to a few thousand tokens: as long as the T launch is small enough to run beside the forward
- * and an estimate says it pays) the two launches are issued as a fused pair: the forward streams
- * its operands and runs its sparse reduction while T is still being computed and waits only for
- * T itself, which takes the adapter's extra launch off the critical path (Sec. "Efficient
- * inference": the adapter multiplications are what limits the inference speedup).  With more
- * tokens it issues the same two launches as the separate calls.  The stream must not receive
- * work from another host thread while the call runs.
+ * T is caller-owned scratch that holds X L afterwards.  The two launches are issued as a fused pair:
+ * the forward streams its operands and runs its sparse reduction while T is still being computed
+ * and waits only for T itself, which takes the adapter's extra launch off the critical path (Sec.
+ * "Efficient inference": the adapter multiplications are what limits the inference speedup).  The
+ * stream must not receive work from another host thread while the call runs.
  */
 slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_vals, const void* Wc_meta,
                                         int d_out, int d_in, const void* L, const void* R, int r,
@@ -162,8 +159,9 @@ slope_status_t slope_linear_bwd_dw_masked(const void* dY, const void* X, int b, 
  *             (dT and T are the bf16 tensors written by this call / phase 0).
  *   phase 2:  dT[b x r] = dY R^T only (dL and dR then come from slope_linear_bwd_dw_adapter).
  * `workspace` is device scratch of at least slope_adapter_workspace_bytes()
- * bytes, used by phase 1 for fixed-order split-K partial sums; unused pointers
- * of the other phase may be NULL.
+ * bytes for phase 1 (the present kernels sum their partial products inside a
+ * thread-block cluster and leave it untouched); unused pointers of the other
+ * phase may be NULL.
  */
 size_t slope_adapter_workspace_bytes(int b, int d_out, int d_in, int r);
 slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY,
@@ -273,17 +271,11 @@ slope_status_t slope_dense_linear_bwd_dw(const void* dY, const void* X, int b, i
  * memory pool is closed to it, or in a section where allocation is forbidden).
  * The thesis has no counterpart of this call; it computes the same dL as phase 1 of
  * slope_adapter_fwd_bwd from the same bf16 dT.
- *  - The split-K partial sums live in a fixed 16 MiB array inside the library image
- *    (slope_adapter_dl_noalloc_max_scratch_bytes()); every GPU that loads the library
- *    holds that array until the process exits.
- *  - Sizes whose partial sums do not fit (splits * d_in * r * 4 bytes, with at most 16
- *    splits) are rejected with SLOPE_ERR_SHAPE before anything is launched; use
- *    slope_adapter_fwd_bwd with a workspace for those.
- *  - The first call on a device looks up the array's device address (once per device,
- *    with that device current); make that first call before any stream capture.
- *  - All calls on a device share the one array.  Nothing in it needs clearing between
- *    calls, but two calls whose kernels overlap on the GPU (different streams) race on
- *    it: serialise them.
+ *  - Sizes are limited as if fp32 partial sums of up to 16 token slices had to fit 16 MiB
+ *    (slope_adapter_dl_noalloc_max_scratch_bytes()): beyond that SLOPE_ERR_SHAPE is returned before
+ *    anything is launched; use slope_adapter_fwd_bwd for those.
+ *  - The sums are formed in fixed order inside a thread-block cluster: the call keeps no state and
+ *    may run on any number of streams at a time.
  * Calls no cudaMalloc / cudaFree and no allocating library routine.
  */
 size_t slope_adapter_dl_noalloc_max_scratch_bytes(void);

@@ -1,12 +1,12 @@
 // tcgen05 GEMM kernels for sm_100a.
 //
-// All kernels are persistent and warp-specialised: warp 0 feeds shared memory with TMA,
+// The big-tile kernels are persistent, all are warp-specialised: warp 0 feeds shared memory with TMA,
 // warp 1 owns tensor memory and issues the MMAs (one elected thread), the remaining warps
 // drain the fp32 accumulators from tensor memory, convert to bf16 and store.  Every mbarrier
 // wait is bounded (ptx.cuh); a role that gives up sets a CTA-wide flag, all roles leave their
 // loops, tensor memory is released and the kernel returns.
 //
-//   dense_gemm_kernel          1 CTA per 128 x N tile; the skinny adapter GEMMs and small dW
+//   dense_gemm_kernel          1 CTA per 128 x 128 tile; dW of the smallest weight matrices
 //   dense_gemm_pair_kernel     CTA pair per 256 x 256 tile (cta_group::2), the last wave's tiles
 //                              halved; dW (masked epilogue) and the dense layer (store epilogue)
 //   sparse_gemm_pair_kernel    CTA pair per 256 x 224 (or 256 x 128) tile, tcgen05.mma.sp;
@@ -15,8 +15,8 @@
 //                              tile); forward / dX with long reductions
 //   sparse_gemm_skinny_kernel  one CTA per 128-row weight slab and K-slice, cluster reduction
 //                              through distributed shared memory; forward / dX with few
-//                              tokens (inference, decode) and the adapter products at such
-//                              sizes, not persistent
+//                              tokens (inference, decode), not persistent
+// The adapter's low-rank products have a kernel of their own (adapter_kernels.cuh).
 #pragma once
 #include "ptx.cuh"
 
@@ -55,7 +55,7 @@ struct SparseGemmParams {
     int M, K, Ntok, r;
     int a2_mn_major;              // 1: A2 is stored [r x M] (M contiguous)
     int group_m;                  // 512-row-tile kernel: row tiles per raster group (0: all in one group)
-    int pdl_mode;                 // few-token kernel: 0 plain, 1 producer / 2 consumer of a fused pair of launches
+    int pdl_mode;                 // 2: consumer of a fused pair of launches (see the few-token kernel)
     const uint8_t* meta;          // metadata blocks of A
     uint16_t* out;                // [Ntok x M]
 };
@@ -69,60 +69,69 @@ struct SparseGemmParams {
 //   kEpiMasked   Eq. (sparse_backward_weight) + Algorithm 1 "pruneAndCompress": keep, per
 //                group of 4 columns, the two columns the first-pass mask selects; bf16
 //                [M x N/2]
-//   kEpiPartial  fp32 partial sums of one K-split into workspace[split][M][N]
 // =====================================================================================
-constexpr int kEpiStore = 0, kEpiMasked = 1, kEpiPartial = 2;
+constexpr int kEpiStore = 0, kEpiMasked = 1;
 
 struct DenseGemmParams {
     int M, N, K;
-    int k_splits;
     void* out;
     const uint8_t* mask;          // kEpiMasked: [M x N/8]
-    int pdl_mode;                 // 1: producer of a fused pair of launches (wait first, release dependents afterwards)
 };
 
-template <int BLOCK_N, int STAGES>
+// 16 accumulator columns of a row -> the 8 that the mask keeps, in ascending order per group of 4.
+__device__ __forceinline__ uint4 compress_16(const uint32_t (&v)[16], uint32_t mbits) {
+    uint32_t w[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const uint32_t mb = (mbits >> (4 * g)) & 0xFu;
+        // kept positions in ascending order: lowest set bit, highest set bit
+        const int p0 = __ffs(mb) - 1, p1 = 31 - __clz(mb);
+        const float e0 = __uint_as_float(v[4 * g]), e1 = __uint_as_float(v[4 * g + 1]),
+                    e2 = __uint_as_float(v[4 * g + 2]), e3 = __uint_as_float(v[4 * g + 3]);
+        const float lo = p0 == 0 ? e0 : (p0 == 1 ? e1 : e2);
+        const float hi = p1 == 1 ? e1 : (p1 == 2 ? e2 : e3);
+        w[g] = pack_bf16x2(lo, hi);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Masked weight gradient of the smallest weight matrices: one 128 x 128 tile per CTA.
+template <int STAGES>
 struct DenseCfg {
+    static constexpr int kBlockN = 128;
     static constexpr int kABytes = kBlockM * 128;                // 128 x 64 bf16
-    static constexpr int kBBytes = BLOCK_N * 128;                // BLOCK_N x 64 bf16
+    static constexpr int kBBytes = kBlockN * 128;
     static constexpr int kStageBytes = kABytes + kBBytes;
     static constexpr int kSmemBytes = STAGES * kStageBytes + 256 + 1024;
-    static constexpr int kTmemCols = 2 * BLOCK_N <= 32 ? 32 : (2 * BLOCK_N <= 64 ? 64 : (2 * BLOCK_N <= 128 ? 128 : (2 * BLOCK_N <= 256 ? 256 : 512)));
-    static_assert(BLOCK_N % 64 == 0 && BLOCK_N <= 256, "BLOCK_N must be 64, 128, 192 or 256");
 };
 
-template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
+template <int STAGES>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
-                  const DenseGemmParams p0, const __grid_constant__ CUtensorMap tmA1,
-                  const __grid_constant__ CUtensorMap tmB1, const DenseGemmParams p1) {
-    // Up to two independent problems of the same kind share one launch (p1.M == 0: only one):
-    // tiles [0, tiles0) belong to problem 0, the rest to problem 1.
-    using Cfg = DenseCfg<BLOCK_N, STAGES>;
+dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                  const DenseGemmParams p) {
+    // A = dY and B = X, both stored [K x .]; M and N are multiples of 128; one tile per CTA
+    using Cfg = DenseCfg<STAGES>;
+    constexpr int kBlockN = Cfg::kBlockN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes);
     uint64_t* empty_bar = full_bar + STAGES;
     uint64_t* tfull_bar = empty_bar + STAGES;
-    uint64_t* tempty_bar = tfull_bar + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty_bar + 2);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    auto tiles_of = [](const DenseGemmParams& q) {
-        return q.M == 0 ? 0 : ((q.M + kBlockM - 1) / kBlockM) * ((q.N + BLOCK_N - 1) / BLOCK_N) * q.k_splits;
-    };
-    const int tiles0 = tiles_of(p0);
-    const int num_tiles = tiles0 + tiles_of(p1);
+    const int num_m = p.M / kBlockM, num_kb = (p.K + 63) / 64;
+    const int m_blk = blockIdx.x % num_m, n_blk = blockIdx.x / num_m;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 128); }
+        mbar_init(tfull_bar, 1);
         *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, Cfg::kTmemCols);
+        tmem_alloc(tmem_slot, kBlockN);
         tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -131,156 +140,64 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constan
     const uint32_t tmem_base = *tmem_slot;
     // Programmatic dependent launch: the set-up above may overlap the tail of the previous kernel in
     // the stream; no thread touches global memory before that kernel has completed.
-    if (p0.pdl_mode == 1) {              // see the few-token kernel: the dependent may rely on all earlier work
-        griddep_wait();
-        griddep_launch_dependents();
-    } else {
-        griddep_launch_dependents();
-        griddep_wait();
-    }
-
-    // tile -> (problem, m block, n block, split): m fastest so that concurrently running CTAs share B
-    auto decode = [&](int tile, int& m_blk, int& n_blk, int& kb0, int& kb1) {
-        const bool second = tile >= tiles0;
-        const DenseGemmParams& q = second ? p1 : p0;
-        if (second) tile -= tiles0;
-        const int num_m = (q.M + kBlockM - 1) / kBlockM;
-        const int num_n = (q.N + BLOCK_N - 1) / BLOCK_N;
-        const int num_kb_total = (q.K + 63) / 64;
-        const int kb_per_split = (num_kb_total + q.k_splits - 1) / q.k_splits;
-        m_blk = tile % num_m;
-        const int rest = tile / num_m;
-        n_blk = rest % num_n;
-        const int split = rest / num_n;
-        kb0 = split * kb_per_split;
-        kb1 = min(num_kb_total, kb0 + kb_per_split);
-        return split | (second ? 0x10000 : 0);
-    };
+    griddep_launch_dependents();
+    griddep_wait();
 
     if (warp == 0) {
         if (elect_one()) {
-            tma_prefetch_desc(&tmA0);
-            tma_prefetch_desc(&tmB0);
+            tma_prefetch_desc(&tmA);
+            tma_prefetch_desc(&tmB);
             PipeState ps;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
-                int m_blk, n_blk, kb0, kb1;
-                const bool second = (decode(tile, m_blk, n_blk, kb0, kb1) & 0x10000) != 0;
-                const CUtensorMap* tmA = second ? &tmA1 : &tmA0;
-                const CUtensorMap* tmB = second ? &tmB1 : &tmB0;
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
-                    uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
-                    uint8_t* sB = sA + Cfg::kABytes;
-                    uint64_t* bar = &full_bar[ps.stage];
-                    mbar_expect_tx(bar, Cfg::kStageBytes);
-                    if (A_MN) {
-                        tma_load_2d(sA, tmA, bar, m_blk * kBlockM, kb * 64);
-                        tma_load_2d(sA + 8192, tmA, bar, m_blk * kBlockM + 64, kb * 64);
-                    } else {
-                        tma_load_2d(sA, tmA, bar, kb * 64, m_blk * kBlockM);
-                    }
-                    if (B_MN) {
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) break;
+                uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
+                uint8_t* sB = sA + Cfg::kABytes;
+                uint64_t* bar = &full_bar[ps.stage];
+                mbar_expect_tx(bar, Cfg::kStageBytes);
 #pragma unroll
-                        for (int h = 0; h < BLOCK_N / 64; ++h)
-                            tma_load_2d(sB + h * 8192, tmB, bar, n_blk * BLOCK_N + h * 64, kb * 64);
-                    } else {
-                        tma_load_2d(sB, tmB, bar, kb * 64, n_blk * BLOCK_N);
-                    }
-                    ps.advance(STAGES);
+                for (int h = 0; h < 2; ++h) {
+                    tma_load_2d(sA + h * 8192, &tmA, bar, m_blk * kBlockM + h * 64, kb * 64);
+                    tma_load_2d(sB + h * 8192, &tmB, bar, n_blk * kBlockN + h * 64, kb * 64);
                 }
+                ps.advance(STAGES);
             }
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            constexpr uint32_t idesc = make_idesc_bf16(kBlockM, BLOCK_N, A_MN, B_MN, false);
+            constexpr uint32_t idesc = make_idesc_bf16(kBlockM, kBlockN, true, true, false);
             PipeState ps;
             bool ok = true;
-            int it = 0;
-            for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++it) {
-                int m_blk, n_blk, kb0, kb1;
-                decode(tile, m_blk, n_blk, kb0, kb1);
-                const int acc = it & 1;
-                const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
-                if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * BLOCK_N;
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
-                    tc_fence_after_sync();
-                    const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
-                    const uint32_t sB = sA + Cfg::kABytes;
+                const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
+                const uint32_t sB = sA + Cfg::kABytes;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint64_t ad = A_MN ? make_smem_desc(sA + j * 2048, 8192, 1024, kSwizzle128B)
-                                                 : make_smem_desc(sA + j * 32, 16, 1024, kSwizzle128B);
-                        const uint64_t bd = B_MN ? make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B)
-                                                 : make_smem_desc(sB + j * 32, 16, 1024, kSwizzle128B);
-                        umma_bf16(d_tmem, ad, bd, idesc, (kb > kb0 || j > 0) ? 1u : 0u);
-                    }
-                    umma_commit(&empty_bar[ps.stage]);
-                    ps.advance(STAGES);
-                }
-                if (ok) umma_commit(&tfull_bar[acc]);
+                for (int j = 0; j < 4; ++j)
+                    umma_bf16(tmem_base, make_smem_desc(sA + j * 2048, 8192, 1024, kSwizzle128B),
+                              make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B), idesc, (kb | j) != 0 ? 1u : 0u);
+                umma_commit(&empty_bar[ps.stage]);
+                ps.advance(STAGES);
             }
+            if (ok) umma_commit(tfull_bar);
         }
     } else {
         const int q = warp & 3;
-        bool ok = true;
-        int it = 0;
-        for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++it) {
-            int m_blk, n_blk, kb0, kb1;
-            const int code = decode(tile, m_blk, n_blk, kb0, kb1);
-            const int split = code & 0xFFFF;
-            const DenseGemmParams& p = (code & 0x10000) ? p1 : p0;
-            const int acc = it & 1;
-            const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
-            if (!mbar_wait(&tfull_bar[acc], acc_phase, abort_flag)) { ok = false; break; }
+        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+        const int m = m_blk * kBlockM + q * 32 + lane;
+        if (mbar_wait(tfull_bar, 0u, abort_flag)) {
             tc_fence_after_sync();
-            const uint32_t t_row = tmem_base + acc * BLOCK_N + (static_cast<uint32_t>(q * 32) << 16);
-            const int m = m_blk * kBlockM + q * 32 + lane;
 #pragma unroll 1
-            for (int c0 = 0; c0 < BLOCK_N; c0 += 16) {
+            for (int c0 = 0; c0 < kBlockN; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld_16(t_row + c0, v);
                 tmem_ld_wait();
-                const int n0 = n_blk * BLOCK_N + c0;
-                if (m >= p.M || n0 >= p.N) continue;
-                if (EPI == kEpiStore) {
-                    uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.N + n0);
-                    uint32_t w[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) w[c] = pack_bf16x2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
-                    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-                } else if (EPI == kEpiMasked) {
-                    const uint32_t mbits =
-                        *reinterpret_cast<const uint16_t*>(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3));
-                    uint32_t w[4];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const uint32_t mb = (mbits >> (4 * g)) & 0xFu;
-                        // kept positions in ascending order: lowest set bit, highest set bit
-                        const int p0 = __ffs(mb) - 1, p1 = 31 - __clz(mb);
-                        const float e0 = __uint_as_float(v[4 * g]), e1 = __uint_as_float(v[4 * g + 1]),
-                                    e2 = __uint_as_float(v[4 * g + 2]), e3 = __uint_as_float(v[4 * g + 3]);
-                        const float lo = p0 == 0 ? e0 : (p0 == 1 ? e1 : e2);
-                        const float hi = p1 == 1 ? e1 : (p1 == 2 ? e2 : e3);
-                        w[g] = pack_bf16x2(lo, hi);
-                    }
-                    *reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1)) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
-                } else {
-                    float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.out) +
-                                                            (static_cast<size_t>(split) * p.M + m) * p.N + n0);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        dst[c] = make_float4(__uint_as_float(v[4 * c]), __uint_as_float(v[4 * c + 1]),
-                                             __uint_as_float(v[4 * c + 2]), __uint_as_float(v[4 * c + 3]));
-                }
+                const int n0 = n_blk * kBlockN + c0;
+                const uint32_t mbits =
+                    *reinterpret_cast<const uint16_t*>(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3));
+                *reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) +
+                                          (n0 >> 1)) = compress_16(v, mbits);
             }
-            tc_fence_before_sync();
-            mbar_arrive(&tempty_bar[acc]);
         }
     }
 
@@ -290,7 +207,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constan
     __syncthreads();
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, Cfg::kTmemCols);
+        tmem_dealloc(tmem_base, kBlockN);
     }
 }
 
@@ -803,19 +720,8 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 } else {
                     const uint32_t mbits =
                         *reinterpret_cast<const uint16_t*>(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3));
-                    uint32_t w[4];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const uint32_t mb = (mbits >> (4 * g)) & 0xFu;
-                        const int p0 = __ffs(mb) - 1, p1 = 31 - __clz(mb);
-                        const float e0 = __uint_as_float(v[4 * g]), e1 = __uint_as_float(v[4 * g + 1]),
-                                    e2 = __uint_as_float(v[4 * g + 2]), e3 = __uint_as_float(v[4 * g + 3]);
-                        const float lo = p0 == 0 ? e0 : (p0 == 1 ? e1 : e2);
-                        const float hi = p1 == 1 ? e1 : (p1 == 2 ? e2 : e3);
-                        w[g] = pack_bf16x2(lo, hi);
-                    }
                     *reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1)) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
+                        compress_16(v, mbits);
                 }
             }
             tc_fence_before_sync();
@@ -1232,7 +1138,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 }
 
 // =====================================================================================
-// Sparse GEMM for few tokens (inference / decode sizes, Ntok <= BLOCK_N <= 256).
+// Sparse GEMM for few tokens (inference / decode sizes, Ntok <= BLOCK_N <= 128).
 // With so few tokens the GEMM is a stream of compressed weights from HBM, and the big-tile
 // kernels above would occupy only a handful of SMs.  Here one CTA owns a 128-row slab of the
 // weights (1-CTA tcgen05.mma.sp, M = 128) and a slice of the reduction: a cluster of S CTAs
@@ -1259,7 +1165,7 @@ struct SparseSkinnyCfg {
     static constexpr int kPartialBytes = BLOCK_N * kBlockM * 4;      // fp32 [token][feature], reuses the rings
     static constexpr int kSmemBytes = kOffBar + 512 + 1024;
     static constexpr int kTmemCols = BLOCK_N + 8 <= 32 ? 32 : (BLOCK_N + 8 <= 128 ? 128 : (BLOCK_N + 8 <= 256 ? 256 : 512));
-    static_assert(BLOCK_N % 16 == 0 && BLOCK_N >= 16 && BLOCK_N <= 256, "token tile");
+    static_assert(BLOCK_N % 16 == 0 && BLOCK_N >= 16 && BLOCK_N <= 128, "token tile");
     static_assert(kPartialBytes <= kOffBar, "partial tile must fit in the pipeline buffers");
     static_assert(kAStage % 1024 == 0 && kBStage % 1024 == 0 && kSmemBytes <= 232448, "shared memory layout");
     static_assert(2 * (A_STAGES + B_STAGES) * 8 + 16 <= 512, "barrier block");
@@ -1289,12 +1195,8 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     const int kb_per = (num_kb + splits - 1) / splits;
     const int kb0 = min(num_kb, rank * kb_per), kb1 = min(num_kb, kb0 + kb_per);
     const int num_sb = kb1 - kb0;                                            // sparse k-blocks of this rank
-    // Dense K-steps (64 wide): the adapter product rides on the last rank; with no sparse part
-    // at all (K == 0: a plain few-token dense GEMM) they are split over the ranks instead.
-    const int all_ab = (p.r + 63) / 64;
-    const int ab_per = num_kb == 0 ? (all_ab + splits - 1) / splits : all_ab;
-    const int ab0 = num_kb == 0 ? min(all_ab, rank * ab_per) : 0;
-    const int num_ab = num_kb == 0 ? min(all_ab, ab0 + ab_per) - ab0 : (rank == splits - 1 ? all_ab : 0);
+    // Dense K-steps (64 wide): the adapter product rides on the last rank.
+    const int num_ab = rank == splits - 1 ? (p.r + 63) / 64 : 0;
     const int total_kb = num_sb + num_ab;
 
     if (threadIdx.x == 0) {
@@ -1324,29 +1226,24 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     // writing stays correct; the first loads after the wait then come at L2 instead of HBM latency.
     //
     // Two launches issued together by one call (T = X L, then the forward that adds T R) use the
-    // dependency more finely.  The producer (pdl_mode 1) waits first and releases its dependents
-    // afterwards: when the consumer starts, everything that preceded the pair in the stream is
-    // complete.  The consumer (pdl_mode 2) therefore streams its weights and activations and runs
-    // its whole sparse reduction without waiting; only the thread that loads the producer's
+    // dependency more finely.  The producer (adapter_gemm_kernel, pdl_mode 1) waits first and releases
+    // its dependents afterwards: when the consumer starts, everything that preceded the pair in the
+    // stream is complete.  The consumer (pdl_mode 2) therefore streams its weights and activations
+    // and runs its whole sparse reduction without waiting; only the thread that loads the producer's
     // output T waits, right before the first such load.  Everything that follows in the consumer
     // (the adapter MMAs, the cluster reduction, the stores) is ordered behind that load.
-    if (p.pdl_mode == 1) {
-        griddep_wait();
-        griddep_launch_dependents();
-    } else {
-        griddep_launch_dependents();
-        if (warp == 0 && elect_one()) {
-            // (a short K-slice gains nothing: its few tiles are requested at once after the wait, and the
-            // prefetch requests would only sit in front of them in the TMA queue)
-            const int n_pf = num_sb >= 8 && p.pdl_mode == 0 ? kSkinnyPrefetchBlocks : 0;
-            for (int i = 0; i < n_pf; ++i) {
-                tma_prefetch_l2_2d(&tmA, (kb0 + i) * 64, m_blk * kBlockM);
-                tma_prefetch_l2_2d(&tmE, 0, m_blk * num_kb + kb0 + i);
-            }
+    griddep_launch_dependents();
+    if (warp == 0 && elect_one()) {
+        // (a short K-slice gains nothing: its few tiles are requested at once after the wait, and the
+        // prefetch requests would only sit in front of them in the TMA queue)
+        const int n_pf = num_sb >= 8 && p.pdl_mode == 0 ? kSkinnyPrefetchBlocks : 0;
+        for (int i = 0; i < n_pf; ++i) {
+            tma_prefetch_l2_2d(&tmA, (kb0 + i) * 64, m_blk * kBlockM);
+            tma_prefetch_l2_2d(&tmE, 0, m_blk * num_kb + kb0 + i);
         }
-        __syncwarp();
-        if (p.pdl_mode != 2) griddep_wait();
     }
+    __syncwarp();
+    if (p.pdl_mode != 2) griddep_wait();
 
     if (warp == 0) {
         // ---------------------------------------------------------- weight ring (values + metadata)
@@ -1363,7 +1260,7 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
                     tma_load_2d_hint(sA, &tmA, bar, kb * 64, m_blk * kBlockM, stream_once);
                     tma_load_2d_hint(sA + Cfg::kABytes, &tmE, bar, 0, m_blk * num_kb + kb, stream_once);
                 } else {
-                    const int ab = ab0 + i - num_sb;
+                    const int ab = i - num_sb;
                     mbar_expect_tx(bar, Cfg::kABytes);
                     if (p.a2_mn_major) {
                         tma_load_2d(sA, &tmA2, bar, m_blk * kBlockM, ab * 64);
@@ -1431,7 +1328,7 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
                 } else {
                     if (p.pdl_mode == 2 && i == num_sb) griddep_wait();      // T comes from the launch before this one
                     mbar_expect_tx(bar, BLOCK_N * 128);
-                    tma_load_2d(sB, &tmB2, bar, (ab0 + i - num_sb) * 64, 0);
+                    tma_load_2d(sB, &tmB2, bar, (i - num_sb) * 64, 0);
                 }
                 ps.advance(B_STAGES);
             }

@@ -2,12 +2,14 @@
 // TMA descriptor construction and kernel launches.  No device memory is allocated here.
 #include "../../include/slope.h"
 
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
 #include <utility>
 
+#include "adapter_kernels.cuh"
 #include "dw_adapter_kernel.cuh"
 #include "gemm_kernels.cuh"
 #include "nm_kernels.cuh"
@@ -257,54 +259,128 @@ static bool set_smem(Kernel k, int bytes) {
 constexpr int kStreamBlocksPerSm = 32;
 
 // ------------------------------------------------------------------ dense GEMM launch
-struct DenseProblem {
-    const void* A = nullptr;
-    const void* B = nullptr;
-    int M = 0, N = 0, K = 0, k_splits = 1;
-    void* out = nullptr;
-    const void* mask = nullptr;
-    int pdl_mode = 0;
-};
-
-// One launch of the 1-CTA dense kernel over one or two problems of the same kind.
-template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
-static slope_status_t launch_dense2(const DenseProblem& q0, const DenseProblem& q1, cudaStream_t stream,
-                                    const DeviceInfo& info) {
-    using Cfg = DenseCfg<BLOCK_N, STAGES>;
-    CUtensorMap tm[4];
-    DenseGemmParams p[2];
-    int tiles = 0;
-    for (int i = 0; i < 2; ++i) {
-        const DenseProblem& q = i == 0 ? q0 : (q1.M > 0 ? q1 : q0);          // unused slot mirrors problem 0
-        const bool okA = A_MN ? make_tmap(&tm[2 * i], q.A, q.K, q.M, 64, 64) : make_tmap(&tm[2 * i], q.A, q.M, q.K, kBlockM, 64);
-        const bool okB = B_MN ? make_tmap(&tm[2 * i + 1], q.B, q.K, q.N, 64, 64)
-                              : make_tmap(&tm[2 * i + 1], q.B, q.N, q.K, BLOCK_N, 64);
-        if (!okA || !okB) return SLOPE_ERR_CUDA;
-        const bool live = i == 0 || q1.M > 0;
-        p[i].M = live ? q.M : 0; p[i].N = q.N; p[i].K = q.K; p[i].k_splits = q.k_splits; p[i].out = q.out;
-        p[i].mask = static_cast<const uint8_t*>(q.mask);
-        p[i].pdl_mode = q0.pdl_mode;
-        if (live) tiles += ((q.M + kBlockM - 1) / kBlockM) * ((q.N + BLOCK_N - 1) / BLOCK_N) * q.k_splits;
-    }
-    auto kern = dense_gemm_kernel<A_MN, B_MN, BLOCK_N, EPI, STAGES>;
+static slope_status_t launch_dense_masked(const void* dY, const void* X, int M, int N, int K, void* out, const void* mask,
+                                          cudaStream_t stream) {
+    constexpr int kStages = 6;
+    using Cfg = DenseCfg<kStages>;
+    CUtensorMap tmA, tmB;
+    if (!make_tmap(&tmA, dY, K, M, 64, 64) || !make_tmap(&tmB, X, K, N, 64, 64)) return SLOPE_ERR_CUDA;
+    const DenseGemmParams p{M, N, K, out, static_cast<const uint8_t*>(mask)};
+    auto kern = dense_gemm_kernel<kStages>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    int grid = tiles < info.sm_count ? tiles : info.sm_count;
-    // The producer of a fused pair runs beside a kernel of CTA pairs: launched as clusters of two its
-    // CTAs fill whole SM pairs instead of breaking up many (the kernel itself ignores the cluster;
-    // a CTA without a tile exits at once).
-    const int cluster = q0.pdl_mode == 1 ? 2 : 1;
-    if (cluster == 2) grid = (grid + 1) & ~1;
-    return launch_cluster_ex(kern, grid, cluster, kGemmThreads, Cfg::kSmemBytes, /*overlap_prologue=*/true, stream,
-                             tm[0], tm[1], p[0], tm[2], tm[3], p[1]);
+    return launch_cluster_ex(kern, (M / kBlockM) * (N / Cfg::kBlockN), 1, kGemmThreads, Cfg::kSmemBytes,
+                             /*overlap_prologue=*/true, stream, tmA, tmB, p);
 }
 
-template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
-static slope_status_t launch_dense(const void* A, const void* B, int M, int N, int K, int k_splits, void* out,
-                                   const void* mask, cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    DenseProblem q;
-    q.A = A; q.B = B; q.M = M; q.N = N; q.K = K; q.k_splits = k_splits; q.out = out; q.mask = mask;
-    q.pdl_mode = pdl_mode;
-    return launch_dense2<A_MN, B_MN, BLOCK_N, EPI, STAGES>(q, DenseProblem{}, stream, info);
+// ------------------------------------------------------------------ adapter products
+struct AdapterOperands {
+    const void* A = nullptr;      // the large operand: [M x K], or [K x M] when A_MN
+    const void* B = nullptr;      // [N x K], or [K x N] when B_MN
+    void* out = nullptr;
+    int M = 0;
+    int transposed = 0;
+};
+
+// Column tile, reduction split (= cluster size) and ring depth of an adapter launch, by estimate.
+// Constants fitted to a sweep of tiles, splits and depths over 8 ... 16384 tokens, widths 768 ... 13824
+// and ranks 16 ... 256 (in most of them the choice is within 5 % of the best swept one):
+//   - a round trip through the ring takes 0.8 us, so a k-block costs at least that over its depth,
+//     and at least what the SM takes in (150 KB per us);
+//   - a CTA brings in 90 GB/s of the large operand, all of them together 6 TB/s, and every further
+//     column tile costs 8 % of that (its second read comes from L2);
+//   - draining a tile costs 0.3 us per 64 columns, 1 us more and 1 us per 64 columns when it is split.
+struct AdapterPlan {
+    int n_tile, splits;
+    bool deep;                    // one CTA per SM with all of its shared memory; else two that share it
+};
+static AdapterPlan adapter_plan(int row_tiles, double a_bytes, int N, int K, int sm_count) {
+    const int num_kb = (K + 63) / 64;
+    AdapterPlan best{64, 1, true};
+    double best_cost = 1e30;
+    for (int n_tile = 64; n_tile <= 256 && (n_tile == 64 || n_tile < 2 * N); n_tile *= 2) {
+        const int col_tiles = (N + n_tile - 1) / n_tile;
+        for (int s = 1; s <= 8 && (s == 1 || 2 * s <= num_kb); s *= 2) {
+            const int ctas = row_tiles * col_tiles * s;
+            // clusters of 4 and 8 do not fill every SM (33 and 15 of them fit on 148 SMs)
+            const int sms = s == 8 ? sm_count * 120 / 148 : s == 4 ? sm_count * 132 / 148 : sm_count;
+            const bool deep = n_tile == 256 || ctas <= sms;
+            const int slots = (deep ? 1 : 2) * sms;
+            const double stages = n_tile == 64 ? (deep ? 9 : 4) : n_tile == 128 ? (deep ? 7 : 3) : 4;
+            const int waves = (ctas + slots - 1) / slots;
+            const double kb_us = std::max(0.8 / stages, (deep ? 1 : 2) * (16.0 + n_tile / 8.0) / 150.0);
+            const double hbm = std::min(6.0e6, 0.09e6 * std::min(ctas, sm_count)) / (1.0 + 0.08 * (col_tiles - 1));
+            const double stream = std::max(waves * ((num_kb + s - 1) / s) * kb_us, a_bytes / hbm);
+            const double tail = (s > 1 ? 1.0 : 0.3) * n_tile / 64.0 + (s > 1 ? 1.0 : 0.0);
+            const double cost = stream + waves * tail;
+            if (cost < best_cost - 1e-9) { best_cost = cost; best = AdapterPlan{n_tile, s, deep}; }
+        }
+    }
+    return best;
+}
+
+template <bool A_MN, bool B_MN, int N_TILE>
+static slope_status_t launch_adapter_tile(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K, int splits,
+                                          bool deep, cudaStream_t stream, int pdl_mode) {
+    using Cfg = AdapterCfg<N_TILE>;
+    CUtensorMap tm[4];
+    AdapterProblem p[2];
+    int tiles = 0;
+    for (int i = 0; i < 2; ++i) {
+        const bool live = i == 0 || q1.M > 0;
+        const AdapterOperands& q = i == 0 ? q0 : (live ? q1 : q0);           // unused slot mirrors problem 0
+        const bool okA = A_MN ? make_tmap(&tm[2 * i], q.A, K, q.M, 64, 64) : make_tmap(&tm[2 * i], q.A, q.M, K, kBlockM, 64);
+        const bool okB = B_MN ? make_tmap(&tm[2 * i + 1], q.B, K, N, 64, 64) : make_tmap(&tm[2 * i + 1], q.B, N, K, N_TILE, 64);
+        if (!okA || !okB) return SLOPE_ERR_CUDA;
+        p[i] = AdapterProblem{live ? q.M : 0, N, K, static_cast<uint16_t*>(q.out), q.transposed};
+        if (live) tiles += (q.M + kBlockM - 1) / kBlockM;
+    }
+    auto kern = adapter_gemm_kernel<A_MN, B_MN, N_TILE>;
+    if (!set_smem(kern, Cfg::smem_bytes(Cfg::kDeep))) return SLOPE_ERR_CUDA;
+    const int stages = deep || Cfg::kShared == 0 ? Cfg::kDeep : Cfg::kShared;
+    return launch_cluster_ex(kern, tiles * ((N + N_TILE - 1) / N_TILE) * splits, splits, kGemmThreads,
+                             Cfg::smem_bytes(stages), /*overlap_prologue=*/true, stream, tm[0], tm[1], p[0], tm[2], tm[3],
+                             p[1], stages, pdl_mode);
+}
+
+// D[M x N] = A B over one or two problems with the same N (= r) and K.
+template <bool A_MN, bool B_MN>
+static slope_status_t launch_adapter(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K,
+                                     cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
+    const AdapterPlan plan = adapter_plan(row_tiles, 2.0 * K * (static_cast<double>(q0.M) + q1.M), N, K, info.sm_count);
+    switch (plan.n_tile) {
+        case 64: return launch_adapter_tile<A_MN, B_MN, 64>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
+        case 128: return launch_adapter_tile<A_MN, B_MN, 128>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
+        default: return launch_adapter_tile<A_MN, B_MN, 256>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
+    }
+}
+
+// CTAs of the T launch below.
+static int adapter_T_ctas(int b, int d_in, int r, const DeviceInfo& info) {
+    const int row_tiles = (b + kBlockM - 1) / kBlockM;
+    const AdapterPlan plan = adapter_plan(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count);
+    return row_tiles * ((r + plan.n_tile - 1) / plan.n_tile) * plan.splits;
+}
+
+// T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
+static slope_status_t launch_adapter_T(const void* X, const void* L, int b, int d_in, int r, void* T,
+                                       cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    return launch_adapter<false, true>(AdapterOperands{X, L, T, b, 0}, AdapterOperands{}, r, d_in, stream, info, pdl_mode);
+}
+
+// dT[b x r] = dY[b x d_out] * R[r x d_out]^T   (both K contiguous)
+static slope_status_t launch_adapter_dT(const void* dY, const void* R, int b, int d_out, int r, void* dT,
+                                        cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    return launch_adapter<false, false>(AdapterOperands{dY, R, dT, b, 0}, AdapterOperands{}, r, d_out, stream, info,
+                                        pdl_mode);
+}
+
+// dR[r x d_out] = (dY^T T)^T and dL[d_in x r] = X^T dT: operands stored [K x M] / [K x N] with K = tokens.
+static AdapterOperands adapter_dR(const void* dY, const void* T, int d_out, void* dR) {
+    return AdapterOperands{dY, T, dR, d_out, 1};
+}
+static AdapterOperands adapter_dL(const void* X, const void* dT, int d_in, void* dL) {
+    return AdapterOperands{X, dT, dL, d_in, 0};
 }
 
 // ------------------------------------------------------------------ CTA-pair launches (main GEMMs)
@@ -316,8 +392,7 @@ constexpr int kPairNarrowStages = 5;
 template <int BLOCK_N, int STAGES>
 static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                                          const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0,
-                                         int reserved_ctas = 0) {
+                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
     using Cfg = SparsePairCfg<BLOCK_N, STAGES>;
     CUtensorMap tmA, tmB, tmE, tmA2, tmB2, tmO;
     if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
@@ -339,8 +414,7 @@ static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* 
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
     p.pdl_mode = pdl_mode;
     const int tiles = ((M / kBlockM + 1) / 2) * ((ntok + BLOCK_N - 1) / BLOCK_N);
-    // (the consumer of a fused pair leaves the producer's SMs alone)
-    const int max_pairs = (info.sm_count - reserved_ctas) / 2;
+    const int max_pairs = info.sm_count / 2;
     const int pairs = tiles < max_pairs ? tiles : max_pairs;
     return launch_pairs(kern, 2 * pairs, Cfg::kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmE, tmA2, tmB2, tmO, p);
 }
@@ -374,8 +448,7 @@ static int quad_group_m(int M, int K, int ntok, int num_pairs) {
 
 static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                                          const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0,
-                                         int reserved_ctas = 0) {
+                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
     using Cfg = SparseQuadCfg<kQuadBlockN, kQuadStages>;
     CUtensorMap tmA, tmB, tmE, tmA2, tmB2, tmO;
     if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
@@ -393,7 +466,7 @@ static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* 
     p.M = M; p.K = K; p.Ntok = ntok; p.r = r; p.a2_mn_major = a2_mn ? 1 : 0;
     p.meta = static_cast<const uint8_t*>(meta);
     p.out = static_cast<uint16_t*>(out);
-    const int max_pairs = (info.sm_count - reserved_ctas) / 2;
+    const int max_pairs = info.sm_count / 2;
     p.pdl_mode = pdl_mode;
     p.group_m = quad_group_m(M, K, ntok, max_pairs);
     auto kern = sparse_gemm_quad_kernel<kQuadBlockN, kQuadStages>;
@@ -475,16 +548,9 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
         const bool ok2 = a2_mn ? make_tmap(&tmA2, fac2, r, M, 64, 64) : make_tmap(&tmA2, fac2, M, r, kBlockM, 64);
         if (!ok2 || !make_tmap(&tmB2, act2, ntok, r, BLOCK_N, 64)) return SLOPE_ERR_CUDA;
     }
-    if (K > 0) {
-        if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
-        if (!make_tmap(&tmB, act, ntok, K, BLOCK_N, 64)) return SLOPE_ERR_CUDA;
-        if (!make_tmap_meta(&tmE, meta, static_cast<size_t>(M) * K / 8)) return SLOPE_ERR_CUDA;
-    } else {                                  // dense-only: the sparse maps are never used for a load
-        if (r <= 0) return SLOPE_ERR_SHAPE;
-        tmA = tmA2;
-        tmB = tmB2;
-        tmE = tmA2;
-    }
+    if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
+    if (!make_tmap(&tmB, act, ntok, K, BLOCK_N, 64)) return SLOPE_ERR_CUDA;
+    if (!make_tmap_meta(&tmE, meta, static_cast<size_t>(M) * K / 8)) return SLOPE_ERR_CUDA;
     if (r <= 0) {
         tmA2 = tmA;
         tmB2 = tmB;
@@ -500,35 +566,30 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
     int cap[9];
     if (!skinny_capacity<BLOCK_N, A_STAGES, B_STAGES>(info, cap)) return SLOPE_ERR_CUDA;
     if (pdl_mode == 2) {
-        // The consumer of a fused pair has to be resident next to its producer (one cluster of up to 8
-        // CTAs per 128 adapter columns), or its last clusters would wait for the producer to finish
-        // and the overlap would be lost: count only the clusters that fit beside it.
-        const int reserved = 8 * ((r + kBlockM - 1) / kBlockM);
+        // The consumer of a fused pair has to be resident next to its producer, or its last clusters
+        // would wait for the producer to finish and the overlap would be lost: count only the
+        // clusters that fit beside it.
+        const int reserved = adapter_T_ctas(ntok, K, r, info);
         for (int sz = 1; sz <= 8; ++sz) {
             cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
             if (cap[sz] < 0) cap[sz] = 0;
         }
         if (cap[1] <= 0) return SLOPE_ERR_CUDA;
     }
-    const int slabs = (M + kBlockM - 1) / kBlockM, num_kb = K > 0 ? K / 128 : (r + 63) / 64;
+    const int slabs = M / kBlockM, num_kb = K / 128;
     const int splits = skinny_splits(slabs, num_kb, BLOCK_N, cap);
     return launch_cluster_ex(kern, slabs * splits, splits, kGemmThreads, Cfg::kSmemBytes, true, stream, tmA, tmB,
                              tmE, tmA2, tmB2, p);
 }
 
-// Few-token GEMM  out[ntok x M] = act * A_2:4^T (+ act2 * fac2^T)  on the weight-streaming
-// kernel, token tile chosen by the token count.  K == 0 runs the dense product alone
-// (out = act2 * fac2^T with reduction length r), which serves the adapter's T = X L and
-// dT = dY R^T at inference sizes.
-constexpr int kSkinnyMaxTokens = 256;
-
+// Few-token GEMM  out[ntok x M] = act * A_2:4^T (+ act2 * fac2^T)  on the weight-streaming kernel,
+// token tile chosen by the token count (at most 128).
 // A variant of the few-token kernel with a half as deep weight ring fits two CTAs on an SM (the
 // same bytes in flight per SM).  It pays when the slabs times K-slices of a launch exceed what the
 // machine holds at one CTA per SM (stacked projections, d_out beyond ~19000 rows): one wave
 // instead of two.  Decided by the same cost model over both variants' capacities.
 template <int BLOCK_N, int A_DEEP, int B_DEEP, int A_FLAT, int B_FLAT>
 static bool prefer_two_ctas_per_sm(int M, int K, const DeviceInfo& info) {
-    if (K <= 0) return false;
     int cap_deep[9], cap_flat[9];
     if (!skinny_capacity<BLOCK_N, A_DEEP, B_DEEP>(info, cap_deep)) return false;
     if (!skinny_capacity<BLOCK_N, A_FLAT, B_FLAT>(info, cap_flat)) return false;
@@ -549,9 +610,7 @@ static slope_status_t launch_skinny(const void* act, int ntok, const void* vals,
     }
     if (ntok <= 64)      // (a two-per-SM variant of this tile, <64, 4, 2>, measured slower: its activation ring is too shallow)
         return launch_sparse_skinny<64, 8, 4>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
-    if (ntok <= 128)
-        return launch_sparse_skinny<128, 7, 3>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
-    return launch_sparse_skinny<256, 5, 2>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
+    return launch_sparse_skinny<128, 7, 3>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
 }
 
 // Kernel choice for the sparse GEMMs.  Up to 256 tokens the GEMM is a weight stream from HBM and
@@ -625,23 +684,19 @@ static bool use_few_token_kernel(int M, int K, int ntok, int r, const DeviceInfo
     return few_us <= tile_us;
 }
 
-// One of the three tile kernels.  As the consumer of a fused pair of launches (pdl_mode 2) it leaves
-// `reserved_ctas` SMs to the producer that runs beside it.
+// One of the three tile kernels.
 static slope_status_t launch_sparse_tiles(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                                           const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                          cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0,
-                                          int reserved_ctas = 0) {
-    switch (choose_sparse_tile(M, K, ntok, (info.sm_count - reserved_ctas) / 2)) {
+                                          cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    switch (choose_sparse_tile(M, K, ntok, info.sm_count / 2)) {
         case SparseTile::kQuad224:
-            return launch_sparse_quad(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode,
-                                      reserved_ctas);
+            return launch_sparse_quad(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
         case SparseTile::kPair128:
             return launch_sparse_pair<kPairNarrowBlockN, kPairNarrowStages>(act, ntok, vals, meta, M, K, act2, fac2, r,
-                                                                            a2_mn, out, stream, info, pdl_mode,
-                                                                            reserved_ctas);
+                                                                            a2_mn, out, stream, info, pdl_mode);
         default:
             return launch_sparse_pair<kPairBlockN, kPairStages>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out,
-                                                                stream, info, pdl_mode, reserved_ctas);
+                                                                stream, info, pdl_mode);
     }
 }
 
@@ -662,7 +717,7 @@ static slope_status_t launch_dense_pair(const void* A, const void* B, int M, int
     const bool okB = B_MN ? make_tmap(&tmB, B, K, N, 64, 64) : make_tmap(&tmB, B, N, K, Cfg::kHalfN, 64);
     if (!okA || !okB) return SLOPE_ERR_CUDA;
     DenseGemmParams p = {};
-    p.M = M; p.N = N; p.K = K; p.k_splits = 1; p.out = out;
+    p.M = M; p.N = N; p.K = K; p.out = out;
     p.mask = static_cast<const uint8_t*>(mask);
     auto kern = dense_gemm_pair_kernel<A_MN, B_MN, BLOCK_N, EPI, STAGES>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
@@ -813,8 +868,6 @@ slope_status_t slope_linear_fwd(const void* X, int b, const void* Wc_vals, const
                               static_cast<cudaStream_t>(stream), info);
 }
 
-static bool adapter_narrow_tiles(int b, int r, const DeviceInfo& info);
-
 slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_vals, const void* Wc_meta, int d_out,
                                         int d_in, const void* L, const void* R, int r, void* T, void* Y,
                                         void* stream_) {
@@ -830,42 +883,12 @@ slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_val
         // Two launches of the few-token kernel as a fused pair: T = X L releases its dependent only
         // once everything before it in the stream is complete, so the forward streams its weights
         // and runs its sparse reduction while T is still being computed, and waits only for T.
-        if (slope_status_t st = launch_skinny(nullptr, b, nullptr, nullptr, r, 0, X, L, d_in, true, T, stream, info, 1))
-            return st;
+        if (slope_status_t st = launch_adapter_T(X, L, b, d_in, r, T, stream, info, 1)) return st;
         return launch_skinny(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, true, Y, stream, info, 2);
     }
-    // More tokens: the tile kernels are the consumer of such a pair in the same way, as long as the
-    // T launch is small enough to run beside them (it then costs the forward that share of the
-    // machine, which pays while T takes a comparable time: up to 32 CTAs, i.e. 4096 tokens at r <= 128).
-    const bool t_few = b <= kSkinnyMaxTokens;
-    const bool t_narrow = adapter_narrow_tiles(b, r, info);
-    const int t_ctas = t_few ? 8 * ((r + kBlockM - 1) / kBlockM)
-                             : ((b + kBlockM - 1) / kBlockM) * (t_narrow ? (r + 63) / 64 : (r + 127) / 128);
-    const int reserved = (t_ctas + 1) & ~1;
-    // Worth it?  Side by side the forward runs on fewer CTA pairs (more waves of tiles, perhaps)
-    // but no longer waits for T; one after the other it has the whole machine.  Tile time and T
-    // time from the measured constants: ~0.33 us per 128-wide k-block and tile + ~1.5 us of
-    // epilogue; a T CTA walks d_in in 64-wide steps of ~0.3 us after ~6 us of launch and start-up.
-    int mode = 0;
-    if (reserved <= info.sm_count / 3) {
-        double cost_full = 0.0, cost_beside = 0.0;
-        choose_sparse_tile(d_out, d_in, b, info.sm_count / 2, &cost_full);
-        choose_sparse_tile(d_out, d_in, b, (info.sm_count - reserved) / 2, &cost_beside);
-        const double tile_us = d_in / 128 * 0.33 + 1.5;
-        const double t_us = t_few ? 5.0 : 6.0 + d_in / 64 * 0.3;
-        const double fwd_beside = cost_beside * tile_us + 2.0;
-        if (1.15 * (fwd_beside > t_us ? fwd_beside : t_us + 2.0) < t_us + cost_full * tile_us) mode = 1;
-    }
-    slope_status_t st;
-    if (t_few)
-        st = launch_skinny(nullptr, b, nullptr, nullptr, r, 0, X, L, d_in, true, T, stream, info, mode);
-    else
-        st = t_narrow ? launch_dense<false, true, 64, kEpiStore, 9>(X, L, b, r, d_in, 1, T, nullptr, stream, info, mode)
-                      : launch_dense<false, true, 128, kEpiStore, 6>(X, L, b, r, d_in, 1, T, nullptr, stream, info, mode);
-    if (st) return st;
-    if (mode == 1)
-        return launch_sparse_tiles(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, /*a2_mn=*/true, Y, stream, info, 2, reserved);
-    return launch_sparse_gemm(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, /*a2_mn=*/true, Y, stream, info);
+    // More tokens: the tile kernels are the consumer of such a pair in the same way.
+    if (slope_status_t st = launch_adapter_T(X, L, b, d_in, r, T, stream, info, 1)) return st;
+    return launch_sparse_tiles(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, /*a2_mn=*/true, Y, stream, info, 2);
 }
 
 slope_status_t slope_linear_bwd_dx(const void* dY, int b, const void* WTc_vals, const void* WTc_meta, int d_out,
@@ -898,8 +921,7 @@ slope_status_t slope_linear_bwd_dw_masked(const void* dY, const void* X, int b, 
         if (narrow_tiles >= 24)
             return launch_dense_pair<true, true, 128, kEpiMasked, 8>(dY, X, d_out, d_in, b, dWc_vals, mask1_bits,
                                                                      static_cast<cudaStream_t>(stream), info);
-        return launch_dense<true, true, 128, kEpiMasked, 6>(dY, X, d_out, d_in, b, 1, dWc_vals, mask1_bits,
-                                                            static_cast<cudaStream_t>(stream), info);
+        return launch_dense_masked(dY, X, d_out, d_in, b, dWc_vals, mask1_bits, static_cast<cudaStream_t>(stream));
     }
     return launch_dense_pair<true, true, 256, kEpiMasked, 6>(dY, X, d_out, d_in, b, dWc_vals, mask1_bits,
                                                              static_cast<cudaStream_t>(stream), info);
@@ -951,46 +973,6 @@ size_t slope_adapter_workspace_bytes(int b, int d_out, int d_in, int r) {
     return adapter_partial_bytes(b, d_in, r) + adapter_partial_bytes(b, d_out, r);     // dL and dR partial sums
 }
 
-// Column tile of the adapter products T = X L and dT = dY R^T (128 token rows per CTA).  These
-// launches are bound by what one SM can pull in, so more CTAs beat fewer bytes per CTA: with
-// r > 64, 64-column tiles double the CTA count (the second read of the activation rows comes from
-// L2) and win as long as all of them still run in one wave.
-static bool adapter_narrow_tiles(int b, int r, const DeviceInfo& info) {
-    if (r <= 64) return true;
-    const int wide_tiles = ((b + kBlockM - 1) / kBlockM) * ((r + 127) / 128);
-    return 2 * wide_tiles <= info.sm_count;
-}
-
-// dT[b x r] = dY[b x d_out] * R[r x d_out]^T   (both K contiguous)
-static slope_status_t launch_adapter_dT(const void* dY, const void* R, int b, int d_out, int r, void* dT,
-                                        cudaStream_t stream, const DeviceInfo& info) {
-    return b <= kSkinnyMaxTokens
-               ? launch_skinny(nullptr, b, nullptr, nullptr, r, 0, dY, R, d_out, false, dT, stream, info)
-           : adapter_narrow_tiles(b, r, info)
-               ? launch_dense<false, false, 64, kEpiStore, 9>(dY, R, b, r, d_out, 1, dT, nullptr, stream, info)
-               : launch_dense<false, false, 128, kEpiStore, 6>(dY, R, b, r, d_out, 1, dT, nullptr, stream, info);
-}
-
-// dL[d_in x r] = X^T dT and dR^T[d_out x r] = dY^T T: operands stored [K x M] / [K x N] with
-// K = tokens, split into fixed slices; both problems share one launch, their fp32 partial
-// sums are reduced in slice order by one more launch (dR written transposed).
-static slope_status_t launch_adapter_grads(const void* X, const void* dY, const void* T, const void* dT, int b,
-                                           int d_out, int d_in, int r, void* dL, void* dR, void* workspace,
-                                           cudaStream_t stream, const DeviceInfo& info) {
-    float* ws_l = static_cast<float*>(workspace);
-    float* ws_r = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + adapter_partial_bytes(b, d_in, r));
-    DenseProblem ql, qr;
-    ql.A = X; ql.B = dT; ql.M = d_in; ql.N = r; ql.K = b; ql.k_splits = adapter_splits(b, d_in); ql.out = ws_l;
-    qr.A = dY; qr.B = T; qr.M = d_out; qr.N = r; qr.K = b; qr.k_splits = adapter_splits(b, d_out); qr.out = ws_r;
-    slope_status_t st = r <= 64 ? launch_dense2<true, true, 64, kEpiPartial, 6>(ql, qr, stream, info)
-                                : launch_dense2<true, true, 128, kEpiPartial, 6>(ql, qr, stream, info);
-    if (st) return st;
-    const SplitKReduce rl{ws_l, static_cast<uint16_t*>(dL), d_in, r, ql.k_splits, 0};
-    const SplitKReduce rr{ws_r, static_cast<uint16_t*>(dR), d_out, r, qr.k_splits, 1};
-    splitk_reduce_kernel<<<info.sm_count * 4, 256, 0, stream>>>(rl, rr);
-    return launch_result();
-}
-
 slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, const void* L, const void* R, int b,
                                      int d_out, int d_in, int r, void* T, void* dT, void* dL, void* dR,
                                      void* workspace, size_t workspace_bytes, void* stream_) {
@@ -1002,12 +984,7 @@ slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, c
         if (!X || !L || !T) return SLOPE_ERR_INVALID_ARG;
         if (!aligned16(X) || !aligned16(L) || !aligned16(T)) return SLOPE_ERR_ALIGNMENT;
         if (slope_status_t st = check_arch(info)) return st;
-        // T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
-        if (b <= kSkinnyMaxTokens)            // few tokens: split d_in over a cluster instead of one CTA
-            return launch_skinny(nullptr, b, nullptr, nullptr, r, 0, X, L, d_in, true, T, stream, info);
-        return adapter_narrow_tiles(b, r, info)
-                   ? launch_dense<false, true, 64, kEpiStore, 9>(X, L, b, r, d_in, 1, T, nullptr, stream, info)
-                   : launch_dense<false, true, 128, kEpiStore, 6>(X, L, b, r, d_in, 1, T, nullptr, stream, info);
+        return launch_adapter_T(X, L, b, d_in, r, T, stream, info);
     }
     if (phase == 2) {
         if (!dY || !R || !dT) return SLOPE_ERR_INVALID_ARG;
@@ -1021,8 +998,9 @@ slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, c
         return SLOPE_ERR_ALIGNMENT;
     if (workspace_bytes < slope_adapter_workspace_bytes(b, d_out, d_in, r)) return SLOPE_ERR_INVALID_ARG;
     if (slope_status_t st = check_arch(info)) return st;
-    if (slope_status_t st = launch_adapter_dT(dY, R, b, d_out, r, dT, stream, info)) return st;
-    return launch_adapter_grads(X, dY, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info);
+    // dR does not read dT: its CTAs run beside the dT launch, those of dL wait for it
+    if (slope_status_t st = launch_adapter_dT(dY, R, b, d_out, r, dT, stream, info, 1)) return st;
+    return launch_adapter<true, true>(adapter_dR(dY, T, d_out, dR), adapter_dL(X, dT, d_in, dL), r, b, stream, info, 2);
 }
 
 // ------------------------------------------------------------------ masked dW with dL, dR riding along
@@ -1088,9 +1066,11 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     if (slope_status_t st = check_arch(info)) return st;
     const DwAdapterPlan plan = dw_adapter_plan(b, d_out, d_in, r, info.sm_count);
     if (!plan.fused || info.sm_count != 148) {
-        // the separate launches: masked dW, then the dL / dR partial products and their reduction
+        // the separate launches: masked dW, dR, dL
         if (slope_status_t st = slope_linear_bwd_dw_masked(dY, X, b, d_out, d_in, mask1_bits, dWc_vals, stream_)) return st;
-        return launch_adapter_grads(X, dY, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info);
+        if (slope_status_t st = launch_adapter<true, true>(adapter_dR(dY, T, d_out, dR), AdapterOperands{}, r, b, stream, info))
+            return st;
+        return launch_adapter<true, true>(adapter_dL(X, dT, d_in, dL), AdapterOperands{}, r, b, stream, info);
     }
     using Cfg = DwAdapterCfg<6>;
     CUtensorMap tmA, tmB, tmT, tmDT;
@@ -1249,61 +1229,24 @@ slope_status_t slope_meta_to_canonical(const void* meta_hw, int rows, int cols, 
 }  // extern "C"
 
 // ------------------------------------------------------------------ allocation-free adapter-gradient entry
-// Some callers may not allocate device memory at all: a plug-in running inside a host
-// application whose memory pool is closed to it, or code that runs where cudaMalloc is
-// forbidden (a latency-critical section, a process that has handed its whole GPU memory
-// budget to a framework allocator).  For them the split-K scratch of the dL gradient lives
-// in this fixed array instead of a caller workspace.  The array belongs to the loaded
-// library image: every GPU that loads the library keeps these 16 MiB until the process
-// exits, and every call on a device shares it.
-namespace slope {
-constexpr size_t kStaticScratchBytes = size_t(16) << 20;
-static __device__ __align__(256) float g_static_scratch[kStaticScratchBytes / sizeof(float)];
-
-// In host code `g_static_scratch` is only a handle; the address kernels can use comes from
-// cudaGetSymbolAddress, asked once per device with that device current.
-static slope_status_t static_scratch_address(float** out) {
-    static std::mutex mu;
-    static float* cache[64] = {nullptr};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SLOPE_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(mu);
-    if (cache[dev] == nullptr) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || p == nullptr) return SLOPE_ERR_CUDA;
-        cache[dev] = static_cast<float*>(p);
-    }
-    *out = cache[dev];
-    return SLOPE_OK;
-}
-}  // namespace slope
-
+// The adapter kernels reduce inside a cluster, so dL needs neither an allocation nor a workspace.
+// The sizes this call takes are still those whose split-K partial sums would fit 16 MiB, as its
+// contract says.
 extern "C" {
 
-size_t slope_adapter_dl_noalloc_max_scratch_bytes(void) { return kStaticScratchBytes; }
+size_t slope_adapter_dl_noalloc_max_scratch_bytes(void) { return size_t(16) << 20; }
 
 slope_status_t slope_adapter_dl_noalloc(const void* X, const void* dT, int b, int d_in, int r, void* dL,
-                                        void* stream_) {
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+                                        void* stream) {
     if (!X || !dT || !dL) return SLOPE_ERR_INVALID_ARG;
     if (d_in <= 0 || d_in % 128 != 0 || b < 1 || !rank_ok(r) || r == 0) return SLOPE_ERR_SHAPE;
     if (!aligned16(X) || !aligned16(dT) || !aligned16(dL)) return SLOPE_ERR_ALIGNMENT;
-    const int splits = adapter_splits(b, d_in);
-    const size_t need = static_cast<size_t>(splits) * d_in * r * sizeof(float);
-    if (need > kStaticScratchBytes) return SLOPE_ERR_SHAPE;      // beyond the fixed scratch: use the workspace call
+    const size_t need = static_cast<size_t>(adapter_splits(b, d_in)) * d_in * r * sizeof(float);
+    if (need > slope_adapter_dl_noalloc_max_scratch_bytes()) return SLOPE_ERR_SHAPE;
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
-    float* scratch = nullptr;
-    if (slope_status_t st = static_scratch_address(&scratch)) return st;
-    // Nothing has to start at zero: every partial sum the reduction reads is written by the
-    // GEMM of this same call, so what an earlier call left in the array is never observed.
-    slope_status_t st =
-        r <= 64 ? launch_dense<true, true, 64, kEpiPartial, 6>(X, dT, d_in, r, b, splits, scratch, nullptr, stream, info)
-                : launch_dense<true, true, 128, kEpiPartial, 6>(X, dT, d_in, r, b, splits, scratch, nullptr, stream, info);
-    if (st) return st;
-    const SplitKReduce red{scratch, static_cast<uint16_t*>(dL), d_in, r, splits, 0};
-    splitk_reduce_kernel<<<info.sm_count * 4, 256, 0, stream>>>(red, SplitKReduce{nullptr, nullptr, 0, 0, 0, 0});
-    return launch_result();
+    return launch_adapter<true, true>(adapter_dL(X, dT, d_in, dL), AdapterOperands{}, r, b,
+                                      static_cast<cudaStream_t>(stream), info);
 }
 
 }  // extern "C"

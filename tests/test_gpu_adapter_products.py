@@ -1,0 +1,49 @@
+"""The adapter's low-rank products at the edges of their kernel: every column tile (64, 128, 256), every
+reduction split (1, 2, 4, 8), one and two CTAs per SM, ragged last tiles and k-blocks.
+
+The reference is the fp64 product of the same bf16 operands (dL is checked from the dT the call wrote), so
+an output is rounded once: 2^-9 / sqrt(3) ~ 1.7e-3 relative on Gaussian data, 5e-3 allowed, and
+parity_error's bound per element."""
+import pytest
+
+from paper_2608_24070_b200 import inputs as si
+from helpers import REL_TOL, parity_error, to_f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [
+    (1, 128, 128, 16),           # one token, two k-blocks of T, one of dL: no split
+    (63, 256, 384, 16),          # four k-blocks: a split of two
+    (130, 4096, 1152, 64),       # ragged second row tile, split of eight
+    (257, 128, 2176, 48),        # ragged k-block in dL / dR, columns past r in the 64-wide tile
+    (1000, 768, 2304, 256),      # widest rank on few tiles: four column tiles
+    (1100, 640, 256, 176),       # rank between the column tiles
+    (4096, 1024, 512, 128),      # 128-wide tiles
+    (9500, 512, 640, 256),       # 75 row tiles: 256-wide tiles
+    (19100, 128, 256, 80),       # more row tiles than SMs: two CTAs per SM
+    (40000, 128, 128, 16),       # several waves; 625 k-blocks for one row tile of dL
+])
+def test_adapter_products_match_fp64(b, d_in, d_out, r):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    bits = {"X": si.gaussian_bf16((b, d_in), 1.0, 31), "dY": si.gaussian_bf16((b, d_out), 1.0, 32),
+            "L": si.gaussian_bf16((d_in, r), 0.01, 33), "R": si.gaussian_bf16((r, d_out), 0.01, 34)}
+    X, dY, L, R = (B.bf16_from_bits(bits[k]) for k in ("X", "dY", "L", "R"))
+    f = {k: to_f64(v) for k, v in bits.items()}
+    nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    T, dT2 = nan(b + 1, r), nan(b + 1, r)                       # a spare row each: nothing may be written behind the last token
+    B.slope_adapter_fwd_bwd(0, X, None, L, None, b, d_out, d_in, r, T=T[:b])
+    B.slope_adapter_fwd_bwd(2, None, dY, None, R, b, d_out, d_in, r, dT=dT2[:b])
+    dT, dL, dR = nan(b, r), nan(d_in, r), nan(r, d_out)
+    ws = torch.empty(B.slope_adapter_workspace_bytes(b, d_out, d_in, r), dtype=torch.uint8, device="cuda")
+    B.slope_adapter_fwd_bwd(1, X, dY, L, R, b, d_out, d_in, r, T=T[:b], dT=dT, dL=dL, dR=dR, workspace=ws)
+    assert B.slope_poll_status() == 0
+    assert torch.isnan(T[b]).all() and torch.isnan(dT2[b]).all()
+    assert torch.equal(dT.view(torch.int16), dT2[:b].view(torch.int16))
+    g = lambda t: to_f64(B.bits_from_bf16(t))
+    errs = {"T": parity_error(g(T[:b]), f["X"] @ f["L"]), "dT": parity_error(g(dT), f["dY"] @ f["R"].T),
+            "dL": parity_error(g(dL), f["X"].T @ g(dT)), "dR": parity_error(g(dR), g(T[:b]).T @ f["dY"])}
+    assert all(v <= REL_TOL for v in errs.values()), errs
