@@ -83,16 +83,46 @@ __device__ __forceinline__ uint4 compress_16(const uint32_t (&v)[16], uint32_t m
     uint32_t w[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-        const uint32_t mb = (mbits >> (4 * g)) & 0xFu;
-        // kept positions in ascending order: lowest set bit, highest set bit
-        const int p0 = __ffs(mb) - 1, p1 = 31 - __clz(mb);
-        const float e0 = __uint_as_float(v[4 * g]), e1 = __uint_as_float(v[4 * g + 1]),
-                    e2 = __uint_as_float(v[4 * g + 2]), e3 = __uint_as_float(v[4 * g + 3]);
-        const float lo = p0 == 0 ? e0 : (p0 == 1 ? e1 : e2);
-        const float hi = p1 == 1 ? e1 : (p1 == 2 ? e2 : e3);
-        w[g] = pack_bf16x2(lo, hi);
+        // two of the four bits are set: the lower one is bit 0, 1 or 2, the higher one bit 3, 2 or 1
+        const uint32_t e0 = v[4 * g], e1 = v[4 * g + 1], e2 = v[4 * g + 2], e3 = v[4 * g + 3];
+        const uint32_t lo = mbits & (1u << (4 * g)) ? e0 : (mbits & (2u << (4 * g)) ? e1 : e2);
+        const uint32_t hi = mbits & (8u << (4 * g)) ? e3 : (mbits & (4u << (4 * g)) ? e2 : e1);
+        w[g] = pack_bf16x2(__uint_as_float(lo), __uint_as_float(hi));
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Epilogue warps of the dense kernels: two per tensor-memory lane quadrant, each takes half of a tile's columns.
+constexpr int kDenseEpiWarps = 8;
+constexpr int kDenseThreads = 64 + 32 * kDenseEpiWarps;
+
+// A row's mask bits of `cols` (64 or 128) columns, fetched before the accumulator is ready: loaded where they are
+// used, 16 columns at a time, every load put an L2 round trip into the drain.
+__device__ __forceinline__ uint4 load_mask_bits(const uint8_t* row, int cols) {
+    if (cols == 128) return __ldg(reinterpret_cast<const uint4*>(row));
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(row));
+    return make_uint4(v.x, v.y, 0u, 0u);
+}
+
+// Drains `cols` (64 or 128) accumulator columns of this thread's row, 64 at a time, so that the tensor-memory loads
+// share one wait.  With few tokens the drain, not the main loop, paces the kernel (double-buffered
+// accumulators): four warps that took 16 columns at a time, a mask load and a wait each, needed ~9 us
+// for a 256 x 256 tile; as it is, 4096 x 4096 with 300 tokens went from 43 to 13 us, 8320 -> 6400 with
+// 740 from 141 to 58, 512 x 512 with 256 from 7.8 to 3.0 (16384 tokens: unchanged).
+__device__ __forceinline__ void drain_masked(uint32_t t_row, int cols, const uint4& bits, uint16_t* dst) {
+    const uint32_t mw[4] = {bits.x, bits.y, bits.z, bits.w};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (64 * i < cols) {
+            uint32_t v[4][16];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tmem_ld_16(t_row + 64 * i + 16 * k, v[k]);
+            tmem_ld_wait();
+            uint4* d = reinterpret_cast<uint4*>(dst + 32 * i);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = compress_16(v[k], mw[2 * i + (k >> 1)] >> (16 * (k & 1)));
+        }
+    }
 }
 
 // Masked weight gradient of the smallest weight matrices: one 128 x 128 tile per CTA.
@@ -106,7 +136,7 @@ struct DenseCfg {
 };
 
 template <int STAGES>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const DenseGemmParams p) {
     // A = dY and B = X, both stored [K x .]; M and N are multiples of 128; one tile per CTA
@@ -130,6 +160,10 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         *abort_flag = 0;
         fence_mbar_init();
     }
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
     if (warp == 1) {
         tmem_alloc(tmem_slot, kBlockN);
         tmem_relinquish();
@@ -145,8 +179,6 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
     if (warp == 0) {
         if (elect_one()) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
             PipeState ps;
             for (int kb = 0; kb < num_kb; ++kb) {
                 if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) break;
@@ -182,22 +214,13 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (ok) umma_commit(tfull_bar);
         }
     } else {
-        const int q = warp & 3;
-        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-        const int m = m_blk * kBlockM + q * 32 + lane;
+        const int q = warp & 3, c0 = ((warp - 2) >> 2) * (kBlockN / 2);
+        const int m = m_blk * kBlockM + q * 32 + lane, n0 = n_blk * kBlockN + c0;
+        const uint4 bits = load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), kBlockN / 2);
         if (mbar_wait(tfull_bar, 0u, abort_flag)) {
             tc_fence_after_sync();
-#pragma unroll 1
-            for (int c0 = 0; c0 < kBlockN; c0 += 16) {
-                uint32_t v[16];
-                tmem_ld_16(t_row + c0, v);
-                tmem_ld_wait();
-                const int n0 = n_blk * kBlockN + c0;
-                const uint32_t mbits =
-                    *reinterpret_cast<const uint16_t*>(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3));
-                *reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) +
-                                          (n0 >> 1)) = compress_16(v, mbits);
-            }
+            drain_masked(tmem_base + c0 + (static_cast<uint32_t>(q * 32) << 16), kBlockN / 2, bits,
+                         static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1));
         }
     }
 
@@ -335,6 +358,11 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         *abort_flag = 0;
         fence_mbar_init();
     }
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+        tma_prefetch_desc(&tmE);
+    }
     if (warp == 1) {
         tmem_alloc_pair(tmem_slot, 512);
         tmem_relinquish_pair();
@@ -354,9 +382,6 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
         if (elect_one()) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
-            tma_prefetch_desc(&tmE);
             const uint64_t keep = l2_policy_evict_last();
             PipeState ps;
             bool ok = true;
@@ -572,7 +597,7 @@ struct DensePairCfg {
 };
 
 template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const DenseGemmParams p) {
     using Cfg = DensePairCfg<BLOCK_N, STAGES>;
@@ -597,9 +622,13 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 8); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 2 * kDenseEpiWarps); }
         *abort_flag = 0;
         fence_mbar_init();
+    }
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
     }
     if (warp == 1) {
         tmem_alloc_pair(tmem_slot, kTmemCols);
@@ -617,8 +646,6 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 
     if (warp == 0) {
         if (elect_one()) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
             PipeState ps;
             bool ok = true;
             PairWork w;
@@ -690,38 +717,44 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             if (pair_id == 0) probe.end(kClockDense);
         }
     } else {
-        const int q = warp & 3;
+        const int q = warp & 3, half = (warp - 2) >> 2;
         bool ok = true;
         int it = 0;
         PairWork w;
         for (int item = pair_id; ok && pair_work<BLOCK_N, kSplitTail>(item, num_pairs, num_m, num_n, w);
              item += num_pairs, ++it) {
-            const int m_pair = w.m_pair;
             const int acc = it & 1;
             const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
+            const int m = (w.m_pair * 2 + static_cast<int>(cta)) * kBlockM + q * 32 + lane;
+            const int cols = w.width / 2, n0 = w.n0 + half * cols;
+            const bool live = m < p.M && n0 < p.N;           // (kEpiMasked: the same for all rows of a CTA)
+            uint4 bits = make_uint4(0u, 0u, 0u, 0u);
+            if (EPI == kEpiMasked && live)
+                bits = load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), cols);
             if (!mbar_wait(&tfull_bar[acc], acc_phase, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
-            const uint32_t t_row = tmem_base + acc * BLOCK_N + (static_cast<uint32_t>(q * 32) << 16);
-            const int m = (m_pair * 2 + static_cast<int>(cta)) * kBlockM + q * 32 + lane;
+            const uint32_t t_row = tmem_base + acc * BLOCK_N + half * cols + (static_cast<uint32_t>(q * 32) << 16);
+            if (EPI == kEpiMasked) {
+                if (live)
+                    drain_masked(t_row, cols, bits, static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1));
+            } else if (n0 < p.N) {
+                uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.N + n0);
 #pragma unroll 1
-            for (int c0 = 0; c0 < w.width; c0 += 16) {
-                uint32_t v[16];
-                tmem_ld_16(t_row + c0, v);
-                tmem_ld_wait();
-                const int n0 = w.n0 + c0;
-                if (m >= p.M || n0 >= p.N) continue;
-                if (EPI == kEpiStore) {
-                    uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.N + n0);
-                    uint32_t w[8];
+                for (int c0 = 0; c0 < cols; c0 += 64) {
+                    uint32_t v[4][16];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) w[c] = pack_bf16x2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
-                    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-                } else {
-                    const uint32_t mbits =
-                        *reinterpret_cast<const uint16_t*>(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3));
-                    *reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1)) =
-                        compress_16(v, mbits);
+                    for (int k = 0; k < 4; ++k) tmem_ld_16(t_row + c0 + 16 * k, v[k]);
+                    tmem_ld_wait();
+                    if (live) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const uint32_t* e = v[k >> 1] + 8 * (k & 1);
+                            dst[c0 / 8 + k] = make_uint4(pack_bf16x2(__uint_as_float(e[0]), __uint_as_float(e[1])),
+                                                         pack_bf16x2(__uint_as_float(e[2]), __uint_as_float(e[3])),
+                                                         pack_bf16x2(__uint_as_float(e[4]), __uint_as_float(e[5])),
+                                                         pack_bf16x2(__uint_as_float(e[6]), __uint_as_float(e[7])));
+                        }
+                    }
                 }
             }
             tc_fence_before_sync();
@@ -830,6 +863,11 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         *abort_flag = 0;
         fence_mbar_init();
     }
+    if (warp == 0 && elect_one()) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+        tma_prefetch_desc(&tmE);
+    }
     if (warp == 1) {
         tmem_alloc_pair(tmem_slot, 512);
         tmem_relinquish_pair();
@@ -849,9 +887,6 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
         if (elect_one()) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
-            tma_prefetch_desc(&tmE);
             const uint64_t keep = l2_policy_evict_last();
             PipeState ps;
             bool ok = true;

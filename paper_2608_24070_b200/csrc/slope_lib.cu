@@ -268,7 +268,7 @@ static slope_status_t launch_dense_masked(const void* dY, const void* X, int M, 
     const DenseGemmParams p{M, N, K, out, static_cast<const uint8_t*>(mask)};
     auto kern = dense_gemm_kernel<kStages>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    return launch_cluster_ex(kern, (M / kBlockM) * (N / Cfg::kBlockN), 1, kGemmThreads, Cfg::kSmemBytes,
+    return launch_cluster_ex(kern, (M / kBlockM) * (N / Cfg::kBlockN), 1, kDenseThreads, Cfg::kSmemBytes,
                              /*overlap_prologue=*/true, stream, tmA, tmB, p);
 }
 
@@ -724,7 +724,7 @@ static slope_status_t launch_dense_pair(const void* A, const void* B, int M, int
     const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + BLOCK_N - 1) / BLOCK_N);
     const int max_pairs = info.sm_count / 2;
     const int pairs = tiles < max_pairs ? tiles : max_pairs;
-    return launch_pairs(kern, 2 * pairs, kGemmThreads, Cfg::kSmemBytes, stream, tmA, tmB, p);
+    return launch_pairs(kern, 2 * pairs, kDenseThreads, Cfg::kSmemBytes, stream, tmA, tmB, p);
 }
 
 static int adapter_splits(int b, int rows) {

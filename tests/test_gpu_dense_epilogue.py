@@ -1,0 +1,60 @@
+"""Weight-gradient and dense GEMM epilogues at the edges of their tiles: every tile width (128 x 128 of one CTA,
+256 x 128 and 256 x 256 of a pair, halved items of the last wave), last tiles that are half empty in either
+dimension, few tokens (one k-block, a ragged one).
+
+The reference is the fp64 product of the same bf16 operands; outputs are rounded once (2^-9 / sqrt(3) ~ 1.7e-3
+relative on Gaussian data, 5e-3 allowed, and parity_error's bound per element)."""
+import pytest
+
+from paper_2608_24070_b200 import inputs as si
+from helpers import REL_TOL, parity_error, to_f64
+
+pytestmark = pytest.mark.gpu
+
+
+def _operands(b, d_in, d_out):
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    bits = [si.gaussian_bf16((b, d_in), 1.0, 41), si.gaussian_bf16((b, d_out), 1.0, 42),
+            si.gaussian_bf16((d_out, d_in), 0.02, 43)]
+    return B, [B.bf16_from_bits(x) for x in bits], [to_f64(x) for x in bits]
+
+
+@pytest.mark.parametrize("b,d_in,d_out", [
+    (1, 128, 128),               # one 128 x 128 tile, one token
+    (65, 384, 640),              # one-CTA tiles, a k-block and one token
+    (200, 1152, 1920),           # 256 x 128 tiles of pairs, last row tile half empty
+    (70, 2176, 2432),            # 256 x 256 tiles, half empty in both dimensions
+    (90, 4096, 4096),            # 256 tiles: the last wave's are halved
+])
+def test_masked_weight_gradient(b, d_in, d_out):
+    import numpy as np
+    import torch
+
+    B, (X, dY, W), (fX, fdY, _) = _operands(b, d_in, d_out)
+    vals, meta, mask = B.alloc_compressed(d_out, d_in)
+    B.slope_prune_24(W, vals, meta, mask)
+    dWc = torch.full((d_out, d_in // 2), float("nan"), dtype=torch.bfloat16, device="cuda")
+    B.slope_linear_bwd_dw_masked(dY, X, mask, dWc)
+    assert B.slope_poll_status() == 0
+    kept = np.unpackbits(mask.cpu().numpy(), axis=1, bitorder="little").astype(bool)
+    ref = (fdY.T @ fX)[kept].reshape(d_out, d_in // 2)
+    assert parity_error(to_f64(B.bits_from_bf16(dWc)), ref) <= REL_TOL
+
+
+@pytest.mark.parametrize("b,d_in,d_out", [(1, 128, 128), (130, 256, 384), (300, 1152, 640), (513, 384, 2176)])
+def test_dense_layer(b, d_in, d_out):
+    import torch
+
+    B, (X, dY, W), (fX, fdY, fW) = _operands(b, d_in, d_out)
+    nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    Y, dX, dW = nan(b + 1, d_out), nan(b + 1, d_in), nan(d_out, d_in)       # a spare row: nothing behind the last token
+    B.slope_dense_linear_fwd(X, W, Y[:b])
+    B.slope_dense_linear_bwd_dx(dY, W, dX[:b])
+    B.slope_dense_linear_bwd_dw(dY, X, dW)
+    assert B.slope_poll_status() == 0
+    assert torch.isnan(Y[b]).all() and torch.isnan(dX[b]).all()
+    g = lambda t: to_f64(B.bits_from_bf16(t))
+    for got, ref in ((Y[:b], fX @ fW.T), (dX[:b], fdY @ fW), (dW, fdY.T @ fX)):
+        assert parity_error(g(got), ref) <= REL_TOL
