@@ -9,10 +9,10 @@
 //   dense_gemm_kernel          1 CTA per 128 x 128 tile; dW of the smallest weight matrices
 //   dense_gemm_pair_kernel     CTA pair per 256 x 256 tile (cta_group::2), the last wave's tiles
 //                              halved; dW (masked epilogue) and the dense layer (store epilogue)
-//   sparse_gemm_pair_kernel    CTA pair per 256 x 224 (or 256 x 128) tile, tcgen05.mma.sp;
+//   sparse_gemm_pair_kernel    CTA pair per tile of 256 rows x 32 ... 224 tokens, tcgen05.mma.sp;
 //                              forward / dX with short reductions or few tiles
-//   sparse_gemm_quad_kernel    CTA pair per 512 x 224 tile (two MMA sub-tiles per activation
-//                              tile); forward / dX with long reductions
+//   sparse_gemm_quad_kernel    CTA pair per tile of 512 rows x 32 ... 224 tokens (two MMA sub-tiles per
+//                              activation tile); forward / dX with long reductions
 //   sparse_gemm_skinny_kernel  one CTA per 128-row weight slab and K-slice, cluster reduction
 //                              through distributed shared memory; forward / dX with few
 //                              tokens (inference, decode), not persistent
@@ -30,6 +30,16 @@ struct PipeState {
     uint32_t phase = 0;
     __device__ __forceinline__ void advance(int nstages) {
         if (++stage == nstages) { stage = 0; phase ^= 1u; }
+    }
+};
+
+// The same with the byte offset of the stage kept along (stage size and count are launch parameters).
+struct RingState {
+    int stage = 0;
+    uint32_t phase = 0, off = 0;
+    __device__ __forceinline__ void advance(int nstages, uint32_t stage_bytes) {
+        off += stage_bytes;
+        if (++stage == nstages) { stage = 0; off = 0; phase ^= 1u; }
     }
 };
 
@@ -54,6 +64,9 @@ __device__ __forceinline__ void drain_after_abort() {
 struct SparseGemmParams {
     int M, K, Ntok, r;
     int a2_mn_major;              // 1: A2 is stored [r x M] (M contiguous)
+    int width;                    // tile kernels: tokens per tile, a multiple of 32, at most kMaxTokenTile
+    int num_n;                    // tile kernels: token tiles
+    int stages;                   // tile kernels: pipeline stages that fit at that width
     int group_m;                  // 512-row-tile kernel: row tiles per raster group (0: all in one group)
     int pdl_mode;                 // 2: consumer of a fused pair of launches (see the few-token kernel)
     const uint8_t* meta;          // metadata blocks of A
@@ -160,7 +173,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         *abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == 0 && elect_one()) {
+    if (warp == 2 && elect_one()) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
@@ -294,49 +307,51 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const SplitKReduce r
 // the barriers of both CTAs; the epilogues release an accumulator stage by arriving on the
 // leader's barrier through the cluster shared-memory window.
 // =====================================================================================
-// Token tiles are BLOCK_N wide except the last one of a ragged token count, which is only as wide
-// as the tokens that are left (rounded up to the 32-token block of the epilogue): the MMAs run
-// with that N, the second CTA's half of the activations starts at its middle, and the epilogue
-// stops there.  A 2048-token forward on 224-token tiles ends in a 32-token tile that costs a
-// fraction of a full one instead of a whole wave of the machine.
-__device__ __forceinline__ int token_tile_width(int ntok, int n0, int block_n) {
+// Tokens per tile of the sparse tile kernels.  The width is chosen per launch (any multiple of 32, the epilogue's
+// block and the step of N for an MMA of 256 rows), so that the tiles of a token count come out equal
+// and fill the waves of the machine; narrower tiles leave room for more pipeline stages.  224 is what
+// tensor memory (two accumulators and the metadata columns) and shared memory (four, or three
+// 512-row, stages) hold.  The last tile is only as wide as the tokens that are left, rounded up to 32:
+// the MMAs run with that N, the second CTA's half starts at its middle, and the epilogue stops there.
+constexpr int kMaxTokenTile = 224;
+__device__ __forceinline__ int token_tile_width(int ntok, int n0, int tile_width) {
     const int left = ntok - n0;
-    return left >= block_n ? block_n : ((left + 31) & ~31);
+    return left >= tile_width ? tile_width : ((left + 31) & ~31);
 }
 
-template <int BLOCK_N, int STAGES>
+constexpr int kMaxTileStages = 8;
 struct SparsePairCfg {
-    static constexpr int kHalfN = BLOCK_N / 2;
     static constexpr int kABytes = kBlockM * 128;
-    static constexpr int kBBytes = kHalfN * 256;
     static constexpr int kEBytes = 2048;
-    static constexpr int kStageBytes = kABytes + kBBytes + kEBytes;
     static constexpr int kStoreRows = 32;                         // tokens per TMA store
     static constexpr int kStoreCols = 32;                         // features per TMA store (one warp's lanes)
     static constexpr int kStoreBytes = kStoreRows * kStoreCols * 2;
     static constexpr int kEpiWarps = 8;                           // two warps per tensor-memory lane quadrant
     static constexpr int kThreads = 64 + 32 * kEpiWarps;
-    static constexpr int kOffStore = STAGES * kStageBytes;
-    static constexpr int kOffBar = kOffStore + kEpiWarps * 2 * kStoreBytes;
-    static constexpr int kSmemBytes = kOffBar + 256 + 1024;
-    static constexpr int kECol = 2 * BLOCK_N;
-    static_assert(BLOCK_N % 32 == 0 && kHalfN % 8 == 0 && 2 * BLOCK_N + 8 <= 512, "tile does not fit tensor memory");
-    static_assert(kStageBytes % 1024 == 0, "stage must keep 1024-byte alignment");
-    static_assert(kSmemBytes <= 232448, "shared memory budget");
+    static constexpr int kStagingBytes = kEpiWarps * 2 * kStoreBytes;
+    static constexpr int kECol = 2 * kMaxTokenTile;
+    __host__ __device__ static constexpr int b_bytes(int width) { return width * 128; }          // per CTA: width / 2 tokens x 128
+    __host__ __device__ static constexpr int stage_bytes(int width) { return kABytes + b_bytes(width) + kEBytes; }
+    __host__ __device__ static constexpr int smem_bytes(int width, int stages) {
+        return stages * stage_bytes(width) + kStagingBytes + 256 + 1024;
+    }
+    static_assert(kMaxTokenTile % 32 == 0 && 2 * kMaxTokenTile + 8 <= 512, "tile does not fit tensor memory");
 };
 
-template <int BLOCK_N, int STAGES>
-__global__ void __launch_bounds__(SparsePairCfg<BLOCK_N, STAGES>::kThreads, 1)
+__global__ void __launch_bounds__(SparsePairCfg::kThreads, 1)
 sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmE, const __grid_constant__ CUtensorMap tmA2,
                         const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmO,
                         const SparseGemmParams p) {
-    using Cfg = SparsePairCfg<BLOCK_N, STAGES>;
+    using Cfg = SparsePairCfg;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBar);
-    uint64_t* empty_bar = full_bar + STAGES;
-    uint64_t* tfull_bar = empty_bar + STAGES;
+    const int stages = p.stages, stage_bytes = Cfg::stage_bytes(p.width);
+    const uint32_t b_half = p.width * 64;                    // bytes of one 64-column half of the activation tile
+    uint8_t* staging = smem + stages * stage_bytes;
+    uint64_t* full_bar = reinterpret_cast<uint64_t*>(staging + Cfg::kStagingBytes);
+    uint64_t* empty_bar = full_bar + kMaxTileStages;
+    uint64_t* tfull_bar = empty_bar + kMaxTileStages;
     uint64_t* tempty_bar = tfull_bar + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty_bar + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -346,19 +361,20 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const int pair_id = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int num_mb = p.M / kBlockM;                        // 128-row blocks of A
     const int num_m = (num_mb + 1) / 2;                      // 256-row pair tiles
-    const int num_n = (p.Ntok + BLOCK_N - 1) / BLOCK_N;
+    const int num_n = p.num_n;
     const int num_tiles = num_m * num_n;
     const int num_kb = p.K / 128;
     const int num_ab = (p.r + 63) / 64;
     const int total_kb = num_kb + num_ab;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+#pragma unroll
+        for (int s = 0; s < kMaxTileStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 2 * Cfg::kEpiWarps); }
         *abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == 0 && elect_one()) {
+    if (warp == 2 && elect_one()) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         tma_prefetch_desc(&tmE);
@@ -383,26 +399,26 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // ------------------------------------------------------------ TMA producer (both CTAs)
         if (elect_one()) {
             const uint64_t keep = l2_policy_evict_last();
-            PipeState ps;
+            RingState ps;
             bool ok = true;
             bool waited = false;
             for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
                 const int m_pair = tile % num_m, n_blk = tile / num_m;
                 const int mb = m_pair * 2 + static_cast<int>(cta);           // this CTA's 128-row block
                 const int mb_e = mb < num_mb ? mb : num_mb - 1;              // rows past M: any valid metadata block
-                const int width = token_tile_width(p.Ntok, n_blk * BLOCK_N, BLOCK_N);
-                const int n_row0 = n_blk * BLOCK_N + static_cast<int>(cta) * (width / 2);
+                const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
+                const int n_row0 = n_blk * p.width + static_cast<int>(cta) * (width / 2);
                 for (int kb = 0; kb < total_kb; ++kb) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
-                    uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
+                    uint8_t* sA = smem + ps.off;
                     uint8_t* sB = sA + Cfg::kABytes;
-                    uint8_t* sE = sB + Cfg::kBBytes;
+                    uint8_t* sE = sB + 2 * b_half;
                     const uint32_t bar = mapa_shared(smem_u32(&full_bar[ps.stage]), 0);
                     if (kb < num_kb) {
-                        if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], 2 * Cfg::kStageBytes);
+                        if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], 2 * stage_bytes);
                         tma_load_2d_pair_hint(sA, &tmA, bar, kb * 64, mb * kBlockM, keep);
                         tma_load_2d_pair(sB, &tmB, bar, kb * 128, n_row0);
-                        tma_load_2d_pair(sB + Cfg::kHalfN * 128, &tmB, bar, kb * 128 + 64, n_row0);
+                        tma_load_2d_pair(sB + b_half, &tmB, bar, kb * 128 + 64, n_row0);
                         tma_load_2d_pair_hint(sE, &tmE, bar, 0, mb_e * num_kb + kb, keep);
                     } else {
                         const int ab = kb - num_kb;
@@ -410,7 +426,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                             griddep_wait();
                             waited = true;
                         }
-                        if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], 2 * (Cfg::kABytes + Cfg::kHalfN * 128));
+                        if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], 2 * (Cfg::kABytes + b_half));
                         if (p.a2_mn_major) {
                             tma_load_2d_pair(sA, &tmA2, bar, mb * kBlockM, ab * 64);
                             tma_load_2d_pair(sA + 8192, &tmA2, bar, mb * kBlockM + 64, ab * 64);
@@ -419,41 +435,43 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         }
                         tma_load_2d_pair(sB, &tmB2, bar, ab * 64, n_row0);
                     }
-                    ps.advance(STAGES);
+                    ps.advance(stages, stage_bytes);
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (leader CTA only)
         if (cta == 0 && elect_one()) {
-            PipeState ps;
+            RingState ps;
             bool ok = true;
             int it = 0;
             ClockProbe probe;
             if (pair_id == 0) probe.begin();
             for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs, ++it) {
-                const int width = token_tile_width(p.Ntok, (tile / num_m) * BLOCK_N, BLOCK_N);
+                const int width = token_tile_width(p.Ntok, (tile / num_m) * p.width, p.width);
                 const uint32_t idesc_sp = make_idesc_bf16(2 * kBlockM, width, false, false, true);
                 const uint32_t idesc_ad = make_idesc_bf16(2 * kBlockM, width, p.a2_mn_major != 0, false, false);
                 const int acc = it & 1;
                 const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
                 if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * BLOCK_N;
+                const uint32_t d_tmem = tmem_base + acc * kMaxTokenTile;
                 for (int kb = 0; kb < total_kb; ++kb) {
                     if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                     tc_fence_after_sync();
-                    const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
+                    const uint32_t sA = smem_u32(smem + ps.off);
                     const uint32_t sB = sA + Cfg::kABytes;
-                    const uint32_t sE = sB + Cfg::kBBytes;
+                    const uint32_t sE = sB + 2 * b_half;
                     if (kb < num_kb) {
                         const uint32_t e_tmem = tmem_base + Cfg::kECol + (kb & 1) * 4;
                         tmem_cp_128x128b_pair(e_tmem, make_smem_desc(sE, 128, 128, kSwizzleNone));
+                        // (a step along K adds to the start address, the descriptor's lowest field, in 16-byte units)
+                        const uint64_t a0 = make_smem_desc(sA, 16, 1024, kSwizzle128B);
+                        const uint64_t b0 = make_smem_desc(sB, 16, 1024, kSwizzle128B);
+                        const uint64_t b2 = b0 + (b_half >> 4);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            const uint64_t ad = make_smem_desc(sA + j * 32, 16, 1024, kSwizzle128B);
-                            const uint64_t bd = make_smem_desc(sB + (j >> 1) * (Cfg::kHalfN * 128) + (j & 1) * 64, 16,
-                                                               1024, kSwizzle128B);
+                            const uint64_t ad = a0 + 2 * j, bd = (j < 2 ? b0 : b2) + 4 * (j & 1);
                             umma_bf16_sp_pair(d_tmem, ad, bd, e_tmem + (j & 2), idesc_sp | (j & 1),
                                               (kb | j) != 0 ? 1u : 0u);
                         }
@@ -468,7 +486,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         }
                     }
                     umma_commit_pair(&empty_bar[ps.stage], 3);
-                    ps.advance(STAGES);
+                    ps.advance(stages, stage_bytes);
                 }
                 if (ok) umma_commit_pair(&tfull_bar[acc], 3);
             }
@@ -485,7 +503,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         const int q = warp & 3;
         const int ew = warp - 2;
         const int half = ew >> 2;
-        uint8_t* my_buf = smem + Cfg::kOffStore + ew * 2 * Cfg::kStoreBytes;
+        uint8_t* my_buf = staging + ew * 2 * Cfg::kStoreBytes;
         const uint64_t stream_out = l2_policy_evict_first();
         bool ok = true;
         int it = 0;
@@ -496,9 +514,9 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
             if (!mbar_wait(&tfull_bar[acc], acc_phase, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
-            const uint32_t t_row = tmem_base + acc * BLOCK_N + (static_cast<uint32_t>(q * 32) << 16);
+            const uint32_t t_row = tmem_base + acc * kMaxTokenTile + (static_cast<uint32_t>(q * 32) << 16);
             const int m0 = (m_pair * 2 + static_cast<int>(cta)) * kBlockM + q * 32;
-            const int width = token_tile_width(p.Ntok, n_blk * BLOCK_N, BLOCK_N);
+            const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
 #pragma unroll 1
             for (int c0 = half * Cfg::kStoreRows; c0 < width; c0 += 2 * Cfg::kStoreRows) {
                 uint32_t v0[16], v1[16];                         // features 0..15 and 16..31 of the quadrant
@@ -523,7 +541,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0 && m0 < p.M) {
-                    tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n_blk * BLOCK_N + c0, stream_out);
+                    tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n_blk * p.width + c0, stream_out);
                     tma_store_commit();
                 }
                 buf ^= 1u;
@@ -626,7 +644,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         *abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == 0 && elect_one()) {
+    if (warp == 2 && elect_one()) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
@@ -779,34 +797,29 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 // ONE staged activation tile, so every activation byte pulled from L2 feeds twice as many
 // MMAs (L2 -> SM bytes per FLOP drop by 31 % against the 256-row tile; that fabric, not DRAM
 // or the tensor pipe, is what bounds these GEMMs).  Tensor memory then holds one accumulator
-// per sub-tile (2 x BLOCK_N columns) plus the metadata columns, so accumulators are single
+// per sub-tile (2 x 224 columns) plus the metadata columns, so accumulators are single
 // buffered; the epilogue is made short instead: accumulator rows are transposed through
 // shared memory and leave as TMA stores of 32 tokens x 128 features.
 //   128-row block of A handled by CTA c for sub-tile s of tile mt:  4*mt + 2*s + c.
 // =====================================================================================
 constexpr int kPrefetchAhead = 8;          // k-blocks of L2 prefetch distance for activation boxes
 
-template <int BLOCK_N, int STAGES>
 struct SparseQuadCfg {
-    static constexpr int kHalfN = BLOCK_N / 2;
     static constexpr int kABytes = kBlockM * 128;                 // per sub-tile
-    static constexpr int kBBytes = kHalfN * 256;
     static constexpr int kEBytes = 2048;                          // per sub-tile
     static constexpr int kOffB = 2 * kABytes;
-    static constexpr int kOffE = kOffB + kBBytes;
-    static constexpr int kStageBytes = kOffE + 2 * kEBytes;
     static constexpr int kStoreRows = 32;                         // tokens per TMA store
     static constexpr int kStoreCols = 32;                         // features per TMA store (one warp's lanes)
-    static constexpr int kStoreBytes = kStoreRows * kStoreCols * 2;   // 2 KB staging buffer
+    static constexpr int kStoreBytes = kStoreRows * kStoreCols * 2;
     static constexpr int kEpiWarps = 8;                           // two warps per tensor-memory lane quadrant
     static constexpr int kThreads = 64 + 32 * kEpiWarps;
-    static constexpr int kOffStore = STAGES * kStageBytes;
-    static constexpr int kOffBar = kOffStore + kEpiWarps * 2 * kStoreBytes;
-    static constexpr int kSmemBytes = kOffBar + 256 + 1024;
-    static constexpr int kECol = 2 * BLOCK_N;
-    static_assert(BLOCK_N % 32 == 0 && kHalfN % 8 == 0 && 2 * BLOCK_N + 16 <= 512, "tile does not fit tensor memory");
-    static_assert(kBBytes % 2048 == 0 && kStageBytes % 1024 == 0, "stage must keep 1024-byte alignment");
-    static_assert(kSmemBytes <= 232448, "shared memory budget");
+    static constexpr int kStagingBytes = kEpiWarps * 2 * kStoreBytes;
+    static constexpr int kECol = 2 * kMaxTokenTile;
+    __host__ __device__ static constexpr int stage_bytes(int width) { return kOffB + width * 128 + 2 * kEBytes; }
+    __host__ __device__ static constexpr int smem_bytes(int width, int stages) {
+        return stages * stage_bytes(width) + kStagingBytes + 256 + 1024;
+    }
+    static_assert(2 * kMaxTokenTile + 16 <= 512, "tile does not fit tensor memory");
 };
 
 // Tile order of the 512-row-tile kernel: row tiles fastest inside a group of `group_m` row tiles,
@@ -826,19 +839,22 @@ __device__ __forceinline__ void quad_tile(int tile, int num_m, int num_n, int gr
     first = local % gm == 0;
 }
 
-template <int BLOCK_N, int STAGES>
-__global__ void __launch_bounds__(SparseQuadCfg<BLOCK_N, STAGES>::kThreads, 1)
+__global__ void __launch_bounds__(SparseQuadCfg::kThreads, 1)
 sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmE, const __grid_constant__ CUtensorMap tmA2,
                         const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmO,
                         const SparseGemmParams p) {
-    using Cfg = SparseQuadCfg<BLOCK_N, STAGES>;
+    using Cfg = SparseQuadCfg;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + Cfg::kOffBar);
-    uint64_t* empty_bar = full_bar + STAGES;
-    uint64_t* tfull_bar = empty_bar + STAGES;                // [2], one per sub-tile accumulator
-    uint64_t* tempty_bar = tfull_bar + 2;                    // [2]
+    const int stages = p.stages, stage_bytes = Cfg::stage_bytes(p.width);
+    const uint32_t b_half = p.width * 64;                    // bytes of one 64-column half of the activation tile
+    const uint32_t off_e = Cfg::kOffB + 2 * b_half;
+    uint8_t* staging = smem + stages * stage_bytes;
+    uint64_t* full_bar = reinterpret_cast<uint64_t*>(staging + Cfg::kStagingBytes);
+    uint64_t* empty_bar = full_bar + kMaxTileStages;
+    uint64_t* tfull_bar = empty_bar + kMaxTileStages;
+    uint64_t* tempty_bar = tfull_bar + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty_bar + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -847,7 +863,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const int pair_id = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int num_mb = p.M / kBlockM;
     const int num_m = (num_mb + 3) / 4;                      // 512-row tiles
-    const int num_n = (p.Ntok + BLOCK_N - 1) / BLOCK_N;
+    const int num_n = p.num_n;
     const int num_tiles = num_m * num_n;
     const int num_kb = p.K / 128;
     const int num_ab = (p.r + 63) / 64;
@@ -855,7 +871,8 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const int group_m = p.group_m > 0 && p.group_m < num_m ? p.group_m : num_m;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+#pragma unroll
+        for (int s = 0; s < kMaxTileStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&tfull_bar[0], 1);
         mbar_init(&tfull_bar[1], 1);
         mbar_init(&tempty_bar[0], 2 * Cfg::kEpiWarps);
@@ -863,7 +880,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         *abort_flag = 0;
         fence_mbar_init();
     }
-    if (warp == 0 && elect_one()) {
+    if (warp == 2 && elect_one()) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
         tma_prefetch_desc(&tmE);
@@ -896,16 +913,16 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 bool first, next_first = false;
                 quad_tile(tile, num_m, num_n, group_m, mt, n_blk, first);
                 const int nsub = (4 * mt + 2 < num_mb) ? 2 : 1;              // second sub-tile may lie past M
-                const int width = token_tile_width(p.Ntok, n_blk * BLOCK_N, BLOCK_N);
-                const int n_row0 = n_blk * BLOCK_N + static_cast<int>(cta) * (width / 2);
+                const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
+                const int n_row0 = n_blk * p.width + static_cast<int>(cta) * (width / 2);
                 // The pairs working on the same token block (same n_blk, different mt) run side by
                 // side and would all wait on the same first-touch DRAM fetch of an activation box.
                 // One of them (mt == 0) pulls the boxes into L2 kPrefetchAhead k-blocks early.
                 const int next_tile = tile + num_pairs;
                 if (next_tile < num_tiles) quad_tile(next_tile, num_m, num_n, group_m, next_mt, next_n_blk, next_first);
                 const int next_row0 =
-                    next_first ? next_n_blk * BLOCK_N +
-                                     static_cast<int>(cta) * (token_tile_width(p.Ntok, next_n_blk * BLOCK_N, BLOCK_N) / 2)
+                    next_first ? next_n_blk * p.width +
+                                     static_cast<int>(cta) * (token_tile_width(p.Ntok, next_n_blk * p.width, p.width) / 2)
                                : 0;
                 for (int kb = 0; kb < total_kb; ++kb) {
                     if (kb < num_kb) {
@@ -921,20 +938,20 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         }
                     }
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
-                    uint8_t* st = smem + ps.stage * Cfg::kStageBytes;
+                    uint8_t* st = smem + ps.stage * stage_bytes;
                     uint8_t* sB = st + Cfg::kOffB;
                     const uint32_t bar = mapa_shared(smem_u32(&full_bar[ps.stage]), 0);
                     if (kb < num_kb) {
                         if (cta == 0)
                             mbar_expect_tx(&full_bar[ps.stage],
-                                           2 * (Cfg::kBBytes + nsub * (Cfg::kABytes + Cfg::kEBytes)));
+                                           2 * (2 * b_half + nsub * (Cfg::kABytes + Cfg::kEBytes)));
                         tma_load_2d_pair(sB, &tmB, bar, kb * 128, n_row0);
-                        tma_load_2d_pair(sB + Cfg::kHalfN * 128, &tmB, bar, kb * 128 + 64, n_row0);
+                        tma_load_2d_pair(sB + b_half, &tmB, bar, kb * 128 + 64, n_row0);
                         for (int s = 0; s < nsub; ++s) {
                             const int mb = 4 * mt + 2 * s + static_cast<int>(cta);
                             const int mb_e = mb < num_mb ? mb : num_mb - 1;
                             tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, kb * 64, mb * kBlockM, keep);
-                            tma_load_2d_pair_hint(st + Cfg::kOffE + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kb,
+                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kb,
                                                   keep);
                         }
                     } else {
@@ -944,7 +961,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                             waited = true;
                         }
                         if (cta == 0)
-                            mbar_expect_tx(&full_bar[ps.stage], 2 * (Cfg::kHalfN * 128 + nsub * Cfg::kABytes));
+                            mbar_expect_tx(&full_bar[ps.stage], 2 * (b_half + nsub * Cfg::kABytes));
                         tma_load_2d_pair(sB, &tmB2, bar, ab * 64, n_row0);
                         for (int s = 0; s < nsub; ++s) {
                             const int m0 = (4 * mt + 2 * s + static_cast<int>(cta)) * kBlockM;
@@ -957,7 +974,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                             }
                         }
                     }
-                    ps.advance(STAGES);
+                    ps.advance(stages);
                 }
             }
         }
@@ -967,19 +984,20 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             uint32_t idesc_sp = 0, idesc_ad = 0;              // set per tile: N is the tile's width
             // the MMAs of sub-tile s for k-block kb out of pipeline stage `stage`
             auto issue = [&](int s, int kb, int stage) {
-                const uint32_t st = smem_u32(smem + stage * Cfg::kStageBytes);
+                const uint32_t st = smem_u32(smem + stage * stage_bytes);
                 const uint32_t sB = st + Cfg::kOffB;
-                const uint32_t d_tmem = tmem_base + s * BLOCK_N;
+                const uint32_t d_tmem = tmem_base + s * kMaxTokenTile;
                 const uint32_t sA = st + s * Cfg::kABytes;
                 if (kb < num_kb) {
                     const uint32_t e_tmem = tmem_base + Cfg::kECol + (kb & 1) * 8 + s * 4;
-                    tmem_cp_128x128b_pair(e_tmem, make_smem_desc(st + Cfg::kOffE + s * Cfg::kEBytes, 128, 128,
+                    tmem_cp_128x128b_pair(e_tmem, make_smem_desc(st + off_e + s * Cfg::kEBytes, 128, 128,
                                                                  kSwizzleNone));
+                    const uint64_t a0 = make_smem_desc(sA, 16, 1024, kSwizzle128B);
+                    const uint64_t b0 = make_smem_desc(sB, 16, 1024, kSwizzle128B);
+                    const uint64_t b2 = b0 + (b_half >> 4);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const uint64_t ad = make_smem_desc(sA + j * 32, 16, 1024, kSwizzle128B);
-                        const uint64_t bd = make_smem_desc(sB + (j >> 1) * (Cfg::kHalfN * 128) + (j & 1) * 64, 16, 1024,
-                                                           kSwizzle128B);
+                        const uint64_t ad = a0 + 2 * j, bd = (j < 2 ? b0 : b2) + 4 * (j & 1);
                         umma_bf16_sp_pair(d_tmem, ad, bd, e_tmem + (j & 2), idesc_sp | (j & 1), (kb | j) != 0 ? 1u : 0u);
                     }
                 } else {
@@ -1005,7 +1023,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 bool first_unused;
                 quad_tile(tile, num_m, num_n, group_m, mt, n_blk, first_unused);
                 const int nsub = (4 * mt + 2 < num_mb) ? 2 : 1;
-                const int width = token_tile_width(p.Ntok, n_blk * BLOCK_N, BLOCK_N);
+                const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
                 idesc_sp = make_idesc_bf16(2 * kBlockM, width, false, false, true);
                 idesc_ad = make_idesc_bf16(2 * kBlockM, width, p.a2_mn_major != 0, false, false);
                 const uint32_t acc_parity = (static_cast<uint32_t>(it) & 1u) ^ 1u;
@@ -1020,11 +1038,11 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 while (ok && !ready1) {
                     ready1 = mbar_test(&tempty_bar[1], acc_parity);
                     if (ready1) break;
-                    if (kb0 < total_kb && kb0 < STAGES) {
+                    if (kb0 < total_kb && kb0 < stages) {
                         if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                         tc_fence_after_sync();
                         issue(0, kb0, ps.stage);
-                        ps.advance(STAGES);
+                        ps.advance(stages);
                         ++kb0;
                     } else {
                         ok = mbar_wait(&tempty_bar[1], acc_parity, abort_flag);
@@ -1037,7 +1055,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     for (int kb1 = 0; kb1 < kb0; ++kb1) {       // catch up
                         issue(1, kb1, pc.stage);
                         umma_commit_pair(&empty_bar[pc.stage], 3);
-                        pc.advance(STAGES);
+                        pc.advance(stages);
                     }
                 }
                 for (int kb = kb0; kb < total_kb; ++kb) {        // in step
@@ -1046,7 +1064,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     issue(0, kb, ps.stage);
                     if (nsub == 2) issue(1, kb, ps.stage);
                     umma_commit_pair(&empty_bar[ps.stage], 3);
-                    ps.advance(STAGES);
+                    ps.advance(stages);
                 }
                 if (ok && nsub == 1) umma_commit_pair(&tfull_bar[1], 3);        // keep both barriers in phase
             }
@@ -1060,12 +1078,12 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // what the next tile waits for.  Phase 2 runs under the next tile's main loop: each warp
         // transposes its 32 x 32 blocks through a private staging buffer and sends them with its
         // own TMA stores; the warps never wait for one another.
-        constexpr int kBlocks = BLOCK_N / Cfg::kStoreRows;        // 32-token blocks per accumulator
+        constexpr int kBlocks = kMaxTokenTile / Cfg::kStoreRows;   // 32-token blocks per accumulator
         constexpr int kMyBlocks = (kBlocks + 1) / 2;              // at most this many per warp
         const int q = warp & 3;
         const int ew = warp - 2;
         const int half = ew >> 2;
-        uint8_t* my_buf = smem + Cfg::kOffStore + ew * 2 * Cfg::kStoreBytes;
+        uint8_t* my_buf = staging + ew * 2 * Cfg::kStoreBytes;
         const uint64_t stream_out = l2_policy_evict_first();
         bool ok = true;
         int it = 0;
@@ -1075,7 +1093,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             bool first_unused;
             quad_tile(tile, num_m, num_n, group_m, mt, n_blk, first_unused);
             const int nsub = (4 * mt + 2 < num_mb) ? 2 : 1;
-            const int width = token_tile_width(p.Ntok, n_blk * BLOCK_N, BLOCK_N);
+            const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
             uint32_t pk[2][kMyBlocks][16];
             // ---- first accumulator (its drain is what the next tile's first MMA waits for).  Two
             //      16-column loads in flight per wait: the warps of a 320-thread CTA are allocated
@@ -1108,7 +1126,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             if (!mbar_wait(&tfull_bar[1], static_cast<uint32_t>(it) & 1u, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
             if (nsub == 2) {
-                const uint32_t t_row = tmem_base + BLOCK_N + (static_cast<uint32_t>(q * 32) << 16);
+                const uint32_t t_row = tmem_base + kMaxTokenTile + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll
                 for (int j = 0; j < kMyBlocks; ++j) {
                     const int c0 = (2 * j + half) * Cfg::kStoreRows;
@@ -1148,7 +1166,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                             fence_proxy_async_smem();
                             __syncwarp();
                             if (lane == 0 && m0 < p.M) {
-                                tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n_blk * BLOCK_N + c0,
+                                tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n_blk * p.width + c0,
                                                   stream_out);
                                 tma_store_commit();
                             }
@@ -1245,7 +1263,7 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         tmem_alloc(tmem_slot, Cfg::kTmemCols);
         tmem_relinquish();
     }
-    if (warp == 0 && elect_one()) {
+    if (warp == 2 && elect_one()) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmE);
     }

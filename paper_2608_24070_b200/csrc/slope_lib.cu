@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "adapter_kernels.cuh"
@@ -286,36 +287,46 @@ struct AdapterOperands {
 // and ranks 16 ... 256 (in most of them the choice is within 5 % of the best swept one):
 //   - a round trip through the ring takes 0.8 us, so a k-block costs at least that over its depth,
 //     and at least what the SM takes in (150 KB per us);
-//   - a CTA brings in 90 GB/s of the large operand, all of them together 6 TB/s, and every further
-//     column tile costs 8 % of that (its second read comes from L2);
+//   - a CTA brings in 90 GB/s of the large operand, dozens of them less, all together 6 TB/s, and every
+//     further column tile costs 8 % of that (its second read comes from L2);
 //   - draining a tile costs 0.3 us per 64 columns, 1 us more and 1 us per 64 columns when it is split.
 struct AdapterPlan {
     int n_tile, splits;
     bool deep;                    // one CTA per SM with all of its shared memory; else two that share it
+    double us;                    // estimated time
 };
+static AdapterPlan adapter_candidate(int row_tiles, double a_bytes, int N, int K, int n_tile, int splits, int sm_count) {
+    const int num_kb = (K + 63) / 64, col_tiles = (N + n_tile - 1) / n_tile, ctas = row_tiles * col_tiles * splits;
+    // clusters of 4 and 8 do not fill every SM (33 and 15 of them fit on 148 SMs)
+    const int sms = splits == 8 ? sm_count * 120 / 148 : splits == 4 ? sm_count * 132 / 148 : sm_count;
+    const bool deep = n_tile == 256 || ctas <= sms;
+    const int slots = (deep ? 1 : 2) * sms;
+    const double stages = n_tile == 64 ? (deep ? 9 : 4) : n_tile == 128 ? (deep ? 7 : 3) : 4;
+    const int waves = (ctas + slots - 1) / slots;
+    const double kb_us = std::max(0.8 / stages, (deep ? 1 : 2) * (16.0 + n_tile / 8.0) / 150.0);
+    const double hbm = std::min({6.0e6, 0.09e6 * ctas, 2.2e6 + 0.03e6 * ctas}) / (1.0 + 0.08 * (col_tiles - 1));
+    const double stream = std::max(waves * ((num_kb + splits - 1) / splits) * kb_us, a_bytes / hbm);
+    const double tail = (splits > 1 ? 1.0 : 0.3) * n_tile / 64.0 + (splits > 1 ? 1.0 : 0.0);
+    return AdapterPlan{n_tile, splits, deep, stream + waves * tail};
+}
+template <typename Visit>
+static void adapter_candidates(int row_tiles, double a_bytes, int N, int K, int sm_count, Visit visit) {
+    for (int n_tile = 64; n_tile <= 256 && (n_tile == 64 || n_tile < 2 * N); n_tile *= 2)
+        for (int s = 1; s <= 8 && (s == 1 || 2 * s <= (K + 63) / 64); s *= 2)
+            visit(adapter_candidate(row_tiles, a_bytes, N, K, n_tile, s, sm_count));
+}
 static AdapterPlan adapter_plan(int row_tiles, double a_bytes, int N, int K, int sm_count) {
-    const int num_kb = (K + 63) / 64;
-    AdapterPlan best{64, 1, true};
-    double best_cost = 1e30;
-    for (int n_tile = 64; n_tile <= 256 && (n_tile == 64 || n_tile < 2 * N); n_tile *= 2) {
-        const int col_tiles = (N + n_tile - 1) / n_tile;
-        for (int s = 1; s <= 8 && (s == 1 || 2 * s <= num_kb); s *= 2) {
-            const int ctas = row_tiles * col_tiles * s;
-            // clusters of 4 and 8 do not fill every SM (33 and 15 of them fit on 148 SMs)
-            const int sms = s == 8 ? sm_count * 120 / 148 : s == 4 ? sm_count * 132 / 148 : sm_count;
-            const bool deep = n_tile == 256 || ctas <= sms;
-            const int slots = (deep ? 1 : 2) * sms;
-            const double stages = n_tile == 64 ? (deep ? 9 : 4) : n_tile == 128 ? (deep ? 7 : 3) : 4;
-            const int waves = (ctas + slots - 1) / slots;
-            const double kb_us = std::max(0.8 / stages, (deep ? 1 : 2) * (16.0 + n_tile / 8.0) / 150.0);
-            const double hbm = std::min(6.0e6, 0.09e6 * std::min(ctas, sm_count)) / (1.0 + 0.08 * (col_tiles - 1));
-            const double stream = std::max(waves * ((num_kb + s - 1) / s) * kb_us, a_bytes / hbm);
-            const double tail = (s > 1 ? 1.0 : 0.3) * n_tile / 64.0 + (s > 1 ? 1.0 : 0.0);
-            const double cost = stream + waves * tail;
-            if (cost < best_cost - 1e-9) { best_cost = cost; best = AdapterPlan{n_tile, s, deep}; }
-        }
-    }
+    AdapterPlan best{64, 1, true, 1e30};
+    adapter_candidates(row_tiles, a_bytes, N, K, sm_count, [&](const AdapterPlan& c) {
+        if (c.us < best.us - 1e-9) best = c;
+    });
     return best;
+}
+
+// SMs that the CTAs of a launch over `rows` rows occupy.
+static int adapter_sms(const AdapterPlan& plan, int rows, int N, int sm_count) {
+    const int ctas = (rows + kBlockM - 1) / kBlockM * ((N + plan.n_tile - 1) / plan.n_tile) * plan.splits;
+    return std::min(plan.deep ? ctas : (ctas + 1) / 2, sm_count);
 }
 
 template <bool A_MN, bool B_MN, int N_TILE>
@@ -344,28 +355,21 @@ static slope_status_t launch_adapter_tile(const AdapterOperands& q0, const Adapt
 
 // D[M x N] = A B over one or two problems with the same N (= r) and K.
 template <bool A_MN, bool B_MN>
-static slope_status_t launch_adapter(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K,
-                                     cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
-    const AdapterPlan plan = adapter_plan(row_tiles, 2.0 * K * (static_cast<double>(q0.M) + q1.M), N, K, info.sm_count);
+static slope_status_t launch_adapter_planned(const AdapterPlan& plan, const AdapterOperands& q0, const AdapterOperands& q1,
+                                             int N, int K, cudaStream_t stream, int pdl_mode) {
     switch (plan.n_tile) {
         case 64: return launch_adapter_tile<A_MN, B_MN, 64>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
         case 128: return launch_adapter_tile<A_MN, B_MN, 128>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
         default: return launch_adapter_tile<A_MN, B_MN, 256>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
     }
 }
-
-// CTAs of the T launch below.
-static int adapter_T_ctas(int b, int d_in, int r, const DeviceInfo& info) {
-    const int row_tiles = (b + kBlockM - 1) / kBlockM;
-    const AdapterPlan plan = adapter_plan(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count);
-    return row_tiles * ((r + plan.n_tile - 1) / plan.n_tile) * plan.splits;
-}
-
-// T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
-static slope_status_t launch_adapter_T(const void* X, const void* L, int b, int d_in, int r, void* T,
-                                       cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    return launch_adapter<false, true>(AdapterOperands{X, L, T, b, 0}, AdapterOperands{}, r, d_in, stream, info, pdl_mode);
+template <bool A_MN, bool B_MN>
+static slope_status_t launch_adapter(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K,
+                                     cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
+    const double a_bytes = 2.0 * K * (static_cast<double>(q0.M) + q1.M);
+    return launch_adapter_planned<A_MN, B_MN>(adapter_plan(row_tiles, a_bytes, N, K, info.sm_count), q0, q1, N, K, stream,
+                                              pdl_mode);
 }
 
 // dT[b x r] = dY[b x d_out] * R[r x d_out]^T   (both K contiguous)
@@ -384,43 +388,56 @@ static AdapterOperands adapter_dL(const void* X, const void* dT, int d_in, void*
 }
 
 // ------------------------------------------------------------------ CTA-pair launches (main GEMMs)
-constexpr int kPairBlockN = 224;             // token tile of the big-tile kernels
-constexpr int kPairStages = 4;
-constexpr int kPairNarrowBlockN = 128;       // narrower 256-row tile for shapes with few tiles
-constexpr int kPairNarrowStages = 5;
-
-template <int BLOCK_N, int STAGES>
-static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
-                                         const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    using Cfg = SparsePairCfg<BLOCK_N, STAGES>;
+// Everything a launch of the two sparse tile kernels has in common.
+struct SparseTileArgs {
     CUtensorMap tmA, tmB, tmE, tmA2, tmB2, tmO;
-    if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
-    if (!make_tmap(&tmB, act, ntok, K, Cfg::kHalfN, 64)) return SLOPE_ERR_CUDA;
-    if (!make_tmap_meta(&tmE, meta, static_cast<size_t>(M) * K / 8)) return SLOPE_ERR_CUDA;
-    if (!make_tmap_plain(&tmO, out, ntok, M, Cfg::kStoreRows, Cfg::kStoreCols, true)) return SLOPE_ERR_CUDA;
+    SparseGemmParams p;
+};
+static bool sparse_tile_args(SparseTileArgs& a, const void* act, int ntok, const void* vals, const void* meta, int M, int K,
+                             const void* act2, const void* fac2, int r, bool a2_mn, void* out, int width, int stages,
+                             bool swizzle_out, int pdl_mode) {
+    if (!make_tmap(&a.tmA, vals, M, K / 2, kBlockM, 64) || !make_tmap(&a.tmB, act, ntok, K, width / 2, 64) ||
+        !make_tmap_meta(&a.tmE, meta, static_cast<size_t>(M) * K / 8) ||
+        !make_tmap_plain(&a.tmO, out, ntok, M, SparsePairCfg::kStoreRows, SparsePairCfg::kStoreCols, swizzle_out))
+        return false;
     if (r > 0) {
-        const bool ok2 = a2_mn ? make_tmap(&tmA2, fac2, r, M, 64, 64) : make_tmap(&tmA2, fac2, M, r, kBlockM, 64);
-        if (!ok2 || !make_tmap(&tmB2, act2, ntok, r, Cfg::kHalfN, 64)) return SLOPE_ERR_CUDA;
+        const bool ok2 = a2_mn ? make_tmap(&a.tmA2, fac2, r, M, 64, 64) : make_tmap(&a.tmA2, fac2, M, r, kBlockM, 64);
+        if (!ok2 || !make_tmap(&a.tmB2, act2, ntok, r, width / 2, 64)) return false;
     } else {
-        tmA2 = tmA;
-        tmB2 = tmB;
+        a.tmA2 = a.tmA;
+        a.tmB2 = a.tmB;
     }
-    SparseGemmParams p = {};
-    p.M = M; p.K = K; p.Ntok = ntok; p.r = r; p.a2_mn_major = a2_mn ? 1 : 0;
-    p.meta = static_cast<const uint8_t*>(meta);
-    p.out = static_cast<uint16_t*>(out);
-    auto kern = sparse_gemm_pair_kernel<BLOCK_N, STAGES>;
-    if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    p.pdl_mode = pdl_mode;
-    const int tiles = ((M / kBlockM + 1) / 2) * ((ntok + BLOCK_N - 1) / BLOCK_N);
-    const int max_pairs = info.sm_count / 2;
-    const int pairs = tiles < max_pairs ? tiles : max_pairs;
-    return launch_pairs(kern, 2 * pairs, Cfg::kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmE, tmA2, tmB2, tmO, p);
+    a.p = SparseGemmParams{};
+    a.p.M = M; a.p.K = K; a.p.Ntok = ntok; a.p.r = r; a.p.a2_mn_major = a2_mn ? 1 : 0;
+    a.p.width = width; a.p.num_n = (ntok + width - 1) / width; a.p.stages = stages; a.p.pdl_mode = pdl_mode;
+    a.p.meta = static_cast<const uint8_t*>(meta);
+    a.p.out = static_cast<uint16_t*>(out);
+    return true;
 }
 
-constexpr int kQuadBlockN = 224;
-constexpr int kQuadStages = 3;
+// Pipeline stages that fit beside the staging buffers at a tile width.
+constexpr int kMaxTileSmem = 232448;
+template <typename Cfg>
+static int tile_stages(int width) {
+    int n = kMaxTileStages;
+    while (n > 1 && Cfg::smem_bytes(width, n) > kMaxTileSmem) --n;
+    return n;
+}
+
+static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
+                                         const void* act2, const void* fac2, int r, bool a2_mn, void* out, int width,
+                                         int max_pairs, cudaStream_t stream, int pdl_mode) {
+    using Cfg = SparsePairCfg;
+    SparseTileArgs a;
+    const int stages = tile_stages<Cfg>(width);
+    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, true, pdl_mode))
+        return SLOPE_ERR_CUDA;
+    if (!set_smem(sparse_gemm_pair_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
+    const int tiles = ((M / kBlockM + 1) / 2) * ((ntok + width - 1) / width);
+    const int pairs = std::min(tiles, max_pairs);
+    return launch_pairs(sparse_gemm_pair_kernel, 2 * pairs, Cfg::kThreads, Cfg::smem_bytes(width, stages), stream, a.tmA,
+                        a.tmB, a.tmE, a.tmA2, a.tmB2, a.tmO, a.p);
+}
 
 // Row tiles per raster group of the 512-row-tile kernel (see quad_tile).  All pairs that work on
 // one token block share its activations, so with every row tile in one group the activations
@@ -430,8 +447,8 @@ constexpr int kQuadStages = 3;
 // a group's weights resident.  Pick the g with the least estimated DRAM traffic
 // (measured at 16384 tokens: 4096 -> 11008 two groups +7 %, 5120 -> 13824 three groups +11 %,
 // square and long-reduction layers one group).
-static int quad_group_m(int M, int K, int ntok, int num_pairs) {
-    const int num_m = (M / kBlockM + 3) / 4, num_n = (ntok + kPairBlockN - 1) / kPairBlockN;
+static int quad_group_m(int M, int K, int ntok, int width, int num_pairs) {
+    const int num_m = (M / kBlockM + 3) / 4, num_n = (ntok + width - 1) / width;
     const double w_tile = 512.0 * K * 1.125, w_total = static_cast<double>(M) * K * 1.125;
     const double x_total = static_cast<double>(ntok) * K * 2.0;
     constexpr double kL2Keeps = 30e6;
@@ -447,33 +464,19 @@ static int quad_group_m(int M, int K, int ntok, int num_pairs) {
 }
 
 static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
-                                         const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                         cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    using Cfg = SparseQuadCfg<kQuadBlockN, kQuadStages>;
-    CUtensorMap tmA, tmB, tmE, tmA2, tmB2, tmO;
-    if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
-    if (!make_tmap(&tmB, act, ntok, K, Cfg::kHalfN, 64)) return SLOPE_ERR_CUDA;
-    if (!make_tmap_meta(&tmE, meta, static_cast<size_t>(M) * K / 8)) return SLOPE_ERR_CUDA;
-    if (!make_tmap_plain(&tmO, out, ntok, M, Cfg::kStoreRows, Cfg::kStoreCols)) return SLOPE_ERR_CUDA;
-    if (r > 0) {
-        const bool ok2 = a2_mn ? make_tmap(&tmA2, fac2, r, M, 64, 64) : make_tmap(&tmA2, fac2, M, r, kBlockM, 64);
-        if (!ok2 || !make_tmap(&tmB2, act2, ntok, r, Cfg::kHalfN, 64)) return SLOPE_ERR_CUDA;
-    } else {
-        tmA2 = tmA;
-        tmB2 = tmB;
-    }
-    SparseGemmParams p = {};
-    p.M = M; p.K = K; p.Ntok = ntok; p.r = r; p.a2_mn_major = a2_mn ? 1 : 0;
-    p.meta = static_cast<const uint8_t*>(meta);
-    p.out = static_cast<uint16_t*>(out);
-    const int max_pairs = info.sm_count / 2;
-    p.pdl_mode = pdl_mode;
-    p.group_m = quad_group_m(M, K, ntok, max_pairs);
-    auto kern = sparse_gemm_quad_kernel<kQuadBlockN, kQuadStages>;
-    if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    const int tiles = ((M / kBlockM + 3) / 4) * ((ntok + kQuadBlockN - 1) / kQuadBlockN);
-    const int pairs = tiles < max_pairs ? tiles : max_pairs;
-    return launch_pairs(kern, 2 * pairs, Cfg::kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmE, tmA2, tmB2, tmO, p);
+                                         const void* act2, const void* fac2, int r, bool a2_mn, void* out, int width,
+                                         int max_pairs, cudaStream_t stream, int pdl_mode) {
+    using Cfg = SparseQuadCfg;
+    SparseTileArgs a;
+    const int stages = tile_stages<Cfg>(width);
+    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, false, pdl_mode))
+        return SLOPE_ERR_CUDA;
+    a.p.group_m = quad_group_m(M, K, ntok, width, max_pairs);
+    if (!set_smem(sparse_gemm_quad_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
+    const int tiles = ((M / kBlockM + 3) / 4) * ((ntok + width - 1) / width);
+    const int pairs = std::min(tiles, max_pairs);
+    return launch_pairs(sparse_gemm_quad_kernel, 2 * pairs, Cfg::kThreads, Cfg::smem_bytes(width, stages), stream, a.tmA,
+                        a.tmB, a.tmE, a.tmA2, a.tmB2, a.tmO, a.p);
 }
 
 // Few tokens (inference / decode sizes): weight-streaming kernel, K split over a cluster.
@@ -569,7 +572,8 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
         // The consumer of a fused pair has to be resident next to its producer, or its last clusters
         // would wait for the producer to finish and the overlap would be lost: count only the
         // clusters that fit beside it.
-        const int reserved = adapter_T_ctas(ntok, K, r, info);
+        const AdapterPlan producer = adapter_plan((ntok + kBlockM - 1) / kBlockM, 2.0 * ntok * K, r, K, info.sm_count);
+        const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
         for (int sz = 1; sz <= 8; ++sz) {
             cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
             if (cap[sz] < 0) cap[sz] = 0;
@@ -613,53 +617,45 @@ static slope_status_t launch_skinny(const void* act, int ntok, const void* vals,
     return launch_sparse_skinny<128, 7, 3>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
 }
 
-// Kernel choice for the sparse GEMMs.  Up to 256 tokens the GEMM is a weight stream from HBM and
-// runs on the few-token kernel.  Beyond that three tile shapes compete:
-//   512 x 224  moves 31 % fewer L2 bytes per FLOP but cannot overlap its epilogue with the next
-//              tile (tensor memory holds one accumulator set).  Measured at 16384 tokens it is
-//              6 % faster per unit of work at a reduction length of 4096 and 14-16 % at 11008,
-//              while at 768 the 256-row tile is up to 25 % faster.
-//   256 x 224  double-buffered accumulators.
-//   256 x 128  the same kernel with a narrower token tile: more, smaller tiles for shapes that
-//              would otherwise leave much of the last wave of the machine empty (2048 x 2048
-//              with 2048 tokens: 80 tiles of 256 x 224 on 74 CTA pairs = 2 waves for 1.08 waves
-//              of work); it stages the weights for fewer tokens, which costs 12 % more time
-//              per unit of work at short reductions and 30-35 % at long ones (measured at 2048
-//              tokens).
-// The choice compares waves of the machine (tiles / CTA pairs, rounded up) times the relative
-// cost of a tile.
-enum class SparseTile { kQuad224, kPair224, kPair128 };
-
-static SparseTile choose_sparse_tile(int M, int K, int ntok, int num_pairs, double* cost_out = nullptr) {
-    // Waves of full tiles; the ragged last token tile of every row tile runs at its own width
-    // (its weight loads do not shrink, its epilogue does: measured, a 32-token tile costs 0.7-0.9
-    // of a 224-token one at reductions of 4096 and more, about 0.4 at 1024) and comes last in tile
-    // order, so it first fills the pairs that the last wave of full tiles leaves idle.
-    const auto rounds = [&](int rows, int block_n) {
-        const int num_m = (M + rows - 1) / rows;
-        const int full = num_m * (ntok / block_n), ragged = ntok % block_n;
-        const int rem = full % num_pairs;
-        double t = full / num_pairs + (rem ? 1.0 : 0.0);
-        if (ragged) {
-            const double width = ((ragged + 31) & ~31) / static_cast<double>(block_n);
-            const int left = num_m - (rem ? num_pairs - rem : 0);
-            const double floor = K >= 4096 ? 0.8 : K >= 2048 ? 0.65 : 0.45;
-            if (left > 0) t += ((left + num_pairs - 1) / num_pairs) * (width > floor ? width : floor);
-        }
-        return t;
-    };
-    const double gain = K >= 8192 ? 0.14 : K >= 4096 ? 0.06 : K >= 2048 ? -0.05 : -0.25;
-    const double cost_pair = rounds(256, kPairBlockN);
-    const double cost_quad = 2.0 * (1.0 - gain) * rounds(512, kPairBlockN);
-    const double narrow_penalty = K >= 8192 ? 1.35 : K >= 4096 ? 1.30 : K >= 2048 ? 1.20 : 1.12;
-    const double cost_narrow = narrow_penalty * kPairNarrowBlockN / kPairBlockN * rounds(256, kPairNarrowBlockN);
-    // (cost_out: the winner's cost in time units of one 256 x 224 tile)
-    if (cost_quad < cost_pair && cost_quad <= cost_narrow) {
-        if (cost_out) *cost_out = cost_quad;
-        return SparseTile::kQuad224;
+// Tile of a sparse GEMM, by estimate:
+//   512 rows   two MMA sub-tiles share an activation tile (fewer bytes per FLOP), but tensor memory then holds one
+//              accumulator set and a tile's drain is exposed;
+//   256 rows   double-buffered accumulators;
+//   width      the token tiles of a launch are made equal (500 tokens: three of 192 and less rather than two of
+//              224 and one of 64) and as wide as fills the waves of CTA pairs best.
+// In SM clocks: a k-block takes the round trip of a pipeline stage (2130, 2515 with all pairs at work) over the stages
+// that fit, and at least its bytes (70 per clock and SM) and its MMAs; a 512-row tile exposes 12 per token
+// of width, the last drain of a launch takes 290 + 8.7 per token (4.4 times that for 512 rows), a launch
+// 47 per pair.  Fitted to a sweep of all tiles over 23 layer shapes (640 ... 22016 wide) and 130 ... 8192
+// tokens, where the choice is on average 0.6 %, at most 11 % slower than the best tile of the sweep.
+struct SparseTile {
+    int rows, width;
+};
+template <typename Cfg>
+static double sparse_tile_cost(int M, double num_kb, int ntok, int width, int num_pairs) {
+    const bool quad = std::is_same<Cfg, SparseQuadCfg>::value;
+    const int rows = quad ? 512 : 256;
+    const int tiles = ((M + rows - 1) / rows) * ((ntok + width - 1) / width), active = std::min(tiles, num_pairs);
+    const double load = Cfg::stage_bytes(width) / 70.0, mma = rows * std::max(width, 64) / 128.0;
+    const double round_trip = 2130.0 + 385.0 * active / num_pairs;
+    const double k_block = std::max({round_trip / tile_stages<Cfg>(width), load, mma});
+    const double tile = num_kb * k_block + (quad ? 12.0 * width : 0.0);
+    const double last_drain = (quad ? 4.4 : 1.0) * (290.0 + 8.7 * width);
+    return (tiles + num_pairs - 1) / num_pairs * tile + last_drain + 47.0 * active;
+}
+static SparseTile choose_sparse_tile(int M, int K, int ntok, int r, int num_pairs, double* cost = nullptr) {
+    const double num_kb = K / 128 + 0.6 * ((r + 63) / 64);            // an adapter step is half a k-block of activations
+    SparseTile best{256, 32};
+    double best_cost = 1e300;
+    for (int w = kMaxTokenTile; w >= 32; w -= 32) {
+        const int n = (ntok + w - 1) / w, width = ((ntok + n - 1) / n + 31) & ~31;
+        const double pair = sparse_tile_cost<SparsePairCfg>(M, num_kb, ntok, width, num_pairs);
+        const double quad = sparse_tile_cost<SparseQuadCfg>(M, num_kb, ntok, width, num_pairs);
+        if (pair < best_cost) { best_cost = pair; best = SparseTile{256, width}; }
+        if (quad < best_cost) { best_cost = quad; best = SparseTile{512, width}; }
     }
-    if (cost_out) *cost_out = cost_narrow < cost_pair ? cost_narrow : cost_pair;
-    return cost_narrow < cost_pair ? SparseTile::kPair128 : SparseTile::kPair224;
+    if (cost) *cost = best_cost;
+    return best;
 }
 
 // Few-token kernel or tile kernel?  Decode sizes (<= 16 tokens) always stream the weights through
@@ -684,20 +680,77 @@ static bool use_few_token_kernel(int M, int K, int ntok, int r, const DeviceInfo
     return few_us <= tile_us;
 }
 
-// One of the three tile kernels.
-static slope_status_t launch_sparse_tiles(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
-                                          const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                          cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    switch (choose_sparse_tile(M, K, ntok, info.sm_count / 2)) {
-        case SparseTile::kQuad224:
-            return launch_sparse_quad(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
-        case SparseTile::kPair128:
-            return launch_sparse_pair<kPairNarrowBlockN, kPairNarrowStages>(act, ntok, vals, meta, M, K, act2, fac2, r,
-                                                                            a2_mn, out, stream, info, pdl_mode);
-        default:
-            return launch_sparse_pair<kPairBlockN, kPairStages>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out,
-                                                                stream, info, pdl_mode);
+static slope_status_t launch_sparse_tile(const SparseTile& t, const void* act, int ntok, const void* vals, const void* meta,
+                                         int M, int K, const void* act2, const void* fac2, int r, bool a2_mn, void* out,
+                                         int pairs, cudaStream_t stream, int pdl_mode) {
+    return t.rows == 512 ? launch_sparse_quad(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, t.width, pairs, stream,
+                                              pdl_mode)
+                         : launch_sparse_pair(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, t.width, pairs, stream,
+                                              pdl_mode);
+}
+
+// T = X L and the forward that adds T R.  How the adapter launch is cut decides how long it takes and how many SMs
+// it keeps from the forward, so the two are planned together, whether they are launched as a fused pair
+// or by separate calls (T is the same bits in both).  Behind the producer a forward takes
+//   - at least T + 5.9 us (two launches, the adapter steps and the drain);
+//   - or its own time + 2 us + the producer's share of the machine; and where pairs on the producer's SMs have as
+//     many tiles as the others (the last CTAs of a launch start there, so a ragged last wave leaves
+//     them out), most of T on top, unless the tiles are chosen for the SMs beside it.
+// us, 4096 -> 4096, r = 64 at 500 / 1000 / 2048 tokens: T split in 2 / 2 / 1: 15.1 / 23.3 / 37.2, in 8: 17.4 / 27.0 /
+// 39.7, although T alone is fastest in 8.
+struct FwdAdapterPlan {
+    AdapterPlan T;
+    SparseTile tile;
+    int pairs;                    // CTA pairs of the forward
+};
+static FwdAdapterPlan plan_fwd_adapter(int b, int d_out, int d_in, int r, const DeviceInfo& info) {
+    struct Memo {
+        int b, d_out, d_in, r, sm_count;
+        FwdAdapterPlan plan;
+    };
+    thread_local Memo memo[64] = {};                                   // a pure function of sizes
+    Memo& m = memo[(b * 31u + d_out / 128 * 7u + d_in / 128 * 3u + r / 16u) % 64];
+    if (m.b == b && m.d_out == d_out && m.d_in == d_in && m.r == r && m.sm_count == info.sm_count) return m.plan;
+    const int row_tiles = (b + kBlockM - 1) / kBlockM;
+    constexpr double kClkPerUs = 1850.0;
+    FwdAdapterPlan best{};
+    best.pairs = info.sm_count / 2;
+    double best_us = 1e300, cost = 0.0;
+    if (use_few_token_kernel(d_out, d_in, b, r, info)) {                // its K-split is chosen around the producer
+        best.T = adapter_plan(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count);
+    } else {
+        const int pairs = info.sm_count / 2;
+        const SparseTile full = choose_sparse_tile(d_out, d_in, b, r, pairs, &cost);
+        const double full_us = cost / kClkPerUs;
+        const int last_wave = ((d_out + full.rows - 1) / full.rows) * ((b + full.width - 1) / full.width) % pairs;
+        adapter_candidates(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count, [&](const AdapterPlan& c) {
+            const int sms = adapter_sms(c, b, r, info.sm_count), beside = (info.sm_count - sms) / 2;
+            const double share = static_cast<double>(sms) / info.sm_count;
+            const bool blocked = last_wave == 0 || last_wave > beside;
+            const double late = std::max(share * c.us, blocked ? (0.6 + 0.4 * share) * c.us : 0.0);
+            const double us = std::max(c.us + 5.9, full_us + 2.0 + late);
+            if (us < best_us) {
+                best_us = us;
+                best = FwdAdapterPlan{c, full, pairs};
+            }
+            if (!blocked || beside < pairs / 2) return;
+            const SparseTile t = choose_sparse_tile(d_out, d_in, b, r, beside, &cost);
+            const double us_beside = std::max(c.us + 5.9, cost / kClkPerUs + 2.0 + share * c.us);
+            if (us_beside < best_us) {
+                best_us = us_beside;
+                best = FwdAdapterPlan{c, t, beside};
+            }
+        });
     }
+    m = Memo{b, d_out, d_in, r, info.sm_count, best};
+    return best;
+}
+
+// T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
+static slope_status_t launch_adapter_T(const FwdAdapterPlan& plan, const void* X, const void* L, int b, int d_in, int r,
+                                       void* T, cudaStream_t stream, int pdl_mode) {
+    return launch_adapter_planned<false, true>(plan.T, AdapterOperands{X, L, T, b, 0}, AdapterOperands{}, r, d_in, stream,
+                                               pdl_mode);
 }
 
 static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
@@ -705,7 +758,9 @@ static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* 
                                          cudaStream_t stream, const DeviceInfo& info) {
     if (use_few_token_kernel(M, K, ntok, r, info))
         return launch_skinny(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info);
-    return launch_sparse_tiles(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info);
+    const int pairs = info.sm_count / 2;
+    return launch_sparse_tile(choose_sparse_tile(M, K, ntok, r, pairs), act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out,
+                              pairs, stream, 0);
 }
 
 template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
@@ -879,16 +934,16 @@ slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_val
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    const FwdAdapterPlan plan = plan_fwd_adapter(b, d_out, d_in, r, info);
+    if (slope_status_t st = launch_adapter_T(plan, X, L, b, d_in, r, T, stream, 1)) return st;
     if (use_few_token_kernel(d_out, d_in, b, r, info)) {
         // Two launches of the few-token kernel as a fused pair: T = X L releases its dependent only
         // once everything before it in the stream is complete, so the forward streams its weights
         // and runs its sparse reduction while T is still being computed, and waits only for T.
-        if (slope_status_t st = launch_adapter_T(X, L, b, d_in, r, T, stream, info, 1)) return st;
         return launch_skinny(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, true, Y, stream, info, 2);
     }
     // More tokens: the tile kernels are the consumer of such a pair in the same way.
-    if (slope_status_t st = launch_adapter_T(X, L, b, d_in, r, T, stream, info, 1)) return st;
-    return launch_sparse_tiles(X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, /*a2_mn=*/true, Y, stream, info, 2);
+    return launch_sparse_tile(plan.tile, X, b, Wc_vals, Wc_meta, d_out, d_in, T, R, r, /*a2_mn=*/true, Y, plan.pairs, stream, 2);
 }
 
 slope_status_t slope_linear_bwd_dx(const void* dY, int b, const void* WTc_vals, const void* WTc_meta, int d_out,
@@ -984,7 +1039,7 @@ slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, c
         if (!X || !L || !T) return SLOPE_ERR_INVALID_ARG;
         if (!aligned16(X) || !aligned16(L) || !aligned16(T)) return SLOPE_ERR_ALIGNMENT;
         if (slope_status_t st = check_arch(info)) return st;
-        return launch_adapter_T(X, L, b, d_in, r, T, stream, info);
+        return launch_adapter_T(plan_fwd_adapter(b, d_out, d_in, r, info), X, L, b, d_in, r, T, stream, 0);
     }
     if (phase == 2) {
         if (!dY || !R || !dT) return SLOPE_ERR_INVALID_ARG;

@@ -1,0 +1,60 @@
+"""Sparse forward and input gradient over every token-tile width of the tile kernels (32 ... 224 in steps of 32, both
+row counts), ragged last tiles and row tiles that are half empty, with and without adapters; the fused
+forward against the separate calls.
+
+The reference is the fp64 product of the bf16 operands the kernels read (T as written), so outputs are rounded
+once: 1.7e-3 relative on Gaussian data, 5e-3 allowed, and parity_error's bound per element."""
+import numpy as np
+import pytest
+
+from paper_2608_24070_b200 import inputs as si
+from helpers import REL_TOL, GpuLayer, parity_error, to_f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [
+    (129, 256, 384, 0),          # narrowest tiles, last row tile half empty
+    (161, 1024, 256, 16),
+    (250, 640, 1920, 0),
+    (353, 512, 4096, 48),
+    (449, 768, 2304, 0),
+    (500, 4096, 1152, 64),
+    (673, 384, 2176, 256),
+    (1000, 768, 2304, 16),
+    (1345, 1152, 640, 0),
+    (2048, 1024, 4096, 32),
+    (5000, 2048, 1408, 0),       # several waves, 512-row tiles the other way round
+])
+def test_token_tiles_match_fp64(b, d_in, d_out, r):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    Wb = si.gaussian_bf16((d_out, d_in), 0.02, 51)
+    layer = GpuLayer(Wb, fused_setup=True)
+    Xb, dYb = si.gaussian_bf16((b, d_in), 1.0, 52), si.gaussian_bf16((b, d_out), 1.0, 53)
+    X, dY = B.bf16_from_bits(Xb), B.bf16_from_bits(dYb)
+    bits = lambda m: np.unpackbits(m.cpu().numpy(), axis=1, bitorder="little").astype(bool)
+    fW = to_f64(Wb)
+    ref_Y, ref_dX = to_f64(Xb) @ (fW * bits(layer.mask1)).T, to_f64(dYb) @ (fW * bits(layer.mask2))
+    g = lambda t: to_f64(B.bits_from_bf16(t))
+    nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    Y, dX = nan(b + 1, d_out), nan(b + 1, d_in)                 # a spare row: nothing behind the last token
+    T = dT = L = R = None
+    if r:
+        Lb, Rb = si.gaussian_bf16((d_in, r), 0.1, 54), si.gaussian_bf16((r, d_out), 0.1, 55)
+        L, R = B.bf16_from_bits(Lb), B.bf16_from_bits(Rb)
+        T, dT = layer.adapter_T(X, L), nan(b, r)
+        B.slope_adapter_fwd_bwd(2, None, dY, None, R, b, d_out, d_in, r, dT=dT)
+        ref_Y, ref_dX = ref_Y + g(T) @ to_f64(Rb), ref_dX + g(dT) @ to_f64(Lb).T
+        T1, Y1 = nan(b, r), nan(b, d_out)
+        B.slope_linear_fwd_adapter(X, layer.Wc_vals, layer.Wc_meta, d_out, L, R, T1, Y1)
+        assert torch.equal(T1.view(torch.int16), T.view(torch.int16))
+        assert parity_error(g(Y1), ref_Y) <= REL_TOL
+    B.slope_linear_fwd(X, layer.Wc_vals, layer.Wc_meta, d_out, Y[:b], T, R)
+    B.slope_linear_bwd_dx(dY, layer.WTc_vals, layer.WTc_meta, d_in, dX[:b], dT, L)
+    layer.poll()
+    assert torch.isnan(Y[b]).all() and torch.isnan(dX[b]).all()
+    assert parity_error(g(Y[:b]), ref_Y) <= REL_TOL
+    assert parity_error(g(dX[:b]), ref_dX) <= REL_TOL
