@@ -2,8 +2,9 @@
 
 Each function has the name of the C entry point it calls (``include/slope.h``), takes
 torch CUDA tensors (bf16 / uint8 / int16 / float32 storage, contiguous) and launches
-on torch's current stream.  Nothing is computed here; if the library is missing the
-import of this module's functions fails loudly -- there is no fallback.
+on torch's current stream.  Nothing is computed here; the calls that take part in a step are
+marshalled by the native module ``_slope`` (``csrc/py_binding.cpp``).  If either library is
+missing the first call fails loudly -- there is no fallback.
 """
 from __future__ import annotations
 
@@ -16,6 +17,7 @@ import torch
 _PKG = Path(__file__).resolve().parent
 _LIB_PATH = _PKG / "libslope.so"
 _lib: Optional[ctypes.CDLL] = None
+_native = None                                       # the module _slope once lib() has attached it to the library
 
 SLOPE_OK = 0
 STATUS_NAMES = {0: "SLOPE_OK", 1: "SLOPE_ERR_INVALID_ARG", 2: "SLOPE_ERR_SHAPE", 3: "SLOPE_ERR_ALIGNMENT",
@@ -44,7 +46,7 @@ class SlopeError(RuntimeError):
 
 def lib() -> ctypes.CDLL:
     """Load libslope.so (built by ``build.build()``); raises if it is not there."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not _LIB_PATH.exists():
             raise RuntimeError(f"{_LIB_PATH} is missing: build it with `python -m paper_2608_24070_b200.build` "
@@ -104,8 +106,20 @@ def lib() -> ctypes.CDLL:
                      "slope_linear_bwd_dw_masked", "slope_adapter_fwd_bwd", "slope_meta_to_canonical",
                      "slope_poll_status"):
             getattr(L, name).restype = ci
+        try:
+            from . import _slope
+        except ImportError as e:
+            raise RuntimeError("the binding's native module _slope.so is missing or does not load: build it with "
+                               f"`python -m paper_2608_24070_b200.build` ({e})") from e
+        _slope.attach(L._handle)
+        _native = _slope
         _lib = L
     return _lib
+
+
+def _calls():
+    lib()
+    return _native
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -145,51 +159,46 @@ def slope_mask_bytes(rows: int, cols: int) -> int:
 
 
 def slope_prune_24(W, Wc_vals, Wc_meta, mask1_bits=None):
-    d_out, d_in = W.shape
-    _check("slope_prune_24", lib().slope_prune_24(_ptr(W), d_out, d_in, _ptr(Wc_vals), _ptr(Wc_meta),
-                                                  _ptr(mask1_bits), _stream()))
+    st = (_native or _calls()).slope_prune_24(W, Wc_vals, Wc_meta, mask1_bits)
+    if st:
+        _check("slope_prune_24", st)
 
 
 def slope_double_prune(W, mask1_bits, WTc_vals, WTc_meta, mask2_bits=None):
-    d_out, d_in = W.shape
-    _check("slope_double_prune", lib().slope_double_prune(_ptr(W), _ptr(mask1_bits), d_out, d_in, _ptr(WTc_vals),
-                                                          _ptr(WTc_meta), _ptr(mask2_bits), _stream()))
+    st = (_native or _calls()).slope_double_prune(W, mask1_bits, WTc_vals, WTc_meta, mask2_bits)
+    if st:
+        _check("slope_double_prune", st)
 
 
 def slope_prune_24_double(W, Wc_vals, Wc_meta, mask1_bits, WTc_vals, WTc_meta, mask2_bits=None):
-    d_out, d_in = W.shape
-    _check("slope_prune_24_double", lib().slope_prune_24_double(_ptr(W), d_out, d_in, _ptr(Wc_vals), _ptr(Wc_meta),
-                                                                _ptr(mask1_bits), _ptr(WTc_vals), _ptr(WTc_meta),
-                                                                _ptr(mask2_bits), _stream()))
+    st = (_native or _calls()).slope_prune_24_double(W, Wc_vals, Wc_meta, mask1_bits, WTc_vals, WTc_meta, mask2_bits)
+    if st:
+        _check("slope_prune_24_double", st)
 
 
 def slope_linear_fwd(X, Wc_vals, Wc_meta, d_out, Y, T=None, R=None):
-    b, d_in = X.shape
-    r = 0 if T is None else T.shape[1]
-    _check("slope_linear_fwd", lib().slope_linear_fwd(_ptr(X), b, _ptr(Wc_vals), _ptr(Wc_meta), d_out, d_in,
-                                                      _ptr(T), _ptr(R), r, _ptr(Y), _stream()))
+    st = (_native or _calls()).slope_linear_fwd(X, Wc_vals, Wc_meta, d_out, Y, T, R)
+    if st:
+        _check("slope_linear_fwd", st)
 
 
 def slope_linear_fwd_adapter(X, Wc_vals, Wc_meta, d_out, L, R, T, Y):
-    """T = X L and Y = X (W^R)^T + T R in one call (a fused pair of launches at inference sizes)."""
-    b, d_in = X.shape
-    _check("slope_linear_fwd_adapter", lib().slope_linear_fwd_adapter(
-        _ptr(X), b, _ptr(Wc_vals), _ptr(Wc_meta), d_out, d_in, _ptr(L), _ptr(R), L.shape[1], _ptr(T), _ptr(Y),
-        _stream()))
+    """T = X L and Y = X (W^R)^T + T R in one call (a fused pair of launches)."""
+    st = (_native or _calls()).slope_linear_fwd_adapter(X, Wc_vals, Wc_meta, d_out, L, R, T, Y)
+    if st:
+        _check("slope_linear_fwd_adapter", st)
 
 
 def slope_linear_bwd_dx(dY, WTc_vals, WTc_meta, d_in, dX, dT=None, L=None):
-    b, d_out = dY.shape
-    r = 0 if dT is None else dT.shape[1]
-    _check("slope_linear_bwd_dx", lib().slope_linear_bwd_dx(_ptr(dY), b, _ptr(WTc_vals), _ptr(WTc_meta), d_out, d_in,
-                                                            _ptr(dT), _ptr(L), r, _ptr(dX), _stream()))
+    st = (_native or _calls()).slope_linear_bwd_dx(dY, WTc_vals, WTc_meta, d_in, dX, dT, L)
+    if st:
+        _check("slope_linear_bwd_dx", st)
 
 
 def slope_linear_bwd_dw_masked(dY, X, mask1_bits, dWc_vals):
-    b, d_out = dY.shape
-    d_in = X.shape[1]
-    _check("slope_linear_bwd_dw_masked", lib().slope_linear_bwd_dw_masked(_ptr(dY), _ptr(X), b, d_out, d_in,
-                                                                          _ptr(mask1_bits), _ptr(dWc_vals), _stream()))
+    st = (_native or _calls()).slope_linear_bwd_dw_masked(dY, X, mask1_bits, dWc_vals)
+    if st:
+        _check("slope_linear_bwd_dw_masked", st)
 
 
 def slope_bwd_dw_adapter_workspace_bytes(b: int, d_out: int, d_in: int, r: int) -> int:
@@ -197,11 +206,9 @@ def slope_bwd_dw_adapter_workspace_bytes(b: int, d_out: int, d_in: int, r: int) 
 
 
 def slope_linear_bwd_dw_adapter(dY, X, T, dT, mask1_bits, dWc_vals, dL, dR, workspace):
-    b, d_out = dY.shape
-    d_in, r = X.shape[1], T.shape[1]
-    _check("slope_linear_bwd_dw_adapter", lib().slope_linear_bwd_dw_adapter(
-        _ptr(dY), _ptr(X), _ptr(T), _ptr(dT), b, d_out, d_in, r, _ptr(mask1_bits), _ptr(dWc_vals), _ptr(dL), _ptr(dR),
-        _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()))
+    st = (_native or _calls()).slope_linear_bwd_dw_adapter(dY, X, T, dT, mask1_bits, dWc_vals, dL, dR, workspace)
+    if st:
+        _check("slope_linear_bwd_dw_adapter", st)
 
 
 def slope_kernel_clock_mhz(kind: int) -> float:
@@ -217,15 +224,13 @@ def slope_adapter_workspace_bytes(b: int, d_out: int, d_in: int, r: int) -> int:
 
 
 def slope_adapter_fwd_bwd(phase, X, dY, L, R, b, d_out, d_in, r, T=None, dT=None, dL=None, dR=None, workspace=None):
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check("slope_adapter_fwd_bwd", lib().slope_adapter_fwd_bwd(
-        phase, _ptr(X), _ptr(dY), _ptr(L), _ptr(R), b, d_out, d_in, r, _ptr(T), _ptr(dT), _ptr(dL), _ptr(dR),
-        _ptr(workspace), ws_bytes, _stream()))
+    st = (_native or _calls()).slope_adapter_fwd_bwd(phase, X, dY, L, R, b, d_out, d_in, r, T, dT, dL, dR, workspace)
+    if st:
+        _check("slope_adapter_fwd_bwd", st)
 
 
 def slope_adapter_dl_noalloc(X, dT, dL):
-    """dL = X^T dT with the split-K scratch in the library's fixed device array (no allocation,
-    no workspace argument).  For callers that are not allowed to allocate GPU memory."""
+    """dL = X^T dT without allocation or workspace.  For callers that are not allowed to allocate GPU memory."""
     b, d_in = X.shape
     r = dT.shape[1]
     _check("slope_adapter_dl_noalloc", lib().slope_adapter_dl_noalloc(_ptr(X), _ptr(dT), b, d_in, r, _ptr(dL),
@@ -237,32 +242,33 @@ def slope_adapter_dl_noalloc_max_scratch_bytes() -> int:
 
 
 def slope_sparse_add(A_vals, B_vals, beta, gamma, out_vals):
-    rows, half = A_vals.shape
-    _check("slope_sparse_add", lib().slope_sparse_add(_ptr(A_vals), _ptr(B_vals), float(beta), float(gamma), rows,
-                                                      half * 2, _ptr(out_vals), _stream()))
+    st = (_native or _calls()).slope_sparse_add(A_vals, B_vals, beta, gamma, out_vals)
+    if st:
+        _check("slope_sparse_add", st)
 
 
 def slope_update_sparse_matrix(Wc_vals, mask1_bits, WTc_meta, WTc_vals):
-    d_out, half = Wc_vals.shape
-    _check("slope_update_sparse_matrix", lib().slope_update_sparse_matrix(
-        _ptr(Wc_vals), _ptr(mask1_bits), _ptr(WTc_meta), d_out, half * 2, _ptr(WTc_vals), _stream()))
+    st = (_native or _calls()).slope_update_sparse_matrix(Wc_vals, mask1_bits, WTc_meta, WTc_vals)
+    if st:
+        _check("slope_update_sparse_matrix", st)
 
 
 def slope_dense_linear_fwd(X, W, Y):
-    (b, d_in), d_out = X.shape, W.shape[0]
-    _check("slope_dense_linear_fwd", lib().slope_dense_linear_fwd(_ptr(X), b, _ptr(W), d_out, d_in, _ptr(Y), _stream()))
+    st = (_native or _calls()).slope_dense_linear_fwd(X, W, Y)
+    if st:
+        _check("slope_dense_linear_fwd", st)
 
 
 def slope_dense_linear_bwd_dx(dY, W, dX):
-    (b, d_out), d_in = dY.shape, W.shape[1]
-    _check("slope_dense_linear_bwd_dx", lib().slope_dense_linear_bwd_dx(_ptr(dY), b, _ptr(W), d_out, d_in, _ptr(dX),
-                                                                        _stream()))
+    st = (_native or _calls()).slope_dense_linear_bwd_dx(dY, W, dX)
+    if st:
+        _check("slope_dense_linear_bwd_dx", st)
 
 
 def slope_dense_linear_bwd_dw(dY, X, dW):
-    (b, d_out), d_in = dY.shape, X.shape[1]
-    _check("slope_dense_linear_bwd_dw", lib().slope_dense_linear_bwd_dw(_ptr(dY), _ptr(X), b, d_out, d_in, _ptr(dW),
-                                                                        _stream()))
+    st = (_native or _calls()).slope_dense_linear_bwd_dw(dY, X, dW)
+    if st:
+        _check("slope_dense_linear_bwd_dw", st)
 
 
 def slope_mask_difference(mask_a, mask_b, count_out):
@@ -272,20 +278,21 @@ def slope_mask_difference(mask_a, mask_b, count_out):
 
 
 def slope_prune_nm(W, n, m, W_R, mask1_bits=None):
-    d_out, d_in = W.shape
-    _check("slope_prune_nm", lib().slope_prune_nm(_ptr(W), d_out, d_in, int(n), int(m), _ptr(W_R), _ptr(mask1_bits),
-                                                  _stream()))
+    st = (_native or _calls()).slope_prune_nm(W, int(n), int(m), W_R, mask1_bits)
+    if st:
+        _check("slope_prune_nm", st)
 
 
 def slope_double_prune_nm(W, mask1_bits, n, m, W_RC, mask2_bits=None):
-    d_out, d_in = W.shape
-    _check("slope_double_prune_nm", lib().slope_double_prune_nm(_ptr(W), _ptr(mask1_bits), d_out, d_in, int(n), int(m),
-                                                                _ptr(W_RC), _ptr(mask2_bits), _stream()))
+    st = (_native or _calls()).slope_double_prune_nm(W, mask1_bits, int(n), int(m), W_RC, mask2_bits)
+    if st:
+        _check("slope_double_prune_nm", st)
 
 
 def slope_apply_mask(G, mask_bits, out):
-    d_out, d_in = G.shape
-    _check("slope_apply_mask", lib().slope_apply_mask(_ptr(G), _ptr(mask_bits), d_out, d_in, _ptr(out), _stream()))
+    st = (_native or _calls()).slope_apply_mask(G, mask_bits, out)
+    if st:
+        _check("slope_apply_mask", st)
 
 
 def slope_meta_to_canonical(meta_hw, rows, cols, meta_canon):

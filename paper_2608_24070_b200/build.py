@@ -1,10 +1,12 @@
-"""Build ``libslope.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Build in-tree: ``libslope.so`` (the C-ABI CUDA library, nvcc for sm_100a) and ``_slope.so`` (the binding's native
+argument marshalling, g++ against torch's headers)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -12,6 +14,8 @@ CSRC = PKG / "csrc"
 LIB = PKG / "libslope.so"
 SOURCES = [CSRC / "slope_lib.cu"]
 HEADERS = sorted(CSRC.glob("*.cuh")) + [PKG.parent / "include" / "slope.h"]
+NATIVE = PKG / "_slope.so"
+NATIVE_SOURCES = [CSRC / "py_binding.cpp", PKG.parent / "include" / "slope.h"]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -27,20 +31,39 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found; cannot build libslope.so")
 
 
-def up_to_date() -> bool:
-    if not LIB.exists():
+def _newer(target: Path, sources) -> bool:
+    if not target.exists():
         return False
-    t = LIB.stat().st_mtime
-    return all(p.stat().st_mtime <= t for p in SOURCES + HEADERS)
+    t = target.stat().st_mtime
+    return all(p.stat().st_mtime <= t for p in sources)
+
+
+def up_to_date() -> bool:
+    return _newer(LIB, SOURCES + HEADERS) and _newer(NATIVE, NATIVE_SOURCES)
+
+
+def _compile(cmd, target: Path) -> None:
+    tmp = target.with_suffix(f".{os.getpid()}.tmp")
+    subprocess.check_call([*cmd, "-o", str(tmp)])
+    os.replace(tmp, target)
+
+
+def native_command():
+    import torch
+
+    root = Path(torch.__file__).resolve().parent
+    cuda = Path(nvcc_path()).resolve().parent.parent
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
+            f"-I{root / 'include'}", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda / 'include'}",
+            str(NATIVE_SOURCES[0]), f"-L{root / 'lib'}", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
-    if not force and up_to_date():
-        return LIB
-    tmp = LIB.with_suffix(f".{os.getpid()}.tmp")
-    cmd = [nvcc_path(), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), "-o", str(tmp), *map(str, SOURCES)]
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    if force or not _newer(LIB, SOURCES + HEADERS):
+        _compile([nvcc_path(), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), *map(str, SOURCES)], LIB)
+    if force or not _newer(NATIVE, NATIVE_SOURCES):
+        _compile(native_command(), NATIVE)
     return LIB
 
 

@@ -23,25 +23,47 @@ static std::atomic<unsigned long long> g_launches{0};
 // ------------------------------------------------------------------ device / driver set-up
 struct DeviceInfo {
     bool ok = false;
+    int dev = 0;
     int sm_count = 0;
     int cc_major = 0;
 };
 
 static DeviceInfo device_info() {
-    static std::mutex mu;
-    static DeviceInfo cache[64];
+    thread_local DeviceInfo cache[64];                       // (per host thread: no lock on every call)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return DeviceInfo{};
-    std::lock_guard<std::mutex> lock(mu);
     if (!cache[dev].ok) {
         cudaDeviceProp prop;
         if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return DeviceInfo{};
-        cache[dev].sm_count = prop.multiProcessorCount;
-        cache[dev].cc_major = prop.major;
-        cache[dev].ok = true;
+        cache[dev] = DeviceInfo{true, dev, prop.multiProcessorCount, prop.major};
     }
     return cache[dev];
 }
+
+// Results of the estimates below, which are pure functions of sizes and of the device: a layer asks for the same ones
+// step after step, and working one out costs the host 0.5 ... 5 us.  A small direct-mapped table per host
+// thread and estimate.
+template <typename V>
+struct SizeMemo {
+    struct Slot {
+        bool valid;
+        int key[6];
+        V value;
+    };
+    Slot slots[64] = {};
+    template <typename Make>
+    const V& get(const int (&key)[6], Make make) {
+        unsigned h = 2166136261u;
+        for (int k : key) h = (h ^ static_cast<unsigned>(k)) * 16777619u;
+        Slot& s = slots[(h ^ (h >> 15)) % 64];
+        if (!s.valid || std::memcmp(s.key, key, sizeof(key)) != 0) {
+            s.value = make();
+            std::memcpy(s.key, key, sizeof(key));
+            s.valid = true;
+        }
+        return s.value;
+    }
+};
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -368,8 +390,10 @@ static slope_status_t launch_adapter(const AdapterOperands& q0, const AdapterOpe
                                      cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
     const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
     const double a_bytes = 2.0 * K * (static_cast<double>(q0.M) + q1.M);
-    return launch_adapter_planned<A_MN, B_MN>(adapter_plan(row_tiles, a_bytes, N, K, info.sm_count), q0, q1, N, K, stream,
-                                              pdl_mode);
+    thread_local SizeMemo<AdapterPlan> memo;
+    const AdapterPlan& plan = memo.get({q0.M, q1.M, N, K, info.sm_count, 0},
+                                       [&] { return adapter_plan(row_tiles, a_bytes, N, K, info.sm_count); });
+    return launch_adapter_planned<A_MN, B_MN>(plan, q0, q1, N, K, stream, pdl_mode);
 }
 
 // dT[b x r] = dY[b x d_out] * R[r x d_out]^T   (both K contiguous)
@@ -566,22 +590,26 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
     auto kern = sparse_gemm_skinny_kernel<BLOCK_N, A_STAGES, B_STAGES>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
 
+    const int slabs = M / kBlockM;
     int cap[9];
     if (!skinny_capacity<BLOCK_N, A_STAGES, B_STAGES>(info, cap)) return SLOPE_ERR_CUDA;
-    if (pdl_mode == 2) {
-        // The consumer of a fused pair has to be resident next to its producer, or its last clusters
-        // would wait for the producer to finish and the overlap would be lost: count only the
-        // clusters that fit beside it.
-        const AdapterPlan producer = adapter_plan((ntok + kBlockM - 1) / kBlockM, 2.0 * ntok * K, r, K, info.sm_count);
-        const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
-        for (int sz = 1; sz <= 8; ++sz) {
-            cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
-            if (cap[sz] < 0) cap[sz] = 0;
+    thread_local SizeMemo<int> memo;                         // (0: nothing fits beside the producer)
+    const int splits = memo.get({M, K, pdl_mode == 2 ? ntok : 0, pdl_mode == 2 ? r : 0, pdl_mode, info.dev}, [&] {
+        if (pdl_mode == 2) {
+            // The consumer of a fused pair has to be resident next to its producer, or its last clusters
+            // would wait for the producer to finish and the overlap would be lost: count only the
+            // clusters that fit beside it.
+            const AdapterPlan producer = adapter_plan((ntok + kBlockM - 1) / kBlockM, 2.0 * ntok * K, r, K, info.sm_count);
+            const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
+            for (int sz = 1; sz <= 8; ++sz) {
+                cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
+                if (cap[sz] < 0) cap[sz] = 0;
+            }
+            if (cap[1] <= 0) return 0;
         }
-        if (cap[1] <= 0) return SLOPE_ERR_CUDA;
-    }
-    const int slabs = M / kBlockM, num_kb = K / 128;
-    const int splits = skinny_splits(slabs, num_kb, BLOCK_N, cap);
+        return skinny_splits(slabs, K / 128, BLOCK_N, cap);
+    });
+    if (splits == 0) return SLOPE_ERR_CUDA;
     return launch_cluster_ex(kern, slabs * splits, splits, kGemmThreads, Cfg::kSmemBytes, true, stream, tmA, tmB,
                              tmE, tmA2, tmB2, p);
 }
@@ -608,7 +636,8 @@ static slope_status_t launch_skinny(const void* act, int ntok, const void* vals,
                                     const void* act2, const void* fac2, int r, bool a2_mn, void* out,
                                     cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
     if (ntok <= 16) {
-        if (prefer_two_ctas_per_sm<16, 10, 4, 5, 2>(M, K, info))
+        thread_local SizeMemo<bool> memo;
+        if (memo.get({M, K, info.dev, 0, 0, 0}, [&] { return prefer_two_ctas_per_sm<16, 10, 4, 5, 2>(M, K, info); }))
             return launch_sparse_skinny<16, 5, 2>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
         return launch_sparse_skinny<16, 10, 4>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
     }
@@ -704,16 +733,9 @@ struct FwdAdapterPlan {
     int pairs;                    // CTA pairs of the forward
 };
 static FwdAdapterPlan plan_fwd_adapter(int b, int d_out, int d_in, int r, const DeviceInfo& info) {
-    struct Memo {
-        int b, d_out, d_in, r, sm_count;
-        FwdAdapterPlan plan;
-    };
-    thread_local Memo memo[64] = {};                                   // a pure function of sizes
-    Memo& m = memo[(b * 31u + d_out / 128 * 7u + d_in / 128 * 3u + r / 16u) % 64];
-    if (m.b == b && m.d_out == d_out && m.d_in == d_in && m.r == r && m.sm_count == info.sm_count) return m.plan;
     const int row_tiles = (b + kBlockM - 1) / kBlockM;
     constexpr double kClkPerUs = 1850.0;
-    FwdAdapterPlan best{};
+    FwdAdapterPlan best{};                                  // (no tile rows: the few-token kernel)
     best.pairs = info.sm_count / 2;
     double best_us = 1e300, cost = 0.0;
     if (use_few_token_kernel(d_out, d_in, b, r, info)) {                // its K-split is chosen around the producer
@@ -742,8 +764,11 @@ static FwdAdapterPlan plan_fwd_adapter(int b, int d_out, int d_in, int r, const 
             }
         });
     }
-    m = Memo{b, d_out, d_in, r, info.sm_count, best};
     return best;
+}
+static FwdAdapterPlan fwd_adapter_plan(int b, int d_out, int d_in, int r, const DeviceInfo& info) {
+    thread_local SizeMemo<FwdAdapterPlan> memo;
+    return memo.get({b, d_out, d_in, r, info.dev, 0}, [&] { return plan_fwd_adapter(b, d_out, d_in, r, info); });
 }
 
 // T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
@@ -756,11 +781,13 @@ static slope_status_t launch_adapter_T(const FwdAdapterPlan& plan, const void* X
 static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                                          const void* act2, const void* fac2, int r, bool a2_mn, void* out,
                                          cudaStream_t stream, const DeviceInfo& info) {
-    if (use_few_token_kernel(M, K, ntok, r, info))
-        return launch_skinny(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info);
     const int pairs = info.sm_count / 2;
-    return launch_sparse_tile(choose_sparse_tile(M, K, ntok, r, pairs), act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out,
-                              pairs, stream, 0);
+    thread_local SizeMemo<SparseTile> memo;                  // (no rows: the few-token kernel)
+    const SparseTile& t = memo.get({M, K, ntok, r, info.dev, 0}, [&] {
+        return use_few_token_kernel(M, K, ntok, r, info) ? SparseTile{0, 0} : choose_sparse_tile(M, K, ntok, r, pairs);
+    });
+    if (t.rows == 0) return launch_skinny(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info);
+    return launch_sparse_tile(t, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, pairs, stream, 0);
 }
 
 template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
@@ -934,9 +961,9 @@ slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_val
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    const FwdAdapterPlan plan = plan_fwd_adapter(b, d_out, d_in, r, info);
+    const FwdAdapterPlan plan = fwd_adapter_plan(b, d_out, d_in, r, info);
     if (slope_status_t st = launch_adapter_T(plan, X, L, b, d_in, r, T, stream, 1)) return st;
-    if (use_few_token_kernel(d_out, d_in, b, r, info)) {
+    if (plan.tile.rows == 0) {
         // Two launches of the few-token kernel as a fused pair: T = X L releases its dependent only
         // once everything before it in the stream is complete, so the forward streams its weights
         // and runs its sparse reduction while T is still being computed, and waits only for T.
@@ -1039,7 +1066,7 @@ slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, c
         if (!X || !L || !T) return SLOPE_ERR_INVALID_ARG;
         if (!aligned16(X) || !aligned16(L) || !aligned16(T)) return SLOPE_ERR_ALIGNMENT;
         if (slope_status_t st = check_arch(info)) return st;
-        return launch_adapter_T(plan_fwd_adapter(b, d_out, d_in, r, info), X, L, b, d_in, r, T, stream, 0);
+        return launch_adapter_T(fwd_adapter_plan(b, d_out, d_in, r, info), X, L, b, d_in, r, T, stream, 0);
     }
     if (phase == 2) {
         if (!dY || !R || !dT) return SLOPE_ERR_INVALID_ARG;
