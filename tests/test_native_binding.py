@@ -1,4 +1,4 @@
-"""The binding's native marshalling refuses what it cannot hand to the C ABI, before anything is launched (no GPU)."""
+"""The binding's native marshalling refuses what it cannot hand to the C ABI, before anything is launched."""
 import pytest
 import torch
 
@@ -29,6 +29,7 @@ def test_arguments_of_the_wrong_kind(B):
         B.slope_adapter_fwd_bwd(1 << 40, None, None, None, None, 1, 128, 128, 16)
 
 
+@pytest.mark.gpu
 def test_statuses_of_the_library_become_errors(B):
     with pytest.raises(B.SlopeError) as e:                       # all pointers missing: refused by the argument checks
         B.slope_adapter_fwd_bwd(0, None, None, None, None, 1, 128, 128, 16)
