@@ -104,7 +104,7 @@ slope_status_t slope_prune_24_double(const void* W, int d_out, int d_in,
  * With few tokens (inference, decode: the paper's forward-only inference measurements; always up
  * to 16 tokens, up to 128 where it is estimated faster than the tile kernels) the same call
  * runs on a kernel that streams the compressed weight once from HBM and splits the
- * reduction over a thread-block cluster.  All GEMM launches of this library are issued with
+ * reduction over a thread-block cluster.  The compute launches of this library are issued with
  * programmatic stream serialisation (their set-up may overlap the previous kernel's tail) and
  * synchronise on the device before they touch memory (the second launch of
  * slope_linear_fwd_adapter relies on its first one having done so and waits only for that one's

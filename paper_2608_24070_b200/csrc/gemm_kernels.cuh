@@ -112,8 +112,8 @@ constexpr int kDenseThreads = 64 + 32 * kDenseEpiWarps;
 // A row's mask bits of `cols` (64 or 128) columns, fetched before the accumulator is ready: loaded where they are
 // used, 16 columns at a time, every load put an L2 round trip into the drain.
 __device__ __forceinline__ uint4 load_mask_bits(const uint8_t* row, int cols) {
-    if (cols == 128) return __ldg(reinterpret_cast<const uint4*>(row));
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(row));
+    if (cols == 128) return ld_v4(row);
+    const uint2 v = ld_v2(row);
     return make_uint4(v.x, v.y, 0u, 0u);
 }
 

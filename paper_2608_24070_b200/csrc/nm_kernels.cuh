@@ -55,13 +55,14 @@ template <int M>
 __global__ void __launch_bounds__(256)
 prune_nm_kernel(const uint4* W, size_t n_chunks, int n, uint4* out, uint16_t* __restrict__ mask) {
     constexpr int kChunks = M == 16 ? 2 : 1;
+    griddep_stream();
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t t0 = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; t0 < n_chunks / kChunks; t0 += stride) {
         const size_t c = kChunks == 1 ? t0 : (t0 & ~size_t(31)) * 2 + (t0 & 31);
         uint32_t w[8 * kChunks];
 #pragma unroll
         for (int k = 0; k < kChunks; ++k) {
-            const uint4 a = __ldcs(W + 2 * (c + 32 * k)), b = __ldcs(W + 2 * (c + 32 * k) + 1);       // streamed: read once
+            const uint4 a = ld_stream_v4(W + 2 * (c + 32 * k)), b = ld_stream_v4(W + 2 * (c + 32 * k) + 1);
             w[8 * k] = a.x; w[8 * k + 1] = a.y; w[8 * k + 2] = a.z; w[8 * k + 3] = a.w;
             w[8 * k + 4] = b.x; w[8 * k + 5] = b.y; w[8 * k + 6] = b.z; w[8 * k + 7] = b.w;
         }
@@ -104,23 +105,25 @@ prune_nm_kernel(const uint4* W, size_t n_chunks, int n, uint4* out, uint16_t* __
 // 512 contiguous bytes of a row) or 16 rows x 4 columns (8-byte loads; two neighbours share a mask byte), which
 // keeps the registers of the 16-row pattern under 128; output in the same orientation.  mask2 = kept by
 // both passes.  `out` may be `W` itself.
+// (Ordinary loads through unrestricted pointers: they stay behind griddep_stream(), and unlike volatile ones the
+// compiler may place them, without which the kernel spills.)
 template <int WORDS>
 __device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&w)[WORDS]) {
     if constexpr (WORDS == 4) {
-        const uint4 v = __ldcs(reinterpret_cast<const uint4*>(p));
+        const uint4 v = *reinterpret_cast<const uint4*>(p);
         w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
     } else {
-        const uint2 v = __ldcs(reinterpret_cast<const uint2*>(p));
+        const uint2 v = *reinterpret_cast<const uint2*>(p);
         w[0] = v.x; w[1] = v.y;
     }
 }
 template <int M>
 __global__ void __launch_bounds__(256, M == 16 ? 2 : M == 8 ? 3 : 4)
-double_prune_nm_kernel(const uint4* W, const uint8_t* __restrict__ mask1, int d_out, int d_in, int n,
-                       uint4* out, uint8_t* __restrict__ mask2) {
+double_prune_nm_kernel(const uint4* W, const uint8_t* mask1, int d_out, int d_in, int n, uint4* out, uint8_t* mask2) {
     constexpr int kWords = M == 16 ? 2 : 4;
     const int per_row = d_in / (2 * kWords);                   // threads per row: a multiple of 32
     const size_t total = static_cast<size_t>(d_out / M) * per_row;
+    griddep_stream();
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total; idx += stride) {
         const size_t h = idx / per_row, c = idx % per_row;
@@ -173,11 +176,12 @@ double_prune_nm_kernel(const uint4* W, const uint8_t* __restrict__ mask1, int d_
 // N:M pattern).  A thread owns 16 consecutive entries; `out` may be `G` itself.
 __global__ void __launch_bounds__(256)
 apply_mask_kernel(const uint4* G, const uint16_t* __restrict__ mask, size_t n_chunks, uint4* out) {
+    griddep_stream();
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t c = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; c < n_chunks; c += stride) {
-        const uint4 a = __ldcs(G + 2 * c), b = __ldcs(G + 2 * c + 1);
+        const uint4 a = ld_stream_v4(G + 2 * c), b = ld_stream_v4(G + 2 * c + 1);
         uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        const uint32_t keep = mask[c];
+        const uint32_t keep = ld_u16(mask + c);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const uint32_t lo = (keep >> (2 * q)) & 1u ? 0x0000FFFFu : 0u;

@@ -81,13 +81,14 @@ __global__ void __launch_bounds__(256) prune24_kernel(const uint4* __restrict__ 
     const int u = tid & 7, r0 = tid >> 3;                 // 16-column slot, row within a pass of 32 rows
     const size_t row_u4 = static_cast<size_t>(d_in) >> 3;
 
+    griddep_stream();
     uint4 w[4][2];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const size_t row = static_cast<size_t>(rb) * 128 + i * 32 + r0;
         const uint4* src = W + row * row_u4 + cb * 16 + 2 * u;
-        w[i][0] = __ldg(src);
-        w[i][1] = __ldg(src + 1);
+        w[i][0] = ld_v4(src);
+        w[i][1] = ld_v4(src + 1);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -140,13 +141,14 @@ __global__ void __launch_bounds__(256, 4) double_prune_kernel(const uint4* __res
     const size_t row_u4 = static_cast<size_t>(d_in) >> 3;
     const size_t mrow = static_cast<size_t>(d_in) >> 3;      // mask bytes per row
 
+    griddep_stream();
     uint4 w[8];
     uint32_t mb[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const size_t row = static_cast<size_t>(rb) * 128 + ig * 8 + t;
-        w[t] = __ldg(W + row * row_u4 + cb * 16 + c8);
-        mb[t] = __ldg(mask1 + row * mrow + cb * 16 + c8);
+        w[t] = ld_v4(W + row * row_u4 + cb * 16 + c8);
+        mb[t] = ld_u8(mask1 + row * mrow + cb * 16 + c8);
     }
 
     uint32_t sel_bits[8] = {0, 0, 0, 0, 0, 0, 0, 0};         // per row: which of the 8 columns the second pass keeps
@@ -226,9 +228,10 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
     const size_t mrow = static_cast<size_t>(d_in) >> 3;      // mask bytes (= uint2 of values) per row
     const size_t at0 = (static_cast<size_t>(rb) * 128 + ig * 8) * row_u4 + cb * 16 + c8;
 
+    griddep_stream();
     uint4 w[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) w[t] = __ldg(W + at0 + t * row_u4);
+    for (int t = 0; t < 8; ++t) w[t] = ld_v4(W + at0 + t * row_u4);
 
     // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place
     uint32_t mb[8];
@@ -321,9 +324,10 @@ __global__ void __launch_bounds__(256) meta_to_canonical_kernel(const uint16_t* 
 // `out` may be A or B (every thread reads its vectors before it writes them), hence no __restrict__.
 __global__ void __launch_bounds__(256) sparse_add_kernel(const uint4* A, const uint4* B, float beta, float gamma,
                                                          size_t n_vec, uint4* out) {
+    griddep_stream();
     for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < n_vec;
          idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const uint4 a = A[idx], b = B[idx];
+        const uint4 a = ld_v4(A + idx), b = ld_v4(B + idx);
         const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
         uint32_t r[4];
 #pragma unroll
@@ -381,6 +385,7 @@ update_transposed_kernel(const uint2* __restrict__ Wc_new, const uint8_t* __rest
     const int num_tiles = ncb * nrb;
 
     if (tid < 16) s_expand[tid] = make_uint2(expand_selector(tid), expand_selector(tid) >> 16);
+    griddep_stream();
 
     uint2 cw[8];
     uint32_t mb[8];
@@ -389,10 +394,10 @@ update_transposed_kernel(const uint2* __restrict__ Wc_new, const uint8_t* __rest
         const uint32_t at = (static_cast<uint32_t>(rb) * 128u + ig * 8u) * row_u2 + cb * 16u + c8;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            cw[t] = __ldg(Wc_new + (at + t * row_u2));
-            mb[t] = __ldg(mask1 + (at + t * row_u2));
+            cw[t] = ld_v2(Wc_new + (at + t * row_u2));
+            mb[t] = ld_u8(mask1 + (at + t * row_u2));
         }
-        if (tid < 128) m = __ldg(metaT + ((static_cast<uint32_t>(cb) * nrb + rb) * 128u + tid));
+        if (tid < 128) m = ld_v4(metaT + ((static_cast<uint32_t>(cb) * nrb + rb) * 128u + tid));
     };
 
     // tile = blockIdx.x, blockIdx.x + gridDim.x, ...: (cb, rb) advance without a division per tile

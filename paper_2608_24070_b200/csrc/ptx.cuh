@@ -227,6 +227,13 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
 // on has finished and its writes are visible (no-op for an ordinary launch);
 // `griddep_launch_dependents` lets a dependent launch that opted in begin its own prologue.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch_dependents();
+// The start of a streaming kernel: its blocks are set up while the preceding kernel drains, and the next kernel's
+// blocks move in as this one's leave.
+__device__ __forceinline__ void griddep_stream() {
+    griddep_launch_dependents();
+    griddep_wait();
+}
 __device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float4 ld_shared_v4(uint32_t saddr) {
@@ -237,6 +244,36 @@ __device__ __forceinline__ float4 ld_shared_v4(uint32_t saddr) {
                  : "memory");
     return v;
 }
+// Global loads of kernels launched with programmatic stream serialisation.  Ordinary loads through const __restrict__
+// pointers (or __ldg) may be moved up past griddep_wait(), behind which alone the preceding kernel's writes
+// are visible; volatile asm statements stay in order.
+__device__ __forceinline__ uint4 ld_v4(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_v2(const void* p) {
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_u8(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_u16(const void* p) {
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+// streamed: read once
+__device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // Read four consecutive fp32 (16-byte aligned) from the shared memory of a CTA of the cluster.
 __device__ __forceinline__ float4 ld_shared_cluster_v4(uint32_t cluster_saddr) {
     float4 v;

@@ -277,9 +277,32 @@ static bool set_smem(Kernel k, int bytes) {
     return true;
 }
 
+// Streaming kernels are launched with programmatic stream serialisation too: every thread waits for the preceding
+// kernel before it touches memory (griddep_stream), but the blocks are already resident, and the ramp-up and
+// tail of back-to-back passes overlap.
+template <typename... KArgs, typename... Args>
+static slope_status_t launch_stream(void (*kern)(KArgs...), dim3 grid, cudaStream_t stream, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? SLOPE_OK : SLOPE_ERR_CUDA;
+}
+
 // Grid of the grid-stride streaming kernels: many short blocks per SM keep the tail of the last
 // wave short (masked copy of a 90 MB matrix: 78 % of the HBM peak with 8 blocks per SM, 91 % with 32).
 constexpr int kStreamBlocksPerSm = 32;
+static unsigned stream_grid(size_t threads, const DeviceInfo& info) {
+    const size_t blocks = (threads + 255) / 256, most = static_cast<size_t>(info.sm_count) * kStreamBlocksPerSm;
+    return static_cast<unsigned>(blocks < most ? blocks : most);
+}
 
 // ------------------------------------------------------------------ dense GEMM launch
 static slope_status_t launch_dense_masked(const void* dY, const void* X, int M, int N, int K, void* out, const void* mask,
@@ -897,10 +920,9 @@ slope_status_t slope_prune_24(const void* W, int d_out, int d_in, void* Wc_vals,
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     dim3 grid(d_in / 128, d_out / 128);
-    prune24_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+    return launch_stream(prune24_kernel, grid, static_cast<cudaStream_t>(stream),
         static_cast<const uint4*>(W), d_out, d_in, static_cast<uint4*>(Wc_vals), static_cast<uint4*>(Wc_meta),
         static_cast<uint4*>(mask1_bits));
-    return launch_result();
 }
 
 slope_status_t slope_double_prune(const void* W, const void* mask1_bits, int d_out, int d_in, void* WTc_vals,
@@ -913,10 +935,9 @@ slope_status_t slope_double_prune(const void* W, const void* mask1_bits, int d_o
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     dim3 grid(d_in / 128, d_out / 128);
-    double_prune_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+    return launch_stream(double_prune_kernel, grid, static_cast<cudaStream_t>(stream),
         static_cast<const uint4*>(W), static_cast<const uint8_t*>(mask1_bits), d_out, d_in,
         static_cast<uint4*>(WTc_vals), static_cast<uint4*>(WTc_meta), static_cast<uint8_t*>(mask2_bits));
-    return launch_result();
 }
 
 slope_status_t slope_prune_24_double(const void* W, int d_out, int d_in, void* Wc_vals, void* Wc_meta,
@@ -929,11 +950,10 @@ slope_status_t slope_prune_24_double(const void* W, int d_out, int d_in, void* W
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     dim3 grid(d_in / 128, d_out / 128);
-    prune24_double_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+    return launch_stream(prune24_double_kernel, grid, static_cast<cudaStream_t>(stream),
         static_cast<const uint4*>(W), d_out, d_in, static_cast<uint2*>(Wc_vals), static_cast<uint4*>(Wc_meta),
         static_cast<uint4*>(mask1_bits), static_cast<uint4*>(WTc_vals), static_cast<uint4*>(WTc_meta),
         static_cast<uint8_t*>(mask2_bits));
-    return launch_result();
 }
 
 slope_status_t slope_linear_fwd(const void* X, int b, const void* Wc_vals, const void* Wc_meta, int d_out, int d_in,
@@ -1188,10 +1208,9 @@ slope_status_t slope_sparse_add(const void* A_vals, const void* B_vals, float be
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     const size_t n_vec = static_cast<size_t>(rows) * cols / 2 / 8;
-    sparse_add_kernel<<<info.sm_count * kStreamBlocksPerSm, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint4*>(A_vals), static_cast<const uint4*>(B_vals), beta, gamma, n_vec,
-        static_cast<uint4*>(out_vals));
-    return launch_result();
+    return launch_stream(sparse_add_kernel, dim3(stream_grid(n_vec, info)), static_cast<cudaStream_t>(stream),
+                         static_cast<const uint4*>(A_vals), static_cast<const uint4*>(B_vals), beta, gamma, n_vec,
+                         static_cast<uint4*>(out_vals));
 }
 
 slope_status_t slope_update_sparse_matrix(const void* Wc_vals, const void* mask1_bits, const void* WTc_meta,
@@ -1205,10 +1224,9 @@ slope_status_t slope_update_sparse_matrix(const void* Wc_vals, const void* mask1
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     const int tiles = (d_in / 128) * (d_out / 128), slots = info.sm_count * kUpdateBlocksPerSm;
-    update_transposed_kernel<<<tiles < slots ? tiles : slots, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint2*>(Wc_vals), static_cast<const uint8_t*>(mask1_bits),
-        static_cast<const uint4*>(WTc_meta), d_out, d_in, static_cast<uint4*>(WTc_vals));
-    return launch_result();
+    return launch_stream(update_transposed_kernel, dim3(tiles < slots ? tiles : slots), static_cast<cudaStream_t>(stream),
+                         static_cast<const uint2*>(Wc_vals), static_cast<const uint8_t*>(mask1_bits),
+                         static_cast<const uint4*>(WTc_meta), d_out, d_in, static_cast<uint4*>(WTc_vals));
 }
 
 // ------------------------------------------------------------------ general N:M (masked dense)
@@ -1223,17 +1241,12 @@ slope_status_t slope_prune_nm(const void* W, int d_out, int d_in, int n, int m, 
     if (slope_status_t st = check_arch(info)) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const size_t chunks = static_cast<size_t>(d_out) * d_in / 16;
-    const int grid = info.sm_count * kStreamBlocksPerSm;
     const uint4* in = static_cast<const uint4*>(W);
     uint4* out = static_cast<uint4*>(W_R);
     uint16_t* mask = static_cast<uint16_t*>(mask1_bits);
-    switch (m) {
-        case 2: prune_nm_kernel<2><<<grid, 256, 0, stream>>>(in, chunks, n, out, mask); break;
-        case 4: prune_nm_kernel<4><<<grid, 256, 0, stream>>>(in, chunks, n, out, mask); break;
-        case 8: prune_nm_kernel<8><<<grid, 256, 0, stream>>>(in, chunks, n, out, mask); break;
-        default: prune_nm_kernel<16><<<grid, 256, 0, stream>>>(in, chunks, n, out, mask); break;
-    }
-    return launch_result();
+    const dim3 grid(stream_grid(m == 16 ? chunks / 2 : chunks, info));
+    auto kern = m == 2 ? prune_nm_kernel<2> : m == 4 ? prune_nm_kernel<4> : m == 8 ? prune_nm_kernel<8> : prune_nm_kernel<16>;
+    return launch_stream(kern, grid, stream, in, chunks, n, out, mask);
 }
 
 slope_status_t slope_double_prune_nm(const void* W, const void* mask1_bits, int d_out, int d_in, int n, int m,
@@ -1245,18 +1258,14 @@ slope_status_t slope_double_prune_nm(const void* W, const void* mask1_bits, int 
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    const int grid = info.sm_count * kStreamBlocksPerSm;
     const uint4* in = static_cast<const uint4*>(W);
     const uint8_t* m1 = static_cast<const uint8_t*>(mask1_bits);
     uint4* out = static_cast<uint4*>(W_RC);
     uint8_t* m2 = static_cast<uint8_t*>(mask2_bits);
-    switch (m) {
-        case 2: double_prune_nm_kernel<2><<<grid, 256, 0, stream>>>(in, m1, d_out, d_in, n, out, m2); break;
-        case 4: double_prune_nm_kernel<4><<<grid, 256, 0, stream>>>(in, m1, d_out, d_in, n, out, m2); break;
-        case 8: double_prune_nm_kernel<8><<<grid, 256, 0, stream>>>(in, m1, d_out, d_in, n, out, m2); break;
-        default: double_prune_nm_kernel<16><<<grid, 256, 0, stream>>>(in, m1, d_out, d_in, n, out, m2); break;
-    }
-    return launch_result();
+    const dim3 grid(stream_grid(static_cast<size_t>(d_out / m) * (d_in / (m == 16 ? 4 : 8)), info));
+    auto kern = m == 2 ? double_prune_nm_kernel<2> : m == 4 ? double_prune_nm_kernel<4>
+                                                   : m == 8 ? double_prune_nm_kernel<8> : double_prune_nm_kernel<16>;
+    return launch_stream(kern, grid, stream, in, m1, d_out, d_in, n, out, m2);
 }
 
 slope_status_t slope_apply_mask(const void* G, const void* mask_bits, int d_out, int d_in, void* out, void* stream) {
@@ -1265,10 +1274,9 @@ slope_status_t slope_apply_mask(const void* G, const void* mask_bits, int d_out,
     if (!aligned16(G) || !aligned16(mask_bits) || !aligned16(out)) return SLOPE_ERR_ALIGNMENT;
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
-    apply_mask_kernel<<<info.sm_count * kStreamBlocksPerSm, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint4*>(G), static_cast<const uint16_t*>(mask_bits),
-        static_cast<size_t>(d_out) * d_in / 16, static_cast<uint4*>(out));
-    return launch_result();
+    const size_t chunks = static_cast<size_t>(d_out) * d_in / 16;
+    return launch_stream(apply_mask_kernel, dim3(stream_grid(chunks, info)), static_cast<cudaStream_t>(stream),
+                         static_cast<const uint4*>(G), static_cast<const uint16_t*>(mask_bits), chunks, static_cast<uint4*>(out));
 }
 
 slope_status_t slope_mask_difference(const void* mask_a, const void* mask_b, int rows, int cols, void* count_out,
@@ -1282,7 +1290,7 @@ slope_status_t slope_mask_difference(const void* mask_a, const void* mask_b, int
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (cudaMemsetAsync(count_out, 0, sizeof(unsigned long long), stream) != cudaSuccess) return SLOPE_ERR_CUDA;
     const size_t n_vec = static_cast<size_t>(rows) * cols / 8 / 16;
-    mask_difference_kernel<<<info.sm_count * kStreamBlocksPerSm, 256, 0, stream>>>(
+    mask_difference_kernel<<<stream_grid(n_vec, info), 256, 0, stream>>>(
         static_cast<const uint4*>(mask_a), static_cast<const uint4*>(mask_b), n_vec,
         static_cast<unsigned long long*>(count_out));
     return launch_result();
