@@ -1,4 +1,4 @@
-"""Sparse forward and input gradient over every token-tile width of the tile kernels (32 ... 224 in steps of 32, both
+"""Sparse forward and input gradient: the few-token kernel where it does not split, every token-tile width of the tile kernels (32 ... 224 in steps of 32, both
 row counts), ragged last tiles and row tiles that are half empty, with and without adapters; the fused
 forward against the separate calls.
 
@@ -14,6 +14,11 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("b,d_in,d_out,r", [
+    (1, 128, 384, 0),            # few-token kernel without a split: one k-block, one token
+    (5, 128, 256, 16),
+    (16, 256, 19200, 0),         # more slabs than SMs
+    (17, 128, 640, 64),
+    (128, 256, 512, 32),
     (129, 256, 384, 0),          # narrowest tiles, last row tile half empty
     (161, 1024, 256, 16),
     (250, 640, 1920, 0),
