@@ -120,7 +120,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             PipeState ps, ps2;
             bool ok = true;
             PairWork w;
-            for (int item = pair_id; ok && pair_work<BLOCK_N, true>(item, num_pairs, num_m, num_n, w); item += num_pairs) {
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w); item += num_pairs) {
                 bool carry_r, carry_l;
                 int n_blk;
                 carries(w, carry_r, carry_l, n_blk);
@@ -166,7 +166,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             bool ok = true;
             int it = 0;
             PairWork w;
-            for (int item = pair_id; ok && pair_work<BLOCK_N, true>(item, num_pairs, num_m, num_n, w);
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w);
                  item += num_pairs, ++it) {
                 bool carry_r, carry_l;
                 int n_blk;
@@ -225,7 +225,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         bool ok = true;
         int it = 0;
         PairWork w;
-        for (int item = pair_id; ok && pair_work<BLOCK_N, true>(item, num_pairs, num_m, num_n, w); item += num_pairs, ++it) {
+        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w); item += num_pairs, ++it) {
             bool carry_r, carry_l;
             int n_blk;
             carries(w, carry_r, carry_l, n_blk);

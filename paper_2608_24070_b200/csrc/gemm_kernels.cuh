@@ -6,9 +6,10 @@
 // wait is bounded (ptx.cuh); a role that gives up sets a CTA-wide flag, all roles leave their
 // loops, tensor memory is released and the kernel returns.
 //
-//   dense_gemm_kernel          1 CTA per 128 x 128 tile; dW of the smallest weight matrices
-//   dense_gemm_pair_kernel     CTA pair per 256 x 256 tile (cta_group::2), the last wave's tiles
-//                              halved; dW (masked epilogue) and the dense layer (store epilogue)
+//   dense_gemm_kernel          1 CTA per 128 x 128 tile; the same products while they are small
+//   dense_gemm_pair_kernel     CTA pair per tile of 256 rows x 64 ... 256 columns (cta_group::2), a
+//                              half-empty last wave's tiles halved; dW (masked epilogue) and the dense
+//                              layer (store epilogue)
 //   sparse_gemm_pair_kernel    CTA pair per tile of 256 rows x 32 ... 224 tokens, tcgen05.mma.sp;
 //                              forward / dX with short reductions or few tiles
 //   sparse_gemm_quad_kernel    CTA pair per tile of 512 rows x 32 ... 224 tokens (two MMA sub-tiles per
@@ -87,6 +88,8 @@ constexpr int kEpiStore = 0, kEpiMasked = 1;
 
 struct DenseGemmParams {
     int M, N, K;
+    int width;                    // columns per tile: 64, 128, 192 or 256
+    int stages;                   // pipeline stages that fit at that width
     void* out;
     const uint8_t* mask;          // kEpiMasked: [M x N/8]
 };
@@ -109,36 +112,69 @@ __device__ __forceinline__ uint4 compress_16(const uint32_t (&v)[16], uint32_t m
 constexpr int kDenseEpiWarps = 8;
 constexpr int kDenseThreads = 64 + 32 * kDenseEpiWarps;
 
-// A row's mask bits of `cols` (64 or 128) columns, fetched before the accumulator is ready: loaded where they are
+// A row's mask bits of `cols` (32, 64 or 128) columns, fetched before the accumulator is ready: loaded where they are
 // used, 16 columns at a time, every load put an L2 round trip into the drain.
-__device__ __forceinline__ uint4 load_mask_bits(const uint8_t* row, int cols) {
-    if (cols == 128) return ld_v4(row);
-    const uint2 v = ld_v2(row);
-    return make_uint4(v.x, v.y, 0u, 0u);
-}
-
-// Drains `cols` (64 or 128) accumulator columns of this thread's row, 64 at a time, so that the tensor-memory loads
-// share one wait.  With few tokens the drain, not the main loop, paces the kernel (double-buffered
-// accumulators): four warps that took 16 columns at a time, a mask load and a wait each, needed ~9 us
-// for a 256 x 256 tile; as it is, 4096 x 4096 with 300 tokens went from 43 to 13 us, 8320 -> 6400 with
-// 740 from 141 to 58, 512 x 512 with 256 from 7.8 to 3.0 (16384 tokens: unchanged).
-__device__ __forceinline__ void drain_masked(uint32_t t_row, int cols, const uint4& bits, uint16_t* dst) {
-    const uint32_t mw[4] = {bits.x, bits.y, bits.z, bits.w};
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        if (64 * i < cols) {
-            uint32_t v[4][16];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) tmem_ld_16(t_row + 64 * i + 16 * k, v[k]);
-            tmem_ld_wait();
-            uint4* d = reinterpret_cast<uint4*>(dst + 32 * i);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = compress_16(v[k], mw[2 * i + (k >> 1)] >> (16 * (k & 1)));
-        }
+__device__ __forceinline__ void load_mask_bits(const uint8_t* row, int cols, uint32_t (&mw)[4]) {
+    if (cols == 128) {
+        const uint4 v = ld_v4(row);
+        mw[0] = v.x; mw[1] = v.y; mw[2] = v.z; mw[3] = v.w;
+    } else if (cols == 64) {
+        const uint2 v = ld_v2(row);
+        mw[0] = v.x; mw[1] = v.y;
+    } else {
+        mw[0] = ld_u32(row);
     }
 }
 
-// Masked weight gradient of the smallest weight matrices: one 128 x 128 tile per CTA.
+// Drains `cols` accumulator columns of this thread's row, up to 64 at a time, so that the tensor-memory loads share one
+// wait.  With few tokens the drain, not the main loop, paces the kernel (double-buffered accumulators): four
+// warps that took 16 columns at a time, a mask load and a wait each, needed ~9 us for a 256 x 256 tile; as
+// it is, 4096 x 4096 with 300 tokens went from 43 to 13 us, 8320 -> 6400 with 740 from 141 to 58, 512 x 512
+// with 256 from 7.8 to 3.0 (16384 tokens: unchanged).
+template <int COLS, typename Store>
+__device__ __forceinline__ void drain_block(uint32_t t_row, int first, Store store) {
+    uint32_t v[COLS / 16][16];
+#pragma unroll
+    for (int k = 0; k < COLS / 16; ++k) tmem_ld_16(t_row + 16 * (first + k), v[k]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < COLS / 16; ++k) store(first + k, v[k]);
+}
+template <typename Store>
+__device__ __forceinline__ void drain_columns(uint32_t t_row, int cols, Store store) {
+    if (cols >= 64) drain_block<64>(t_row, 0, store);
+    if (cols == 128) drain_block<64>(t_row, 4, store);
+    else if (cols == 96) drain_block<32>(t_row, 4, store);
+    else if (cols == 32) drain_block<32>(t_row, 0, store);
+}
+
+// Writes `cols` drained accumulator columns of output row m from column n0 on, as bf16 (kEpiStore; rows past M take part
+// in the warp-wide tensor-memory loads, but store nothing) or the half that the mask bits select (kEpiMasked).
+template <int EPI>
+__device__ __forceinline__ void drain_row(uint32_t t_row, int cols, const DenseGemmParams& p, int m, int n0, const uint32_t (&mw)[4]) {
+    if (EPI == kEpiMasked) {
+        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1));
+        drain_columns(t_row, cols, [&](int c, const uint32_t (&v)[16]) { dst[c] = compress_16(v, mw[c >> 1] >> (16 * (c & 1))); });
+    } else {
+        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.N + n0);
+        drain_columns(t_row, cols, [&](int c, const uint32_t (&v)[16]) {
+            if (m >= p.M) return;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t* e = v + 8 * k;
+                dst[2 * c + k] = make_uint4(pack_bf16x2(__uint_as_float(e[0]), __uint_as_float(e[1])),
+                                            pack_bf16x2(__uint_as_float(e[2]), __uint_as_float(e[3])),
+                                            pack_bf16x2(__uint_as_float(e[4]), __uint_as_float(e[5])),
+                                            pack_bf16x2(__uint_as_float(e[6]), __uint_as_float(e[7])));
+            }
+        });
+    }
+}
+
+// Dense GEMM with one 128 x 128 tile per CTA, for products whose tiles all run at once and whose reduction is short: no
+// cluster to launch and to synchronise.  us, against the best width of the CTA-pair kernel: masked weight
+// gradient 512 x 512 with 256 tokens 3.1 / 3.5, 768 -> 2304 with 1000 tokens 6.0 / 6.9, 1024 -> 2048 with 2048 tokens
+// 8.5 / 9.2; with 4096 tokens 16.0 / 15.3, as a CTA then pulls twice the pair's bytes per FLOP.
 template <int STAGES>
 struct DenseCfg {
     static constexpr int kBlockN = 128;
@@ -148,11 +184,11 @@ struct DenseCfg {
     static constexpr int kSmemBytes = STAGES * kStageBytes + 256 + 1024;
 };
 
-template <int STAGES>
+template <bool A_MN, bool B_MN, int EPI, int STAGES>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const DenseGemmParams p) {
-    // A = dY and B = X, both stored [K x .]; M and N are multiples of 128; one tile per CTA
+    // N is a multiple of 128; one tile per CTA
     using Cfg = DenseCfg<STAGES>;
     constexpr int kBlockN = Cfg::kBlockN;
     extern __shared__ uint8_t smem_raw[];
@@ -164,7 +200,7 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_m = p.M / kBlockM, num_kb = (p.K + 63) / 64;
+    const int num_m = (p.M + kBlockM - 1) / kBlockM, num_kb = (p.K + 63) / 64;
     const int m_blk = blockIdx.x % num_m, n_blk = blockIdx.x / num_m;
 
     if (threadIdx.x == 0) {
@@ -199,41 +235,52 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 uint8_t* sB = sA + Cfg::kABytes;
                 uint64_t* bar = &full_bar[ps.stage];
                 mbar_expect_tx(bar, Cfg::kStageBytes);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    tma_load_2d(sA + h * 8192, &tmA, bar, m_blk * kBlockM + h * 64, kb * 64);
-                    tma_load_2d(sB + h * 8192, &tmB, bar, n_blk * kBlockN + h * 64, kb * 64);
+                if (A_MN) {
+                    tma_load_2d(sA, &tmA, bar, m_blk * kBlockM, kb * 64);
+                    tma_load_2d(sA + 8192, &tmA, bar, m_blk * kBlockM + 64, kb * 64);
+                } else {
+                    tma_load_2d(sA, &tmA, bar, kb * 64, m_blk * kBlockM);
+                }
+                if (B_MN) {
+                    tma_load_2d(sB, &tmB, bar, n_blk * kBlockN, kb * 64);
+                    tma_load_2d(sB + 8192, &tmB, bar, n_blk * kBlockN + 64, kb * 64);
+                } else {
+                    tma_load_2d(sB, &tmB, bar, kb * 64, n_blk * kBlockN);
                 }
                 ps.advance(STAGES);
             }
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            constexpr uint32_t idesc = make_idesc_bf16(kBlockM, kBlockN, true, true, false);
+            constexpr uint32_t idesc = make_idesc_bf16(kBlockM, kBlockN, A_MN, B_MN, false);
             PipeState ps;
             bool ok = true;
+            ClockProbe probe;
+            if (blockIdx.x == 0) probe.begin();
             for (int kb = 0; kb < num_kb; ++kb) {
                 if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
                 const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
                 const uint32_t sB = sA + Cfg::kABytes;
+                const uint64_t a0 = A_MN ? make_smem_desc(sA, 8192, 1024, kSwizzle128B) : make_smem_desc(sA, 16, 1024, kSwizzle128B);
+                const uint64_t b0 = B_MN ? make_smem_desc(sB, 8192, 1024, kSwizzle128B) : make_smem_desc(sB, 16, 1024, kSwizzle128B);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    umma_bf16(tmem_base, make_smem_desc(sA + j * 2048, 8192, 1024, kSwizzle128B),
-                              make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B), idesc, (kb | j) != 0 ? 1u : 0u);
+                    umma_bf16(tmem_base, a0 + j * (A_MN ? 128 : 2), b0 + j * (B_MN ? 128 : 2), idesc, (kb | j) != 0 ? 1u : 0u);
                 umma_commit(&empty_bar[ps.stage]);
                 ps.advance(STAGES);
             }
             if (ok) umma_commit(tfull_bar);
+            if (blockIdx.x == 0) probe.end(kClockDense);
         }
     } else {
         const int q = warp & 3, c0 = ((warp - 2) >> 2) * (kBlockN / 2);
         const int m = m_blk * kBlockM + q * 32 + lane, n0 = n_blk * kBlockN + c0;
-        const uint4 bits = load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), kBlockN / 2);
+        uint32_t mw[4];
+        if (EPI == kEpiMasked) load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), kBlockN / 2, mw);
         if (mbar_wait(tfull_bar, 0u, abort_flag)) {
             tc_fence_after_sync();
-            drain_masked(tmem_base + c0 + (static_cast<uint32_t>(q * 32) << 16), kBlockN / 2, bits,
-                         static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1));
+            drain_row<EPI>(tmem_base + c0 + (static_cast<uint32_t>(q * 32) << 16), kBlockN / 2, p, m, n0, mw);
         }
     }
 
@@ -587,44 +634,48 @@ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, int&
 struct PairWork {
     int m_pair, n0, width;
 };
-template <int BLOCK_N, bool SPLIT_TAIL>
-__device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, int num_n, PairWork& w) {
+__device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, int num_n, int width, bool split_tail,
+                                          PairWork& w) {
     const int num_tiles = num_m * num_n;
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
-    const bool split = SPLIT_TAIL && rem > 0 && 2 * rem <= num_pairs;
+    const bool split = split_tail && rem > 0 && 2 * rem <= num_pairs;
     if (item >= (split ? full + 2 * rem : num_tiles)) return false;
     const bool halved = split && item >= full;
     const int tile = halved ? full + ((item - full) >> 1) : item;
     int n_blk;
     raster_tile(tile, num_m, num_n, w.m_pair, n_blk);
-    w.width = halved ? BLOCK_N / 2 : BLOCK_N;
-    w.n0 = n_blk * BLOCK_N + (halved && ((item - full) & 1) ? BLOCK_N / 2 : 0);
+    w.width = halved ? width / 2 : width;
+    w.n0 = n_blk * width + (halved && ((item - full) & 1) ? width / 2 : 0);
     return true;
 }
 
-// Dense CTA-pair GEMM: D[M x N] = A[M x K] * B[N x K]^T with a 256 x BLOCK_N tile per pair
-// (each CTA: 128 rows of A, BLOCK_N/2 rows of B, 128 x BLOCK_N accumulator rows).
-template <int BLOCK_N, int STAGES>
+// Dense CTA-pair GEMM: D[M x N] = A[M x K] * B[N x K]^T with a tile of 256 rows x 64 ... 256 columns per pair (each CTA:
+// 128 rows of A, half of the columns of B, 128 accumulator rows).  The width is chosen per launch so that a small
+// matrix has tiles for all pairs; a [K x N] operand is loaded in chunks of 64 columns (a width of 64 or 192
+// leaves half of a chunk unused).
 struct DensePairCfg {
-    static constexpr int kHalfN = BLOCK_N / 2;
     static constexpr int kABytes = kBlockM * 128;
-    static constexpr int kBBytes = kHalfN * 128;
-    static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kSmemBytes = STAGES * kStageBytes + 256 + 1024;
-    static_assert(BLOCK_N % 128 == 0 && BLOCK_N <= 256, "BLOCK_N must be 128 or 256");
+    static constexpr int kMaxWidth = 256, kMaxStages = 8;
+    __host__ __device__ static constexpr int chunks(int width) { return (width / 2 + 63) / 64; }
+    __host__ __device__ static constexpr int b_bytes(bool b_mn, int width) { return b_mn ? chunks(width) * 8192 : width * 64; }
+    __host__ __device__ static constexpr int stage_bytes(bool b_mn, int width) { return kABytes + b_bytes(b_mn, width); }
+    __host__ __device__ static constexpr int smem_bytes(bool b_mn, int width, int stages) {
+        return stages * stage_bytes(b_mn, width) + 256 + 1024;
+    }
 };
 
-template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
+template <bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const DenseGemmParams p) {
-    using Cfg = DensePairCfg<BLOCK_N, STAGES>;
-    constexpr int kTmemCols = 2 * BLOCK_N;                       // 256 or 512
+    using Cfg = DensePairCfg;
+    constexpr int kTmemCols = 2 * Cfg::kMaxWidth;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes);
-    uint64_t* empty_bar = full_bar + STAGES;
-    uint64_t* tfull_bar = empty_bar + STAGES;
+    const int stages = p.stages, stage_bytes = Cfg::stage_bytes(B_MN, p.width);
+    uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + stages * stage_bytes);
+    uint64_t* empty_bar = full_bar + Cfg::kMaxStages;
+    uint64_t* tfull_bar = empty_bar + Cfg::kMaxStages;
     uint64_t* tempty_bar = tfull_bar + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty_bar + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -633,13 +684,14 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const uint32_t cta = cluster_ctarank();
     const int pair_id = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int num_m = (p.M + 2 * kBlockM - 1) / (2 * kBlockM);
-    const int num_n = (p.N + BLOCK_N - 1) / BLOCK_N;
+    const int num_n = (p.N + p.width - 1) / p.width;
     const int num_kb = (p.K + 63) / 64;
     // halving needs B loads of any width: the [K x N] operand is loaded in 64-column chunks
-    constexpr bool kSplitTail = B_MN && BLOCK_N == 256;
+    const bool split_tail = B_MN && p.width == 256;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+#pragma unroll
+        for (int s = 0; s < Cfg::kMaxStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&tfull_bar[a], 1); mbar_init(&tempty_bar[a], 2 * kDenseEpiWarps); }
         *abort_flag = 0;
         fence_mbar_init();
@@ -664,20 +716,22 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 
     if (warp == 0) {
         if (elect_one()) {
-            PipeState ps;
+            RingState ps;
             bool ok = true;
             PairWork w;
-            for (int item = pair_id; ok && pair_work<BLOCK_N, kSplitTail>(item, num_pairs, num_m, num_n, w);
+            const uint32_t leader_bar = mapa_shared(smem_u32(full_bar), 0);
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
                  item += num_pairs) {
                 const int half_w = w.width / 2;                       // B rows (columns of D) this CTA stages
                 const int m0 = (w.m_pair * 2 + static_cast<int>(cta)) * kBlockM;
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
-                const uint32_t stage_tx = kSplitTail ? 2 * (Cfg::kABytes + half_w * 128) : 2 * Cfg::kStageBytes;
+                const bool two_chunks = Cfg::chunks(w.width) == 2;
+                const uint32_t stage_tx = 2 * (Cfg::kABytes + Cfg::b_bytes(B_MN, w.width));
                 for (int kb = 0; kb < num_kb; ++kb) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
-                    uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
+                    uint8_t* sA = smem + ps.off;
                     uint8_t* sB = sA + Cfg::kABytes;
-                    const uint32_t bar = mapa_shared(smem_u32(&full_bar[ps.stage]), 0);
+                    const uint32_t bar = leader_bar + 8 * ps.stage;
                     if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], stage_tx);
                     if (A_MN) {
                         tma_load_2d_pair(sA, &tmA, bar, m0, kb * 64);
@@ -686,49 +740,45 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                         tma_load_2d_pair(sA, &tmA, bar, kb * 64, m0);
                     }
                     if (B_MN) {
-#pragma unroll
-                        for (int h = 0; h < Cfg::kHalfN / 64; ++h)
-                            if (h * 64 < half_w) tma_load_2d_pair(sB + h * 8192, &tmB, bar, n0 + h * 64, kb * 64);
+                        tma_load_2d_pair(sB, &tmB, bar, n0, kb * 64);
+                        if (two_chunks) tma_load_2d_pair(sB + 8192, &tmB, bar, n0 + 64, kb * 64);
                     } else {
                         tma_load_2d_pair(sB, &tmB, bar, kb * 64, n0);
                     }
-                    ps.advance(STAGES);
+                    ps.advance(stages, stage_bytes);
                 }
             }
         }
     } else if (warp == 1) {
         if (cta == 0 && elect_one()) {
-            constexpr uint32_t idesc_full = make_idesc_bf16(2 * kBlockM, BLOCK_N, A_MN, B_MN, false);
-            constexpr uint32_t idesc_half = make_idesc_bf16(2 * kBlockM, BLOCK_N / 2, A_MN, B_MN, false);
-            PipeState ps;
+            RingState ps;
             bool ok = true;
             int it = 0;
             PairWork w;
             ClockProbe probe;
             if (pair_id == 0) probe.begin();
-            for (int item = pair_id; ok && pair_work<BLOCK_N, kSplitTail>(item, num_pairs, num_m, num_n, w);
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
                  item += num_pairs, ++it) {
-                const uint32_t idesc = w.width == BLOCK_N ? idesc_full : idesc_half;
+                const uint32_t idesc = make_idesc_bf16(2 * kBlockM, w.width, A_MN, B_MN, false);
                 const int acc = it & 1;
                 const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
                 if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * BLOCK_N;
+                const uint32_t d_tmem = tmem_base + acc * Cfg::kMaxWidth;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                     tc_fence_after_sync();
-                    const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
+                    const uint32_t sA = smem_u32(smem + ps.off);
                     const uint32_t sB = sA + Cfg::kABytes;
+                    const uint64_t a0 = A_MN ? make_smem_desc(sA, 8192, 1024, kSwizzle128B) : make_smem_desc(sA, 16, 1024, kSwizzle128B);
+                    const uint64_t b0 = B_MN ? make_smem_desc(sB, 8192, 1024, kSwizzle128B) : make_smem_desc(sB, 16, 1024, kSwizzle128B);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint64_t ad = A_MN ? make_smem_desc(sA + j * 2048, 8192, 1024, kSwizzle128B)
-                                                 : make_smem_desc(sA + j * 32, 16, 1024, kSwizzle128B);
-                        const uint64_t bd = B_MN ? make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B)
-                                                 : make_smem_desc(sB + j * 32, 16, 1024, kSwizzle128B);
+                    for (int j = 0; j < 4; ++j) {              // steps along K, in 16-byte units of the start address
+                        const uint64_t ad = a0 + j * (A_MN ? 128 : 2), bd = b0 + j * (B_MN ? 128 : 2);
                         umma_bf16_pair(d_tmem, ad, bd, idesc, (kb | j) != 0 ? 1u : 0u);
                     }
                     umma_commit_pair(&empty_bar[ps.stage], 3);
-                    ps.advance(STAGES);
+                    ps.advance(stages, stage_bytes);
                 }
                 if (ok) umma_commit_pair(&tfull_bar[acc], 3);
             }
@@ -739,42 +789,22 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         bool ok = true;
         int it = 0;
         PairWork w;
-        for (int item = pair_id; ok && pair_work<BLOCK_N, kSplitTail>(item, num_pairs, num_m, num_n, w);
+        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
              item += num_pairs, ++it) {
             const int acc = it & 1;
             const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
             const int m = (w.m_pair * 2 + static_cast<int>(cta)) * kBlockM + q * 32 + lane;
             const int cols = w.width / 2, n0 = w.n0 + half * cols;
-            const bool live = m < p.M && n0 < p.N;           // (kEpiMasked: the same for all rows of a CTA)
-            uint4 bits = make_uint4(0u, 0u, 0u, 0u);
+            // columns inside the matrix: N is a multiple of 128, so a part of them only at a width of 192 (kEpiStore)
+            const int left = min(cols, p.N - n0);
+            const bool live = m < p.M && left > 0;           // (kEpiMasked: the same for all rows of a CTA)
+            uint32_t mw[4];
             if (EPI == kEpiMasked && live)
-                bits = load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), cols);
+                load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n0 >> 3), cols, mw);
             if (!mbar_wait(&tfull_bar[acc], acc_phase, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
-            const uint32_t t_row = tmem_base + acc * BLOCK_N + half * cols + (static_cast<uint32_t>(q * 32) << 16);
-            if (EPI == kEpiMasked) {
-                if (live)
-                    drain_masked(t_row, cols, bits, static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * (p.N >> 1) + (n0 >> 1));
-            } else if (n0 < p.N) {
-                uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + static_cast<size_t>(m) * p.N + n0);
-#pragma unroll 1
-                for (int c0 = 0; c0 < cols; c0 += 64) {
-                    uint32_t v[4][16];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) tmem_ld_16(t_row + c0 + 16 * k, v[k]);
-                    tmem_ld_wait();
-                    if (live) {
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const uint32_t* e = v[k >> 1] + 8 * (k & 1);
-                            dst[c0 / 8 + k] = make_uint4(pack_bf16x2(__uint_as_float(e[0]), __uint_as_float(e[1])),
-                                                         pack_bf16x2(__uint_as_float(e[2]), __uint_as_float(e[3])),
-                                                         pack_bf16x2(__uint_as_float(e[4]), __uint_as_float(e[5])),
-                                                         pack_bf16x2(__uint_as_float(e[6]), __uint_as_float(e[7])));
-                        }
-                    }
-                }
-            }
+            const uint32_t t_row = tmem_base + acc * Cfg::kMaxWidth + half * cols + (static_cast<uint32_t>(q * 32) << 16);
+            if (EPI == kEpiMasked ? live : left > 0) drain_row<EPI>(t_row, left, p, m, n0, mw);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[acc]), 0));

@@ -257,6 +257,11 @@ __device__ __forceinline__ uint2 ld_v2(const void* p) {
     asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
+__device__ __forceinline__ uint32_t ld_u32(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint32_t ld_u8(const void* p) {
     uint32_t v;
     asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));

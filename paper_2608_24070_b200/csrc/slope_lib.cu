@@ -304,20 +304,6 @@ static unsigned stream_grid(size_t threads, const DeviceInfo& info) {
     return static_cast<unsigned>(blocks < most ? blocks : most);
 }
 
-// ------------------------------------------------------------------ dense GEMM launch
-static slope_status_t launch_dense_masked(const void* dY, const void* X, int M, int N, int K, void* out, const void* mask,
-                                          cudaStream_t stream) {
-    constexpr int kStages = 6;
-    using Cfg = DenseCfg<kStages>;
-    CUtensorMap tmA, tmB;
-    if (!make_tmap(&tmA, dY, K, M, 64, 64) || !make_tmap(&tmB, X, K, N, 64, 64)) return SLOPE_ERR_CUDA;
-    const DenseGemmParams p{M, N, K, out, static_cast<const uint8_t*>(mask)};
-    auto kern = dense_gemm_kernel<kStages>;
-    if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    return launch_cluster_ex(kern, (M / kBlockM) * (N / Cfg::kBlockN), 1, kDenseThreads, Cfg::kSmemBytes,
-                             /*overlap_prologue=*/true, stream, tmA, tmB, p);
-}
-
 // ------------------------------------------------------------------ adapter products
 struct AdapterOperands {
     const void* A = nullptr;      // the large operand: [M x K], or [K x M] when A_MN
@@ -813,23 +799,68 @@ static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* 
     return launch_sparse_tile(t, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, pairs, stream, 0);
 }
 
-template <bool A_MN, bool B_MN, int BLOCK_N, int EPI, int STAGES>
-static slope_status_t launch_dense_pair(const void* A, const void* B, int M, int N, int K, void* out,
-                                        const void* mask, cudaStream_t stream, const DeviceInfo& info) {
-    using Cfg = DensePairCfg<BLOCK_N, STAGES>;
+static int dense_stages(bool b_mn, int width) {
+    int n = DensePairCfg::kMaxStages;
+    while (n > 1 && DensePairCfg::smem_bytes(b_mn, width, n) > 232448) --n;
+    return n;
+}
+// Columns per tile of the dense CTA-pair kernel, by estimate.  Narrow tiles give a small matrix enough of them for the
+// pairs; wide ones move fewer bytes per FLOP.  In SM clocks: a k-block of 64 takes its bytes at 70 per clock and its
+// MMAs (2.36 per column, no fewer than 80 columns' worth), a tile no less than its drain, a launch one more drain
+// and 47 per pair.  (192 columns of a [K x N] operand cost the bytes of 256 and are not taken.)  Fitted to a sweep over
+// 12 layer shapes (512 ... 9728) and 64 ... 8192 tokens: 0.2 % slower on average than the best width, where 256 x 256
+// throughout is 24 %.  us, 256 x 256 -> now: forward / input gradient of a dense layer 500 tokens 1024 x 1024 9.5 / 9.6 ->
+// 4.9 / 5.6, 740 tokens 8320 -> 6400 forward 84 -> 68, 700 tokens 2048 -> 6144 input gradient 32.6 -> 21.1.
+static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int num_pairs) {
+    const int num_m = (M + 255) / 256, num_kb = (K + 63) / 64;
+    int best = 256;
+    double best_cost = 1e300;
+    for (int width = 256; width >= 64; width -= 64) {
+        if (b_mn && width == 192) continue;
+        const int tiles = num_m * ((N + width - 1) / width), rem = tiles % num_pairs;
+        const bool halves = b_mn && width == 256 && tiles > num_pairs && 2 * rem <= num_pairs;      // see pair_work
+        const double waves = tiles / num_pairs + (rem == 0 ? 0.0 : halves ? 0.5 : 1.0);
+        const double k_block = std::max(DensePairCfg::stage_bytes(b_mn, width) / 70.0, 2.36 * std::max(width, 80));
+        const double drain = masked ? 850.0 + 11.8 * width : 780.0 + 24.2 * width;
+        const double cost = waves * std::max(num_kb * k_block, drain) + drain + 47.0 * std::min(tiles, num_pairs);
+        if (cost < best_cost) { best_cost = cost; best = width; }
+    }
+    return best;
+}
+
+// D[M x N] on 128 x 128 tiles of single CTAs while they all run at once and the reduction is at most
+// 2048 long (measured on both sides of either line: dense_gemm_kernel), else on the CTA-pair kernel; a dense layer with
+// fewer than 64 such tiles has more CTAs of the pair kernel's 64-column tiles (256 tokens 512 x 512: 3.7 against 4.3 us).
+template <bool A_MN, bool B_MN, int EPI>
+static slope_status_t launch_dense(const void* A, const void* B, int M, int N, int K, void* out,
+                                   const void* mask, cudaStream_t stream, const DeviceInfo& info) {
+    const int max_pairs = info.sm_count / 2, small_tiles = ((M + kBlockM - 1) / kBlockM) * (N / 128);
+    const bool small = small_tiles <= info.sm_count && K <= 2048 && (EPI == kEpiMasked || small_tiles >= 64);
+    thread_local SizeMemo<int> memo;
+    const int width = small ? 128 : memo.get({M, N, K, info.sm_count, 0, 0}, [&] {
+        return choose_dense_width(M, N, K, B_MN, EPI == kEpiMasked, max_pairs);
+    });
     CUtensorMap tmA, tmB;
     const bool okA = A_MN ? make_tmap(&tmA, A, K, M, 64, 64) : make_tmap(&tmA, A, M, K, kBlockM, 64);
-    const bool okB = B_MN ? make_tmap(&tmB, B, K, N, 64, 64) : make_tmap(&tmB, B, N, K, Cfg::kHalfN, 64);
+    const bool okB = B_MN ? make_tmap(&tmB, B, K, N, 64, 64) : make_tmap(&tmB, B, N, K, small ? 128 : width / 2, 64);
     if (!okA || !okB) return SLOPE_ERR_CUDA;
-    DenseGemmParams p = {};
-    p.M = M; p.N = N; p.K = K; p.out = out;
-    p.mask = static_cast<const uint8_t*>(mask);
-    auto kern = dense_gemm_pair_kernel<A_MN, B_MN, BLOCK_N, EPI, STAGES>;
-    if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
-    const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + BLOCK_N - 1) / BLOCK_N);
-    const int max_pairs = info.sm_count / 2;
-    const int pairs = tiles < max_pairs ? tiles : max_pairs;
-    return launch_pairs(kern, 2 * pairs, kDenseThreads, Cfg::kSmemBytes, stream, tmA, tmB, p);
+    if (small) {
+        constexpr int kStages = 6;
+        using Cfg = DenseCfg<kStages>;
+        const DenseGemmParams p{M, N, K, width, kStages, out, static_cast<const uint8_t*>(mask)};
+        auto kern = dense_gemm_kernel<A_MN, B_MN, EPI, kStages>;
+        if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
+        return launch_cluster_ex(kern, small_tiles, 1, kDenseThreads, Cfg::kSmemBytes, /*overlap_prologue=*/true, stream, tmA,
+                                 tmB, p);
+    }
+    using Cfg = DensePairCfg;
+    const int stages = dense_stages(B_MN, width);
+    const DenseGemmParams p{M, N, K, width, stages, out, static_cast<const uint8_t*>(mask)};
+    auto kern = dense_gemm_pair_kernel<A_MN, B_MN, EPI>;
+    if (!set_smem(kern, 232448)) return SLOPE_ERR_CUDA;
+    const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + width - 1) / width);
+    const int pairs = std::min(tiles, max_pairs);
+    return launch_pairs(kern, 2 * pairs, kDenseThreads, Cfg::smem_bytes(B_MN, width, stages), stream, tmA, tmB, p);
 }
 
 static int adapter_splits(int b, int rows) {
@@ -1014,19 +1045,8 @@ slope_status_t slope_linear_bwd_dw_masked(const void* dY, const void* X, int b, 
     if (!aligned16(dY) || !aligned16(X) || !aligned16(mask1_bits) || !aligned16(dWc_vals)) return SLOPE_ERR_ALIGNMENT;
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
-    // Small weight matrices do not have enough 256 x 256 tiles for the 74 CTA pairs.  They run on
-    // 256 x 128 tiles of CTA pairs (each CTA stages half of the X tile: GPT-2-small 33 -> 29.5 us) or,
-    // when even those are few, on 128 x 128 tiles of one CTA each.
-    const int pair_tiles = ((d_out + 255) / 256) * ((d_in + 255) / 256);
-    if (pair_tiles * 2 <= info.sm_count) {
-        const int narrow_tiles = ((d_out + 255) / 256) * ((d_in + 127) / 128);
-        if (narrow_tiles >= 24)
-            return launch_dense_pair<true, true, 128, kEpiMasked, 8>(dY, X, d_out, d_in, b, dWc_vals, mask1_bits,
-                                                                     static_cast<cudaStream_t>(stream), info);
-        return launch_dense_masked(dY, X, d_out, d_in, b, dWc_vals, mask1_bits, static_cast<cudaStream_t>(stream));
-    }
-    return launch_dense_pair<true, true, 256, kEpiMasked, 6>(dY, X, d_out, d_in, b, dWc_vals, mask1_bits,
-                                                             static_cast<cudaStream_t>(stream), info);
+    return launch_dense<true, true, kEpiMasked>(dY, X, d_out, d_in, b, dWc_vals, mask1_bits,
+                                                     static_cast<cudaStream_t>(stream), info);
 }
 
 // ------------------------------------------------------------------ dense layer on the same pipeline
@@ -1042,7 +1062,7 @@ slope_status_t slope_dense_linear_fwd(const void* X, int b, const void* W, int d
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     // Y[b x d_out] = X[b x d_in] * W[d_out x d_in]^T: both operands K-contiguous
-    return launch_dense_pair<false, false, 256, kEpiStore, 6>(X, W, b, d_out, d_in, Y, nullptr,
+    return launch_dense<false, false, kEpiStore>(X, W, b, d_out, d_in, Y, nullptr,
                                                               static_cast<cudaStream_t>(stream), info);
 }
 
@@ -1052,7 +1072,7 @@ slope_status_t slope_dense_linear_bwd_dx(const void* dY, int b, const void* W, i
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     // dX[b x d_in] = dY[b x d_out] * W[d_out x d_in]: W is the [K x N] operand
-    return launch_dense_pair<false, true, 256, kEpiStore, 6>(dY, W, b, d_in, d_out, dX, nullptr,
+    return launch_dense<false, true, kEpiStore>(dY, W, b, d_in, d_out, dX, nullptr,
                                                              static_cast<cudaStream_t>(stream), info);
 }
 
@@ -1062,7 +1082,7 @@ slope_status_t slope_dense_linear_bwd_dw(const void* dY, const void* X, int b, i
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     // dW[d_out x d_in] = dY[b x d_out]^T * X[b x d_in]: both operands stored [K x .]
-    return launch_dense_pair<true, true, 256, kEpiStore, 6>(dY, X, d_out, d_in, b, dW, nullptr,
+    return launch_dense<true, true, kEpiStore>(dY, X, d_out, d_in, b, dW, nullptr,
                                                             static_cast<cudaStream_t>(stream), info);
 }
 

@@ -1,6 +1,5 @@
-"""Weight-gradient and dense GEMM epilogues at the edges of their tiles: every tile width (128 x 128 of one CTA,
-256 x 128 and 256 x 256 of a pair, halved items of the last wave), last tiles that are half empty in either
-dimension, few tokens (one k-block, a ragged one).
+"""Weight-gradient and dense GEMM epilogues at the edges of their tiles: every tile width (64, 128, 192, 256), halved
+items of the last wave, last tiles that are partly empty in either dimension, few tokens (one k-block, a ragged one).
 
 The reference is the fp64 product of the same bf16 operands; outputs are rounded once (2^-9 / sqrt(3) ~ 1.7e-3
 relative on Gaussian data, 5e-3 allowed, and parity_error's bound per element)."""
@@ -22,10 +21,11 @@ def _operands(b, d_in, d_out):
 
 
 @pytest.mark.parametrize("b,d_in,d_out", [
-    (1, 128, 128),               # one 128 x 128 tile, one token
-    (65, 384, 640),              # one-CTA tiles, a k-block and one token
-    (200, 1152, 1920),           # 256 x 128 tiles of pairs, last row tile half empty
-    (70, 2176, 2432),            # 256 x 256 tiles, half empty in both dimensions
+    (1, 128, 128),               # 64 wide, half empty, one token
+    (65, 384, 640),              # 64 wide, a k-block and one token
+    (200, 1152, 1920),           # 128 wide, last row tile half empty
+    (70, 2176, 2432),
+    (200, 3200, 2688),           # 256 wide, half empty in both dimensions
     (90, 4096, 4096),            # 256 tiles: the last wave's are halved
 ])
 def test_masked_weight_gradient(b, d_in, d_out):
@@ -43,7 +43,8 @@ def test_masked_weight_gradient(b, d_in, d_out):
     assert parity_error(to_f64(B.bits_from_bf16(dWc)), ref) <= REL_TOL
 
 
-@pytest.mark.parametrize("b,d_in,d_out", [(1, 128, 128), (130, 256, 384), (300, 1152, 640), (513, 384, 2176)])
+@pytest.mark.parametrize("b,d_in,d_out", [(1, 128, 128), (130, 256, 384), (300, 1152, 640), (513, 384, 2176),
+                                        (700, 2048, 4224), (600, 3200, 2688)])
 def test_dense_layer(b, d_in, d_out):
     import torch
 
