@@ -102,7 +102,7 @@ slope_status_t slope_prune_24_double(const void* W, int d_out, int d_in,
  * Wc_vals / Wc_meta come from slope_prune_24.  T = X L is produced by
  * slope_adapter_fwd_bwd(phase 0).  r = 0 (T, R ignored) leaves the adapter out.
  * With few tokens (inference, decode: the paper's forward-only inference measurements; always up
- * to 16 tokens, up to 128 where it is estimated faster than the tile kernels) the same call
+ * to 16 tokens, up to 128 for long reductions on few rows) the same call
  * runs on a kernel that streams the compressed weight once from HBM and splits the
  * reduction over a thread-block cluster.  The compute launches of this library are issued with
  * programmatic stream serialisation (their set-up may overlap the previous kernel's tail) and

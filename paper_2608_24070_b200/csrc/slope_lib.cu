@@ -696,26 +696,16 @@ static SparseTile choose_sparse_tile(int M, int K, int ntok, int r, int num_pair
     return best;
 }
 
-// Few-token kernel or tile kernel?  Decode sizes (<= 16 tokens) always stream the weights through
-// the few-token kernel.  Up to 128 tokens the two are compared by estimate: the few-token kernel's
-// own cost model against a tile kernel that has one token tile, i.e. M / 256 tiles which each
-// walk the whole reduction (measured: ~4 us per launch plus 0.32 us per k-block and wave of the
-// machine).  A tall weight (4096 -> 11008) then has enough tiles for the tile kernel, a long
-// reduction on few rows (11008 -> 4096) wants the K-split of the few-token kernel.  Beyond 128
-// tokens the 256-token variant of the few-token kernel pays 512 row requests per k-block for
-// its activations and loses almost everywhere (measured), so the tile kernels take over.
-static bool use_few_token_kernel(int M, int K, int ntok, int r, const DeviceInfo& info) {
+// Few-token kernel or tile kernel?  Decode sizes (<= 16 tokens) stream the weights through the few-token kernel.  From 17 to
+// 128 tokens it is the better one only for a long reduction on few rows, where its K-split fills the machine and a
+// tile kernel has a handful of tiles that each walk the whole reduction; a tall weight has tiles enough, narrow ones
+// for few tokens.  us, few-token / tile kernel: 32 tokens 4096 -> 4096 7.7 / 8.6, 1024 -> 1024 4.1 / 3.8, 3072 -> 768 4.4 / 6.2,
+// 4096 -> 12288 14.3 / 12.2; 64 tokens 2048 -> 2048 5.6 / 5.4, 4096 -> 4096 8.3 / 8.6, 4096 -> 22016 33 / 23; 80 tokens 4096 -> 4096
+// 9.3 / 8.9, 8192 -> 2560 10.2 / 13.4; 128 tokens 11008 -> 4096 15.8 / 17.9, 2048 -> 6144 10.2 / 7.1.
+static bool use_few_token_kernel(int M, int K, int ntok) {
     if (ntok <= 16) return true;
     if (ntok > 128) return false;
-    int cap[9];
-    const bool ok = ntok <= 64 ? skinny_capacity<64, 8, 4>(info, cap) : skinny_capacity<128, 7, 3>(info, cap);
-    if (!ok) return false;
-    double few_us = 0.0;
-    skinny_splits(M / kBlockM, K / 128, ntok <= 64 ? 64 : 128, cap, &few_us);
-    const int num_pairs = info.sm_count / 2;
-    const int tiles = (M + 255) / 256;
-    const double tile_us = 4.0 + ((tiles + num_pairs - 1) / num_pairs) * (K / 128 + (r + 63) / 64) * 0.32;
-    return few_us <= tile_us;
+    return K >= 2 * M || (ntok <= 64 && K >= M && K >= 2048);
 }
 
 static slope_status_t launch_sparse_tile(const SparseTile& t, const void* act, int ntok, const void* vals, const void* meta,
@@ -747,7 +737,7 @@ static FwdAdapterPlan plan_fwd_adapter(int b, int d_out, int d_in, int r, const 
     FwdAdapterPlan best{};                                  // (no tile rows: the few-token kernel)
     best.pairs = info.sm_count / 2;
     double best_us = 1e300, cost = 0.0;
-    if (use_few_token_kernel(d_out, d_in, b, r, info)) {                // its K-split is chosen around the producer
+    if (use_few_token_kernel(d_out, d_in, b)) {                // its K-split is chosen around the producer
         best.T = adapter_plan(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count);
     } else {
         const int pairs = info.sm_count / 2;
@@ -793,7 +783,7 @@ static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* 
     const int pairs = info.sm_count / 2;
     thread_local SizeMemo<SparseTile> memo;                  // (no rows: the few-token kernel)
     const SparseTile& t = memo.get({M, K, ntok, r, info.dev, 0}, [&] {
-        return use_few_token_kernel(M, K, ntok, r, info) ? SparseTile{0, 0} : choose_sparse_tile(M, K, ntok, r, pairs);
+        return use_few_token_kernel(M, K, ntok) ? SparseTile{0, 0} : choose_sparse_tile(M, K, ntok, r, pairs);
     });
     if (t.rows == 0) return launch_skinny(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info);
     return launch_sparse_tile(t, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, pairs, stream, 0);
