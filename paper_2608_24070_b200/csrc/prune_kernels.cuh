@@ -22,44 +22,43 @@ namespace slope {
 //   - an element is kept when it beats at least two of the other three (majority of three
 //     comparison bits, one LOP3 each);
 //   - prmt's sign-replication mode turns the keep bits into half-word masks.
+// These kernels are bound by the logic pipe, so what a pass does not need is not computed (the first pass wants mask and
+// metadata bytes, the second two codes), bits that are masked or shifted out anyway are not cleared, and fixed shifts are
+// folded into multiplies.  Both passes in one launch 17.7 -> 16.4 us at 4096 x 4096 and 42.1 -> 39.2 at 4096 x 11008 (4.5 and
+// 5.0 TB/s), the second pass alone 14.1 -> 11.6 and 30.9 -> 26.3.
 // ---------------------------------------------------------------------------------------
 struct PackedPick {
     uint32_t out0, out1;      // kept pair of group 0 / group 1: first kept in the low half
-    uint32_t mask_byte;       // 4 keep bits of group 0 | 4 keep bits of group 1 << 4
-    uint32_t meta_byte;       // code p0 | p1<<2 of group 0 | code of group 1 << 4
     uint32_t keep[4];         // element i kept: 0xFFFF in the low half (group 0) / high half (group 1)
+    uint32_t code;            // p0 | p1 << 2 of group 0 in bits 0..3, of group 1 in bits 16..19
 };
 
 __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (a & c) | (b & c); }
 __device__ __forceinline__ uint32_t bitsel(uint32_t m, uint32_t a, uint32_t b) { return (m & a) | (~m & b); }
 
 __device__ __forceinline__ PackedPick pick2of4_packed(uint32_t E0, uint32_t E1, uint32_t E2, uint32_t E3) {
-    constexpr uint32_t G = 0x80008000u;
-    const uint32_t M0 = E0 & 0x7FFF7FFFu, M1 = E1 & 0x7FFF7FFFu, M2 = E2 & 0x7FFF7FFFu, M3 = E3 & 0x7FFF7FFFu;
-    const uint32_t c01 = M0 + G - M1, c02 = M0 + G - M2, c03 = M0 + G - M3;
-    const uint32_t c12 = M1 + G - M2, c13 = M1 + G - M3, c23 = M2 + G - M3;
-    // keep flags in bits 15 / 31
-    const uint32_t k0 = maj3(c01, c02, c03);
-    const uint32_t k1 = maj3(~c01, c12, c13);
-    const uint32_t k2 = maj3(~c02, ~c12, c23);
-    const uint32_t k3 = maj3(~c03, ~c13, ~c23);
-    // half-word masks (0xFFFF where kept): bytes 0,1 <- sign of byte 1; bytes 2,3 <- sign of byte 3
-    const uint32_t m0 = prmt(k0, 0u, 0xBB99u), m1 = prmt(k1, 0u, 0xBB99u);
-    const uint32_t m2 = prmt(k2, 0u, 0xBB99u), m3 = prmt(k3, 0u, 0xBB99u);
+    constexpr uint32_t G = 0x80008000u, V = 0x7FFF7FFFu;
+    const uint32_t A0 = E0 | G, A1 = E1 | G, A2 = E2 | G, M1 = E1 & V, M2 = E2 & V, M3 = E3 & V;
+    const uint32_t c01 = A0 - M1, c02 = A0 - M2, c03 = A0 - M3, c12 = A1 - M2, c13 = A1 - M3, c23 = A2 - M3;
+    // keep flags in bits 15 / 31, then half-word masks (bytes 0,1 <- sign of byte 1; bytes 2,3 <- sign of byte 3)
+    const uint32_t m0 = prmt(maj3(c01, c02, c03), 0u, 0xBB99u), m1 = prmt(maj3(~c01, c12, c13), 0u, 0xBB99u);
+    const uint32_t m2 = prmt(maj3(~c02, ~c12, c23), 0u, 0xBB99u), m3 = prmt(maj3(~c03, ~c13, ~c23), 0u, 0xBB99u);
     const uint32_t first = bitsel(m0, E0, bitsel(m1, E1, E2));      // lowest kept position
     const uint32_t second = bitsel(m3, E3, bitsel(m2, E2, E1));     // highest kept position
     PackedPick r;
     r.out0 = prmt(first, second, 0x5410u);
     r.out1 = prmt(first, second, 0x7632u);
-    const uint32_t t = (m0 & 0x00010001u) | (m1 & 0x00020002u) | (m2 & 0x00040004u) | (m3 & 0x00080008u);
-    r.mask_byte = (t | (t >> 12)) & 0xFFu;
-    const uint32_t p0 = ~m0 & bitsel(m1, 0x00010001u, 0x00020002u);
-    const uint32_t p1 = bitsel(m3, 0x00030003u, bitsel(m2, 0x00020002u, 0x00010001u));
-    const uint32_t c = p0 | (p1 << 2);
-    r.meta_byte = (c | (c >> 12)) & 0xFFu;
+    r.code = (~m0 & bitsel(m1, 0x00010001u, 0x00020002u)) | bitsel(m3, 0x000C000Cu, bitsel(m2, 0x00080008u, 0x00040004u));
     r.keep[0] = m0; r.keep[1] = m1; r.keep[2] = m2; r.keep[3] = m3;
     return r;
 }
+// 4 keep bits of group 0 | 4 keep bits of group 1 << 4 (above bit 7: undefined)
+__device__ __forceinline__ uint32_t mask_byte(const PackedPick& r) {
+    const uint32_t t = (r.keep[0] & 0x00010001u) | (r.keep[1] & 0x00020002u) | (r.keep[2] & 0x00040004u) | (r.keep[3] & 0x00080008u);
+    return t | (t >> 12);
+}
+// code of group 0 | code of group 1 << 4 (above bit 7: undefined)
+__device__ __forceinline__ uint32_t meta_byte(const PackedPick& r) { return r.code | (r.code >> 12); }
 
 // Byte offset, inside a 2 KB metadata block, of the byte holding the codes of local
 // row rr (0..127) and local 8-column slot c8 (0..15).
@@ -100,8 +99,8 @@ __global__ void __launch_bounds__(256) prune24_kernel(const uint4* __restrict__ 
         const PackedPick b = pick2of4_packed(prmt(w[i][1].x, w[i][1].z, 0x5410u), prmt(w[i][1].x, w[i][1].z, 0x7632u),
                                              prmt(w[i][1].y, w[i][1].w, 0x5410u), prmt(w[i][1].y, w[i][1].w, 0x7632u));
         vals[row * (row_u4 >> 1) + cb * 8 + u] = make_uint4(a.out0, a.out1, b.out0, b.out1);
-        s_meta[meta_byte_offset(rr, 2 * u) >> 1] = static_cast<uint16_t>(a.meta_byte | (b.meta_byte << 8));
-        s_mask[rr * 8 + u] = static_cast<uint16_t>(a.mask_byte | (b.mask_byte << 8));
+        s_meta[meta_byte_offset(rr, 2 * u) >> 1] = static_cast<uint16_t>(prmt(meta_byte(a), meta_byte(b), 0x0040u));
+        s_mask[rr * 8 + u] = static_cast<uint16_t>(prmt(mask_byte(a), mask_byte(b), 0x0040u));
     }
     __syncthreads();
     if (tid < 128) {
@@ -114,6 +113,27 @@ __global__ void __launch_bounds__(256) prune24_kernel(const uint4* __restrict__ 
     }
 }
 
+// What the second pass of two columns jl, jh of a thread's 8 x 8 patch leaves behind: a and b are the picks of rows 0..3 and
+// 4..7, column jl in the low, jh in the high half-words.
+__device__ __forceinline__ void second_pass_store(const PackedPick& a, const PackedPick& b, int jl, int jh, int ig, int c8,
+                                                  uint8_t* s_out, uint8_t* s_meta) {
+    const int slot = (ig ^ c8) * 8;                                            // (j >> 3) & 15 == c8 for both columns
+    *reinterpret_cast<uint2*>(s_out + (c8 * 8 + jl) * 128 + slot) = make_uint2(a.out0, b.out0);
+    *reinterpret_cast<uint2*>(s_out + (c8 * 8 + jh) * 128 + slot) = make_uint2(a.out1, b.out1);
+    const uint32_t codes = a.code + b.code * 16u;                              // (a multiply-add: not the logic pipe)
+    s_meta[16 * jl] = static_cast<uint8_t>(codes);
+    s_meta[16 * jh] = static_cast<uint8_t>(codes >> 16);
+}
+// Adds, for each of the 8 rows, bit jl (in the low half-word) and bit jh (in the high one) where the pass keeps it.
+__device__ __forceinline__ void second_pass_select(const PackedPick& a, const PackedPick& b, int jl, int jh, uint32_t (&sel)[8]) {
+    const uint32_t bits = (1u << jl) | (0x10000u << jh);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        sel[i] |= a.keep[i] & bits;
+        sel[4 + i] |= b.keep[i] & bits;
+    }
+}
+
 // Second pass.  Tile (rb, cb) of W (rows = d_out, cols = d_in) produces tile (cb, rb) of the
 // compressed transposed matrix.  A thread owns 8 rows x 8 columns of the tile, read straight
 // from global memory (eight 16-byte loads, rows 256 B apart per half-warp).  Groups run down
@@ -123,7 +143,8 @@ __global__ void __launch_bounds__(256) prune24_kernel(const uint4* __restrict__ 
 // an XOR-swizzled 16 KB staging tile whose 64-bit stores are conflict free.
 __device__ __forceinline__ uint32_t halfword_mask_from_bits(uint32_t mask_byte, int w) {
     // bit 2w of the byte -> low half-word, bit 2w+1 -> high half-word (all ones where kept)
-    const uint32_t z = (mask_byte << (15 - 2 * w)) | (mask_byte << (30 - 2 * w));
+    // (one multiply for two shifts and an or: the shifted bytes do not overlap)
+    const uint32_t z = mask_byte * ((1u << (15 - 2 * w)) + (1u << (30 - 2 * w)));
     return prmt(z, 0u, 0xBB99u);
 }
 
@@ -151,7 +172,7 @@ __global__ void __launch_bounds__(256, 4) double_prune_kernel(const uint4* __res
         mb[t] = ld_u8(mask1 + row * mrow + cb * 16 + c8);
     }
 
-    uint32_t sel_bits[8] = {0, 0, 0, 0, 0, 0, 0, 0};         // per row: which of the 8 columns the second pass keeps
+    uint32_t sel[8] = {0, 0, 0, 0, 0, 0, 0, 0};              // per row: which of the 8 columns the second pass keeps
     const int meta_base = meta_byte_offset(c8 * 8, ig);      // + 16 per column inside the 8-column slot
 #pragma unroll
     for (int wi = 0; wi < 4; ++wi) {
@@ -163,25 +184,14 @@ __global__ void __launch_bounds__(256, 4) double_prune_kernel(const uint4* __res
         }
         const PackedPick a = pick2of4_packed(e[0], e[1], e[2], e[3]);        // rows 0..3 of columns 2wi, 2wi+1
         const PackedPick b = pick2of4_packed(e[4], e[5], e[6], e[7]);        // rows 4..7
-        const int j0 = c8 * 8 + 2 * wi;
-        const int slot = (ig ^ c8) * 8;                                        // (j >> 3) & 15 == c8 for both columns
-        *reinterpret_cast<uint2*>(s_out + j0 * 128 + slot) = make_uint2(a.out0, b.out0);
-        *reinterpret_cast<uint2*>(s_out + (j0 + 1) * 128 + slot) = make_uint2(a.out1, b.out1);
-        s_meta[meta_base + 16 * (2 * wi)] = static_cast<uint8_t>((a.meta_byte & 0xFu) | ((b.meta_byte & 0xFu) << 4));
-        s_meta[meta_base + 16 * (2 * wi + 1)] = static_cast<uint8_t>((a.meta_byte >> 4) | (b.meta_byte & 0xF0u));
-        if (mask2 != nullptr) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                sel_bits[i] |= (((a.mask_byte >> i) & 1u) << (2 * wi)) | (((a.mask_byte >> (4 + i)) & 1u) << (2 * wi + 1));
-                sel_bits[4 + i] |= (((b.mask_byte >> i) & 1u) << (2 * wi)) | (((b.mask_byte >> (4 + i)) & 1u) << (2 * wi + 1));
-            }
-        }
+        second_pass_store(a, b, 2 * wi, 2 * wi + 1, ig, c8, s_out, s_meta + meta_base);
+        if (mask2 != nullptr) second_pass_select(a, b, 2 * wi, 2 * wi + 1, sel);
     }
     if (mask2 != nullptr) {
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const size_t row = static_cast<size_t>(rb) * 128 + ig * 8 + t;
-            mask2[row * mrow + cb * 16 + c8] = static_cast<uint8_t>(sel_bits[t] & mb[t]);
+            mask2[row * mrow + cb * 16 + c8] = static_cast<uint8_t>((sel[t] | (sel[t] >> 16)) & mb[t]);
         }
     }
     __syncthreads();
@@ -233,52 +243,41 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
 #pragma unroll
     for (int t = 0; t < 8; ++t) w[t] = ld_v4(W + at0 + t * row_u4);
 
-    // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place
-    uint32_t mb[8];
+    // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place.  (Leaving it in the
+    //      packed order would save its four byte permutes per row, but an and that feeds another logic operation is merged
+    //      into it, which carries element and mask apart into the second pass: 204 bytes of spills, 22 us instead of 18 at
+    //      4096 x 4096.)
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        const PackedPick a = pick2of4_packed(prmt(w[t].x, w[t].z, 0x5410u), prmt(w[t].x, w[t].z, 0x7632u),
-                                             prmt(w[t].y, w[t].w, 0x5410u), prmt(w[t].y, w[t].w, 0x7632u));
+        const uint32_t E0 = prmt(w[t].x, w[t].z, 0x5410u), E1 = prmt(w[t].x, w[t].z, 0x7632u);
+        const uint32_t E2 = prmt(w[t].y, w[t].w, 0x5410u), E3 = prmt(w[t].y, w[t].w, 0x7632u);
+        const PackedPick a = pick2of4_packed(E0, E1, E2, E3);
         const int rr = ig * 8 + t;
         vals[at0 + t * mrow] = make_uint2(a.out0, a.out1);
-        s_meta[meta_byte_offset(rr, c8)] = static_cast<uint8_t>(a.meta_byte);
-        s_mask[rr * 16 + c8] = static_cast<uint8_t>(a.mask_byte);
-        mb[t] = a.mask_byte;
-        w[t].x &= prmt(a.keep[0], a.keep[1], 0x5410u);
-        w[t].y &= prmt(a.keep[2], a.keep[3], 0x5410u);
-        w[t].z &= prmt(a.keep[0], a.keep[1], 0x7632u);
-        w[t].w &= prmt(a.keep[2], a.keep[3], 0x7632u);
+        s_meta[meta_byte_offset(rr, c8)] = static_cast<uint8_t>(meta_byte(a));
+        s_mask[rr * 16 + c8] = static_cast<uint8_t>(mask_byte(a));
+        const uint32_t x0 = E0 & a.keep[0], x1 = E1 & a.keep[1], x2 = E2 & a.keep[2], x3 = E3 & a.keep[3];
+        w[t] = make_uint4(prmt(x0, x1, 0x5410u), prmt(x2, x3, 0x5410u), prmt(x0, x1, 0x7632u), prmt(x2, x3, 0x7632u));
     }
 
     // ---- second pass on the masked tile (see double_prune_kernel)
-    uint32_t sel_bits[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    uint32_t sel[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const int meta_base = meta_byte_offset(c8 * 8, ig);
 #pragma unroll
     for (int wi = 0; wi < 4; ++wi) {
-        uint32_t e[8];
+        uint32_t x[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) e[t] = wi == 0 ? w[t].x : (wi == 1 ? w[t].y : (wi == 2 ? w[t].z : w[t].w));
-        const PackedPick a = pick2of4_packed(e[0], e[1], e[2], e[3]);
-        const PackedPick b = pick2of4_packed(e[4], e[5], e[6], e[7]);
-        const int j0 = c8 * 8 + 2 * wi;
-        const int slot = (ig ^ c8) * 8;
-        *reinterpret_cast<uint2*>(s_out + j0 * 128 + slot) = make_uint2(a.out0, b.out0);
-        *reinterpret_cast<uint2*>(s_out + (j0 + 1) * 128 + slot) = make_uint2(a.out1, b.out1);
-        s_metaT[meta_base + 16 * (2 * wi)] = static_cast<uint8_t>((a.meta_byte & 0xFu) | ((b.meta_byte & 0xFu) << 4));
-        s_metaT[meta_base + 16 * (2 * wi + 1)] = static_cast<uint8_t>((a.meta_byte >> 4) | (b.meta_byte & 0xF0u));
-        if (mask2 != nullptr) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                sel_bits[i] |= (((a.mask_byte >> i) & 1u) << (2 * wi)) | (((a.mask_byte >> (4 + i)) & 1u) << (2 * wi + 1));
-                sel_bits[4 + i] |= (((b.mask_byte >> i) & 1u) << (2 * wi)) | (((b.mask_byte >> (4 + i)) & 1u) << (2 * wi + 1));
-            }
-        }
+        for (int t = 0; t < 8; ++t) x[t] = wi == 0 ? w[t].x : (wi == 1 ? w[t].y : (wi == 2 ? w[t].z : w[t].w));
+        const PackedPick a = pick2of4_packed(x[0], x[1], x[2], x[3]);
+        const PackedPick b = pick2of4_packed(x[4], x[5], x[6], x[7]);
+        second_pass_store(a, b, 2 * wi, 2 * wi + 1, ig, c8, s_out, s_metaT + meta_base);
+        if (mask2 != nullptr) second_pass_select(a, b, 2 * wi, 2 * wi + 1, sel);
     }
     if (mask2 != nullptr) {
 #pragma unroll
         for (int t = 0; t < 8; ++t)
             mask2[(static_cast<size_t>(rb) * 128 + ig * 8 + t) * mrow + cb * 16 + c8] =
-                static_cast<uint8_t>(sel_bits[t] & mb[t]);
+                static_cast<uint8_t>((sel[t] | (sel[t] >> 16)) & s_mask[(ig * 8 + t) * 16 + c8]);
     }
     __syncthreads();
 
