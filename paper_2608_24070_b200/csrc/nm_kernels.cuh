@@ -55,7 +55,7 @@ template <int M>
 __global__ void __launch_bounds__(256)
 prune_nm_kernel(const uint4* W, size_t n_chunks, int n, uint4* out, uint16_t* __restrict__ mask) {
     constexpr int kChunks = M == 16 ? 2 : 1;
-    griddep_stream();
+    griddep_stream(8);
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t t0 = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; t0 < n_chunks / kChunks; t0 += stride) {
         const size_t c = kChunks == 1 ? t0 : (t0 & ~size_t(31)) * 2 + (t0 & 31);
@@ -105,7 +105,7 @@ prune_nm_kernel(const uint4* W, size_t n_chunks, int n, uint4* out, uint16_t* __
 // 512 contiguous bytes of a row) or 16 rows x 4 columns (8-byte loads; two neighbours share a mask byte), which
 // keeps the registers of the 16-row pattern under 128; output in the same orientation.  mask2 = kept by
 // both passes.  `out` may be `W` itself.
-// (Ordinary loads through unrestricted pointers: they stay behind griddep_stream(), and unlike volatile ones the
+// (Ordinary loads through unrestricted pointers: they stay behind griddep_stream, and unlike volatile ones the
 // compiler may place them, without which the kernel spills.)
 template <int WORDS>
 __device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&w)[WORDS]) {
@@ -123,7 +123,7 @@ double_prune_nm_kernel(const uint4* W, const uint8_t* mask1, int d_out, int d_in
     constexpr int kWords = M == 16 ? 2 : 4;
     const int per_row = d_in / (2 * kWords);                   // threads per row: a multiple of 32
     const size_t total = static_cast<size_t>(d_out / M) * per_row;
-    griddep_stream();
+    griddep_stream(M == 16 ? 2 : M == 8 ? 3 : 4);
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total; idx += stride) {
         const size_t h = idx / per_row, c = idx % per_row;
@@ -176,7 +176,7 @@ double_prune_nm_kernel(const uint4* W, const uint8_t* mask1, int d_out, int d_in
 // N:M pattern).  A thread owns 16 consecutive entries; `out` may be `G` itself.
 __global__ void __launch_bounds__(256)
 apply_mask_kernel(const uint4* G, const uint16_t* __restrict__ mask, size_t n_chunks, uint4* out) {
-    griddep_stream();
+    griddep_stream(8);
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
     for (size_t c = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; c < n_chunks; c += stride) {
         const uint4 a = ld_stream_v4(G + 2 * c), b = ld_stream_v4(G + 2 * c + 1);

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) prune24_kernel(const uint4* __restrict__ 
     const int u = tid & 7, r0 = tid >> 3;                 // 16-column slot, row within a pass of 32 rows
     const size_t row_u4 = static_cast<size_t>(d_in) >> 3;
 
-    griddep_stream();
+    griddep_stream(4);
     uint4 w[4][2];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256, 4) double_prune_kernel(const uint4* __res
     const size_t row_u4 = static_cast<size_t>(d_in) >> 3;
     const size_t mrow = static_cast<size_t>(d_in) >> 3;      // mask bytes per row
 
-    griddep_stream();
+    griddep_stream(4);
     uint4 w[8];
     uint32_t mb[8];
 #pragma unroll
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
     const size_t mrow = static_cast<size_t>(d_in) >> 3;      // mask bytes (= uint2 of values) per row
     const size_t at0 = (static_cast<size_t>(rb) * 128 + ig * 8) * row_u4 + cb * 16 + c8;
 
-    griddep_stream();
+    griddep_stream(4);
     uint4 w[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) w[t] = ld_v4(W + at0 + t * row_u4);
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(256) meta_to_canonical_kernel(const uint16_t* 
 // `out` may be A or B (every thread reads its vectors before it writes them), hence no __restrict__.
 __global__ void __launch_bounds__(256) sparse_add_kernel(const uint4* A, const uint4* B, float beta, float gamma,
                                                          size_t n_vec, uint4* out) {
-    griddep_stream();
+    griddep_stream(8);
     for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < n_vec;
          idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
         const uint4 a = ld_v4(A + idx), b = ld_v4(B + idx);
@@ -384,7 +384,7 @@ update_transposed_kernel(const uint2* __restrict__ Wc_new, const uint8_t* __rest
     const int num_tiles = ncb * nrb;
 
     if (tid < 16) s_expand[tid] = make_uint2(expand_selector(tid), expand_selector(tid) >> 16);
-    griddep_stream();
+    griddep_wait();
 
     uint2 cw[8];
     uint32_t mb[8];

@@ -227,14 +227,20 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
 // on has finished and its writes are visible (no-op for an ordinary launch);
 // `griddep_launch_dependents` lets a dependent launch that opted in begin its own prologue.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_launch_dependents();
-// The start of a streaming kernel: its blocks are set up while the preceding kernel drains, and the next kernel's
-// blocks move in as this one's leave.
-__device__ __forceinline__ void griddep_stream() {
-    griddep_launch_dependents();
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The start of a streaming kernel with room for `resident` blocks per SM: its blocks are set up while the preceding kernel
+// drains.  It lets the next kernel's blocks in before its own have left only when it fills the GPU about once itself: the
+// next blocks go wherever a slot is free, and beside a partial wave that puts most of them on a few SMs.
+// us per launch, back to back, early / not: first pass of 768 x 3072 (144 blocks) 3.7 / 2.3, of 2048 x 2048 (256) 3.5 / 3.2,
+// of 3072 x 3072 (576) 5.4 / 5.7, of 4096 x 4096 (1024) 10.5 / 11.4; masked copy of 1024 x 1024 (512) 2.6 / 1.5.
+__device__ __forceinline__ void griddep_stream(uint32_t resident) {
+    // (predicated, not a branch: the kernels' register allocation is tight)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ge.u32 p, %0, %1;\n\t@p griddepcontrol.launch_dependents;\n\t}"
+        ::"r"(gridDim.x * gridDim.y), "r"(128u * resident)
+        : "memory");
     griddep_wait();
 }
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float4 ld_shared_v4(uint32_t saddr) {
     float4 v;

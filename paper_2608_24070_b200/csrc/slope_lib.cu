@@ -278,8 +278,8 @@ static bool set_smem(Kernel k, int bytes) {
 }
 
 // Streaming kernels are launched with programmatic stream serialisation too: every thread waits for the preceding
-// kernel before it touches memory (griddep_stream), but the blocks are already resident, and the ramp-up and
-// tail of back-to-back passes overlap.
+// kernel before it touches memory (griddep_stream), but the blocks are set up by then, and on large grids the
+// ramp-up and tail of back-to-back passes overlap.
 template <typename... KArgs, typename... Args>
 static slope_status_t launch_stream(void (*kern)(KArgs...), dim3 grid, cudaStream_t stream, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
