@@ -1398,18 +1398,19 @@ sparse_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         // ---------------------------------------------------------- activation ring
         if (elect_one()) {
             PipeState ps;
+            const uint32_t half_bytes = p.width * 128;                   // p.width token rows (see launch_sparse_skinny)
             for (int i = 0; i < total_kb; ++i) {
                 if (!mbar_wait(&emptyB[ps.stage], ps.phase ^ 1u, abort_flag)) break;
                 uint8_t* sB = smem + Cfg::kOffB + ps.stage * Cfg::kBStage;
                 uint64_t* bar = &fullB[ps.stage];
                 if (i < num_sb) {
                     const int kb = kb0 + i;
-                    mbar_expect_tx(bar, Cfg::kBStage);
+                    mbar_expect_tx(bar, 2 * half_bytes);
                     tma_load_2d(sB, &tmB, bar, kb * 128, 0);
                     tma_load_2d(sB + BLOCK_N * 128, &tmB, bar, kb * 128 + 64, 0);
                 } else {
                     if (p.pdl_mode == 2 && i == num_sb) griddep_wait();      // T comes from the launch before this one
-                    mbar_expect_tx(bar, BLOCK_N * 128);
+                    mbar_expect_tx(bar, half_bytes);
                     tma_load_2d(sB, &tmB2, bar, (i - num_sb) * 64, 0);
                 }
                 ps.advance(B_STAGES);

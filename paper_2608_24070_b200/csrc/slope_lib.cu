@@ -523,7 +523,7 @@ constexpr double kSkinnySmUs = 0.23, kSkinnyHbmUs = 0.0028, kSkinnyWaveUs = 4.0,
                  kSkinnyReducePerRankUs = 0.07;
 
 // A k-block costs an SM its weight tile (kSkinnySmUs) plus the activation tile's TMA row
-// requests (2 per token of the tile, ~2 ns each).
+// requests (2 per token, ~2 ns each, counted here for a full tile).
 constexpr double kSkinnyTokenUs = 0.004;
 
 static int skinny_splits(int slabs, int num_kb, int block_n, const int (&cap)[9], double* est_us = nullptr) {
@@ -579,13 +579,17 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
                                            const void* act2, const void* fac2, int r, bool a2_mn, void* out,
                                            cudaStream_t stream, const DeviceInfo& info, int pdl_mode) {
     using Cfg = SparseSkinnyCfg<BLOCK_N, A_STAGES, B_STAGES>;
+    // An activation box has a row per token and no more: an SM takes about one 128-byte row of any box per 2 clocks, inside
+    // the matrix or not, and what the MMAs read beyond them only reaches accumulator columns that are never stored.  us at one
+    // token, boxes of 16 rows / of 1: 4096 -> 22016 23.2 / 20.0, 4096 -> 12288 13.3 / 12.3, 4096 -> 4096 7.1 / 6.9.
+    const int rows = std::min(ntok, BLOCK_N);
     CUtensorMap tmA, tmB, tmE, tmA2, tmB2;
     if (r > 0) {
         const bool ok2 = a2_mn ? make_tmap(&tmA2, fac2, r, M, 64, 64) : make_tmap(&tmA2, fac2, M, r, kBlockM, 64);
-        if (!ok2 || !make_tmap(&tmB2, act2, ntok, r, BLOCK_N, 64)) return SLOPE_ERR_CUDA;
+        if (!ok2 || !make_tmap(&tmB2, act2, ntok, r, rows, 64)) return SLOPE_ERR_CUDA;
     }
     if (!make_tmap(&tmA, vals, M, K / 2, kBlockM, 64)) return SLOPE_ERR_CUDA;
-    if (!make_tmap(&tmB, act, ntok, K, BLOCK_N, 64)) return SLOPE_ERR_CUDA;
+    if (!make_tmap(&tmB, act, ntok, K, rows, 64)) return SLOPE_ERR_CUDA;
     if (!make_tmap_meta(&tmE, meta, static_cast<size_t>(M) * K / 8)) return SLOPE_ERR_CUDA;
     if (r <= 0) {
         tmA2 = tmA;
@@ -593,7 +597,7 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
     }
     SparseGemmParams p = {};
     p.M = M; p.K = K; p.Ntok = ntok; p.r = r; p.a2_mn_major = a2_mn ? 1 : 0;
-    p.pdl_mode = pdl_mode;
+    p.pdl_mode = pdl_mode; p.width = rows;
     p.meta = static_cast<const uint8_t*>(meta);
     p.out = static_cast<uint16_t*>(out);
     auto kern = sparse_gemm_skinny_kernel<BLOCK_N, A_STAGES, B_STAGES>;

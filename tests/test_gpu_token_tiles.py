@@ -63,3 +63,28 @@ def test_token_tiles_match_fp64(b, d_in, d_out, r):
     assert torch.isnan(Y[b]).all() and torch.isnan(dX[b]).all()
     assert parity_error(g(Y[:b]), ref_Y) <= REL_TOL
     assert parity_error(g(dX[:b]), ref_dX) <= REL_TOL
+
+
+@pytest.mark.parametrize("b,before", [(1, 16), (7, 16), (13, 16), (17, 64), (63, 64), (65, 128), (127, 128)])
+def test_few_tokens_do_not_see_what_an_earlier_launch_left_in_shared_memory(b, before):
+    """Activation tiles are loaded for as many tokens as there are; the MMAs also read the rows behind them."""
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    d_in, d_out, r = 2048, 1024, 32
+    layer = GpuLayer(si.gaussian_bf16((d_out, d_in), 0.02, 56), fused_setup=True)
+    L, R = (B.bf16_from_bits(si.gaussian_bf16(s, 0.1, 57)) for s in ((d_in, r), (r, d_out)))
+    X = B.bf16_from_bits(si.gaussian_bf16((b, d_in), 1.0, 58))
+    out = []
+    for fill in (0.0, float("nan")):
+        noise, T0, Y0 = (torch.full((before, n), fill, dtype=torch.bfloat16, device="cuda") for n in (d_in, r, d_out))
+        for _ in range(3):                                       # on every SM
+            B.slope_linear_fwd(noise, layer.Wc_vals, layer.Wc_meta, d_out, Y0, T0, R)
+        T, Y = (torch.empty((b, n), dtype=torch.bfloat16, device="cuda") for n in (r, d_out))
+        B.slope_linear_fwd_adapter(X, layer.Wc_vals, layer.Wc_meta, d_out, L, R, T, Y)
+        out.append((T, Y))
+    (T, Y), (T1, Y1) = out
+    assert torch.isfinite(Y).all() and torch.equal(Y.view(torch.int16), Y1.view(torch.int16))
+    assert torch.equal(T.view(torch.int16), T1.view(torch.int16))
+    assert B.slope_poll_status() == 0
