@@ -157,19 +157,18 @@ static bool make_tmap_meta(CUtensorMap* tm, const void* base, size_t total_bytes
     });
 }
 
-// 2-D bf16 tensor map for TMA stores of output tiles: unswizzled, or (for a box 64 bytes wide) with
-// the 64-byte swizzle the transposing epilogues write their staging tiles in.
-static bool make_tmap_plain(CUtensorMap* tm, const void* base, int rows, int cols, int box_rows, int box_cols,
-                            bool swizzle64 = false) {
+// 2-D bf16 tensor map for the TMA stores of the transposing epilogues: boxes 64 bytes wide, with the 64-byte swizzle their
+// staging tiles are written in.
+static bool make_tmap_out(CUtensorMap* tm, const void* base, int rows, int cols, int box_rows, int box_cols) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
     const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
     const cuuint64_t gstride[1] = {static_cast<cuuint64_t>(cols) * 2};
     const cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), static_cast<cuuint32_t>(box_rows)};
     const cuuint32_t estr[2] = {1, 1};
-    return tmap_memo(tm, TmapKey{base, rows, cols, box_rows, box_cols, swizzle64 ? 3 : 2}, [&](CUtensorMap* out) {
+    return tmap_memo(tm, TmapKey{base, rows, cols, box_rows, box_cols, 3}, [&](CUtensorMap* out) {
         return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                   CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     });
@@ -428,10 +427,10 @@ struct SparseTileArgs {
 };
 static bool sparse_tile_args(SparseTileArgs& a, const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                              const void* act2, const void* fac2, int r, bool a2_mn, void* out, int width, int stages,
-                             bool swizzle_out, int pdl_mode) {
+                             int pdl_mode) {
     if (!make_tmap(&a.tmA, vals, M, K / 2, kBlockM, 64) || !make_tmap(&a.tmB, act, ntok, K, width / 2, 64) ||
         !make_tmap_meta(&a.tmE, meta, static_cast<size_t>(M) * K / 8) ||
-        !make_tmap_plain(&a.tmO, out, ntok, M, SparsePairCfg::kStoreRows, SparsePairCfg::kStoreCols, swizzle_out))
+        !make_tmap_out(&a.tmO, out, ntok, M, SparsePairCfg::kStoreRows, SparsePairCfg::kStoreCols))
         return false;
     if (r > 0) {
         const bool ok2 = a2_mn ? make_tmap(&a.tmA2, fac2, r, M, 64, 64) : make_tmap(&a.tmA2, fac2, M, r, kBlockM, 64);
@@ -463,7 +462,7 @@ static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* 
     using Cfg = SparsePairCfg;
     SparseTileArgs a;
     const int stages = tile_stages<Cfg>(width);
-    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, true, pdl_mode))
+    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, pdl_mode))
         return SLOPE_ERR_CUDA;
     if (!set_smem(sparse_gemm_pair_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
     const int tiles = ((M / kBlockM + 1) / 2) * ((ntok + width - 1) / width);
@@ -502,7 +501,7 @@ static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* 
     using Cfg = SparseQuadCfg;
     SparseTileArgs a;
     const int stages = tile_stages<Cfg>(width);
-    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, false, pdl_mode))
+    if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, pdl_mode))
         return SLOPE_ERR_CUDA;
     a.p.group_m = quad_group_m(M, K, ntok, width, max_pairs);
     if (!set_smem(sparse_gemm_quad_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
