@@ -589,8 +589,9 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const uint32_t t_row = tmem_base + acc * kMaxTokenTile + (static_cast<uint32_t>(q * 32) << 16);
             const int m0 = (m_pair * 2 + static_cast<int>(cta)) * kBlockM + q * 32;
             const int width = token_tile_width(p.Ntok, n_blk * p.width, p.width);
+            // (rows past M are not staged either: the wait for a staging buffer counts stores)
 #pragma unroll 1
-            for (int c0 = half * Cfg::kStoreRows; c0 < width; c0 += 2 * Cfg::kStoreRows) {
+            for (int c0 = half * Cfg::kStoreRows; m0 < p.M && c0 < width; c0 += 2 * Cfg::kStoreRows) {
                 uint32_t block[16];
                 load_packed_block(t_row + c0, block);
                 // the staging buffer about to be overwritten must have been read by its TMA store
@@ -599,7 +600,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 stage_packed_block(smem_u32(my_buf + buf * Cfg::kStoreBytes), lane, block);
                 fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0 && m0 < p.M) {
+                if (lane == 0) {
                     tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n_blk * p.width + c0, stream_out);
                     tma_store_commit();
                 }
@@ -1134,13 +1135,16 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         int it = 0;
         uint32_t buf = 0;
         auto store_block = [&](const uint32_t (&block)[16], int m0, int n0) {
+            // (Rows past M are not staged either: the wait below counts stores, and a block that is staged but not stored
+            // would let the one after it overwrite a buffer whose store is still reading.)
+            if (m0 >= p.M) return;
             // the staging buffer about to be overwritten must have been read by its TMA store
             if (lane == 0) tma_store_wait_read<1>();
             __syncwarp();
             stage_packed_block(smem_u32(my_buf + buf * Cfg::kStoreBytes), lane, block);
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0 && m0 < p.M) {
+            if (lane == 0) {
                 tma_store_2d_hint(&tmO, my_buf + buf * Cfg::kStoreBytes, m0, n0, stream_out);
                 tma_store_commit();
             }

@@ -30,6 +30,7 @@ pytestmark = pytest.mark.gpu
     (1345, 1152, 640, 0),
     (2048, 1024, 4096, 32),
     (5000, 2048, 1408, 0),       # several waves, 512-row tiles the other way round
+    (15257, 512, 3968, 0),       # 31 row blocks: in the last 512-row tile one CTA has rows for one sub-tile only
 ])
 def test_token_tiles_match_fp64(b, d_in, d_out, r):
     import torch
