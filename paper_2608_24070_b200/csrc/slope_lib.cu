@@ -665,10 +665,10 @@ static slope_status_t launch_skinny(const void* act, int ntok, const void* vals,
 //   width      the token tiles of a launch are made equal (500 tokens: three of 192 and less rather than two of
 //              224 and one of 64) and as wide as fills the waves of CTA pairs best.
 // In SM clocks: a k-block takes the round trip of a pipeline stage (2130, 2515 with all pairs at work) over the stages
-// that fit, and at least its bytes (70 per clock and SM) and its MMAs; a 512-row tile exposes 12 per token
-// of width, the last drain of a launch takes 290 + 8.7 per token (4.4 times that for 512 rows), a launch
-// 47 per pair.  Fitted to a sweep of all tiles over 23 layer shapes (640 ... 22016 wide) and 130 ... 8192
-// tokens, where the choice is on average 0.6 %, at most 11 % slower than the best tile of the sweep.
+// that fit, and at least its bytes (70 per clock and SM) and its MMAs; a 512-row tile exposes 3.3 per token
+// of width, the last drain of a launch takes 290 + 8.7 per token (2.4 times that for 512 rows), a launch
+// 47 per pair.  Fitted to a sweep of all tiles over 18 layer shapes (768 ... 22016 wide) and 160 ... 8192
+// tokens, where the choice is on average 0.7 %, at most 12 % slower than the best tile of the sweep.
 struct SparseTile {
     int rows, width;
 };
@@ -680,8 +680,8 @@ static double sparse_tile_cost(int M, double num_kb, int ntok, int width, int nu
     const double load = Cfg::stage_bytes(width) / 70.0, mma = rows * std::max(width, 64) / 128.0;
     const double round_trip = 2130.0 + 385.0 * active / num_pairs;
     const double k_block = std::max({round_trip / tile_stages<Cfg>(width), load, mma});
-    const double tile = num_kb * k_block + (quad ? 12.0 * width : 0.0);
-    const double last_drain = (quad ? 4.4 : 1.0) * (290.0 + 8.7 * width);
+    const double tile = num_kb * k_block + (quad ? 3.3 * width : 0.0);
+    const double last_drain = (quad ? 2.4 : 1.0) * (290.0 + 8.7 * width);
     return (tiles + num_pairs - 1) / num_pairs * tile + last_drain + 47.0 * active;
 }
 static SparseTile choose_sparse_tile(int M, int K, int ntok, int r, int num_pairs, double* cost = nullptr) {
