@@ -792,9 +792,9 @@ static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* 
     return launch_sparse_tile(t, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, pairs, stream, 0);
 }
 
-static int dense_stages(bool b_mn, int width) {
+static int dense_stages(bool b_mn, int epi, int width) {
     int n = DensePairCfg::kMaxStages;
-    while (n > 1 && DensePairCfg::smem_bytes(b_mn, width, n) > 232448) --n;
+    while (n > 1 && DensePairCfg::smem_bytes(b_mn, epi, width, n) > 232448) --n;
     return n;
 }
 // Columns per tile of the dense CTA-pair kernel, by estimate.  Narrow tiles give a small matrix enough of them for the
@@ -847,13 +847,16 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
                                  tmB, p);
     }
     using Cfg = DensePairCfg;
-    const int stages = dense_stages(B_MN, width);
+    CUtensorMap tmO = tmA;
+    if (EPI == kEpiStore && !make_tmap_out(&tmO, out, M, N, 32, 32)) return SLOPE_ERR_CUDA;
+    const int stages = dense_stages(B_MN, EPI, width);
     const DenseGemmParams p{M, N, K, width, stages, out, static_cast<const uint8_t*>(mask)};
     auto kern = dense_gemm_pair_kernel<A_MN, B_MN, EPI>;
     if (!set_smem(kern, 232448)) return SLOPE_ERR_CUDA;
     const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + width - 1) / width);
     const int pairs = std::min(tiles, max_pairs);
-    return launch_pairs(kern, 2 * pairs, kDenseThreads, Cfg::smem_bytes(B_MN, width, stages), stream, tmA, tmB, p);
+    return launch_pairs(kern, 2 * pairs, kDenseThreads, Cfg::smem_bytes(B_MN, EPI, width, stages), stream, tmA, tmB,
+                        tmO, p);
 }
 
 static int adapter_splits(int b, int rows) {

@@ -44,7 +44,8 @@ def test_masked_weight_gradient(b, d_in, d_out):
 
 
 @pytest.mark.parametrize("b,d_in,d_out", [(1, 128, 128), (130, 256, 384), (300, 1152, 640), (513, 384, 2176),
-                                        (700, 2048, 4224), (600, 3200, 2688)])
+                                        (700, 2048, 4224), (600, 3200, 2688),
+                                        (3000, 256, 4992)])
 def test_dense_layer(b, d_in, d_out):
     import torch
 
