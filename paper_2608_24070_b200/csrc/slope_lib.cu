@@ -802,7 +802,8 @@ static int dense_stages(bool b_mn, int epi, int width) {
 // MMAs (2.36 per column, no fewer than 80 columns' worth), a tile no less than its drain, a launch one more drain
 // and 47 per pair.  (192 columns of a [K x N] operand cost the bytes of 256 and are not taken.)  Fitted to a sweep over
 // 12 layer shapes (512 ... 9728) and 64 ... 8192 tokens: 0.2 % slower on average than the best width, where 256 x 256
-// throughout is 24 %.  us, 256 x 256 -> now: forward / input gradient of a dense layer 500 tokens 1024 x 1024 9.5 / 9.6 ->
+// throughout is 24 % (the plain store's drain was 24 per column then; halved since, which moves weight gradients of 256 tokens
+// 4096 x 4096 12.8 -> 10.9, 486 tokens 4224 x 2560 13.2 -> 12.1, 700 tokens 2048 x 6144 18.2 -> 16.4).  us, 256 x 256 -> now: forward / input gradient of a dense layer 500 tokens 1024 x 1024 9.5 / 9.6 ->
 // 4.9 / 5.6, 740 tokens 8320 -> 6400 forward 84 -> 68, 700 tokens 2048 -> 6144 input gradient 32.6 -> 21.1.
 static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int num_pairs) {
     const int num_m = (M + 255) / 256, num_kb = (K + 63) / 64;
@@ -814,7 +815,7 @@ static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int n
         const bool halves = b_mn && width == 256 && tiles > num_pairs && 2 * rem <= num_pairs;      // see pair_work
         const double waves = tiles / num_pairs + (rem == 0 ? 0.0 : halves ? 0.5 : 1.0);
         const double k_block = std::max(DensePairCfg::stage_bytes(b_mn, width) / 70.0, 2.36 * std::max(width, 80));
-        const double drain = masked ? 850.0 + 11.8 * width : 780.0 + 24.2 * width;
+        const double drain = masked ? 850.0 + 11.8 * width : 780.0 + 12.0 * width;
         const double cost = waves * std::max(num_kb * k_block, drain) + drain + 47.0 * std::min(tiles, num_pairs);
         if (cost < best_cost) { best_cost = cost; best = width; }
     }
