@@ -237,16 +237,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             const bool live = m < p.M && n_first < p.N;
             // first-pass mask bits of this thread's columns, fetched before the accumulator is ready
             uint32_t mbits[4] = {0u, 0u, 0u, 0u};
-            if (live) {
-                const uint8_t* mp = p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n_first >> 3);
-                if (w.width == BLOCK_N) {
-                    const uint4 v = __ldg(reinterpret_cast<const uint4*>(mp));
-                    mbits[0] = v.x; mbits[1] = v.y; mbits[2] = v.z; mbits[3] = v.w;
-                } else {
-                    const uint2 v = __ldg(reinterpret_cast<const uint2*>(mp));
-                    mbits[0] = v.x; mbits[1] = v.y;
-                }
-            }
+            if (live) load_mask_bits(p.mask + static_cast<size_t>(m) * (p.N >> 3) + (n_first >> 3), w.width / 2, mbits);
             if (!mbar_wait(tfull_bar, static_cast<uint32_t>(it) & 1u, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
             const uint32_t t_row = tmem_base + (static_cast<uint32_t>(q * 32) << 16);

@@ -32,3 +32,35 @@ def test_chained_passes_wait_for_each_other(d_out, d_in):
     for a, b in zip(chain(False), chain(True)):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
     assert B.slope_poll_status() == 0
+
+
+@pytest.mark.parametrize("d_out,d_in", [(4096, 4096), (3840, 2560)])
+@pytest.mark.parametrize("r", [32, 256])                        # adapter gradients inside the weight-gradient launch / beside it
+def test_gradients_wait_for_the_mask(d_out, d_in, r):
+    """The weight gradient reads the mask that the pruning pass in front of it writes, in an array that held another mask."""
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    b = 96
+    gen = torch.Generator("cuda").manual_seed(7)
+    new = lambda *shape: torch.randn(shape, generator=gen, dtype=torch.bfloat16, device="cuda")
+    Ws, X, dY, T, dT = [new(d_out, d_in), new(d_out, d_in)], new(b, d_in), new(b, d_out), new(b, r), new(b, r)
+    ws = torch.empty(B.slope_bwd_dw_adapter_workspace_bytes(b, d_out, d_in, r), dtype=torch.uint8, device="cuda")
+
+    def chain(settle):
+        v, m, k = B.alloc_compressed(d_out, d_in)
+        out = []
+        for W in Ws * 2:
+            dWc, dL, dR = (torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((d_out, d_in // 2), (d_in, r), (r, d_out)))
+            B.slope_prune_24(W, v, m, k)
+            if settle:
+                torch.cuda.synchronize()
+            B.slope_linear_bwd_dw_adapter(dY, X, T, dT, k, dWc, dL, dR, ws)
+            out += [dWc, dL, dR]
+        torch.cuda.synchronize()
+        return out
+
+    for x, y in zip(chain(False), chain(True)):
+        assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+    assert B.slope_poll_status() == 0
