@@ -351,10 +351,10 @@ def kernel_sources_sha256():
 # sources reports traffic = null (tests/test_bench_line.py fails until the capture is refreshed or
 # cleared).
 NCU_TRAFFIC = {
-    "sources": "7789ed6cc30292ef38521fe9213e30ee0e33c0058cbf348bce32188120fada05",
+    "sources": None,
     "captured_tokens": 16384,
-    "sparse_bytes_per_launch": 496199314,     # mean over the 14 sparse GEMM launches of one step
-    "dense_bytes_per_launch": 1220423278,     # mean over the 7 weight-gradient launches of one step
+    "sparse_bytes_per_launch": None,     # mean over the 14 sparse GEMM launches of one step
+    "dense_bytes_per_launch": None,     # mean over the 7 weight-gradient launches of one step
 }
 
 

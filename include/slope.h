@@ -159,9 +159,9 @@ slope_status_t slope_linear_bwd_dw_masked(const void* dY, const void* X, int b, 
  *             (dT and T are the bf16 tensors written by this call / phase 0).
  *   phase 2:  dT[b x r] = dY R^T only (dL and dR then come from slope_linear_bwd_dw_adapter).
  * `workspace` is device scratch of at least slope_adapter_workspace_bytes()
- * bytes for phase 1 (the present kernels sum their partial products inside a
- * thread-block cluster and leave it untouched); unused pointers of the other
- * phase may be NULL.
+ * bytes for phase 1: dL and dR may overlap the operands, and are then formed in it
+ * and copied into place (otherwise partial products are summed inside a thread-block
+ * cluster and it is left untouched); unused pointers of the other phase may be NULL.
  */
 size_t slope_adapter_workspace_bytes(int b, int d_out, int d_in, int r);
 slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY,

@@ -47,3 +47,56 @@ def test_adapter_products_match_fp64(b, d_in, d_out, r):
     errs = {"T": parity_error(g(T[:b]), f["X"] @ f["L"]), "dT": parity_error(g(dT), f["dY"] @ f["R"].T),
             "dL": parity_error(g(dL), f["X"].T @ g(dT)), "dR": parity_error(g(dR), g(T[:b]).T @ f["dY"])}
     assert all(v <= REL_TOL for v in errs.values()), errs
+
+
+def _gradient_operands(b, d_in, d_out, r):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(35)
+    new = lambda *shape: torch.randn(shape, generator=gen, dtype=torch.bfloat16, device="cuda")
+    o = {"X": new(b, d_in), "dY": new(b, d_out), "R": new(r, d_out), "T": new(b, r), "dT": new(b, r)}
+    fresh = lambda: {k: v.clone() for k, v in o.items()} | {
+        "dL": torch.empty((d_in, r), dtype=torch.bfloat16, device="cuda"), "dR": torch.empty((r, d_out), dtype=torch.bfloat16, device="cuda")}
+    return B, fresh
+
+
+def _same_gradients(fresh, run, d_in, d_out, r, places):
+    """run(o) with gradients of their own against the same call with dL / dR at the start of an operand's memory."""
+    import torch
+
+    o = fresh()
+    run(o)
+    for dL_in, dR_in in places:
+        q = fresh()
+        if dL_in:
+            q["dL"] = q[dL_in].view(-1)[:d_in * r].view(d_in, r)
+        if dR_in:
+            q["dR"] = q[dR_in].view(-1)[:r * d_out].view(r, d_out)
+        run(q)
+        for k in ("dL", "dR"):
+            assert torch.equal(o[k].view(torch.int16), q[k].view(torch.int16)), (dL_in, dR_in, k)
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [(700, 256, 384, 128), (1000, 768, 2304, 16), (4096, 1024, 2560, 256), (2500, 128, 128, 64)])
+def test_gradients_may_take_the_place_of_operands(b, d_in, d_out, r):
+    B, fresh = _gradient_operands(b, d_in, d_out, r)
+    ws = B.torch.empty(B.slope_adapter_workspace_bytes(b, d_out, d_in, r), dtype=B.torch.uint8, device="cuda")
+    run = lambda o: B.slope_adapter_fwd_bwd(1, o["X"], o["dY"], None, o["R"], b, d_out, d_in, r, T=o["T"], dT=o["dT"], dL=o["dL"],
+                                            dR=o["dR"], workspace=ws)
+    _same_gradients(fresh, run, d_in, d_out, r, [(None, "R"), ("X", "dY"), ("dY", "X"), ("T", "R") if b >= d_in else ("X", "R")])
+    assert B.slope_poll_status() == 0
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [(1000, 768, 2304, 16), (700, 256, 384, 128), (600, 4096, 4096, 32)])
+def test_gradients_beside_the_weight_gradient_may_take_the_place_of_operands(b, d_in, d_out, r):
+    B, fresh = _gradient_operands(b, d_in, d_out, r)
+    W = B.torch.randn((d_out, d_in), dtype=B.torch.bfloat16, device="cuda")
+    v, m, mask = B.alloc_compressed(d_out, d_in)
+    B.slope_prune_24(W, v, m, mask)
+    dWc = B.torch.empty_like(v)
+    ws = B.torch.empty(B.slope_bwd_dw_adapter_workspace_bytes(b, d_out, d_in, r), dtype=B.torch.uint8, device="cuda")
+    run = lambda o: B.slope_linear_bwd_dw_adapter(o["dY"], o["X"], o["T"], o["dT"], mask, dWc, o["dL"], o["dR"], ws)
+    _same_gradients(fresh, run, d_in, d_out, r, [("X", None), (None, "dY"), ("dY", "X")])
+    assert B.slope_poll_status() == 0
