@@ -276,6 +276,9 @@ slope_status_t slope_dense_linear_bwd_dw(const void* dY, const void* X, int b, i
  *    anything is launched; use slope_adapter_fwd_bwd for those.
  *  - The sums are formed in fixed order inside a thread-block cluster: the call keeps no state and
  *    may run on any number of streams at a time.
+ *  - dL may overlap X or dT.  It is then formed in a fixed 8 MiB array of the library image and copied
+ *    into place; such calls on a device share that array, so serialise them, and make the first one
+ *    before any stream capture.
  * Calls no cudaMalloc / cudaFree and no allocating library routine.
  */
 size_t slope_adapter_dl_noalloc_max_scratch_bytes(void);

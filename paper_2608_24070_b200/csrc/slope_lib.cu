@@ -1362,24 +1362,36 @@ slope_status_t slope_meta_to_canonical(const void* meta_hw, int rows, int cols, 
 }  // extern "C"
 
 // ------------------------------------------------------------------ allocation-free adapter-gradient entry
-// The adapter kernels reduce inside a cluster, so dL needs neither an allocation nor a workspace.
-// The sizes this call takes are still those whose split-K partial sums would fit 16 MiB, as its
-// contract says.
+// The adapter kernels reduce inside a cluster, so dL needs neither an allocation nor a workspace -- unless it is to take
+// the place of X or dT: CTAs store their shares while others still read, so it is then formed in a fixed
+// array of the library image and copied.  The sizes this call takes are those whose split-K partial sums
+// would fit 16 MiB, as its contract says; a bf16 dL is at most half of that.
+namespace slope {
+constexpr size_t kDlLimitBytes = size_t(16) << 20;
+static __device__ __align__(256) uint8_t g_dl_scratch[kDlLimitBytes / 2];
+}  // namespace slope
+
 extern "C" {
 
-size_t slope_adapter_dl_noalloc_max_scratch_bytes(void) { return size_t(16) << 20; }
+size_t slope_adapter_dl_noalloc_max_scratch_bytes(void) { return kDlLimitBytes; }
 
 slope_status_t slope_adapter_dl_noalloc(const void* X, const void* dT, int b, int d_in, int r, void* dL,
-                                        void* stream) {
+                                        void* stream_) {
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (!X || !dT || !dL) return SLOPE_ERR_INVALID_ARG;
     if (d_in <= 0 || d_in % 128 != 0 || b < 1 || !rank_ok(r) || r == 0) return SLOPE_ERR_SHAPE;
     if (!aligned16(X) || !aligned16(dT) || !aligned16(dL)) return SLOPE_ERR_ALIGNMENT;
     const size_t need = static_cast<size_t>(adapter_splits(b, d_in)) * d_in * r * sizeof(float);
-    if (need > slope_adapter_dl_noalloc_max_scratch_bytes()) return SLOPE_ERR_SHAPE;
+    if (need > kDlLimitBytes) return SLOPE_ERR_SHAPE;
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
-    return launch_adapter<true, true>(adapter_dL(X, dT, d_in, dL), AdapterOperands{}, r, b,
-                                      static_cast<cudaStream_t>(stream), info);
+    const size_t bytes = sizeof(uint16_t) * d_in * r, rows = b;
+    const bool staged = overlap(dL, bytes, X, sizeof(uint16_t) * rows * d_in) || overlap(dL, bytes, dT, sizeof(uint16_t) * rows * r);
+    void* out = dL;
+    if (staged && cudaGetSymbolAddress(&out, g_dl_scratch) != cudaSuccess) return SLOPE_ERR_CUDA;
+    if (slope_status_t st = launch_adapter<true, true>(adapter_dL(X, dT, d_in, out), AdapterOperands{}, r, b, stream, info)) return st;
+    if (staged && cudaMemcpyAsync(dL, out, bytes, cudaMemcpyDeviceToDevice, stream) != cudaSuccess) return SLOPE_ERR_CUDA;
+    return SLOPE_OK;
 }
 
 }  // extern "C"

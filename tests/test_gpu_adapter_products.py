@@ -100,3 +100,19 @@ def test_gradients_beside_the_weight_gradient_may_take_the_place_of_operands(b, 
     run = lambda o: B.slope_linear_bwd_dw_adapter(o["dY"], o["X"], o["T"], o["dT"], mask, dWc, o["dL"], o["dR"], ws)
     _same_gradients(fresh, run, d_in, d_out, r, [("X", None), (None, "dY"), ("dY", "X")])
     assert B.slope_poll_status() == 0
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [(1000, 768, 128, 16), (300, 256, 128, 256), (2000, 1024, 128, 256)])
+def test_noalloc_gradient_may_take_the_place_of_an_operand(b, d_in, d_out, r):
+    B, fresh = _gradient_operands(b, d_in, d_out, r)
+    run = lambda o: B.slope_adapter_dl_noalloc(o["X"], o["dT"], o["dL"])
+    o = fresh()
+    run(o)
+    for place in ("X", "dT"):
+        q = fresh()
+        if q[place].numel() < d_in * r:
+            continue
+        q["dL"] = q[place].view(-1)[-d_in * r:].view(d_in, r)
+        run(q)
+        assert B.torch.equal(o["dL"].view(B.torch.int16), q["dL"].view(B.torch.int16)), place
+    assert B.slope_poll_status() == 0
