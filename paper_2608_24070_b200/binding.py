@@ -106,6 +106,11 @@ def lib() -> ctypes.CDLL:
                      "slope_linear_bwd_dw_masked", "slope_adapter_fwd_bwd", "slope_meta_to_canonical",
                      "slope_poll_status"):
             getattr(L, name).restype = ci
+        from . import build
+
+        if build.NATIVE.exists() and not build.native_matches():
+            raise RuntimeError("the binding's native module _slope.so was built against another torch or Python: build it again "
+                               "with `python -m paper_2608_24070_b200.build`")
         try:
             from . import _slope
         except ImportError as e:

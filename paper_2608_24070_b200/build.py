@@ -38,8 +38,25 @@ def _newer(target: Path, sources) -> bool:
     return all(p.stat().st_mtime <= t for p in sources)
 
 
+def native_build() -> str:
+    """What _slope.so depends on besides its sources: torch's C++ interface and this interpreter's."""
+    import torch
+
+    return (f"_slope.so for torch {torch.__version__}, C++11 ABI {int(torch._C._GLIBCXX_USE_CXX11_ABI)}, "
+            f"{sysconfig.get_config_var('SOABI')}")
+
+
+def native_matches() -> bool:
+    """_slope.so is there and was compiled against this torch and this Python (it carries native_build() as a string)."""
+    return NATIVE.exists() and native_build().encode() + b"\0" in NATIVE.read_bytes()
+
+
+def _native_current() -> bool:
+    return _newer(NATIVE, NATIVE_SOURCES) and native_matches()
+
+
 def up_to_date() -> bool:
-    return _newer(LIB, SOURCES + HEADERS) and _newer(NATIVE, NATIVE_SOURCES)
+    return _newer(LIB, SOURCES + HEADERS) and _native_current()
 
 
 def _compile(cmd, target: Path) -> None:
@@ -55,6 +72,7 @@ def native_command():
     cuda = Path(nvcc_path()).resolve().parent.parent
     abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
     return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
+            f'-DSLOPE_NATIVE_BUILD="{native_build()}"',
             f"-I{root / 'include'}", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda / 'include'}",
             str(NATIVE_SOURCES[0]), f"-L{root / 'lib'}", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
 
@@ -62,7 +80,7 @@ def native_command():
 def build(force: bool = False, verbose: bool = False) -> Path:
     if force or not _newer(LIB, SOURCES + HEADERS):
         _compile([nvcc_path(), *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), *map(str, SOURCES)], LIB)
-    if force or not _newer(NATIVE, NATIVE_SOURCES):
+    if force or not _native_current():
         _compile(native_command(), NATIVE)
     return LIB
 

@@ -16,6 +16,9 @@
 
 #include "../../include/slope.h"
 
+// The torch and Python this module was compiled against (build.native_build()); build.py and binding.py look for it in the file.
+extern "C" __attribute__((used)) const char slope_native_build[] = SLOPE_NATIVE_BUILD;
+
 namespace {
 
 #define SLOPE_CALLS(X)                                                                                                  \
@@ -97,7 +100,7 @@ int rows(const at::Tensor& t) { return static_cast<int>(t.size(0)); }
 int cols(const at::Tensor& t) { return static_cast<int>(t.size(1)); }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// Runs `body(args)` with Python's lock released around the C call inside it (see SLOPE_CALL).
+// Runs `body(args)`; C++ exceptions become Python ones.
 template <typename Body>
 PyObject* guarded(PyObject* const* args, Py_ssize_t n, Body body) {
     try {

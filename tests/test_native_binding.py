@@ -34,3 +34,14 @@ def test_statuses_of_the_library_become_errors(B):
     with pytest.raises(B.SlopeError) as e:                       # all pointers missing: refused by the argument checks
         B.slope_adapter_fwd_bwd(0, None, None, None, None, 1, 128, 128, 16)
     assert e.value.status == 1
+
+
+def test_a_module_built_against_another_torch_is_neither_kept_nor_loaded(B, monkeypatch):
+    from paper_2608_24070_b200 import build
+
+    assert build.up_to_date()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert not build.up_to_date()
+    monkeypatch.setattr(B, "_lib", None)
+    with pytest.raises(RuntimeError, match="another torch"):
+        B.lib()
