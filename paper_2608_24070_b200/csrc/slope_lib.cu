@@ -1097,12 +1097,12 @@ static bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes
     return b != nullptr && x < y + b_bytes && y < x + a_bytes;
 }
 
-// dR = T^T dY and dL = X^T dT in one launch, pdl_mode 2: behind the dT launch, which reads R.  CTAs store their shares of
-// the gradients while others still read, so gradients that overlap what is being read are formed in the workspace and
-// copied into place.
+// dR = T^T dY and dL = X^T dT: in one launch behind the dT launch, which reads R (`behind_dT`), or in two that are cut each by
+// itself.  CTAs store their shares of the gradients while others still read, so gradients that overlap what is being read
+// are formed in the workspace and copied into place.
 static slope_status_t launch_adapter_grads(const void* X, const void* dY, const void* R, const void* T, const void* dT, int b,
                                            int d_out, int d_in, int r, void* dL, void* dR, void* workspace,
-                                           cudaStream_t stream, const DeviceInfo& info, int pdl_mode) {
+                                           cudaStream_t stream, const DeviceInfo& info, bool behind_dT) {
     const size_t unit = sizeof(uint16_t), rows = b, l_bytes = unit * d_in * r, r_bytes = unit * d_out * r;
     const auto among_operands = [&](const void* g, size_t bytes) {
         return overlap(g, bytes, X, unit * rows * d_in) || overlap(g, bytes, dY, unit * rows * d_out) ||
@@ -1111,9 +1111,12 @@ static slope_status_t launch_adapter_grads(const void* X, const void* dY, const 
     const bool staged = among_operands(dL, l_bytes) || among_operands(dR, r_bytes);
     void* to_l = staged ? workspace : dL;
     void* to_r = staged ? static_cast<uint8_t*>(workspace) + adapter_partial_bytes(b, d_in, r) : dR;
-    if (slope_status_t st = launch_adapter<true, true>(adapter_dR(dY, T, d_out, to_r), adapter_dL(X, dT, d_in, to_l), r, b, stream,
-                                                       info, pdl_mode))
+    const AdapterOperands qr = adapter_dR(dY, T, d_out, to_r), ql = adapter_dL(X, dT, d_in, to_l);
+    if (slope_status_t st = behind_dT ? launch_adapter<true, true>(qr, ql, r, b, stream, info, 2)
+                                      : launch_adapter<true, true>(qr, AdapterOperands{}, r, b, stream, info))
         return st;
+    if (!behind_dT)
+        if (slope_status_t st = launch_adapter<true, true>(ql, AdapterOperands{}, r, b, stream, info)) return st;
     if (staged && (cudaMemcpyAsync(dL, to_l, l_bytes, cudaMemcpyDeviceToDevice, stream) != cudaSuccess ||
                    cudaMemcpyAsync(dR, to_r, r_bytes, cudaMemcpyDeviceToDevice, stream) != cudaSuccess))
         return SLOPE_ERR_CUDA;
@@ -1147,7 +1150,7 @@ slope_status_t slope_adapter_fwd_bwd(int phase, const void* X, const void* dY, c
     if (slope_status_t st = check_arch(info)) return st;
     // dR does not read dT: its CTAs run beside the dT launch, those of dL wait for it
     if (slope_status_t st = launch_adapter_dT(dY, R, b, d_out, r, dT, stream, info, 1)) return st;
-    return launch_adapter_grads(X, dY, R, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info, 2);
+    return launch_adapter_grads(X, dY, R, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info, true);
 }
 
 // ------------------------------------------------------------------ masked dW with dL, dR riding along
@@ -1213,9 +1216,9 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     if (slope_status_t st = check_arch(info)) return st;
     const DwAdapterPlan plan = dw_adapter_plan(b, d_out, d_in, r, info.sm_count);
     if (!plan.fused || info.sm_count != 148) {
-        // the separate launches: masked dW, then dR and dL
+        // the separate launches: masked dW, dR, dL
         if (slope_status_t st = slope_linear_bwd_dw_masked(dY, X, b, d_out, d_in, mask1_bits, dWc_vals, stream_)) return st;
-        return launch_adapter_grads(X, dY, nullptr, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info, 0);
+        return launch_adapter_grads(X, dY, nullptr, T, dT, b, d_out, d_in, r, dL, dR, workspace, stream, info, false);
     }
     using Cfg = DwAdapterCfg<6>;
     CUtensorMap tmA, tmB, tmT, tmDT;
