@@ -21,6 +21,11 @@
 
 namespace slope {
 
+// Rows of a K-contiguous operand's box: no more than the matrix has.  An SM takes about one 128-byte row of any box per two clocks,
+// inside the matrix or not; what the MMAs read behind the last row only reaches accumulator rows or columns that are
+// never stored.
+__host__ __device__ constexpr int adapter_box_rows(int rows, int tile) { return rows < tile ? rows : tile; }
+
 struct AdapterProblem {
     int M, N, K;
     uint16_t* out;                // bf16 [M x N], or [N x M] when `transposed`
@@ -139,14 +144,16 @@ adapter_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_const
     if (warp == 0) {
         if (elect_one()) {
             PipeState ps;
-            const int chunks = B_MN ? (cols + 63) / 64 : N_TILE / 64;        // chunks of 64 columns past N are not loaded
+            const int chunks = (cols + 63) / 64;                             // chunks of 64 columns past N are not loaded
+            const uint32_t stage_tx = 128 * ((A_MN ? kBlockM : adapter_box_rows(p.M, kBlockM)) +
+                                             (B_MN ? 64 * chunks : adapter_box_rows(p.N, N_TILE)));
             for (int i = 0; i < num_kb; ++i) {
                 if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) break;
                 uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
                 uint8_t* sB = sA + Cfg::kABytes;
                 uint64_t* bar = &full_bar[ps.stage];
                 const int k0 = (kb0 + i) * 64;
-                mbar_expect_tx(bar, Cfg::kABytes + chunks * 8192);
+                mbar_expect_tx(bar, stage_tx);
                 if (A_MN) {
                     tma_load_2d(sA, tmA, bar, m_blk * kBlockM, k0);
                     tma_load_2d(sA + 8192, tmA, bar, m_blk * kBlockM + 64, k0);

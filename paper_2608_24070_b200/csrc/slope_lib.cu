@@ -313,44 +313,81 @@ struct AdapterOperands {
 };
 
 // Column tile, reduction split (= cluster size) and ring depth of an adapter launch, by estimate.
-// Constants fitted to a sweep of tiles, splits and depths over 8 ... 16384 tokens, widths 768 ... 13824
-// and ranks 16 ... 256 (in most of them the choice is within 5 % of the best swept one):
-//   - a round trip through the ring takes 0.8 us, so a k-block costs at least that over its depth,
-//     and at least what the SM takes in (150 KB per us);
-//   - a CTA brings in 90 GB/s of the large operand, dozens of them less, all together 6 TB/s, and every
-//     further column tile costs 8 % of that (its second read comes from L2);
-//   - draining a tile costs 0.3 us per 64 columns, 1 us more and 1 us per 64 columns when it is split.
 struct AdapterPlan {
     int n_tile, splits;
     bool deep;                    // one CTA per SM with all of its shared memory; else two that share it
-    double us;                    // estimated time
+    double us;                    // estimated time, less the launch
 };
-static AdapterPlan adapter_candidate(int row_tiles, double a_bytes, int N, int K, int n_tile, int splits, int sm_count) {
-    const int num_kb = (K + 63) / 64, col_tiles = (N + n_tile - 1) / n_tile, ctas = row_tiles * col_tiles * splits;
+struct AdapterShape {
+    int row_tiles, box_rows;      // 128-row tiles of both problems; rows of the large operand's box
+    double a_bytes;               // of the large operands
+    int N, K;
+    bool b_mn;                    // the small operand is loaded in chunks of 64 columns, whatever N is
+};
+// How the CTAs of a launch come to lie on the machine.
+struct AdapterGrid {
+    int ctas, col_tiles, waves, rank_kb;   // rank_kb: k-blocks of a CTA
+    bool deep;
+    double stages, busy;                   // ring depth; share of the SMs that are at work at a time
+};
+static AdapterGrid adapter_grid(const AdapterShape& q, int n_tile, int splits, int sm_count) {
+    const int col_tiles = (q.N + n_tile - 1) / n_tile, ctas = q.row_tiles * col_tiles * splits;
     // clusters of 4 and 8 do not fill every SM (33 and 15 of them fit on 148 SMs)
     const int sms = splits == 8 ? sm_count * 120 / 148 : splits == 4 ? sm_count * 132 / 148 : sm_count;
     const bool deep = n_tile == 256 || ctas <= sms;
-    const int slots = (deep ? 1 : 2) * sms;
+    const int slots = (deep ? 1 : 2) * sms, waves = (ctas + slots - 1) / slots, num_kb = (q.K + 63) / 64;
     const double stages = n_tile == 64 ? (deep ? 9 : 4) : n_tile == 128 ? (deep ? 7 : 3) : 4;
-    const int waves = (ctas + slots - 1) / slots;
-    const double kb_us = std::max(0.8 / stages, (deep ? 1 : 2) * (16.0 + n_tile / 8.0) / 150.0);
-    const double hbm = std::min({6.0e6, 0.09e6 * ctas, 2.2e6 + 0.03e6 * ctas}) / (1.0 + 0.08 * (col_tiles - 1));
-    const double stream = std::max(waves * ((num_kb + splits - 1) / splits) * kb_us, a_bytes / hbm);
+    return AdapterGrid{ctas, col_tiles, waves, (num_kb + splits - 1) / splits, deep, stages,
+                       static_cast<double>(std::min(ctas, slots)) / sm_count};
+}
+// A launch that has the machine to itself.  Constants fitted to a sweep of tiles, splits and depths over 1 ... 16384 tokens,
+// widths 128 ... 13824 and ranks 16 ... 256 (the choice is on average 0.1 %, at most 12 % slower than the best swept one;
+// with a split's cost the same for any number of CTAs and boxes always full, dT of 6158 tokens and width 1408 took 7.8
+// instead of 6.4 us, of 5 tokens and width 896 4.0 instead of 3.5):
+//   - a round trip through the ring takes 1.2 us, a fifth more when all SMs are at it, so a k-block costs at
+//     least that over its depth, and at least the rows of its boxes at 1300 a us;
+//   - all CTAs together bring in 6.6 TB/s of the large operand, few of them less, and every further
+//     column tile costs half of that again;
+//   - draining 64 columns costs 0.75 us; when the tile is split 1.3 us more for the two barriers and, per 64
+//     columns, what the cluster has to sum: the share of 128 rows that is there and the share of SMs in it.
+static AdapterPlan adapter_candidate(const AdapterShape& q, int n_tile, int splits, int sm_count) {
+    const AdapterGrid g = adapter_grid(q, n_tile, splits, sm_count);
+    const int rows = q.box_rows + std::min(n_tile, q.b_mn ? (q.N + 63) / 64 * 64 : q.N);
+    const double kb_us = std::max(1.2 * (1.0 + 0.2 * g.busy) / g.stages, (g.deep ? 1 : 2) * rows / 1300.0);
+    const double hbm = std::min(6.6e6, 3.5e6 + 0.03e6 * g.ctas) / (1.0 + 0.5 * (g.col_tiles - 1));
+    const double cols = n_tile / 64.0, tail = splits > 1 ? 1.3 + (0.3 + q.box_rows / 128.0 + g.busy) * cols : 0.75 * cols;
+    return AdapterPlan{n_tile, splits, g.deep, std::max(g.waves * g.rank_kb * kb_us, q.a_bytes / hbm) + g.waves * tail};
+}
+// A T launch beside the tile kernel that consumes it.  Its constants go with those of plan_fwd_adapter, which weighs the
+// two against each other; with the ones above, which know T alone, forwards of few rows got the wrong share of the
+// machine (3057 tokens 9856 -> 384, r = 64: 32.3 instead of 26.4 us):
+//   - a k-block costs 0.8 us over the ring's depth, and at least what the SM takes in (150 KB per us);
+//   - a CTA brings in 90 GB/s of the large operand, dozens of them less, all together 6 TB/s, and every
+//     further column tile costs 8 % of that (its second read comes from L2);
+//   - draining a tile costs 0.3 us per 64 columns, 1 us more and 1 us per 64 columns when it is split.
+static AdapterPlan adapter_beside_forward(const AdapterShape& q, int n_tile, int splits, int sm_count) {
+    const AdapterGrid g = adapter_grid(q, n_tile, splits, sm_count);
+    const double kb_us = std::max(0.8 / g.stages, (g.deep ? 1 : 2) * (16.0 + n_tile / 8.0) / 150.0);
+    const double hbm = std::min({6.0e6, 0.09e6 * g.ctas, 2.2e6 + 0.03e6 * g.ctas}) / (1.0 + 0.08 * (g.col_tiles - 1));
     const double tail = (splits > 1 ? 1.0 : 0.3) * n_tile / 64.0 + (splits > 1 ? 1.0 : 0.0);
-    return AdapterPlan{n_tile, splits, deep, stream + waves * tail};
+    return AdapterPlan{n_tile, splits, g.deep, std::max(g.waves * g.rank_kb * kb_us, q.a_bytes / hbm) + g.waves * tail};
 }
 template <typename Visit>
-static void adapter_candidates(int row_tiles, double a_bytes, int N, int K, int sm_count, Visit visit) {
-    for (int n_tile = 64; n_tile <= 256 && (n_tile == 64 || n_tile < 2 * N); n_tile *= 2)
-        for (int s = 1; s <= 8 && (s == 1 || 2 * s <= (K + 63) / 64); s *= 2)
-            visit(adapter_candidate(row_tiles, a_bytes, N, K, n_tile, s, sm_count));
+static void adapter_cuts(const AdapterShape& q, Visit visit) {
+    for (int n_tile = 64; n_tile <= 256 && (n_tile == 64 || n_tile < 2 * q.N); n_tile *= 2)
+        for (int s = 1; s <= 8 && (s == 1 || 2 * s <= (q.K + 63) / 64); s *= 2) visit(n_tile, s);
 }
-static AdapterPlan adapter_plan(int row_tiles, double a_bytes, int N, int K, int sm_count) {
+static AdapterPlan adapter_plan(const AdapterShape& q, int sm_count) {
     AdapterPlan best{64, 1, true, 1e30};
-    adapter_candidates(row_tiles, a_bytes, N, K, sm_count, [&](const AdapterPlan& c) {
+    adapter_cuts(q, [&](int n_tile, int splits) {
+        const AdapterPlan c = adapter_candidate(q, n_tile, splits, sm_count);
         if (c.us < best.us - 1e-9) best = c;
     });
     return best;
+}
+// T = X L: `b` tokens of width `d_in`.
+static AdapterShape adapter_T_shape(int b, int d_in, int r) {
+    return AdapterShape{(b + kBlockM - 1) / kBlockM, adapter_box_rows(b, kBlockM), 2.0 * b * d_in, r, d_in, true};
 }
 
 // SMs that the CTAs of a launch over `rows` rows occupy.
@@ -369,8 +406,10 @@ static slope_status_t launch_adapter_tile(const AdapterOperands& q0, const Adapt
     for (int i = 0; i < 2; ++i) {
         const bool live = i == 0 || q1.M > 0;
         const AdapterOperands& q = i == 0 ? q0 : (live ? q1 : q0);           // unused slot mirrors problem 0
-        const bool okA = A_MN ? make_tmap(&tm[2 * i], q.A, K, q.M, 64, 64) : make_tmap(&tm[2 * i], q.A, q.M, K, kBlockM, 64);
-        const bool okB = B_MN ? make_tmap(&tm[2 * i + 1], q.B, K, N, 64, 64) : make_tmap(&tm[2 * i + 1], q.B, N, K, N_TILE, 64);
+        const bool okA = A_MN ? make_tmap(&tm[2 * i], q.A, K, q.M, 64, 64)
+                              : make_tmap(&tm[2 * i], q.A, q.M, K, adapter_box_rows(q.M, kBlockM), 64);
+        const bool okB = B_MN ? make_tmap(&tm[2 * i + 1], q.B, K, N, 64, 64)
+                              : make_tmap(&tm[2 * i + 1], q.B, N, K, adapter_box_rows(N, N_TILE), 64);
         if (!okA || !okB) return SLOPE_ERR_CUDA;
         p[i] = AdapterProblem{live ? q.M : 0, N, K, static_cast<uint16_t*>(q.out), q.transposed};
         if (live) tiles += (q.M + kBlockM - 1) / kBlockM;
@@ -396,11 +435,13 @@ static slope_status_t launch_adapter_planned(const AdapterPlan& plan, const Adap
 template <bool A_MN, bool B_MN>
 static slope_status_t launch_adapter(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K,
                                      cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
-    const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
-    const double a_bytes = 2.0 * K * (static_cast<double>(q0.M) + q1.M);
     thread_local SizeMemo<AdapterPlan> memo;
-    const AdapterPlan& plan = memo.get({q0.M, q1.M, N, K, info.sm_count, 0},
-                                       [&] { return adapter_plan(row_tiles, a_bytes, N, K, info.sm_count); });
+    const AdapterPlan& plan = memo.get({q0.M, q1.M, N, K, info.sm_count, 0}, [&] {
+        const int row_tiles = (q0.M + kBlockM - 1) / kBlockM + (q1.M + kBlockM - 1) / kBlockM;
+        const int box_rows = A_MN ? kBlockM : adapter_box_rows(std::max(q0.M, q1.M), kBlockM);
+        return adapter_plan(AdapterShape{row_tiles, box_rows, 2.0 * K * (static_cast<double>(q0.M) + q1.M), N, K, B_MN},
+                            info.sm_count);
+    });
     return launch_adapter_planned<A_MN, B_MN>(plan, q0, q1, N, K, stream, pdl_mode);
 }
 
@@ -611,7 +652,7 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
             // The consumer of a fused pair has to be resident next to its producer, or its last clusters
             // would wait for the producer to finish and the overlap would be lost: count only the
             // clusters that fit beside it.
-            const AdapterPlan producer = adapter_plan((ntok + kBlockM - 1) / kBlockM, 2.0 * ntok * K, r, K, info.sm_count);
+            const AdapterPlan producer = adapter_plan(adapter_T_shape(ntok, K, r), info.sm_count);
             const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
             for (int sz = 1; sz <= 8; ++sz) {
                 cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
@@ -735,19 +776,20 @@ struct FwdAdapterPlan {
     int pairs;                    // CTA pairs of the forward
 };
 static FwdAdapterPlan plan_fwd_adapter(int b, int d_out, int d_in, int r, const DeviceInfo& info) {
-    const int row_tiles = (b + kBlockM - 1) / kBlockM;
+    const AdapterShape shape = adapter_T_shape(b, d_in, r);
     constexpr double kClkPerUs = 1850.0;
     FwdAdapterPlan best{};                                  // (no tile rows: the few-token kernel)
     best.pairs = info.sm_count / 2;
     double best_us = 1e300, cost = 0.0;
     if (use_few_token_kernel(d_out, d_in, b)) {                // its K-split is chosen around the producer
-        best.T = adapter_plan(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count);
+        best.T = adapter_plan(shape, info.sm_count);
     } else {
         const int pairs = info.sm_count / 2;
         const SparseTile full = choose_sparse_tile(d_out, d_in, b, r, pairs, &cost);
         const double full_us = cost / kClkPerUs;
         const int last_wave = ((d_out + full.rows - 1) / full.rows) * ((b + full.width - 1) / full.width) % pairs;
-        adapter_candidates(row_tiles, 2.0 * b * d_in, r, d_in, info.sm_count, [&](const AdapterPlan& c) {
+        adapter_cuts(shape, [&](int n_tile, int splits) {
+            const AdapterPlan c = adapter_beside_forward(shape, n_tile, splits, info.sm_count);
             const int sms = adapter_sms(c, b, r, info.sm_count), beside = (info.sm_count - sms) / 2;
             const double share = static_cast<double>(sms) / info.sm_count;
             const bool blocked = last_wave == 0 || last_wave > beside;

@@ -49,6 +49,33 @@ def test_adapter_products_match_fp64(b, d_in, d_out, r):
     assert all(v <= REL_TOL for v in errs.values()), errs
 
 
+@pytest.mark.parametrize("b,d_in,d_out,r", [(1, 1024, 896, 16), (5, 640, 1152, 48), (17, 4096, 640, 80), (127, 768, 2304, 256)])
+def test_rows_that_are_not_loaded_are_not_seen(b, d_in, d_out, r):
+    """Boxes hold as many rows of the tokens and of R as there are; the MMAs also read the rows behind them."""
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(36)
+    new = lambda *shape: torch.randn(shape, generator=gen, dtype=torch.bfloat16, device="cuda")
+    full = lambda v, *shape: torch.full(shape, v, dtype=torch.bfloat16, device="cuda")
+    X, dY, L, R, wide = new(b, d_in), new(b, d_out), new(d_in, r), new(r, d_out), 256
+    out = []
+    for fill in (0.0, float("nan")):
+        for _ in range(3):                                       # on every SM
+            B.slope_adapter_fwd_bwd(0, full(fill, 20000, d_in), None, full(fill, d_in, wide), None, 20000, d_out, d_in, wide,
+                                    T=full(0, 20000, wide))
+            B.slope_adapter_fwd_bwd(2, None, full(fill, 20000, d_out), None, full(fill, wide, d_out), 20000, d_out, d_in, wide,
+                                    dT=full(0, 20000, wide))
+        T, dT = full(float("nan"), b, r), full(float("nan"), b, r)
+        B.slope_adapter_fwd_bwd(0, X, None, L, None, b, d_out, d_in, r, T=T)
+        B.slope_adapter_fwd_bwd(2, None, dY, None, R, b, d_out, d_in, r, dT=dT)
+        out.append((T, dT))
+    for x, y in zip(*out):
+        assert torch.isfinite(x).all() and torch.equal(x.view(torch.int16), y.view(torch.int16))
+    assert B.slope_poll_status() == 0
+
+
 def _gradient_operands(b, d_in, d_out, r):
     import torch
     from paper_2608_24070_b200 import binding as B, build
