@@ -741,15 +741,19 @@ static SparseTile choose_sparse_tile(int M, int K, int ntok, int r, int num_pair
 }
 
 // Few-token kernel or tile kernel?  Decode sizes (<= 16 tokens) stream the weights through the few-token kernel.  From 17 to
-// 128 tokens it is the better one only for a long reduction on few rows, where its K-split fills the machine and a
-// tile kernel has a handful of tiles that each walk the whole reduction; a tall weight has tiles enough, narrow ones
-// for few tokens.  us, few-token / tile kernel: 32 tokens 4096 -> 4096 7.7 / 8.6, 1024 -> 1024 4.1 / 3.8, 3072 -> 768 4.4 / 6.2,
-// 4096 -> 12288 14.3 / 12.2; 64 tokens 2048 -> 2048 5.6 / 5.4, 4096 -> 4096 8.3 / 8.6, 4096 -> 22016 33 / 23; 80 tokens 4096 -> 4096
-// 9.3 / 8.9, 8192 -> 2560 10.2 / 13.4; 128 tokens 11008 -> 4096 15.8 / 17.9, 2048 -> 6144 10.2 / 7.1.
+// 128 tokens its K-split has to make up for boxes of every token in every CTA and for a drain that grows with the tokens,
+// which takes a reduction that is the longer the more tokens and the more rows there are; a short one, or a tall weight, has
+// the tile kernels' narrow tiles.  Up to 44 row slabs, which run in three slices side by side, the line is a fit to 760
+// sizes on both kernels (0.2 % slower on average than the better one of the two; by the rule below, which compared the
+// two extents only, 5 %); beyond them waves of slabs decide, and no simple line does.  us, few-token / tile kernel: 32 tokens 4096 -> 4096
+// 7.8 / 9.2, 1024 -> 1024 4.4 / 4.1, 3072 -> 768 4.7 / 6.4; 64 tokens 512 -> 256 5.0 / 3.4, 2048 -> 1024 5.3 / 5.4, 2048 -> 2048
+// 5.8 / 5.4, 4096 -> 4096 8.6 / 9.3; 128 tokens 256 -> 128 7.3 / 3.1, 3072 -> 768 7.0 / 6.5, 4096 -> 512 7.3 / 7.6, 8192 -> 4096
+// 14.2 / 15.1; beyond: 17 tokens 4096 -> 11264 16.8 / 11.2, 64 tokens 8192 -> 6656 15.9 / 16.8, 7808 -> 10752 24.7 / 16.5.
 static bool use_few_token_kernel(int M, int K, int ntok) {
     if (ntok <= 16) return true;
     if (ntok > 128) return false;
-    return K >= 2 * M || (ntok <= 64 && K >= M && K >= 2048);
+    if (M <= 44 * kBlockM) return K >= (850.0 + 4.0 * ntok + 0.11 * ntok * ntok) * (1.0 + M / 4000.0);
+    return K >= 2 * M || (ntok <= 64 && K >= M);
 }
 
 static slope_status_t launch_sparse_tile(const SparseTile& t, const void* act, int ntok, const void* vals, const void* meta,

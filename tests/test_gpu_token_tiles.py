@@ -69,11 +69,20 @@ def test_token_tiles_match_fp64(b, d_in, d_out, r):
 @pytest.mark.parametrize("b,before", [(1, 16), (7, 16), (13, 16), (17, 64), (63, 64), (65, 128), (127, 128)])
 def test_few_tokens_do_not_see_what_an_earlier_launch_left_in_shared_memory(b, before):
     """Activation tiles are loaded for as many tokens as there are; the MMAs also read the rows behind them."""
+    _leftovers_are_not_seen(b, before, 2048)
+
+
+@pytest.mark.parametrize("b,before", [(33, 64), (66, 128), (127, 128)])
+def test_few_tokens_on_long_reductions_do_not_see_them_either(b, before):
+    _leftovers_are_not_seen(b, before, 6144)                     # (127 tokens take the few-token kernel on long reductions only)
+
+
+def _leftovers_are_not_seen(b, before, d_in):
     import torch
     from paper_2608_24070_b200 import binding as B, build
 
     build.build()
-    d_in, d_out, r = 2048, 1024, 32
+    d_out, r = 1024, 32
     layer = GpuLayer(si.gaussian_bf16((d_out, d_in), 0.02, 56), fused_setup=True)
     L, R = (B.bf16_from_bits(si.gaussian_bf16(s, 0.1, 57)) for s in ((d_in, r), (r, d_out)))
     X = B.bf16_from_bits(si.gaussian_bf16((b, d_in), 1.0, 58))
@@ -89,3 +98,13 @@ def test_few_tokens_do_not_see_what_an_earlier_launch_left_in_shared_memory(b, b
     assert torch.isfinite(Y).all() and torch.equal(Y.view(torch.int16), Y1.view(torch.int16))
     assert torch.equal(T.view(torch.int16), T1.view(torch.int16))
     assert B.slope_poll_status() == 0
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [
+    (17, 1152, 256, 0), (17, 896, 256, 16),          # either side of the few-token kernel's line, 17 tokens
+    (64, 2304, 1280, 64), (65, 1792, 1280, 0),       # its 64- and 128-token tiles
+    (128, 4096, 512, 256), (127, 3456, 640, 0),
+    (40, 7808, 5632, 0), (40, 5888, 5760, 32),       # 44 row slabs and 45
+])
+def test_few_token_kernel_on_either_side_of_its_line(b, d_in, d_out, r):
+    test_token_tiles_match_fp64(b, d_in, d_out, r)
