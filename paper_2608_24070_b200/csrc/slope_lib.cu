@@ -881,7 +881,7 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
         return choose_dense_width(M, N, K, B_MN, EPI == kEpiMasked, max_pairs);
     });
     CUtensorMap tmA, tmB;
-    const bool okA = A_MN ? make_tmap(&tmA, A, K, M, 64, 64) : make_tmap(&tmA, A, M, K, kBlockM, 64);
+    const bool okA = A_MN ? make_tmap(&tmA, A, K, M, 64, 64) : make_tmap(&tmA, A, M, K, dense_a_box(M), 64);
     const bool okB = B_MN ? make_tmap(&tmB, B, K, N, 64, 64) : make_tmap(&tmB, B, N, K, small ? 128 : width / 2, 64);
     if (!okA || !okB) return SLOPE_ERR_CUDA;
     if (small) {

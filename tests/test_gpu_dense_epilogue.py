@@ -60,3 +60,29 @@ def test_dense_layer(b, d_in, d_out):
     g = lambda t: to_f64(B.bits_from_bf16(t))
     for got, ref in ((Y[:b], fX @ fW.T), (dX[:b], fdY @ fW), (dW, fdY.T @ fX)):
         assert parity_error(g(got), ref) <= REL_TOL
+
+
+@pytest.mark.parametrize("b,d_in,d_out", [(1, 640, 8320), (9, 8320, 640),     # one-CTA tiles in the forward / the input gradient
+                                          (2, 2304, 640), (127, 1024, 3840)])
+def test_few_tokens_do_not_see_what_an_earlier_launch_left_in_shared_memory(b, d_in, d_out):
+    """Boxes hold as many token rows as there are; the MMAs also read the rows behind them."""
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(44)
+    new = lambda *shape: torch.randn(shape, generator=gen, dtype=torch.bfloat16, device="cuda")
+    X, dY, W = new(b, d_in), new(b, d_out), new(d_out, d_in)
+    out = []
+    for fill in (0.0, float("nan")):
+        for tokens in (128, 4000):                               # both kernels, on every SM
+            noise = lambda n: torch.full((tokens, n), fill, dtype=torch.bfloat16, device="cuda")
+            B.slope_dense_linear_fwd(noise(d_in), W, noise(d_out))
+            B.slope_dense_linear_bwd_dx(noise(d_out), W, noise(d_in))
+        Y, dX = (torch.full((b, n), float("nan"), dtype=torch.bfloat16, device="cuda") for n in (d_out, d_in))
+        B.slope_dense_linear_fwd(X, W, Y)
+        B.slope_dense_linear_bwd_dx(dY, W, dX)
+        out.append((Y, dX))
+    for x, y in zip(*out):
+        assert torch.isfinite(x).all() and torch.equal(x.view(torch.int16), y.view(torch.int16))
+    assert B.slope_poll_status() == 0
