@@ -1,5 +1,6 @@
-"""The adapter's low-rank products at the edges of their kernel: every column tile (64, 128, 256), every
-reduction split (1, 2, 4, 8), one and two CTAs per SM, ragged last tiles and k-blocks.
+"""The adapter's low-rank products at the edges of their kernel: every column tile (64, 128, 256) and every
+reduction split (1, 2, 4, 8) that the estimate gives them, one and two CTAs per SM, ragged last tiles and k-blocks;
+operands whose boxes are not full; gradients that take the place of operands.
 
 The reference is the fp64 product of the same bf16 operands (dL is checked from the dT the call wrote), so
 an output is rounded once: 2^-9 / sqrt(3) ~ 1.7e-3 relative on Gaussian data, 5e-3 allowed, and
@@ -14,15 +15,15 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("b,d_in,d_out,r", [
     (1, 128, 128, 16),           # one token, two k-blocks of T, one of dL: no split
-    (63, 256, 384, 16),          # four k-blocks: a split of two
-    (130, 4096, 1152, 64),       # ragged second row tile, split of eight
-    (257, 128, 2176, 48),        # ragged k-block in dL / dR, columns past r in the 64-wide tile
-    (1000, 768, 2304, 256),      # widest rank on few tiles: four column tiles
+    (63, 256, 384, 16),          # boxes of 63 and of 16 rows, no split
+    (130, 4096, 1152, 64),       # ragged second row tile, T and dT split in eight
+    (257, 128, 2176, 48),        # dT split in eight; ragged k-block in dL / dR, columns past r in the 64-wide tile
+    (1000, 768, 2304, 256),      # widest rank on few tiles: four column tiles; dT split in four
     (1100, 640, 256, 176),       # rank between the column tiles
-    (4096, 1024, 512, 128),      # 128-wide tiles
-    (9500, 512, 640, 256),       # 75 row tiles: 256-wide tiles
-    (19100, 128, 256, 80),       # more row tiles than SMs: two CTAs per SM
-    (40000, 128, 128, 16),       # several waves; 625 k-blocks for one row tile of dL
+    (4096, 1024, 512, 128),      # dL / dR split in four
+    (9500, 512, 640, 256),       # 75 row tiles: 256-wide tiles; dL / dR on 128-wide ones, split in four
+    (19100, 128, 256, 80),       # more row tiles than SMs: two CTAs per SM on 128-wide tiles
+    (40000, 128, 128, 16),       # several waves; 625 k-blocks for two row tiles, split in eight
 ])
 def test_adapter_products_match_fp64(b, d_in, d_out, r):
     import torch
@@ -47,6 +48,35 @@ def test_adapter_products_match_fp64(b, d_in, d_out, r):
     errs = {"T": parity_error(g(T[:b]), f["X"] @ f["L"]), "dT": parity_error(g(dT), f["dY"] @ f["R"].T),
             "dL": parity_error(g(dL), f["X"].T @ g(dT)), "dR": parity_error(g(dR), g(T[:b]).T @ f["dY"])}
     assert all(v <= REL_TOL for v in errs.values()), errs
+
+
+@pytest.mark.parametrize("b,d_in,d_out,r", [
+    # T: column tile / split, in two CTAs per SM where it says shared
+    (1090, 1536, 128, 256),      # 64 / 2
+    (9558, 1664, 128, 16),       # 64 / 2 shared
+    (2974, 1536, 128, 80),       # 64 / 4 shared
+    (1531, 1024, 128, 80),       # 64 / 8 shared
+    (2102, 3584, 128, 256),      # 128 / 2
+    (1067, 2816, 128, 208),      # 128 / 4
+    (150, 4992, 128, 240),       # 128 / 8
+    (2032, 2560, 128, 112),      # 128 / 8 shared
+    (2785, 5376, 384, 256),      # 256 / 2
+    (1328, 5888, 128, 240),      # 256 / 4
+    # dT
+    (1047, 128, 2176, 240),      # 64 / 2
+    (2197, 128, 7168, 48),       # 64 / 8 shared
+    (2387, 128, 5504, 208),      # 128 / 2
+    (1055, 128, 4864, 208),      # 128 / 4
+    # dL and dR
+    (1989, 1024, 128, 208),      # 64 / 2
+    (260, 4864, 128, 256),       # 128 / 1
+    (6391, 128, 2176, 240),      # 128 / 2
+    (8983, 256, 256, 224),       # 128 / 8
+    (13715, 1664, 512, 208),     # 256 / 4
+    (28495, 384, 768, 208),      # 256 / 8
+])
+def test_tiles_and_splits(b, d_in, d_out, r):
+    test_adapter_products_match_fp64(b, d_in, d_out, r)
 
 
 @pytest.mark.parametrize("b,d_in,d_out,r", [(1, 1024, 896, 16), (5, 640, 1152, 48), (17, 4096, 640, 80), (127, 768, 2304, 256)])

@@ -1,5 +1,6 @@
-"""Weight-gradient and dense GEMM epilogues at the edges of their tiles: every tile width (64, 128, 192, 256), halved
-items of the last wave, last tiles that are partly empty in either dimension, few tokens (one k-block, a ragged one).
+"""Weight-gradient and dense GEMM epilogues at the edges of their tiles: the one-CTA kernel and every width of the CTA-pair
+kernel (64, 128, 192, 256), halved items of the last wave, last tiles that are partly empty in either dimension, few tokens
+(one k-block, a ragged one).
 
 The reference is the fp64 product of the same bf16 operands; outputs are rounded once (2^-9 / sqrt(3) ~ 1.7e-3
 relative on Gaussian data, 5e-3 allowed, and parity_error's bound per element)."""
@@ -21,12 +22,16 @@ def _operands(b, d_in, d_out):
 
 
 @pytest.mark.parametrize("b,d_in,d_out", [
-    (1, 128, 128),               # 64 wide, half empty, one token
-    (65, 384, 640),              # 64 wide, a k-block and one token
-    (200, 1152, 1920),           # 128 wide, last row tile half empty
-    (70, 2176, 2432),
+    (1, 128, 128),               # one-CTA kernel, one tile, one token
+    (65, 384, 640),              # one-CTA kernel, a k-block and one token
+    (200, 1152, 1920),           # one-CTA kernel, 135 tiles
+    (70, 2176, 2432),            # 128 wide, last row tile half empty
     (200, 3200, 2688),           # 256 wide, half empty in both dimensions
     (90, 4096, 4096),            # 256 tiles: the last wave's are halved
+    (2049, 128, 128),            # 64 wide, row tile half empty, 33 k-blocks, the last with one token
+    (2111, 512, 512),            # 64 wide
+    (2100, 384, 384),            # 64 wide, last row tile half empty
+    (2200, 1152, 1920),          # 128 wide, last row tile half empty
 ])
 def test_masked_weight_gradient(b, d_in, d_out):
     import numpy as np
@@ -45,7 +50,9 @@ def test_masked_weight_gradient(b, d_in, d_out):
 
 @pytest.mark.parametrize("b,d_in,d_out", [(1, 128, 128), (130, 256, 384), (300, 1152, 640), (513, 384, 2176),
                                         (700, 2048, 4224), (600, 3200, 2688),
-                                        (3000, 256, 4992)])
+                                        (3000, 256, 4992),
+                                        (1000, 1024, 1024),      # one-CTA kernel in all three, last row tile partly empty
+                                        (777, 1024, 1280)])      # and beside a 128-wide input gradient
 def test_dense_layer(b, d_in, d_out):
     import torch
 

@@ -1,6 +1,6 @@
-"""Sparse forward and input gradient: the few-token kernel where it does not split, every token-tile width of the tile kernels (32 ... 224 in steps of 32, both
-row counts), ragged last tiles and row tiles that are half empty, with and without adapters; the fused
-forward against the separate calls.
+"""Sparse forward and input gradient: the few-token kernel where it does not split and on either side of its line, the 256-row
+tiles at every width (32 ... 224 in steps of 32) and the 512-row tiles at the widths that are chosen for them (96 ... 224), ragged last
+tiles and row tiles that are half empty, with and without adapters; the fused forward against the separate calls.
 
 The reference is the fp64 product of the bf16 operands the kernels read (T as written), so outputs are rounded
 once: 1.7e-3 relative on Gaussian data, 5e-3 allowed, and parity_error's bound per element."""
@@ -17,19 +17,25 @@ pytestmark = pytest.mark.gpu
     (1, 128, 384, 0),            # few-token kernel without a split: one k-block, one token
     (5, 128, 256, 16),
     (16, 256, 19200, 0),         # more slabs than SMs
-    (17, 128, 640, 64),
-    (128, 256, 512, 32),
-    (129, 256, 384, 0),          # narrowest tiles, last row tile half empty
-    (161, 1024, 256, 16),
-    (250, 640, 1920, 0),
-    (353, 512, 4096, 48),
-    (449, 768, 2304, 0),
-    (500, 4096, 1152, 64),
-    (673, 384, 2176, 256),
-    (1000, 768, 2304, 16),
-    (1345, 1152, 640, 0),
-    (2048, 1024, 4096, 32),
-    (5000, 2048, 1408, 0),       # several waves, 512-row tiles the other way round
+    # tile rows x width of the forward / the input gradient
+    (17, 128, 640, 64),          # 256x32 / 256x32
+    (128, 256, 512, 32),         # 256x32 / 256x32
+    (129, 256, 384, 0),          # 256x32 / 256x32, last row tile half empty
+    (161, 1024, 256, 16),        # 256x32 / 256x64
+    (250, 640, 1920, 0),         # 256x64 / 256x32
+    (353, 512, 4096, 48),        # 256x128 / 256x32
+    (449, 768, 2304, 0),         # 256x96 / 256x32
+    (500, 4096, 1152, 64),       # 256x64 / 256x128
+    (673, 384, 2176, 256),       # 256x128 / 256x32
+    (1000, 768, 2304, 16),       # 256x128 / 256x64
+    (1345, 1152, 640, 0),        # 256x96 / 256x128
+    (2048, 1024, 4096, 32),      # 256x160 / 256x128
+    (5000, 2048, 1408, 0),       # 512x224, several waves / 256x192
+    (1782, 128, 896, 32),        # 256x224 / 256x64
+    (458, 1152, 6400, 48),       # 512x96 / 256x64
+    (496, 1152, 6528, 0),        # 512x128 / 256x64
+    (1826, 1024, 2560, 16),      # 512x160 / 256x128
+    (3974, 1024, 1408, 0),       # 512x192 / 256x224
     (15257, 512, 3968, 0),       # 31 row blocks: in the last 512-row tile one CTA has rows for one sub-tile only
 ])
 def test_token_tiles_match_fp64(b, d_in, d_out, r):
