@@ -70,7 +70,6 @@ struct SparseGemmParams {
     int stages;                   // tile kernels: pipeline stages that fit at that width
     int group_m;                  // 512-row-tile kernel: row tiles per raster group (0: all in one group)
     int pdl_mode;                 // 2: consumer of a fused pair of launches (see the few-token kernel)
-    const uint8_t* meta;          // metadata blocks of A
     uint16_t* out;                // [Ntok x M]
 };
 
@@ -132,7 +131,7 @@ __device__ __forceinline__ void load_mask_bits(const uint8_t* row, int cols, uin
     }
 }
 
-// Drains `cols` accumulator columns of this thread's row, up to 64 at a time, so that the tensor-memory loads share one
+// Drains `cols` (32, 64 or 128) accumulator columns of this thread's row, up to 64 at a time, so that the tensor-memory loads share one
 // wait.  With few tokens the drain, not the main loop, paces the kernel (double-buffered accumulators): four
 // warps that took 16 columns at a time, a mask load and a wait each, needed ~9 us for a 256 x 256 tile; as
 // it is, 4096 x 4096 with 300 tokens went from 43 to 13 us, 8320 -> 6400 with 740 from 141 to 58, 512 x 512
@@ -150,7 +149,6 @@ template <typename Store>
 __device__ __forceinline__ void drain_columns(uint32_t t_row, int cols, Store store) {
     if (cols >= 64) drain_block<64>(t_row, 0, store);
     if (cols == 128) drain_block<64>(t_row, 4, store);
-    else if (cols == 96) drain_block<32>(t_row, 4, store);
     else if (cols == 32) drain_block<32>(t_row, 0, store);
 }
 
@@ -888,7 +886,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 // or the tensor pipe, is what bounds these GEMMs).  Tensor memory then holds one accumulator
 // per sub-tile (2 x 224 columns) plus the metadata columns, so accumulators are single
 // buffered; the epilogue is made short instead: accumulator rows are transposed through
-// shared memory and leave as TMA stores of 32 tokens x 128 features.
+// shared memory and leave as TMA stores of 32 tokens x 32 features.
 //   128-row block of A handled by CTA c for sub-tile s of tile mt:  4*mt + 2*s + c.
 // =====================================================================================
 constexpr int kPrefetchAhead = 8;          // k-blocks of L2 prefetch distance for activation boxes
@@ -1221,8 +1219,8 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 break;
             }
             uint32_t pk[2][kMyBlocks][16];
-            // ---- first accumulator (its drain is what the next tile's first MMA waits for).  Two loads in flight per
-            //      wait: the warps of a 320-thread CTA are allocated registers as twelve, which caps a thread at 168, and
+            // ---- first accumulator (its drain is what the next tile's first MMA waits for).  One load of 16 registers at a
+            //      time: the warps of a 320-thread CTA are allocated registers as twelve, which caps a thread at 168, and
             //      128 of them hold the two packed accumulators.
             if (!mbar_wait(&tfull_bar[0], static_cast<uint32_t>(it) & 1u, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();

@@ -121,7 +121,7 @@ template <int M>
 __global__ void __launch_bounds__(256, M == 16 ? 2 : M == 8 ? 3 : 4)
 double_prune_nm_kernel(const uint4* W, const uint8_t* mask1, int d_out, int d_in, int n, uint4* out, uint8_t* mask2) {
     constexpr int kWords = M == 16 ? 2 : 4;
-    const int per_row = d_in / (2 * kWords);                   // threads per row: a multiple of 32
+    const int per_row = d_in / (2 * kWords);                   // threads per row: a multiple of 16, of 32 for M = 16
     const size_t total = static_cast<size_t>(d_out / M) * per_row;
     griddep_stream(M == 16 ? 2 : M == 8 ? 3 : 4);
     const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;

@@ -70,9 +70,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 // One try: the hardware may park the thread for up to kSuspendHintNs while the phase is
 // pending (it wakes as soon as the phase completes), so a waiting role costs no issue slots.
 constexpr uint32_t kSuspendHintNs = 20000;

@@ -199,12 +199,6 @@ static slope_status_t launch_cluster_ex(void (*kern)(KArgs...), int grid, int cl
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? SLOPE_OK : SLOPE_ERR_CUDA;
 }
 
-template <typename... KArgs, typename... Args>
-static slope_status_t launch_cluster(void (*kern)(KArgs...), int grid, int cluster, int threads, int smem_bytes,
-                                     cudaStream_t stream, Args&&... args) {
-    return launch_cluster_ex(kern, grid, cluster, threads, smem_bytes, false, stream, std::forward<Args>(args)...);
-}
-
 // How many clusters of `cluster` CTAs of this kernel the device holds at once (0: query failed).
 template <typename Kernel>
 static int max_active_clusters(Kernel kern, int cluster, int threads, int smem_bytes, int sm_count) {
@@ -483,7 +477,6 @@ static bool sparse_tile_args(SparseTileArgs& a, const void* act, int ntok, const
     a.p = SparseGemmParams{};
     a.p.M = M; a.p.K = K; a.p.Ntok = ntok; a.p.r = r; a.p.a2_mn_major = a2_mn ? 1 : 0;
     a.p.width = width; a.p.num_n = (ntok + width - 1) / width; a.p.stages = stages; a.p.pdl_mode = pdl_mode;
-    a.p.meta = static_cast<const uint8_t*>(meta);
     a.p.out = static_cast<uint16_t*>(out);
     return true;
 }
@@ -563,7 +556,7 @@ constexpr double kSkinnySmUs = 0.23, kSkinnyHbmUs = 0.0028, kSkinnyWaveUs = 4.0,
                  kSkinnyReducePerRankUs = 0.07;
 
 // A k-block costs an SM its weight tile (kSkinnySmUs) plus the activation tile's TMA row
-// requests (2 per token, ~2 ns each, counted here for a full tile).
+// requests (2 per token, ~2 ns each; charged for a full tile, as the constants were fitted, although a box has a row per token).
 constexpr double kSkinnyTokenUs = 0.004;
 
 static int skinny_splits(int slabs, int num_kb, int block_n, const int (&cap)[9], double* est_us = nullptr) {
@@ -638,7 +631,6 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
     SparseGemmParams p = {};
     p.M = M; p.K = K; p.Ntok = ntok; p.r = r; p.a2_mn_major = a2_mn ? 1 : 0;
     p.pdl_mode = pdl_mode; p.width = rows;
-    p.meta = static_cast<const uint8_t*>(meta);
     p.out = static_cast<uint16_t*>(out);
     auto kern = sparse_gemm_skinny_kernel<BLOCK_N, A_STAGES, B_STAGES>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
@@ -848,9 +840,10 @@ static int dense_stages(bool b_mn, int epi, int width) {
 // MMAs (2.36 per column, no fewer than 80 columns' worth), a tile no less than its drain, a launch one more drain
 // and 47 per pair.  (192 columns of a [K x N] operand cost the bytes of 256 and are not taken.)  Fitted to a sweep over
 // 12 layer shapes (512 ... 9728) and 64 ... 8192 tokens: 0.2 % slower on average than the best width, where 256 x 256
-// throughout is 24 % (the plain store's drain was 24 per column then; halved since, which moves weight gradients of 256 tokens
-// 4096 x 4096 12.8 -> 10.9, 486 tokens 4224 x 2560 13.2 -> 12.1, 700 tokens 2048 x 6144 18.2 -> 16.4).  us, 256 x 256 -> now: forward / input gradient of a dense layer 500 tokens 1024 x 1024 9.5 / 9.6 ->
-// 4.9 / 5.6, 740 tokens 8320 -> 6400 forward 84 -> 68, 700 tokens 2048 -> 6144 input gradient 32.6 -> 21.1.
+// throughout is 24 %.  us, 256 x 256 / chosen width: forward / input gradient of a dense layer 500 tokens 1024 x 1024
+// 9.5 / 9.6 -> 4.9 / 5.6, 740 tokens 8320 -> 6400 forward 84 -> 68, 700 tokens 2048 -> 6144 input gradient 32.6 -> 21.1.
+// The plain store's drain term is that of tiles that leave as TMA stores; with the direct stores' (24 per column) weight
+// gradients took, before -> now, 256 tokens 4096 x 4096 12.8 -> 10.9, 700 tokens 2048 x 6144 18.2 -> 16.4.
 static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int num_pairs) {
     const int num_m = (M + 255) / 256, num_kb = (K + 63) / 64;
     int best = 256;
