@@ -12,8 +12,8 @@
 // shared memory plus two small tiles of T and dT per carried k-block.
 //
 // Work split.  Tile (m, n) of dW (256 x 256, one CTA pair) carries, besides its own product,
-//   - for n < splits_r: the partial sum of dR^T rows [256 m, 256 m + 256) over the k-blocks kb with
-//     kb mod splits_r == n,
+//   - when it is number p < splits_r of its row of tiles in raster order: the partial sum of dR^T rows
+//     [256 m, 256 m + 256) over the k-blocks kb with kb mod splits_r == p,
 //   - for m < splits_l: the partial sum of dL rows [256 n, 256 n + 256) over kb mod splits_l == m,
 // so that every carrier does the same small share of extra work (an MMA of N = r instead of 256 on
 // one k-block in splits) and no tile is much longer than the others.  The fp32 partial sums go to a
@@ -32,6 +32,7 @@ struct DwAdapterParams {
     int M, N, K;                  // d_out, d_in, tokens
     int r;                        // adapter rank, multiple of 16, <= 128
     int splits_r, splits_l;       // partial sums per dR^T row block / per dL row block
+    int alternate_k;              // as in DenseGemmParams
     uint16_t* dWc;                // [M x N/2]
     const uint8_t* mask;          // [M x N/8]
     float* ws_r;                  // [splits_r][M][r]
@@ -106,7 +107,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     auto carries = [&](const PairWork& w, bool& carry_r, bool& carry_l, int& n_blk) {
         n_blk = w.n0 / BLOCK_N;
         const bool full = w.width == BLOCK_N;
-        carry_r = full && n_blk < p.splits_r;
+        carry_r = full && w.pos < p.splits_r;
         carry_l = full && w.m_pair < p.splits_l;
     };
 
@@ -118,7 +119,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             tma_prefetch_desc(&tmT);
             tma_prefetch_desc(&tmDT);
             PipeState ps, ps2;
-            bool ok = true;
+            bool ok = true, backwards = p.alternate_k != 0;
             PairWork w;
             for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w); item += num_pairs) {
                 bool carry_r, carry_l;
@@ -129,7 +130,8 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
                 const int x_small = static_cast<int>(cta) * (p.r / 2);          // this CTA's half of the r columns
                 const uint32_t stage_tx = 2 * (Cfg::kABytes + half_w * 128);
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int i = 0; i < num_kb; ++i) {
+                    const int kb = backwards ? num_kb - 1 - i : i;
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sA = smem + ps.stage * Cfg::kStageBytes;
                     uint8_t* sB = sA + Cfg::kABytes;
@@ -140,7 +142,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     tma_load_2d_pair(sB, &tmB, bar, n0, kb * 64);
                     if (half_w > 64) tma_load_2d_pair(sB + 8192, &tmB, bar, n0 + 64, kb * 64);
                     ps.advance(STAGES);
-                    const bool kr = carry_r && kb % p.splits_r == n_blk;
+                    const bool kr = carry_r && kb % p.splits_r == w.pos;
                     const bool kl = carry_l && kb % p.splits_l == w.m_pair;
                     if (kr || kl) {
                         if (!mbar_wait(&empty2_bar[ps2.stage], ps2.phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -154,6 +156,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                         ps2.advance(Cfg::kSmallStages);
                     }
                 }
+                backwards ^= p.alternate_k != 0;
             }
         }
     } else if (warp == 1) {
@@ -163,7 +166,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             constexpr uint32_t idesc_half = make_idesc_bf16(2 * kBlockM, BLOCK_N / 2, true, true, false);
             const uint32_t idesc_ad = make_idesc_bf16(2 * kBlockM, p.r, true, true, false);
             PipeState ps, ps2;
-            bool ok = true;
+            bool ok = true, backwards = p.alternate_k != 0;
             int it = 0;
             PairWork w;
             for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w);
@@ -175,7 +178,8 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 if (!mbar_wait(tempty_bar, (static_cast<uint32_t>(it) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
                 uint32_t acc_r = 0, acc_l = 0;
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int i = 0; i < num_kb; ++i) {
+                    const int kb = backwards ? num_kb - 1 - i : i;
                     if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t sA = smem_u32(smem + ps.stage * Cfg::kStageBytes);
@@ -183,8 +187,8 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
                         umma_bf16_pair(tmem_base, make_smem_desc(sA + j * 2048, 8192, 1024, kSwizzle128B),
-                                       make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B), idesc, (kb | j) != 0 ? 1u : 0u);
-                    const bool kr = carry_r && kb % p.splits_r == n_blk;
+                                       make_smem_desc(sB + j * 2048, 8192, 1024, kSwizzle128B), idesc, (i | j) != 0 ? 1u : 0u);
+                    const bool kr = carry_r && kb % p.splits_r == w.pos;
                     const bool kl = carry_l && kb % p.splits_l == w.m_pair;
                     if (kr || kl) {
                         if (!mbar_wait(&full2_bar[ps2.stage], ps2.phase, abort_flag)) { ok = false; break; }
@@ -212,6 +216,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     ps.advance(STAGES);
                 }
                 if (ok) umma_commit_pair(tfull_bar, 3);
+                backwards ^= p.alternate_k != 0;
             }
         }
     } else {
@@ -265,7 +270,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             if (half == 0 ? carry_r : carry_l) {
                 const int row = half == 0 ? m : n_blk * BLOCK_N + static_cast<int>(cta) * kBlockM + row_in_cta;
                 const int rows_total = half == 0 ? p.M : p.N;
-                const int split = half == 0 ? n_blk : w.m_pair;
+                const int split = half == 0 ? w.pos : w.m_pair;
                 float* dst = (half == 0 ? p.ws_r : p.ws_l) + (static_cast<size_t>(split) * rows_total + row) * p.r;
                 const uint32_t t_ad = t_row + (half == 0 ? Cfg::kColR : Cfg::kColL);
 #pragma unroll 1

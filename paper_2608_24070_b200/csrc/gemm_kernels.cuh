@@ -69,6 +69,7 @@ struct SparseGemmParams {
     int num_n;                    // tile kernels: token tiles
     int stages;                   // tile kernels: pipeline stages that fit at that width
     int group_m;                  // 512-row-tile kernel: row tiles per raster group (0: all in one group)
+    int alternate_k;              // 512-row-tile kernel: 1: every other tile of a pair takes the reduction from its end (see quad_tile)
     int pdl_mode;                 // 2: consumer of a fused pair of launches (see the few-token kernel)
     uint16_t* out;                // [Ntok x M]
 };
@@ -89,6 +90,7 @@ struct DenseGemmParams {
     int M, N, K;
     int width;                    // columns per tile: 64, 128, 192 or 256
     int stages;                   // pipeline stages that fit at that width
+    int alternate_k;              // CTA-pair kernel: 1: every other tile of a pair takes the reduction from its end (see raster_tile)
     void* out;
     const uint8_t* mask;          // kEpiMasked: [M x N/8]
 };
@@ -631,16 +633,29 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 // Tile order for GEMMs whose two operands are both streamed once per tile (dW: dY^T X with the
 // tokens as reduction).  The ~74 tiles in flight should form a near-square patch of the output:
 // a patch of gm x gn tiles reads (gm + gn) operand panels, a gm x 1 strip reads gm + 1 for 1/gn
-// of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column.
+// of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column, forwards in one group and
+// backwards in the next: the wave that straddles two groups then has the columns of both in common.
+// These GEMMs run at the power cap, where a byte from HBM costs what some 150 FLOP do, so what a wave can take from L2
+// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on; its last part is still
+// there when the next wave begins, and half of its panels are the next wave's too, so with a long reduction
+// every other tile of a pair takes the k-blocks from the end (alternate_k).  While the panels fit, that order
+// only lengthens the way between two uses of a k-block.  A model of L2 as 60 MB, least recently used first out, which gives the
+// 630 MB that 4096 x 4096 at 16384 tokens read before, has 540 MB now, and 1.45 instead of 1.77 GB for 4096 -> 11008.
+// us under sustained load, every group and tile forwards / now: 16384 tokens 4096 x 4096 427 / 421, 4096 -> 11008 1136 / 1117,
+// 11008 -> 4096 1117 / 1105, 8192 tokens 5120 -> 13824 878 / 862, 12000 tokens 2048 -> 5504 220 / 215.5; the order of the
+// groups alone, 4096 tokens 4096 -> 11008 273.9 / 273.8, 2048 tokens 5120 -> 13824 215.6 / 215.0.
 constexpr int kRasterGroupM = 8;
-__device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, int& m, int& n) {
+constexpr int kAlternateFrom = 6144;          // shortest reduction that is taken from alternating ends
+// (`pos`: how many columns of tiles of the group come before the tile's)
+__host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, int& m, int& n, int& pos) {
     const int group_size = kRasterGroupM * num_n;
     const int g = tile / group_size;
     const int first_m = g * kRasterGroupM;
-    const int gm = min(num_m - first_m, kRasterGroupM);
+    const int gm = num_m - first_m < kRasterGroupM ? num_m - first_m : kRasterGroupM;
     const int local = tile - g * group_size;
     m = first_m + local % gm;
-    n = local / gm;
+    pos = local / gm;
+    n = g & 1 ? num_n - 1 - pos : pos;
 }
 
 // Work items of the persistent CTA-pair GEMM.  Items are tiles in raster order; when the tiles
@@ -649,7 +664,7 @@ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, int&
 // takes half the time instead of a full tile time on a half-empty machine (4096 x 4096 weight
 // gradient: 256 tiles on 74 pairs = 3 waves + 34 tiles -> 68 half items: 3.5 instead of 4 waves).
 struct PairWork {
-    int m_pair, n0, width;
+    int m_pair, n0, width, pos;
 };
 __device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, int num_n, int width, bool split_tail,
                                           PairWork& w) {
@@ -660,7 +675,7 @@ __device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, in
     const bool halved = split && item >= full;
     const int tile = halved ? full + ((item - full) >> 1) : item;
     int n_blk;
-    raster_tile(tile, num_m, num_n, w.m_pair, n_blk);
+    raster_tile(tile, num_m, num_n, w.m_pair, n_blk, w.pos);
     w.width = halved ? width / 2 : width;
     w.n0 = n_blk * width + (halved && ((item - full) & 1) ? width / 2 : 0);
     return true;
@@ -737,7 +752,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     if (warp == 0) {
         if (elect_one()) {
             RingState ps;
-            bool ok = true;
+            bool ok = true, backwards = p.alternate_k != 0;   // (what ran before, the input gradient, read the last tokens last)
             PairWork w;
             const uint32_t leader_bar = mapa_shared(smem_u32(full_bar), 0);
             for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
@@ -752,21 +767,23 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     uint8_t* sA = smem + ps.off;
                     uint8_t* sB = sA + Cfg::kABytes;
                     const uint32_t bar = leader_bar + 8 * ps.stage;
+                    const int k0 = (backwards ? num_kb - 1 - kb : kb) * 64;
                     if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], stage_tx);
                     if (A_MN) {
-                        tma_load_2d_pair(sA, &tmA, bar, m0, kb * 64);
-                        tma_load_2d_pair(sA + 8192, &tmA, bar, m0 + 64, kb * 64);
+                        tma_load_2d_pair(sA, &tmA, bar, m0, k0);
+                        tma_load_2d_pair(sA + 8192, &tmA, bar, m0 + 64, k0);
                     } else {
-                        tma_load_2d_pair(sA, &tmA, bar, kb * 64, m0);
+                        tma_load_2d_pair(sA, &tmA, bar, k0, m0);
                     }
                     if (B_MN) {
-                        tma_load_2d_pair(sB, &tmB, bar, n0, kb * 64);
-                        if (two_chunks) tma_load_2d_pair(sB + 8192, &tmB, bar, n0 + 64, kb * 64);
+                        tma_load_2d_pair(sB, &tmB, bar, n0, k0);
+                        if (two_chunks) tma_load_2d_pair(sB + 8192, &tmB, bar, n0 + 64, k0);
                     } else {
-                        tma_load_2d_pair(sB, &tmB, bar, kb * 64, n0);
+                        tma_load_2d_pair(sB, &tmB, bar, k0, n0);
                     }
                     ps.advance(stages, stage_bytes);
                 }
+                backwards ^= p.alternate_k != 0;
             }
         }
     } else if (warp == 1) {
@@ -913,7 +930,11 @@ struct SparseQuadCfg {
 // then token blocks, then the next group.  The pairs that work on one token block side by side
 // share its activation tile; a group's share of the compressed weight is what has to stay in L2
 // while the token blocks sweep by.  `first` marks the tile that prefetches the block's
-// activations into L2 for its group.
+// activations into L2 for its group.  Where even one group's weights are more than L2 keeps (long reductions), every other
+// tile of a pair takes the k-blocks from the end (alternate_k), so that a wave begins with the weights the last
+// one ended with.  us under sustained load, before / now: 16384 tokens 11008 -> 4096 632 / 617, 8192 tokens 13824 -> 5120 494 / 487,
+// 4000 tokens 11008 -> 4096 157.6 / 155.7.  (Where they fit, the order would only cost: 5120 -> 13824 in two groups 249 -> 306 MB
+// by a model of L2 as 60 MB, least recently used first out.)
 __device__ __forceinline__ void quad_tile(int tile, int num_m, int num_n, int group_m, int& mt, int& n_blk,
                                           bool& first) {
     const int group_size = group_m * num_n;
@@ -994,7 +1015,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const uint64_t keep = l2_policy_evict_last();
             PipeState ps;
             bool ok = true;
-            bool waited = false;
+            bool waited = false, backwards = false;
             for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
                 int mt, n_blk, next_mt, next_n_blk;
                 bool first, next_first = false;
@@ -1011,17 +1032,21 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     next_first ? next_n_blk * p.width +
                                      static_cast<int>(cta) * (token_tile_width(p.Ntok, next_n_blk * p.width, p.width) / 2)
                                : 0;
+                const bool next_backwards = backwards != (p.alternate_k != 0);
+                const auto k_column = [&](int kb, bool from_end) { return (from_end ? num_kb - 1 - kb : kb) * 128; };
                 for (int kb = 0; kb < total_kb; ++kb) {
                     if (kb < num_kb) {
                         const int pk = kb + kPrefetchAhead;
                         if (pk < num_kb) {
                             if (first) {
-                                tma_prefetch_l2_2d(&tmB, pk * 128, n_row0);
-                                tma_prefetch_l2_2d(&tmB, pk * 128 + 64, n_row0);
+                                const int x = k_column(pk, backwards);
+                                tma_prefetch_l2_2d(&tmB, x, n_row0);
+                                tma_prefetch_l2_2d(&tmB, x + 64, n_row0);
                             }
                         } else if (next_first && pk - num_kb < num_kb) {
-                            tma_prefetch_l2_2d(&tmB, (pk - num_kb) * 128, next_row0);
-                            tma_prefetch_l2_2d(&tmB, (pk - num_kb) * 128 + 64, next_row0);
+                            const int x = k_column(pk - num_kb, next_backwards);
+                            tma_prefetch_l2_2d(&tmB, x, next_row0);
+                            tma_prefetch_l2_2d(&tmB, x + 64, next_row0);
                         }
                     }
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -1032,13 +1057,14 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         if (cta == 0)
                             mbar_expect_tx(&full_bar[ps.stage],
                                            2 * (2 * b_half + nsub * (Cfg::kABytes + Cfg::kEBytes)));
-                        tma_load_2d_pair(sB, &tmB, bar, kb * 128, n_row0);
-                        tma_load_2d_pair(sB + b_half, &tmB, bar, kb * 128 + 64, n_row0);
+                        const int x = k_column(kb, backwards);
+                        tma_load_2d_pair(sB, &tmB, bar, x, n_row0);
+                        tma_load_2d_pair(sB + b_half, &tmB, bar, x + 64, n_row0);
                         for (int s = 0; s < nsub; ++s) {
                             const int mb = 4 * mt + 2 * s + static_cast<int>(cta);
                             const int mb_e = mb < num_mb ? mb : num_mb - 1;
-                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, kb * 64, mb * kBlockM, keep);
-                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kb,
+                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, x / 2, mb * kBlockM, keep);
+                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + x / 128,
                                                   keep);
                         }
                     } else {
@@ -1063,6 +1089,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     }
                     ps.advance(stages);
                 }
+                backwards = next_backwards;
             }
         }
     } else if (warp == 1) {

@@ -513,11 +513,12 @@ static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* 
 // a group's weights resident.  Pick the g with the least estimated DRAM traffic
 // (measured at 16384 tokens: 4096 -> 11008 two groups +7 %, 5120 -> 13824 three groups +11 %,
 // square and long-reduction layers one group).
+// Where one group's weights do not fit, tiles alternate the end of the reduction that they begin with (see quad_tile).
+constexpr double kL2Keeps = 30e6;
 static int quad_group_m(int M, int K, int ntok, int width, int num_pairs) {
     const int num_m = (M / kBlockM + 3) / 4, num_n = (ntok + width - 1) / width;
     const double w_tile = 512.0 * K * 1.125, w_total = static_cast<double>(M) * K * 1.125;
     const double x_total = static_cast<double>(ntok) * K * 2.0;
-    constexpr double kL2Keeps = 30e6;
     int best_gm = num_m;
     double best = 1e300;
     for (int g = 1; g <= num_m; ++g) {
@@ -538,6 +539,7 @@ static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* 
     if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, pdl_mode))
         return SLOPE_ERR_CUDA;
     a.p.group_m = quad_group_m(M, K, ntok, width, max_pairs);
+    a.p.alternate_k = a.p.group_m * 512.0 * K * 1.125 > kL2Keeps;
     if (!set_smem(sparse_gemm_quad_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
     const int tiles = ((M / kBlockM + 3) / 4) * ((ntok + width - 1) / width);
     const int pairs = std::min(tiles, max_pairs);
@@ -861,6 +863,9 @@ static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int n
     return best;
 }
 
+// (256 x 256 tiles only: the fused weight and adapter gradients, which have no others, then add up the same sums in the same order)
+static int alternate_k(int K, int width) { return K >= kAlternateFrom && width == 256 ? 1 : 0; }
+
 // D[M x N] on 128 x 128 tiles of single CTAs while they all run at once and the reduction is at most
 // 2048 long (measured on both sides of either line: dense_gemm_kernel), else on the CTA-pair kernel; a dense layer with
 // fewer than 64 such tiles has more CTAs of the pair kernel's 64-column tiles (256 tokens 512 x 512: 3.7 against 4.3 us).
@@ -880,7 +885,7 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
     if (small) {
         constexpr int kStages = 6;
         using Cfg = DenseCfg<kStages>;
-        const DenseGemmParams p{M, N, K, width, kStages, out, static_cast<const uint8_t*>(mask)};
+        const DenseGemmParams p{M, N, K, width, kStages, 0, out, static_cast<const uint8_t*>(mask)};
         auto kern = dense_gemm_kernel<A_MN, B_MN, EPI, kStages>;
         if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
         return launch_cluster_ex(kern, small_tiles, 1, kDenseThreads, Cfg::kSmemBytes, /*overlap_prologue=*/true, stream, tmA,
@@ -890,7 +895,7 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
     CUtensorMap tmO = tmA;
     if (EPI == kEpiStore && !make_tmap_out(&tmO, out, M, N, 32, 32)) return SLOPE_ERR_CUDA;
     const int stages = dense_stages(B_MN, EPI, width);
-    const DenseGemmParams p{M, N, K, width, stages, out, static_cast<const uint8_t*>(mask)};
+    const DenseGemmParams p{M, N, K, width, stages, alternate_k(K, width), out, static_cast<const uint8_t*>(mask)};
     auto kern = dense_gemm_pair_kernel<A_MN, B_MN, EPI>;
     if (!set_smem(kern, 232448)) return SLOPE_ERR_CUDA;
     const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + width - 1) / width);
@@ -1216,12 +1221,10 @@ static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_c
     const int num_pairs = sm_count / 2, num_tiles = num_m * num_n;
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
     if (rem > 0 && 2 * rem <= num_pairs) {
-        for (int tile = full; tile < num_tiles; ++tile) {            // the raster order of raster_tile()
-            const int group_size = kRasterGroupM * num_n, g = tile / group_size, first_m = g * kRasterGroupM;
-            const int gm = num_m - first_m < kRasterGroupM ? num_m - first_m : kRasterGroupM;
-            const int local = tile - g * group_size;
-            const int m = first_m + local % gm, n = local / gm;
-            if (m < plan.splits_l || n < plan.splits_r) return plan;
+        for (int tile = full; tile < num_tiles; ++tile) {
+            int m, n, pos;
+            raster_tile(tile, num_m, num_n, m, n, pos);
+            if (m < plan.splits_l || pos < plan.splits_r) return plan;
         }
     }
     plan.fused = true;
@@ -1267,6 +1270,7 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     DwAdapterParams p = {};
     p.M = d_out; p.N = d_in; p.K = b; p.r = r;
     p.splits_r = plan.splits_r; p.splits_l = plan.splits_l;
+    p.alternate_k = alternate_k(b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
     p.dWc = static_cast<uint16_t*>(dWc_vals);
     p.mask = static_cast<const uint8_t*>(mask1_bits);
     p.ws_r = static_cast<float*>(workspace);
