@@ -33,6 +33,19 @@ struct PackedPick {
     uint32_t code;            // p0 | p1 << 2 of group 0 in bits 0..3, of group 1 in bits 16..19
 };
 
+// A value the compiler takes as it is: left to itself it merges the logic operation that made the value into those that use
+// it, and then carries both operands along.  (A multiply-add by one, which is not the logic pipe; `one` must be opaque too.)
+__device__ __forceinline__ uint32_t opaque_one() {
+    uint32_t v;
+    asm volatile("mov.u32 %0, %%nsmid;\n\tmin.u32 %0, %0, 1;" : "=r"(v));
+    return v;
+}
+__device__ __forceinline__ uint32_t pin(uint32_t x, uint32_t one) {
+    uint32_t v;
+    asm volatile("mad.lo.u32 %0, %1, %2, 0;" : "=r"(v) : "r"(x), "r"(one));
+    return v;
+}
+
 __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (a & c) | (b & c); }
 __device__ __forceinline__ uint32_t bitsel(uint32_t m, uint32_t a, uint32_t b) { return (m & a) | (~m & b); }
 
@@ -243,10 +256,12 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
 #pragma unroll
     for (int t = 0; t < 8; ++t) w[t] = ld_v4(W + at0 + t * row_u4);
 
-    // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place.  (Leaving it in the
-    //      packed order would save its four byte permutes per row, but an and that feeds another logic operation is merged
-    //      into it, which carries element and mask apart into the second pass: 204 bytes of spills, 22 us instead of 18 at
-    //      4096 x 4096.)
+    // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place, in the packed order, in
+    //      which words of the second pass are pairs of columns j, j + 4 (four byte permutes per row less than back in natural
+    //      order).  The masked words are pinned: merged into the second pass they cost 204 bytes of spills, 22 us
+    //      instead of 18 at 4096 x 4096.  us, natural / packed order: 4096 x 4096 16.4 / 16.1, 4096 x 11008 40.2 / 39.5,
+    //      13824 x 5120 62.5 / 61.4, 2048 x 2048 6.27 / 6.10.
+    const uint32_t one = opaque_one();
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const uint32_t E0 = prmt(w[t].x, w[t].z, 0x5410u), E1 = prmt(w[t].x, w[t].z, 0x7632u);
@@ -256,8 +271,7 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
         vals[at0 + t * mrow] = make_uint2(a.out0, a.out1);
         s_meta[meta_byte_offset(rr, c8)] = static_cast<uint8_t>(meta_byte(a));
         s_mask[rr * 16 + c8] = static_cast<uint8_t>(mask_byte(a));
-        const uint32_t x0 = E0 & a.keep[0], x1 = E1 & a.keep[1], x2 = E2 & a.keep[2], x3 = E3 & a.keep[3];
-        w[t] = make_uint4(prmt(x0, x1, 0x5410u), prmt(x2, x3, 0x5410u), prmt(x0, x1, 0x7632u), prmt(x2, x3, 0x7632u));
+        w[t] = make_uint4(pin(E0 & a.keep[0], one), pin(E1 & a.keep[1], one), pin(E2 & a.keep[2], one), pin(E3 & a.keep[3], one));
     }
 
     // ---- second pass on the masked tile (see double_prune_kernel)
@@ -270,8 +284,8 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
         for (int t = 0; t < 8; ++t) x[t] = wi == 0 ? w[t].x : (wi == 1 ? w[t].y : (wi == 2 ? w[t].z : w[t].w));
         const PackedPick a = pick2of4_packed(x[0], x[1], x[2], x[3]);
         const PackedPick b = pick2of4_packed(x[4], x[5], x[6], x[7]);
-        second_pass_store(a, b, 2 * wi, 2 * wi + 1, ig, c8, s_out, s_metaT + meta_base);
-        if (mask2 != nullptr) second_pass_select(a, b, 2 * wi, 2 * wi + 1, sel);
+        second_pass_store(a, b, wi, wi + 4, ig, c8, s_out, s_metaT + meta_base);
+        if (mask2 != nullptr) second_pass_select(a, b, wi, wi + 4, sel);
     }
     if (mask2 != nullptr) {
 #pragma unroll
