@@ -282,6 +282,15 @@ __device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
     return v;
 }
 
+// with an L2 eviction-priority hint
+__device__ __forceinline__ uint4 ld_hint_v4(const void* p, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p), "l"(policy));
+    return v;
+}
+
 // Read four consecutive fp32 (16-byte aligned) from the shared memory of a CTA of the cluster.
 __device__ __forceinline__ float4 ld_shared_cluster_v4(uint32_t cluster_saddr) {
     float4 v;
