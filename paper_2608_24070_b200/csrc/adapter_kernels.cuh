@@ -17,6 +17,8 @@
 // 12.3 / 28.3 -> 6.2 / 8.6; dT + dL + dR at 8192 tokens, 5120 -> 13824, r = 128: 115 -> 92 (82 at the
 // HBM peak); at 1000 tokens, 768 -> 2304, r = 256: 29.8 -> 13.4; T at 16384 x 4096, r = 256: 45 -> 36.
 #pragma once
+#include <type_traits>
+
 #include "gemm_kernels.cuh"
 
 namespace slope {
@@ -76,12 +78,44 @@ __device__ __forceinline__ void adapter_reduce(const AdapterProblem& p, uint32_t
     }
 }
 
-template <bool A_MN, bool B_MN, int N_TILE>
+// Weights of the few-token forward that a T launch is the producer of.  That forward's CTAs come up only when T has let them in, i.e.
+// when everything before the pair is complete, and their first loads 1 to 1.5 us later, in which HBM would have nothing to do;
+// `blocks` further CTAs of the T launch, on SMs that T does not need, ask L2 for the first k-blocks of every slice meanwhile.
+// (4 linears of a block of width 4096 / 11008, r = 64, 8 tokens, us: none 56.96, 3 k-blocks 55.40, 6 55.66, 12 58.19.)
+constexpr int kPairPrefetchBlocks = 3;     // k-blocks of a slice
+struct WeightPrefetch {
+    const uint8_t *vals, *meta;   // compressed values [M x K/2] and their metadata
+    int K, splits, slices;        // K-slices of a 128-row slab; slices of all slabs
+    int blocks;                   // at the end of the grid, whole clusters; 0: none
+};
+__device__ __forceinline__ void prefetch_weights(const WeightPrefetch& w, int block) {
+    const int num_kb = w.K / 128, kb_per = (num_kb + w.splits - 1) / w.splits;
+    for (int slice = block; slice < w.slices; slice += w.blocks) {
+        const int slab = slice / w.splits, kb0 = slice % w.splits * kb_per;
+        const int n = min(kPairPrefetchBlocks, min(num_kb, kb0 + kb_per) - kb0);
+        const uint8_t* v = w.vals + static_cast<size_t>(slab) * kBlockM * w.K + kb0 * 128;
+        for (int i = threadIdx.x; i < kBlockM * n; i += kGemmThreads) prefetch_l2(v + static_cast<size_t>(i / n) * w.K + i % n * 128);
+        const uint8_t* m = w.meta + (static_cast<size_t>(slab) * num_kb + kb0) * 2048;
+        for (int i = threadIdx.x; i < 16 * n; i += kGemmThreads) prefetch_l2(m + i * 128);
+    }
+}
+
+struct NoPrefetch {};                      // (launches without such CTAs do not pay for the test)
+
+template <bool A_MN, bool B_MN, int N_TILE, typename Prefetch>
 __global__ void __launch_bounds__(kGemmThreads, 2)
 adapter_gemm_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0,
                     const AdapterProblem p0, const __grid_constant__ CUtensorMap tmA1,
                     const __grid_constant__ CUtensorMap tmB1, const AdapterProblem p1, const int stages,
-                    const int pdl_mode) {
+                    const int pdl_mode, const Prefetch next) {
+    if constexpr (std::is_same<Prefetch, WeightPrefetch>::value) {
+        if (blockIdx.x >= gridDim.x - next.blocks) {
+            griddep_wait();
+            griddep_launch_dependents();
+            prefetch_weights(next, blockIdx.x - (gridDim.x - next.blocks));
+            return;
+        }
+    }
     // One cluster per tile of 128 rows x N_TILE columns, column tiles of a row tile next to each other.  Up to
     // two problems with the same N and K share a launch (p1.M == 0: only one): the row tiles
     // [0, tiles0) belong to problem 0, the rest to problem 1.

@@ -392,7 +392,7 @@ static int adapter_sms(const AdapterPlan& plan, int rows, int N, int sm_count) {
 
 template <bool A_MN, bool B_MN, int N_TILE>
 static slope_status_t launch_adapter_tile(const AdapterOperands& q0, const AdapterOperands& q1, int N, int K, int splits,
-                                          bool deep, cudaStream_t stream, int pdl_mode) {
+                                          bool deep, cudaStream_t stream, int pdl_mode, const WeightPrefetch& next) {
     using Cfg = AdapterCfg<N_TILE>;
     CUtensorMap tm[4];
     AdapterProblem p[2];
@@ -408,22 +408,28 @@ static slope_status_t launch_adapter_tile(const AdapterOperands& q0, const Adapt
         p[i] = AdapterProblem{live ? q.M : 0, N, K, static_cast<uint16_t*>(q.out), q.transposed};
         if (live) tiles += (q.M + kBlockM - 1) / kBlockM;
     }
-    auto kern = adapter_gemm_kernel<A_MN, B_MN, N_TILE>;
-    if (!set_smem(kern, Cfg::smem_bytes(Cfg::kDeep))) return SLOPE_ERR_CUDA;
     const int stages = deep || Cfg::kShared == 0 ? Cfg::kDeep : Cfg::kShared;
-    return launch_cluster_ex(kern, tiles * ((N + N_TILE - 1) / N_TILE) * splits, splits, kGemmThreads,
-                             Cfg::smem_bytes(stages), /*overlap_prologue=*/true, stream, tm[0], tm[1], p[0], tm[2], tm[3],
-                             p[1], stages, pdl_mode);
+    const int ctas = tiles * ((N + N_TILE - 1) / N_TILE) * splits;
+    const auto launch = [&](auto prefetch, int further) {
+        auto kern = adapter_gemm_kernel<A_MN, B_MN, N_TILE, decltype(prefetch)>;
+        if (!set_smem(kern, Cfg::smem_bytes(Cfg::kDeep))) return SLOPE_ERR_CUDA;
+        return launch_cluster_ex(kern, ctas + further, splits, kGemmThreads, Cfg::smem_bytes(stages), /*overlap_prologue=*/true,
+                                 stream, tm[0], tm[1], p[0], tm[2], tm[3], p[1], stages, pdl_mode, prefetch);
+    };
+    if constexpr (!A_MN && B_MN)                             // (T)
+        if (next.blocks > 0) return launch(next, next.blocks);
+    return launch(NoPrefetch{}, 0);
 }
 
 // D[M x N] = A B over one or two problems with the same N (= r) and K.
 template <bool A_MN, bool B_MN>
 static slope_status_t launch_adapter_planned(const AdapterPlan& plan, const AdapterOperands& q0, const AdapterOperands& q1,
-                                             int N, int K, cudaStream_t stream, int pdl_mode) {
+                                             int N, int K, cudaStream_t stream, int pdl_mode,
+                                             const WeightPrefetch& next = WeightPrefetch{}) {
     switch (plan.n_tile) {
-        case 64: return launch_adapter_tile<A_MN, B_MN, 64>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
-        case 128: return launch_adapter_tile<A_MN, B_MN, 128>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
-        default: return launch_adapter_tile<A_MN, B_MN, 256>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode);
+        case 64: return launch_adapter_tile<A_MN, B_MN, 64>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode, next);
+        case 128: return launch_adapter_tile<A_MN, B_MN, 128>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode, next);
+        default: return launch_adapter_tile<A_MN, B_MN, 256>(q0, q1, N, K, plan.splits, plan.deep, stream, pdl_mode, next);
     }
 }
 template <bool A_MN, bool B_MN>
@@ -609,6 +615,29 @@ static bool skinny_capacity(const DeviceInfo& info, int (&cap)[9]) {
     return cap[1] > 0;
 }
 
+// K-splits of a launch of the few-token kernel (0: the device has no room for it).
+template <int BLOCK_N, int A_STAGES, int B_STAGES>
+static int skinny_split_count(int ntok, int M, int K, int r, const DeviceInfo& info, int pdl_mode) {
+    int cap[9];
+    if (!skinny_capacity<BLOCK_N, A_STAGES, B_STAGES>(info, cap)) return 0;
+    thread_local SizeMemo<int> memo;
+    return memo.get({M, K, pdl_mode == 2 ? ntok : 0, pdl_mode == 2 ? r : 0, pdl_mode, info.dev}, [&] {
+        if (pdl_mode == 2) {
+            // The consumer of a fused pair has to be resident next to its producer, or its last clusters
+            // would wait for the producer to finish and the overlap would be lost: count only the
+            // clusters that fit beside it.
+            const AdapterPlan producer = adapter_plan(adapter_T_shape(ntok, K, r), info.sm_count);
+            const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
+            for (int sz = 1; sz <= 8; ++sz) {
+                cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
+                if (cap[sz] < 0) cap[sz] = 0;
+            }
+            if (cap[1] <= 0) return 0;
+        }
+        return skinny_splits(M / kBlockM, K / 128, BLOCK_N, cap);
+    });
+}
+
 template <int BLOCK_N, int A_STAGES, int B_STAGES>
 static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
                                            const void* act2, const void* fac2, int r, bool a2_mn, void* out,
@@ -637,25 +666,7 @@ static slope_status_t launch_sparse_skinny(const void* act, int ntok, const void
     auto kern = sparse_gemm_skinny_kernel<BLOCK_N, A_STAGES, B_STAGES>;
     if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
 
-    const int slabs = M / kBlockM;
-    int cap[9];
-    if (!skinny_capacity<BLOCK_N, A_STAGES, B_STAGES>(info, cap)) return SLOPE_ERR_CUDA;
-    thread_local SizeMemo<int> memo;                         // (0: nothing fits beside the producer)
-    const int splits = memo.get({M, K, pdl_mode == 2 ? ntok : 0, pdl_mode == 2 ? r : 0, pdl_mode, info.dev}, [&] {
-        if (pdl_mode == 2) {
-            // The consumer of a fused pair has to be resident next to its producer, or its last clusters
-            // would wait for the producer to finish and the overlap would be lost: count only the
-            // clusters that fit beside it.
-            const AdapterPlan producer = adapter_plan(adapter_T_shape(ntok, K, r), info.sm_count);
-            const int reserved = adapter_sms(producer, ntok, r, info.sm_count);
-            for (int sz = 1; sz <= 8; ++sz) {
-                cap[sz] -= (reserved + sz - 1) / sz + (sz > 1 ? 1 : 0);
-                if (cap[sz] < 0) cap[sz] = 0;
-            }
-            if (cap[1] <= 0) return 0;
-        }
-        return skinny_splits(slabs, K / 128, BLOCK_N, cap);
-    });
+    const int slabs = M / kBlockM, splits = skinny_split_count<BLOCK_N, A_STAGES, B_STAGES>(ntok, M, K, r, info, pdl_mode);
     if (splits == 0) return SLOPE_ERR_CUDA;
     return launch_cluster_ex(kern, slabs * splits, splits, kGemmThreads, Cfg::kSmemBytes, true, stream, tmA, tmB,
                              tmE, tmA2, tmB2, p);
@@ -679,18 +690,26 @@ static bool prefer_two_ctas_per_sm(int M, int K, const DeviceInfo& info) {
     return est_flat < 0.93 * est_deep;
 }
 
-static slope_status_t launch_skinny(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
-                                    const void* act2, const void* fac2, int r, bool a2_mn, void* out,
-                                    cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+// Calls visit(token tile, weight stages, activation stages), as integral constants, with the variant for a launch.
+template <typename Visit>
+static auto with_skinny_variant(int ntok, int M, int K, const DeviceInfo& info, Visit visit) {
+    using std::integral_constant;
     if (ntok <= 16) {
         thread_local SizeMemo<bool> memo;
         if (memo.get({M, K, info.dev, 0, 0, 0}, [&] { return prefer_two_ctas_per_sm<16, 10, 4, 5, 2>(M, K, info); }))
-            return launch_sparse_skinny<16, 5, 2>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
-        return launch_sparse_skinny<16, 10, 4>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
+            return visit(integral_constant<int, 16>{}, integral_constant<int, 5>{}, integral_constant<int, 2>{});
+        return visit(integral_constant<int, 16>{}, integral_constant<int, 10>{}, integral_constant<int, 4>{});
     }
     if (ntok <= 64)      // (a two-per-SM variant of this tile, <64, 4, 2>, measured slower: its activation ring is too shallow)
-        return launch_sparse_skinny<64, 8, 4>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
-    return launch_sparse_skinny<128, 7, 3>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
+        return visit(integral_constant<int, 64>{}, integral_constant<int, 8>{}, integral_constant<int, 4>{});
+    return visit(integral_constant<int, 128>{}, integral_constant<int, 7>{}, integral_constant<int, 3>{});
+}
+static slope_status_t launch_skinny(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
+                                    const void* act2, const void* fac2, int r, bool a2_mn, void* out,
+                                    cudaStream_t stream, const DeviceInfo& info, int pdl_mode = 0) {
+    return with_skinny_variant(ntok, M, K, info, [&](auto n, auto a, auto b) {
+        return launch_sparse_skinny<n(), a(), b()>(act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, stream, info, pdl_mode);
+    });
 }
 
 // Tile of a sparse GEMM, by estimate:
@@ -813,11 +832,31 @@ static FwdAdapterPlan fwd_adapter_plan(int b, int d_out, int d_in, int r, const 
     return memo.get({b, d_out, d_in, r, info.dev, 0}, [&] { return plan_fwd_adapter(b, d_out, d_in, r, info); });
 }
 
+// What the T launch in front of a few-token forward asks L2 for: the first k-blocks of weights of at least 40 MB that are tall enough
+// to occupy the SMs without a split, at up to 16 tokens.  Launching the further CTAs costs the pair up to 0.5 us, which a
+// shorter or a split stream does not give back.  us without / with it, r = 64, 8 tokens: 4096 -> 22016 21.2 / 19.5, 5120 -> 35840
+// 34.25 / 33.5; on the other side of the line 4096 -> 12288 13.93 / 14.04, 11008 -> 4096 13.53 / 13.55, and the four linears
+// of a block of width 2048 / 6400 32.3 / 33.1, 1280 / 4096 27.4 / 29.5; of 4096 / 11008 56.9 / 55.3, of 3584 / 9600 49.7 / 48.5.
+constexpr double kPairPrefetchFrom = 40e6;
+constexpr int kPairPrefetchRows = 16384;
+static WeightPrefetch pair_prefetch(const FwdAdapterPlan& plan, int ntok, const void* vals, const void* meta, int M, int K, int r,
+                                    const DeviceInfo& info) {
+    if (plan.tile.rows != 0 || ntok > 16 || M < kPairPrefetchRows || 1.125 * M * K < kPairPrefetchFrom) return WeightPrefetch{};
+    const int splits = with_skinny_variant(ntok, M, K, info, [&](auto n, auto a, auto b) {
+        return skinny_split_count<n(), a(), b()>(ntok, M, K, r, info, 2);
+    });
+    if (splits == 0) return WeightPrefetch{};
+    // (clusters of 8 fill 120 of 148 SMs)
+    const int slices = M / kBlockM * splits, free_sms = info.sm_count * 120 / 148 - adapter_sms(plan.T, ntok, r, info.sm_count);
+    const int blocks = std::max(std::min(slices, free_sms), 0) / plan.T.splits * plan.T.splits;
+    return WeightPrefetch{static_cast<const uint8_t*>(vals), static_cast<const uint8_t*>(meta), K, splits, slices, blocks};
+}
+
 // T[b x r] = X[b x d_in] * L[d_in x r]   (A = X, K contiguous; B = L^T stored [K x N])
 static slope_status_t launch_adapter_T(const FwdAdapterPlan& plan, const void* X, const void* L, int b, int d_in, int r,
-                                       void* T, cudaStream_t stream, int pdl_mode) {
+                                       void* T, cudaStream_t stream, int pdl_mode, const WeightPrefetch& next = WeightPrefetch{}) {
     return launch_adapter_planned<false, true>(plan.T, AdapterOperands{X, L, T, b, 0}, AdapterOperands{}, r, d_in, stream,
-                                               pdl_mode);
+                                               pdl_mode, next);
 }
 
 static slope_status_t launch_sparse_gemm(const void* act, int ntok, const void* vals, const void* meta, int M, int K,
@@ -1054,7 +1093,8 @@ slope_status_t slope_linear_fwd_adapter(const void* X, int b, const void* Wc_val
     if (slope_status_t st = check_arch(info)) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const FwdAdapterPlan plan = fwd_adapter_plan(b, d_out, d_in, r, info);
-    if (slope_status_t st = launch_adapter_T(plan, X, L, b, d_in, r, T, stream, 1)) return st;
+    const WeightPrefetch next = pair_prefetch(plan, b, Wc_vals, Wc_meta, d_out, d_in, r, info);
+    if (slope_status_t st = launch_adapter_T(plan, X, L, b, d_in, r, T, stream, 1, next)) return st;
     if (plan.tile.rows == 0) {
         // Two launches of the few-token kernel as a fused pair: T = X L releases its dependent only
         // once everything before it in the stream is complete, so the forward streams its weights
