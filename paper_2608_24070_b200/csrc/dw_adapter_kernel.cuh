@@ -120,8 +120,9 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             tma_prefetch_desc(&tmDT);
             PipeState ps, ps2;
             bool ok = true, backwards = p.alternate_k != 0;
+            int it = 0;
             PairWork w;
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w); item += num_pairs) {
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, p.alternate_k != 0, w); item += num_pairs, ++it) {
                 bool carry_r, carry_l;
                 int n_blk;
                 carries(w, carry_r, carry_l, n_blk);
@@ -156,7 +157,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                         ps2.advance(Cfg::kSmallStages);
                     }
                 }
-                backwards ^= p.alternate_k != 0;
+                backwards ^= p.alternate_k != 0 && (it & 1);      // (dense_gemm_pair_kernel takes two at a time)
             }
         }
     } else if (warp == 1) {
@@ -169,7 +170,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             bool ok = true, backwards = p.alternate_k != 0;
             int it = 0;
             PairWork w;
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w);
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, p.alternate_k != 0, w);
                  item += num_pairs, ++it) {
                 bool carry_r, carry_l;
                 int n_blk;
@@ -216,7 +217,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     ps.advance(STAGES);
                 }
                 if (ok) umma_commit_pair(tfull_bar, 3);
-                backwards ^= p.alternate_k != 0;
+                backwards ^= p.alternate_k != 0 && (it & 1);      // (dense_gemm_pair_kernel takes two at a time)
             }
         }
     } else {
@@ -230,7 +231,7 @@ dw_adapter_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         bool ok = true;
         int it = 0;
         PairWork w;
-        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, w); item += num_pairs, ++it) {
+        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, BLOCK_N, true, p.alternate_k != 0, w); item += num_pairs, ++it) {
             bool carry_r, carry_l;
             int n_blk;
             carries(w, carry_r, carry_l, n_blk);

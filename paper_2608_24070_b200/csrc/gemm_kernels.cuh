@@ -90,7 +90,7 @@ struct DenseGemmParams {
     int M, N, K;
     int width;                    // columns per tile: 64, 128, 192 or 256
     int stages;                   // pipeline stages that fit at that width
-    int alternate_k;              // CTA-pair kernel: 1: every other tile of a pair takes the reduction from its end (see raster_tile)
+    int alternate_k;              // CTA-pair kernel: 1: long reductions (see raster_tile)
     void* out;
     const uint8_t* mask;          // kEpiMasked: [M x N/8]
 };
@@ -633,21 +633,27 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 // Tile order for GEMMs whose two operands are both streamed once per tile (dW: dY^T X with the
 // tokens as reduction).  The ~74 tiles in flight should form a near-square patch of the output:
 // a patch of gm x gn tiles reads (gm + gn) operand panels, a gm x 1 strip reads gm + 1 for 1/gn
-// of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column, forwards in one group and
-// backwards in the next: the wave that straddles two groups then has the columns of both in common.
+// of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column.
+//
 // These GEMMs run at the power cap, where a byte from HBM costs what some 150 FLOP do, so what a wave can take from L2
-// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on; its last part is still
-// there when the next wave begins, and half of its panels are the next wave's too, so with a long reduction
-// every other tile of a pair takes the k-blocks from the end (alternate_k).  While the panels fit, that order
-// only lengthens the way between two uses of a k-block.  A model of L2 as 60 MB, least recently used first out, which gives the
-// 630 MB that 4096 x 4096 at 16384 tokens read before, has 540 MB now, and 1.45 instead of 1.77 GB for 4096 -> 11008.
-// us under sustained load, every group and tile forwards / now: 16384 tokens 4096 x 4096 427 / 421, 4096 -> 11008 1136 / 1117,
-// 11008 -> 4096 1117 / 1105, 8192 tokens 5120 -> 13824 878 / 862, 12000 tokens 2048 -> 5504 220 / 215.5; the order of the
-// groups alone, 4096 tokens 4096 -> 11008 273.9 / 273.8, 2048 tokens 5120 -> 13824 215.6 / 215.0.
+// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on.  With reductions that long
+// (alternate_k)
+//   - a pair works on two tiles at a time, kInterleaveBlocks k-blocks of one, then of the other (it has two accumulators
+//     anyway): the patch in flight is twice as large and reads a fifth fewer panels per tile, and each accumulator is
+//     drained while the other one's k-blocks run;
+//   - every other two tiles of a pair take the k-blocks from the end: the last part of a wave's panels is still there when
+//     the next wave begins, and half of its panels are the next wave's too;
+//   - every other group is walked backwards: the wave that straddles two groups has the columns of both in common.
+// While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us).
+// DRAM reads in MB, tiles one after the other and forwards / alternating ends only / now: 16384 tokens 4096 x 4096 631 / 534 / 437,
+// 4096 -> 11008 2059 / 1554 / 1288, 11008 -> 4096 1698 / 1452 / 1214.  us under sustained load: 433 / 423 / 411, 1155 / 1114 / 1089,
+// 1126 / 1105 / 1076, 8192 tokens 5120 -> 13824 890 / 855 / 843, 12000 tokens 2048 -> 5504 224 / 216 / 212.  (32 k-blocks at a time:
+// 411, 1102, 1091, 859, 211.)
 constexpr int kRasterGroupM = 8;
 constexpr int kAlternateFrom = 6144;          // shortest reduction that is taken from alternating ends
-// (`pos`: how many columns of tiles of the group come before the tile's)
-__host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, int& m, int& n, int& pos) {
+constexpr int kInterleaveBlocks = 16;
+// (`turn`: every other group backwards; `pos`: how many columns of tiles of the group come before the tile's)
+__host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, bool turn, int& m, int& n, int& pos) {
     const int group_size = kRasterGroupM * num_n;
     const int g = tile / group_size;
     const int first_m = g * kRasterGroupM;
@@ -655,7 +661,7 @@ __host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int nu
     const int local = tile - g * group_size;
     m = first_m + local % gm;
     pos = local / gm;
-    n = g & 1 ? num_n - 1 - pos : pos;
+    n = turn && (g & 1) ? num_n - 1 - pos : pos;
 }
 
 // Work items of the persistent CTA-pair GEMM.  Items are tiles in raster order; when the tiles
@@ -666,7 +672,7 @@ __host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int nu
 struct PairWork {
     int m_pair, n0, width, pos;
 };
-__device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, int num_n, int width, bool split_tail,
+__device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, int num_n, int width, bool split_tail, bool turn,
                                           PairWork& w) {
     const int num_tiles = num_m * num_n;
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
@@ -675,7 +681,7 @@ __device__ __forceinline__ bool pair_work(int item, int num_pairs, int num_m, in
     const bool halved = split && item >= full;
     const int tile = halved ? full + ((item - full) >> 1) : item;
     int n_blk;
-    raster_tile(tile, num_m, num_n, w.m_pair, n_blk, w.pos);
+    raster_tile(tile, num_m, num_n, turn, w.m_pair, n_blk, w.pos);
     w.width = halved ? width / 2 : width;
     w.n0 = n_blk * width + (halved && ((item - full) & 1) ? width / 2 : 0);
     return true;
@@ -723,6 +729,9 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int num_kb = (p.K + 63) / 64;
     // halving needs B loads of any width: the [K x N] operand is loaded in 64-column chunks
     const bool split_tail = B_MN && p.width == 256;
+    // A pair works on `group` items at a time, `chunk` k-blocks of one and then of the other (see raster_tile).
+    const bool turn = p.alternate_k != 0;
+    const int group = turn ? 2 : 1, chunk = turn ? kInterleaveBlocks : num_kb;
 
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -753,16 +762,15 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         if (elect_one()) {
             RingState ps;
             bool ok = true, backwards = p.alternate_k != 0;   // (what ran before, the input gradient, read the last tokens last)
-            PairWork w;
             const uint32_t leader_bar = mapa_shared(smem_u32(full_bar), 0);
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
-                 item += num_pairs) {
+            // k-blocks [kb0, kb1) of an item
+            auto load = [&](const PairWork& w, int kb0, int kb1) {
                 const int half_w = w.width / 2;                       // B rows (columns of D) this CTA stages
                 const int m0 = (w.m_pair * 2 + static_cast<int>(cta)) * kBlockM;
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
                 const bool two_chunks = Cfg::chunks(w.width) == 2;
                 const uint32_t stage_tx = 2 * (dense_a_bytes(A_MN, p.M) + Cfg::b_bytes(B_MN, w.width));
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sA = smem + ps.off;
                     uint8_t* sB = sA + Cfg::kABytes;
@@ -783,6 +791,14 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     }
                     ps.advance(stages, stage_bytes);
                 }
+            };
+            PairWork w0, w1;
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0); item += group * num_pairs) {
+                const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
+                for (int kb = 0; ok && kb < num_kb; kb += chunk) {
+                    load(w0, kb, min(kb + chunk, num_kb));
+                    if (two && ok) load(w1, kb, min(kb + chunk, num_kb));
+                }
                 backwards ^= p.alternate_k != 0;
             }
         }
@@ -791,19 +807,20 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             RingState ps;
             bool ok = true;
             int it = 0;
-            PairWork w;
             ClockProbe probe;
             if (pair_id == 0) probe.begin();
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
-                 item += num_pairs, ++it) {
+            // k-blocks [kb0, kb1) of a pair's item number `it`
+            auto multiply = [&](const PairWork& w, int it, int kb0, int kb1) {
                 const uint32_t idesc = make_idesc_bf16(2 * kBlockM, w.width, A_MN, B_MN, false);
                 const int acc = it & 1;
-                const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
-                if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-                tc_fence_after_sync();
+                if (kb0 == 0) {
+                    const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;
+                    if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, abort_flag)) { ok = false; return; }
+                    tc_fence_after_sync();
+                }
                 const uint32_t d_tmem = tmem_base + acc * Cfg::kMaxWidth;
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; break; }
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    if (!mbar_wait(&full_bar[ps.stage], ps.phase, abort_flag)) { ok = false; return; }
                     tc_fence_after_sync();
                     const uint32_t sA = smem_u32(smem + ps.off);
                     const uint32_t sB = sA + Cfg::kABytes;
@@ -817,7 +834,16 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     umma_commit_pair(&empty_bar[ps.stage], 3);
                     ps.advance(stages, stage_bytes);
                 }
-                if (ok) umma_commit_pair(&tfull_bar[acc], 3);
+                if (kb1 == num_kb) umma_commit_pair(&tfull_bar[acc], 3);
+            };
+            PairWork w0, w1;
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0);
+                 item += group * num_pairs, it += group) {
+                const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
+                for (int kb = 0; ok && kb < num_kb; kb += chunk) {
+                    multiply(w0, it, kb, min(kb + chunk, num_kb));
+                    if (two && ok) multiply(w1, it + 1, kb, min(kb + chunk, num_kb));
+                }
             }
             if (pair_id == 0) probe.end(kClockDense);
         }
@@ -828,7 +854,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         uint32_t buf = 0;
         const uint32_t my_buf = smem_u32(staging + (warp - 2) * 2 * Cfg::kStoreBytes);
         PairWork w;
-        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, w);
+        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w);
              item += num_pairs, ++it) {
             const int acc = it & 1;
             const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;

@@ -1,4 +1,4 @@
-"""Long reductions that every other tile of a CTA pair takes from the end: the weight gradient (masked, dense, with the adapter
+"""Long reductions that CTA pairs take from alternating ends, and of the weight gradient for two tiles in turn: the weight gradient (masked, dense, with the adapter
 gradients) from 6144 tokens on, the sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last k-blocks,
 last row tiles that are half empty, more than one raster group (the second one runs backwards), halved items of the last wave.
 
