@@ -636,21 +636,22 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 // of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column.
 //
 // These GEMMs run at the power cap, where a byte from HBM costs what some 150 FLOP do, so what a wave can take from L2
-// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on.  With reductions that long
-// (alternate_k)
+// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on.  With reductions of 8192 and
+// more (alternate_k)
 //   - a pair works on two tiles at a time, kInterleaveBlocks k-blocks of one, then of the other (it has two accumulators
 //     anyway): the patch in flight is twice as large and reads a fifth fewer panels per tile, and each accumulator is
 //     drained while the other one's k-blocks run;
 //   - every other two tiles of a pair take the k-blocks from the end: the last part of a wave's panels is still there when
 //     the next wave begins, and half of its panels are the next wave's too;
 //   - every other group is walked backwards: the wave that straddles two groups has the columns of both in common.
-// While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us).
+// While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us;
+// in between, 6200 tokens 4096 -> 11008 420 -> 418, 7000 tokens 7168 -> 1408 120.6 -> 121.9).
 // DRAM reads in MB, tiles one after the other and forwards / alternating ends only / now: 16384 tokens 4096 x 4096 631 / 534 / 437,
 // 4096 -> 11008 2059 / 1554 / 1288, 11008 -> 4096 1698 / 1452 / 1214.  us under sustained load: 433 / 423 / 411, 1155 / 1114 / 1089,
 // 1126 / 1105 / 1076, 8192 tokens 5120 -> 13824 890 / 855 / 843, 12000 tokens 2048 -> 5504 224 / 216 / 212.  (32 k-blocks at a time:
 // 411, 1102, 1091, 859, 211.)
 constexpr int kRasterGroupM = 8;
-constexpr int kAlternateFrom = 6144;          // shortest reduction that is taken from alternating ends
+constexpr int kAlternateFrom = 8192;          // shortest reduction that is taken from alternating ends
 constexpr int kInterleaveBlocks = 16;
 // (`turn`: every other group backwards; `pos`: how many columns of tiles of the group come before the tile's)
 __host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, bool turn, int& m, int& n, int& pos) {
@@ -770,12 +771,13 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
                 const bool two_chunks = Cfg::chunks(w.width) == 2;
                 const uint32_t stage_tx = 2 * (dense_a_bytes(A_MN, p.M) + Cfg::b_bytes(B_MN, w.width));
-                for (int kb = kb0; kb < kb1; ++kb) {
+                const int step = backwards ? -64 : 64;
+                int k0 = backwards ? (num_kb - 1 - kb0) * 64 : kb0 * 64;
+                for (int kb = kb0; kb < kb1; ++kb, k0 += step) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sA = smem + ps.off;
                     uint8_t* sB = sA + Cfg::kABytes;
                     const uint32_t bar = leader_bar + 8 * ps.stage;
-                    const int k0 = (backwards ? num_kb - 1 - kb : kb) * 64;
                     if (cta == 0) mbar_expect_tx(&full_bar[ps.stage], stage_tx);
                     if (A_MN) {
                         tma_load_2d_pair(sA, &tmA, bar, m0, k0);
@@ -1059,20 +1061,23 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                                      static_cast<int>(cta) * (token_tile_width(p.Ntok, next_n_blk * p.width, p.width) / 2)
                                : 0;
                 const bool next_backwards = backwards != (p.alternate_k != 0);
-                const auto k_column = [&](int kb, bool from_end) { return (from_end ? num_kb - 1 - kb : kb) * 128; };
-                for (int kb = 0; kb < total_kb; ++kb) {
+                const int dir = backwards ? -1 : 1, next_dir = next_backwards ? -1 : 1;
+                int kx = backwards ? num_kb - 1 : 0;                         // the k-block that step kb takes
+                const int skip = max(kPrefetchAhead - num_kb, 0);            // (of the next tile too little is left to prefetch these)
+                int next_x = (next_backwards ? num_kb - 1 - skip : skip) * 128;
+                for (int kb = 0; kb < total_kb; ++kb, kx += dir) {
                     if (kb < num_kb) {
                         const int pk = kb + kPrefetchAhead;
                         if (pk < num_kb) {
                             if (first) {
-                                const int x = k_column(pk, backwards);
+                                const int x = (kx + kPrefetchAhead * dir) * 128;
                                 tma_prefetch_l2_2d(&tmB, x, n_row0);
                                 tma_prefetch_l2_2d(&tmB, x + 64, n_row0);
                             }
                         } else if (next_first && pk - num_kb < num_kb) {
-                            const int x = k_column(pk - num_kb, next_backwards);
-                            tma_prefetch_l2_2d(&tmB, x, next_row0);
-                            tma_prefetch_l2_2d(&tmB, x + 64, next_row0);
+                            tma_prefetch_l2_2d(&tmB, next_x, next_row0);
+                            tma_prefetch_l2_2d(&tmB, next_x + 64, next_row0);
+                            next_x += 128 * next_dir;
                         }
                     }
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -1083,14 +1088,13 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         if (cta == 0)
                             mbar_expect_tx(&full_bar[ps.stage],
                                            2 * (2 * b_half + nsub * (Cfg::kABytes + Cfg::kEBytes)));
-                        const int x = k_column(kb, backwards);
-                        tma_load_2d_pair(sB, &tmB, bar, x, n_row0);
-                        tma_load_2d_pair(sB + b_half, &tmB, bar, x + 64, n_row0);
+                        tma_load_2d_pair(sB, &tmB, bar, kx * 128, n_row0);
+                        tma_load_2d_pair(sB + b_half, &tmB, bar, kx * 128 + 64, n_row0);
                         for (int s = 0; s < nsub; ++s) {
                             const int mb = 4 * mt + 2 * s + static_cast<int>(cta);
                             const int mb_e = mb < num_mb ? mb : num_mb - 1;
-                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, x / 2, mb * kBlockM, keep);
-                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + x / 128,
+                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, kx * 64, mb * kBlockM, keep);
+                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kx,
                                                   keep);
                         }
                     } else {

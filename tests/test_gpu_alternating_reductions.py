@@ -1,5 +1,5 @@
 """Long reductions that CTA pairs take from alternating ends, and of the weight gradient for two tiles in turn: the weight gradient (masked, dense, with the adapter
-gradients) from 6144 tokens on, the sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last k-blocks,
+gradients) from 8192 tokens on, the sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last k-blocks,
 last row tiles that are half empty, more than one raster group (the second one runs backwards), halved items of the last wave.
 
 The reference is the fp64 product on sampled rows; outputs are rounded once (1.7e-3 relative on Gaussian data, 5e-3 allowed, and
@@ -18,9 +18,9 @@ def _bits(mask):
 
 
 @pytest.mark.parametrize("b,d_in,d_out,r", [
-    (6143, 2304, 2560, 0),       # one token short of it
-    (6144, 2304, 2560, 0),       # 10 x 9 tiles: two raster groups, 16 tiles of the last wave halved
-    (6145, 2432, 2432, 16),      # a last k-block of one token, last row and column of tiles half empty
+    (8128, 2304, 2560, 0),       # a k-block short of it
+    (8192, 2304, 2560, 0),       # 10 x 9 tiles: two raster groups, 16 tiles of the last wave halved
+    (8193, 2432, 2432, 16),      # a last k-block of one token, last row and column of tiles half empty
     (8200, 3328, 3072, 64),      # 13 x 12 tiles, fused with the adapter gradients; 8 of them halved
 ])
 def test_weight_gradient(b, d_in, d_out, r):
