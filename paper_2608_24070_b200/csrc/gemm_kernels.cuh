@@ -90,7 +90,6 @@ struct DenseGemmParams {
     int M, N, K;
     int width;                    // columns per tile: 64, 128, 192 or 256
     int stages;                   // pipeline stages that fit at that width
-    int alternate_k;              // CTA-pair kernel: 1: long reductions (see raster_tile)
     void* out;
     const uint8_t* mask;          // kEpiMasked: [M x N/8]
 };
@@ -637,7 +636,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 //
 // These GEMMs run at the power cap, where a byte from HBM costs what some 150 FLOP do, so what a wave can take from L2
 // instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on.  With reductions of 8192 and
-// more (alternate_k)
+// more, and a full group of tile rows,
 //   - a pair works on two tiles at a time, kInterleaveBlocks k-blocks of one, then of the other (it has two accumulators
 //     anyway): the patch in flight is twice as large and reads a fifth fewer panels per tile, and each accumulator is
 //     drained while the other one's k-blocks run;
@@ -645,7 +644,8 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 //     the next wave begins, and half of its panels are the next wave's too;
 //   - every other group is walked backwards: the wave that straddles two groups has the columns of both in common.
 // While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us;
-// in between, 6200 tokens 4096 -> 11008 420 -> 418, 7000 tokens 7168 -> 1408 120.6 -> 121.9).
+// in between, 6200 tokens 4096 -> 11008 420 -> 418, 7000 tokens 7168 -> 1408 120.6 -> 121.9;
+// with 8500 tokens, but six tile rows, 147.4 -> 148.3).
 // DRAM reads in MB, tiles one after the other and forwards / alternating ends only / now: 16384 tokens 4096 x 4096 631 / 534 / 437,
 // 4096 -> 11008 2059 / 1554 / 1288, 11008 -> 4096 1698 / 1452 / 1214.  us under sustained load: 433 / 423 / 411, 1155 / 1114 / 1089,
 // 1126 / 1105 / 1076, 8192 tokens 5120 -> 13824 890 / 855 / 843, 12000 tokens 2048 -> 5504 224 / 216 / 212.  (32 k-blocks at a time:
@@ -705,7 +705,8 @@ struct DensePairCfg {
     }
 };
 
-template <bool A_MN, bool B_MN, int EPI>
+// LONG: two tiles in turn, from alternating ends (see raster_tile); a kernel of its own, whose loops do not cost the others.
+template <bool A_MN, bool B_MN, int EPI, bool LONG>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmO /* kEpiStore */, const DenseGemmParams p) {
@@ -730,9 +731,10 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int num_kb = (p.K + 63) / 64;
     // halving needs B loads of any width: the [K x N] operand is loaded in 64-column chunks
     const bool split_tail = B_MN && p.width == 256;
-    // A pair works on `group` items at a time, `chunk` k-blocks of one and then of the other (see raster_tile).
-    const bool turn = p.alternate_k != 0;
-    const int group = turn ? 2 : 1, chunk = turn ? kInterleaveBlocks : num_kb;
+    // A pair works on `group` items at a time, `chunk` k-blocks of one and then of the other.
+    constexpr bool turn = LONG;
+    constexpr int group = LONG ? 2 : 1;
+    const int chunk = LONG ? kInterleaveBlocks : num_kb;
 
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -762,7 +764,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     if (warp == 0) {
         if (elect_one()) {
             RingState ps;
-            bool ok = true, backwards = p.alternate_k != 0;   // (what ran before, the input gradient, read the last tokens last)
+            bool ok = true, backwards = LONG;   // (what ran before, the input gradient, read the last tokens last)
             const uint32_t leader_bar = mapa_shared(smem_u32(full_bar), 0);
             // k-blocks [kb0, kb1) of an item
             auto load = [&](const PairWork& w, int kb0, int kb1) {
@@ -771,8 +773,8 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
                 const bool two_chunks = Cfg::chunks(w.width) == 2;
                 const uint32_t stage_tx = 2 * (dense_a_bytes(A_MN, p.M) + Cfg::b_bytes(B_MN, w.width));
-                const int step = backwards ? -64 : 64;
-                int k0 = backwards ? (num_kb - 1 - kb0) * 64 : kb0 * 64;
+                const int step = LONG && backwards ? -64 : 64;
+                int k0 = LONG && backwards ? (num_kb - 1 - kb0) * 64 : kb0 * 64;
                 for (int kb = kb0; kb < kb1; ++kb, k0 += step) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sA = smem + ps.off;
@@ -797,11 +799,12 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             PairWork w0, w1;
             for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0); item += group * num_pairs) {
                 const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
-                for (int kb = 0; ok && kb < num_kb; kb += chunk) {
+                if (!LONG) load(w0, 0, num_kb);
+                for (int kb = 0; LONG && ok && kb < num_kb; kb += chunk) {
                     load(w0, kb, min(kb + chunk, num_kb));
                     if (two && ok) load(w1, kb, min(kb + chunk, num_kb));
                 }
-                backwards ^= p.alternate_k != 0;
+                backwards ^= LONG;
             }
         }
     } else if (warp == 1) {
@@ -842,7 +845,8 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0);
                  item += group * num_pairs, it += group) {
                 const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
-                for (int kb = 0; ok && kb < num_kb; kb += chunk) {
+                if (!LONG) multiply(w0, it, 0, num_kb);
+                for (int kb = 0; LONG && ok && kb < num_kb; kb += chunk) {
                     multiply(w0, it, kb, min(kb + chunk, num_kb));
                     if (two && ok) multiply(w1, it + 1, kb, min(kb + chunk, num_kb));
                 }

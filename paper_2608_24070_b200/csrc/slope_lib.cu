@@ -905,7 +905,9 @@ static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int n
 }
 
 // (256 x 256 tiles only: the fused weight and adapter gradients, which have no others, then add up the same sums in the same order)
-static int alternate_k(int K, int width) { return K >= kAlternateFrom && width == 256 ? 1 : 0; }
+static bool alternate_k(int M, int K, int width) {
+    return K >= kAlternateFrom && width == 256 && M > 2 * kBlockM * (kRasterGroupM - 1);
+}
 
 // D[M x N] on 128 x 128 tiles of single CTAs while they all run at once and the reduction is at most
 // 2048 long (measured on both sides of either line: dense_gemm_kernel), else on the CTA-pair kernel; a dense layer with
@@ -926,7 +928,7 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
     if (small) {
         constexpr int kStages = 6;
         using Cfg = DenseCfg<kStages>;
-        const DenseGemmParams p{M, N, K, width, kStages, 0, out, static_cast<const uint8_t*>(mask)};
+        const DenseGemmParams p{M, N, K, width, kStages, out, static_cast<const uint8_t*>(mask)};
         auto kern = dense_gemm_kernel<A_MN, B_MN, EPI, kStages>;
         if (!set_smem(kern, Cfg::kSmemBytes)) return SLOPE_ERR_CUDA;
         return launch_cluster_ex(kern, small_tiles, 1, kDenseThreads, Cfg::kSmemBytes, /*overlap_prologue=*/true, stream, tmA,
@@ -936,8 +938,8 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
     CUtensorMap tmO = tmA;
     if (EPI == kEpiStore && !make_tmap_out(&tmO, out, M, N, 32, 32)) return SLOPE_ERR_CUDA;
     const int stages = dense_stages(B_MN, EPI, width);
-    const DenseGemmParams p{M, N, K, width, stages, alternate_k(K, width), out, static_cast<const uint8_t*>(mask)};
-    auto kern = dense_gemm_pair_kernel<A_MN, B_MN, EPI>;
+    const DenseGemmParams p{M, N, K, width, stages, out, static_cast<const uint8_t*>(mask)};
+    auto kern = alternate_k(M, K, width) ? dense_gemm_pair_kernel<A_MN, B_MN, EPI, true> : dense_gemm_pair_kernel<A_MN, B_MN, EPI, false>;
     if (!set_smem(kern, 232448)) return SLOPE_ERR_CUDA;
     const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + width - 1) / width);
     const int pairs = std::min(tiles, max_pairs);
@@ -1261,7 +1263,7 @@ static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_c
     if (plan.splits_r > num_kb) plan.splits_r = num_kb;
     if (plan.splits_l > num_kb) plan.splits_l = num_kb;
     const int num_pairs = sm_count / 2, num_tiles = num_m * num_n;
-    const bool turn = alternate_k(b, choose_dense_width(d_out, d_in, b, true, true, num_pairs)) != 0;
+    const bool turn = alternate_k(d_out, b, choose_dense_width(d_out, d_in, b, true, true, num_pairs));
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
     if (rem > 0 && 2 * rem <= num_pairs) {
         for (int tile = full; tile < num_tiles; ++tile) {
@@ -1313,7 +1315,7 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     DwAdapterParams p = {};
     p.M = d_out; p.N = d_in; p.K = b; p.r = r;
     p.splits_r = plan.splits_r; p.splits_l = plan.splits_l;
-    p.alternate_k = alternate_k(b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
+    p.alternate_k = alternate_k(d_out, b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
     p.dWc = static_cast<uint16_t*>(dWc_vals);
     p.mask = static_cast<const uint8_t*>(mask1_bits);
     p.ws_r = static_cast<float*>(workspace);
