@@ -69,7 +69,6 @@ struct SparseGemmParams {
     int num_n;                    // tile kernels: token tiles
     int stages;                   // tile kernels: pipeline stages that fit at that width
     int group_m;                  // 512-row-tile kernel: row tiles per raster group (0: all in one group)
-    int alternate_k;              // 512-row-tile kernel: 1: every other tile of a pair takes the reduction from its end (see quad_tile)
     int pdl_mode;                 // 2: consumer of a fused pair of launches (see the few-token kernel)
     uint16_t* out;                // [Ntok x M]
 };
@@ -962,11 +961,10 @@ struct SparseQuadCfg {
 // then token blocks, then the next group.  The pairs that work on one token block side by side
 // share its activation tile; a group's share of the compressed weight is what has to stay in L2
 // while the token blocks sweep by.  `first` marks the tile that prefetches the block's
-// activations into L2 for its group.  Where even one group's weights are more than L2 keeps (long reductions), every other
-// tile of a pair takes the k-blocks from the end (alternate_k), so that a wave begins with the weights the last
-// one ended with.  us under sustained load, before / now: 16384 tokens 11008 -> 4096 632 / 617, 8192 tokens 13824 -> 5120 494 / 487,
-// 4000 tokens 11008 -> 4096 157.6 / 155.7.  (Where they fit, the order would only cost: 5120 -> 13824 in two groups 249 -> 306 MB
-// by a model of L2 as 60 MB, least recently used first out.)
+// activations into L2 for its group.  Every tile takes the k-blocks from the first to the last: a token's outputs then have
+// the same bits wherever in the batch it stands.  (Where a group's weights are more than L2 keeps, tiles that took them from
+// alternating ends found some 180 of 795 MB still there -- 16384 tokens 11008 -> 4096 631 -> 619 us, 8192 tokens 13824 -> 5120
+// 485 -> 476 -- but two equal tokens could then differ in the last bit.)
 __device__ __forceinline__ void quad_tile(int tile, int num_m, int num_n, int group_m, int& mt, int& n_blk,
                                           bool& first) {
     const int group_size = group_m * num_n;
@@ -1047,7 +1045,7 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const uint64_t keep = l2_policy_evict_last();
             PipeState ps;
             bool ok = true;
-            bool waited = false, backwards = false;
+            bool waited = false;
             for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
                 int mt, n_blk, next_mt, next_n_blk;
                 bool first, next_first = false;
@@ -1064,24 +1062,17 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     next_first ? next_n_blk * p.width +
                                      static_cast<int>(cta) * (token_tile_width(p.Ntok, next_n_blk * p.width, p.width) / 2)
                                : 0;
-                const bool next_backwards = backwards != (p.alternate_k != 0);
-                const int dir = backwards ? -1 : 1, next_dir = next_backwards ? -1 : 1;
-                int kx = backwards ? num_kb - 1 : 0;                         // the k-block that step kb takes
-                const int skip = max(kPrefetchAhead - num_kb, 0);            // (of the next tile too little is left to prefetch these)
-                int next_x = (next_backwards ? num_kb - 1 - skip : skip) * 128;
-                for (int kb = 0; kb < total_kb; ++kb, kx += dir) {
+                for (int kb = 0; kb < total_kb; ++kb) {
                     if (kb < num_kb) {
                         const int pk = kb + kPrefetchAhead;
                         if (pk < num_kb) {
                             if (first) {
-                                const int x = (kx + kPrefetchAhead * dir) * 128;
-                                tma_prefetch_l2_2d(&tmB, x, n_row0);
-                                tma_prefetch_l2_2d(&tmB, x + 64, n_row0);
+                                tma_prefetch_l2_2d(&tmB, pk * 128, n_row0);
+                                tma_prefetch_l2_2d(&tmB, pk * 128 + 64, n_row0);
                             }
                         } else if (next_first && pk - num_kb < num_kb) {
-                            tma_prefetch_l2_2d(&tmB, next_x, next_row0);
-                            tma_prefetch_l2_2d(&tmB, next_x + 64, next_row0);
-                            next_x += 128 * next_dir;
+                            tma_prefetch_l2_2d(&tmB, (pk - num_kb) * 128, next_row0);
+                            tma_prefetch_l2_2d(&tmB, (pk - num_kb) * 128 + 64, next_row0);
                         }
                     }
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -1092,13 +1083,13 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         if (cta == 0)
                             mbar_expect_tx(&full_bar[ps.stage],
                                            2 * (2 * b_half + nsub * (Cfg::kABytes + Cfg::kEBytes)));
-                        tma_load_2d_pair(sB, &tmB, bar, kx * 128, n_row0);
-                        tma_load_2d_pair(sB + b_half, &tmB, bar, kx * 128 + 64, n_row0);
+                        tma_load_2d_pair(sB, &tmB, bar, kb * 128, n_row0);
+                        tma_load_2d_pair(sB + b_half, &tmB, bar, kb * 128 + 64, n_row0);
                         for (int s = 0; s < nsub; ++s) {
                             const int mb = 4 * mt + 2 * s + static_cast<int>(cta);
                             const int mb_e = mb < num_mb ? mb : num_mb - 1;
-                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, kx * 64, mb * kBlockM, keep);
-                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kx,
+                            tma_load_2d_pair_hint(st + s * Cfg::kABytes, &tmA, bar, kb * 64, mb * kBlockM, keep);
+                            tma_load_2d_pair_hint(st + off_e + s * Cfg::kEBytes, &tmE, bar, 0, mb_e * num_kb + kb,
                                                   keep);
                         }
                     } else {
@@ -1123,7 +1114,6 @@ sparse_gemm_quad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     }
                     ps.advance(stages);
                 }
-                backwards = next_backwards;
             }
         }
     } else if (warp == 1) {

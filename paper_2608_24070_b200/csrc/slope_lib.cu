@@ -519,14 +519,11 @@ static slope_status_t launch_sparse_pair(const void* act, int ntok, const void* 
 // a group's weights resident.  Pick the g with the least estimated DRAM traffic
 // (measured at 16384 tokens: 4096 -> 11008 two groups +7 %, 5120 -> 13824 three groups +11 %,
 // square and long-reduction layers one group).
-// Where one group's weights do not fit, tiles alternate the end of the reduction that they begin with (see quad_tile), provided a
-// wave spans at least four token blocks, i.e. the next one takes up the same weights: of few tokens through a tall weight
-// each is read once or twice anyway (500 tokens 4096 -> 22016 55.6 us, alternating 55.8, 1000 tokens 5120 -> 13824 71.2 / 71.6).
-constexpr double kL2Keeps = 30e6;
 static int quad_group_m(int M, int K, int ntok, int width, int num_pairs) {
     const int num_m = (M / kBlockM + 3) / 4, num_n = (ntok + width - 1) / width;
     const double w_tile = 512.0 * K * 1.125, w_total = static_cast<double>(M) * K * 1.125;
     const double x_total = static_cast<double>(ntok) * K * 2.0;
+    constexpr double kL2Keeps = 30e6;
     int best_gm = num_m;
     double best = 1e300;
     for (int g = 1; g <= num_m; ++g) {
@@ -547,7 +544,6 @@ static slope_status_t launch_sparse_quad(const void* act, int ntok, const void* 
     if (!sparse_tile_args(a, act, ntok, vals, meta, M, K, act2, fac2, r, a2_mn, out, width, stages, pdl_mode))
         return SLOPE_ERR_CUDA;
     a.p.group_m = quad_group_m(M, K, ntok, width, max_pairs);
-    a.p.alternate_k = a.p.group_m * 512.0 * K * 1.125 > kL2Keeps && 4 * a.p.group_m <= max_pairs;
     if (!set_smem(sparse_gemm_quad_kernel, kMaxTileSmem)) return SLOPE_ERR_CUDA;
     const int tiles = ((M / kBlockM + 3) / 4) * ((ntok + width - 1) / width);
     const int pairs = std::min(tiles, max_pairs);

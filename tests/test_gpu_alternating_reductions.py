@@ -1,6 +1,6 @@
-"""Long reductions that CTA pairs take from alternating ends, and of the weight gradient for two tiles in turn: the weight gradient (masked, dense, with the adapter
-gradients) from 8192 tokens on, the sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last k-blocks,
-last row tiles that are half empty, more than one raster group (the second one runs backwards), halved items of the last wave.
+"""Long reductions.  The weight gradient (masked, dense, with the adapter gradients) from 8192 tokens on: CTA pairs work on two tiles in
+turn and take them from alternating ends.  The sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last
+k-blocks, last row tiles that are half empty, more than one raster group (the second one runs backwards), halved items of the last wave.
 
 The reference is the fp64 product on sampled rows; outputs are rounded once (1.7e-3 relative on Gaussian data, 5e-3 allowed, and
 parity_error's bound per element), dL and dR from bf16 T and dT."""

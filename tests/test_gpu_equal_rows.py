@@ -1,0 +1,50 @@
+"""Equal token rows of one call give equal bits, wherever in the batch they stand: every tile of a product takes the sums of a row in the
+same order.  Long reductions on many token blocks (several tiles per CTA pair), ragged last tiles, where a kernel could gain from
+taking some of its tiles from another end."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+PERIOD = 61              # no divisor of a tile's rows: each of the distinct rows comes up at every position of a tile
+
+
+def _rows(b, d, seed):
+    import torch
+
+    gen = torch.Generator("cuda").manual_seed(seed)
+    return torch.randn((PERIOD, d), generator=gen, device="cuda", dtype=torch.bfloat16).repeat(-(-b // PERIOD), 1)[:b].contiguous()
+
+
+def _assert_equal_rows(out):
+    import torch
+
+    bits = out.view(torch.int16)
+    assert torch.isfinite(out).all()
+    assert torch.equal(bits[PERIOD:], bits[:-PERIOD])
+
+
+@pytest.mark.parametrize("b,k,m,r", [
+    (5001, 13824, 2560, 64),     # 5 row tiles of 512 in one raster group, a CTA pair works on two token blocks
+    (4500, 11008, 3968, 0),      # 31 row blocks, 168 tiles
+    (9000, 4096, 4096, 16),      # weights that stay in L2
+    (700, 11008, 2048, 0),       # 256-row tiles
+])
+def test_sparse_products(b, k, m, r):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(91)
+    new = lambda *shape, sigma: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16).mul_(sigma)
+    vals, meta, _ = B.alloc_compressed(m, k)
+    B.slope_prune_24(new(m, k, sigma=0.02), vals, meta, None)
+    act = _rows(b, k, 92)
+    low, R, L = (_rows(b, r, 93), new(r, m, sigma=0.1), new(m, r, sigma=0.1)) if r else (None, None, None)
+    Y, dX = (torch.full((b, m), float("nan"), device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    B.slope_linear_fwd(act, vals, meta, m, Y, low, R)
+    B.slope_linear_bwd_dx(act, vals, meta, m, dX, low, L)
+    assert B.slope_poll_status() == 0
+    _assert_equal_rows(Y)
+    _assert_equal_rows(dX)
+    if not r:
+        assert torch.equal(Y, dX)      # without adapters the two calls are one product
