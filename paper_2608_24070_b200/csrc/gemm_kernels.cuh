@@ -639,8 +639,9 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 //   - a pair works on two tiles at a time, kInterleaveBlocks k-blocks of one, then of the other (it has two accumulators
 //     anyway): the patch in flight is twice as large and reads a fifth fewer panels per tile, and each accumulator is
 //     drained while the other one's k-blocks run;
-//   - every other two tiles of a pair take the k-blocks from the end: the last part of a wave's panels is still there when
-//     the next wave begins, and half of its panels are the next wave's too;
+//   - every other two tiles of a pair take the k-blocks from the end, where the reduction runs over tokens: the last part of a
+//     wave's panels is still there when the next wave begins, and half of its panels are the next wave's too.  (Forward and input
+//     gradient of a dense layer gain less than 1 % from it, and a token's outputs would have other bits elsewhere in the batch);
 //   - every other group is walked backwards: the wave that straddles two groups has the columns of both in common.
 // While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us;
 // in between, 6200 tokens 4096 -> 11008 420 -> 418, 7000 tokens 7168 -> 1408 120.6 -> 121.9;
@@ -650,7 +651,7 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 // 1126 / 1105 / 1076, 8192 tokens 5120 -> 13824 890 / 855 / 843, 12000 tokens 2048 -> 5504 224 / 216 / 212.  (32 k-blocks at a time:
 // 411, 1102, 1091, 859, 211.)
 constexpr int kRasterGroupM = 8;
-constexpr int kAlternateFrom = 8192;          // shortest reduction that is taken from alternating ends
+constexpr int kLongFrom = 8192;               // shortest such reduction
 constexpr int kInterleaveBlocks = 16;
 // (`turn`: every other group backwards; `pos`: how many columns of tiles of the group come before the tile's)
 __host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, bool turn, int& m, int& n, int& pos) {
@@ -704,7 +705,8 @@ struct DensePairCfg {
     }
 };
 
-// LONG: two tiles in turn, from alternating ends (see raster_tile); a kernel of its own, whose loops do not cost the others.
+// LONG: two tiles in turn, in the weight gradient from alternating ends (see raster_tile); a kernel of its own, whose loops do not
+// cost the others.
 template <bool A_MN, bool B_MN, int EPI, bool LONG>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -730,10 +732,8 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int num_kb = (p.K + 63) / 64;
     // halving needs B loads of any width: the [K x N] operand is loaded in 64-column chunks
     const bool split_tail = B_MN && p.width == 256;
-    // A pair works on `group` items at a time, `chunk` k-blocks of one and then of the other.
-    constexpr bool turn = LONG;
-    constexpr int group = LONG ? 2 : 1;
-    const int chunk = LONG ? kInterleaveBlocks : num_kb;
+    constexpr int at_a_time = LONG ? 2 : 1;       // items that a pair works on in turn
+    constexpr bool kAlternate = LONG && A_MN;     // every other two from the end of the reduction
 
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -763,7 +763,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     if (warp == 0) {
         if (elect_one()) {
             RingState ps;
-            bool ok = true, backwards = LONG;   // (what ran before, the input gradient, read the last tokens last)
+            bool ok = true, backwards = kAlternate;   // (what ran before, the input gradient, read the last tokens last)
             const uint32_t leader_bar = mapa_shared(smem_u32(full_bar), 0);
             // k-blocks [kb0, kb1) of an item
             auto load = [&](const PairWork& w, int kb0, int kb1) {
@@ -772,8 +772,8 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 const int n0 = w.n0 + static_cast<int>(cta) * half_w;
                 const bool two_chunks = Cfg::chunks(w.width) == 2;
                 const uint32_t stage_tx = 2 * (dense_a_bytes(A_MN, p.M) + Cfg::b_bytes(B_MN, w.width));
-                const int step = LONG && backwards ? -64 : 64;
-                int k0 = LONG && backwards ? (num_kb - 1 - kb0) * 64 : kb0 * 64;
+                const int step = kAlternate && backwards ? -64 : 64;
+                int k0 = kAlternate && backwards ? (num_kb - 1 - kb0) * 64 : kb0 * 64;
                 for (int kb = kb0; kb < kb1; ++kb, k0 += step) {
                     if (!mbar_wait(&empty_bar[ps.stage], ps.phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t* sA = smem + ps.off;
@@ -795,15 +795,20 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     ps.advance(stages, stage_bytes);
                 }
             };
-            PairWork w0, w1;
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0); item += group * num_pairs) {
-                const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
-                if (!LONG) load(w0, 0, num_kb);
-                for (int kb = 0; LONG && ok && kb < num_kb; kb += chunk) {
-                    load(w0, kb, min(kb + chunk, num_kb));
-                    if (two && ok) load(w1, kb, min(kb + chunk, num_kb));
+            PairWork w0;
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, LONG, w0);
+                 item += at_a_time * num_pairs) {
+                if constexpr (LONG) {
+                    PairWork w1;
+                    const bool two = pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, LONG, w1);
+                    for (int kb = 0; ok && kb < num_kb; kb += kInterleaveBlocks) {
+                        load(w0, kb, min(kb + kInterleaveBlocks, num_kb));
+                        if (two && ok) load(w1, kb, min(kb + kInterleaveBlocks, num_kb));
+                    }
+                    backwards ^= kAlternate;
+                } else {
+                    load(w0, 0, num_kb);
                 }
-                backwards ^= LONG;
             }
         }
     } else if (warp == 1) {
@@ -840,14 +845,18 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 }
                 if (kb1 == num_kb) umma_commit_pair(&tfull_bar[acc], 3);
             };
-            PairWork w0, w1;
-            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w0);
-                 item += group * num_pairs, it += group) {
-                const bool two = group == 2 && pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, turn, w1);
-                if (!LONG) multiply(w0, it, 0, num_kb);
-                for (int kb = 0; LONG && ok && kb < num_kb; kb += chunk) {
-                    multiply(w0, it, kb, min(kb + chunk, num_kb));
-                    if (two && ok) multiply(w1, it + 1, kb, min(kb + chunk, num_kb));
+            PairWork w0;
+            for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, LONG, w0);
+                 item += at_a_time * num_pairs, it += at_a_time) {
+                if constexpr (LONG) {
+                    PairWork w1;
+                    const bool two = pair_work(item + num_pairs, num_pairs, num_m, num_n, p.width, split_tail, LONG, w1);
+                    for (int kb = 0; ok && kb < num_kb; kb += kInterleaveBlocks) {
+                        multiply(w0, it, kb, min(kb + kInterleaveBlocks, num_kb));
+                        if (two && ok) multiply(w1, it + 1, kb, min(kb + kInterleaveBlocks, num_kb));
+                    }
+                } else {
+                    multiply(w0, it, 0, num_kb);
                 }
             }
             if (pair_id == 0) probe.end(kClockDense);
@@ -859,7 +868,7 @@ dense_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         uint32_t buf = 0;
         const uint32_t my_buf = smem_u32(staging + (warp - 2) * 2 * Cfg::kStoreBytes);
         PairWork w;
-        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, turn, w);
+        for (int item = pair_id; ok && pair_work(item, num_pairs, num_m, num_n, p.width, split_tail, LONG, w);
              item += num_pairs, ++it) {
             const int acc = it & 1;
             const uint32_t acc_phase = static_cast<uint32_t>(it >> 1) & 1u;

@@ -900,9 +900,10 @@ static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int n
     return best;
 }
 
-// (256 x 256 tiles only: the fused weight and adapter gradients, which have no others, then add up the same sums in the same order)
-static bool alternate_k(int M, int K, int width) {
-    return K >= kAlternateFrom && width == 256 && M > 2 * kBlockM * (kRasterGroupM - 1);
+// Whether a launch takes two tiles in turn, the weight gradient from alternating ends (see raster_tile; 256 x 256 tiles only: the fused
+// weight and adapter gradients, which have no others, then add up the same sums in the same order).
+static bool long_reduction(int M, int K, int width) {
+    return K >= kLongFrom && width == 256 && M > 2 * kBlockM * (kRasterGroupM - 1);
 }
 
 // D[M x N] on 128 x 128 tiles of single CTAs while they all run at once and the reduction is at most
@@ -935,7 +936,7 @@ static slope_status_t launch_dense(const void* A, const void* B, int M, int N, i
     if (EPI == kEpiStore && !make_tmap_out(&tmO, out, M, N, 32, 32)) return SLOPE_ERR_CUDA;
     const int stages = dense_stages(B_MN, EPI, width);
     const DenseGemmParams p{M, N, K, width, stages, out, static_cast<const uint8_t*>(mask)};
-    auto kern = alternate_k(M, K, width) ? dense_gemm_pair_kernel<A_MN, B_MN, EPI, true> : dense_gemm_pair_kernel<A_MN, B_MN, EPI, false>;
+    auto kern = long_reduction(M, K, width) ? dense_gemm_pair_kernel<A_MN, B_MN, EPI, true> : dense_gemm_pair_kernel<A_MN, B_MN, EPI, false>;
     if (!set_smem(kern, 232448)) return SLOPE_ERR_CUDA;
     const int tiles = ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + width - 1) / width);
     const int pairs = std::min(tiles, max_pairs);
@@ -1259,7 +1260,7 @@ static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_c
     if (plan.splits_r > num_kb) plan.splits_r = num_kb;
     if (plan.splits_l > num_kb) plan.splits_l = num_kb;
     const int num_pairs = sm_count / 2, num_tiles = num_m * num_n;
-    const bool turn = alternate_k(d_out, b, choose_dense_width(d_out, d_in, b, true, true, num_pairs));
+    const bool turn = long_reduction(d_out, b, choose_dense_width(d_out, d_in, b, true, true, num_pairs));
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
     if (rem > 0 && 2 * rem <= num_pairs) {
         for (int tile = full; tile < num_tiles; ++tile) {
@@ -1311,7 +1312,7 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     DwAdapterParams p = {};
     p.M = d_out; p.N = d_in; p.K = b; p.r = r;
     p.splits_r = plan.splits_r; p.splits_l = plan.splits_l;
-    p.alternate_k = alternate_k(d_out, b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
+    p.alternate_k = long_reduction(d_out, b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
     p.dWc = static_cast<uint16_t*>(dWc_vals);
     p.mask = static_cast<const uint8_t*>(mask1_bits);
     p.ws_r = static_cast<float*>(workspace);

@@ -48,3 +48,28 @@ def test_sparse_products(b, k, m, r):
     _assert_equal_rows(dX)
     if not r:
         assert torch.equal(Y, dX)      # without adapters the two calls are one product
+
+
+@pytest.mark.parametrize("b,k,m,backward", [
+    (4100, 8320, 4096, False),   # 17 x 16 tiles of 256 x 256, two in turn; a last row tile of four tokens
+    (2500, 8192, 5120, True),    # 10 x 20, the second raster group backwards
+    (1793, 8192, 4992, True),    # eight rows of tiles, the last one with one token; the last wave's tiles halved
+    (1792, 8192, 4992, True),    # seven: one tile after the other
+    (4100, 4096, 4096, False),
+])
+def test_dense_products(b, k, m, backward):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+    from helpers import REL_TOL, parity_error, to_f64
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(94)
+    W = torch.randn((k, m) if backward else (m, k), generator=gen, device="cuda", dtype=torch.bfloat16).mul_(0.02)
+    act = _rows(b, k, 95)
+    out = torch.full((b + 1, m), float("nan"), device="cuda", dtype=torch.bfloat16)
+    (B.slope_dense_linear_bwd_dx if backward else B.slope_dense_linear_fwd)(act, W, out[:b])
+    assert B.slope_poll_status() == 0
+    assert torch.isnan(out[b]).all()
+    _assert_equal_rows(out[:b])
+    g = lambda t: to_f64(B.bits_from_bf16(t))
+    assert parity_error(g(out[:PERIOD]), g(act[:PERIOD]) @ (g(W) if backward else g(W).T)) <= REL_TOL
