@@ -634,8 +634,8 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 // of the work.  Tiles are numbered in groups of kRasterGroupM tile rows, column by column.
 //
 // These GEMMs run at the power cap, where a byte from HBM costs what some 150 FLOP do, so what a wave can take from L2
-// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 6000 tokens on.  With reductions of 8192 and
-// more, and a full group of tile rows,
+// instead is time.  A wave's panels (17 x 256 x K) are more than L2 keeps from some 5500 steps of the reduction on.  From there,
+// and with at least seven tile rows,
 //   - a pair works on two tiles at a time, kInterleaveBlocks k-blocks of one, then of the other (it has two accumulators
 //     anyway): the patch in flight is twice as large and reads a fifth fewer panels per tile, and each accumulator is
 //     drained while the other one's k-blocks run;
@@ -643,15 +643,18 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 //     wave's panels is still there when the next wave begins, and half of its panels are the next wave's too.  (Forward and input
 //     gradient of a dense layer gain less than 1 % from it, and a token's outputs would have other bits elsewhere in the batch);
 //   - every other group is walked backwards: the wave that straddles two groups has the columns of both in common.
-// While the panels fit, all that only lengthens the way between two uses of a k-block (4096 tokens 4096 x 4096 103.2 -> 103.5 us;
-// in between, 6200 tokens 4096 -> 11008 420 -> 418, 7000 tokens 7168 -> 1408 120.6 -> 121.9;
-// with 8500 tokens, but six tile rows, 147.4 -> 148.3).
-// DRAM reads in MB, tiles one after the other and forwards / alternating ends only / now: 16384 tokens 4096 x 4096 631 / 534 / 437,
-// 4096 -> 11008 2059 / 1554 / 1288, 11008 -> 4096 1698 / 1452 / 1214.  us under sustained load: 433 / 423 / 411, 1155 / 1114 / 1089,
-// 1126 / 1105 / 1076, 8192 tokens 5120 -> 13824 890 / 855 / 843, 12000 tokens 2048 -> 5504 224 / 216 / 212.  (32 k-blocks at a time:
-// 411, 1102, 1091, 859, 211.)
+// us under sustained load, one tile after the other / so, medians that repeat within 1 %:
+//   weight gradient, 16384 tokens 4096 x 4096 425 / 406, 4096 -> 11008 1107 / 1076, 11008 -> 4096 1084 / 1055, 8192 tokens
+//     5120 -> 13824 858 / 831; input gradient 4000 tokens 4096 <- 11008 287 / 277, forward 16384 tokens 11008 -> 4096 1130 / 1073;
+//   length, weight gradients 4096 x 4096, 4096 -> 11008, 2560 -> 7680, 11008 -> 4096: 4608 tokens 115.9 / 115.2, 303.2 / 301.6,
+//     138.0 / 138.1, 304.1 / 304.8; 5632 142.1 / 140.2, 375.2 / 367.5, 170.7 / 168.4, 372.0 / 369.4; 7000 181.2 / 177.0, 485.8 / 468.0,
+//     215.5 / 209.7; forward 8192 tokens 5120 -> 4096 258.7 / 258.7, 5632 282.1 / 280.1, 7168 370.9 / 361.9;
+//   tile rows, 16384 tokens 8192 -> 1024, 1536, 1792: 217.2 / 216.5, 323.6 / 318.7, 373.0 / 363.4; but with six 12000 tokens
+//     7168 -> 1408 205.2 / 205.4, 8500 145.2 / 146.2, forward 1536 tokens 11008 -> 4096 115.2 / 116.0, 1792 138.5 / 136.7.
+// DRAM reads in MB, one tile after the other / alternating ends only / so: 16384 tokens 4096 x 4096 631 / 534 / 436, 4096 -> 11008
+// 2059 / 1554 / 1294, 11008 -> 4096 1698 / 1452 / 1231.  (32 k-blocks at a time instead of 16 took 1 to 2 % longer where rows are many.)
 constexpr int kRasterGroupM = 8;
-constexpr int kLongFrom = 8192;               // shortest such reduction
+constexpr int kLongFrom = 5632, kLongTileRows = 7;
 constexpr int kInterleaveBlocks = 16;
 // (`turn`: every other group backwards; `pos`: how many columns of tiles of the group come before the tile's)
 __host__ __device__ __forceinline__ void raster_tile(int tile, int num_m, int num_n, bool turn, int& m, int& n, int& pos) {

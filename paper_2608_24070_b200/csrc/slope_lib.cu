@@ -903,7 +903,7 @@ static int choose_dense_width(int M, int N, int K, bool b_mn, bool masked, int n
 // Whether a launch takes two tiles in turn, the weight gradient from alternating ends (see raster_tile; 256 x 256 tiles only: the fused
 // weight and adapter gradients, which have no others, then add up the same sums in the same order).
 static bool long_reduction(int M, int K, int width) {
-    return K >= kLongFrom && width == 256 && M > 2 * kBlockM * (kRasterGroupM - 1);
+    return K >= kLongFrom && width == 256 && M > 2 * kBlockM * (kLongTileRows - 1);
 }
 
 // D[M x N] on 128 x 128 tiles of single CTAs while they all run at once and the reduction is at most

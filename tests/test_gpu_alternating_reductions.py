@@ -1,4 +1,4 @@
-"""Long reductions.  The weight gradient (masked, dense, with the adapter gradients) from 8192 tokens on: CTA pairs work on two tiles in
+"""Long reductions.  The weight gradient (masked, dense, with the adapter gradients) from 5632 tokens on: CTA pairs work on two tiles in
 turn and take them from alternating ends.  The sparse 512-row tiles where a raster group's weights are more than L2 keeps.  Ragged last
 k-blocks, last row tiles that are half empty, more than one raster group (the second one runs backwards), halved items of the last wave.
 
@@ -18,7 +18,10 @@ def _bits(mask):
 
 
 @pytest.mark.parametrize("b,d_in,d_out,r", [
-    (8128, 2304, 2560, 0),       # a k-block short of it
+    (5631, 2304, 2560, 0),       # a token short of it
+    (5632, 2304, 2560, 0),
+    (8128, 2304, 2560, 0),
+    (6000, 4352, 1664, 0),       # seven tile rows, the last one half empty
     (8192, 2304, 2560, 0),       # 10 x 9 tiles: two raster groups, 16 tiles of the last wave halved
     (8193, 2432, 2432, 16),      # a last k-block of one token, last row and column of tiles half empty
     (8200, 3328, 3072, 64),      # 13 x 12 tiles, fused with the adapter gradients; 8 of them halved

@@ -54,8 +54,10 @@ def test_sparse_products(b, k, m, r):
     (4100, 8320, 4096, False),   # 17 x 16 tiles of 256 x 256, two in turn; a last row tile of four tokens
     (2500, 8192, 5120, True),    # 10 x 20, the second raster group backwards
     (1793, 8192, 4992, True),    # eight rows of tiles, the last one with one token; the last wave's tiles halved
-    (1792, 8192, 4992, True),    # seven: one tile after the other
-    (4100, 4096, 4096, False),
+    (1792, 8192, 4992, True),    # seven
+    (1536, 8192, 5120, True),    # six: one tile after the other
+    (4100, 5632, 4096, False),   # the shortest reduction
+    (4100, 5504, 4096, False),   # shorter: one tile after the other
 ])
 def test_dense_products(b, k, m, backward):
     import torch
