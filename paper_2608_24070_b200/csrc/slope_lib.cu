@@ -324,10 +324,13 @@ struct AdapterGrid {
     bool deep;
     double stages, busy;                   // ring depth; share of the SMs that are at work at a time
 };
+// SMs that clusters of `size` fill (33 of 4 and 15 of 8 fit on 148).
+static int cluster_sms(int size, int sm_count) {
+    return size == 8 ? sm_count * 120 / 148 : size == 4 ? sm_count * 132 / 148 : sm_count;
+}
 static AdapterGrid adapter_grid(const AdapterShape& q, int n_tile, int splits, int sm_count) {
     const int col_tiles = (q.N + n_tile - 1) / n_tile, ctas = q.row_tiles * col_tiles * splits;
-    // clusters of 4 and 8 do not fill every SM (33 and 15 of them fit on 148 SMs)
-    const int sms = splits == 8 ? sm_count * 120 / 148 : splits == 4 ? sm_count * 132 / 148 : sm_count;
+    const int sms = cluster_sms(splits, sm_count);
     const bool deep = n_tile == 256 || ctas <= sms;
     const int slots = (deep ? 1 : 2) * sms, waves = (ctas + slots - 1) / slots, num_kb = (q.K + 63) / 64;
     const double stages = n_tile == 64 ? (deep ? 9 : 4) : n_tile == 128 ? (deep ? 7 : 3) : 4;
@@ -832,9 +835,13 @@ static FwdAdapterPlan fwd_adapter_plan(int b, int d_out, int d_in, int r, const 
 
 // What the T launch in front of a few-token forward asks L2 for: the first k-blocks of weights of at least 40 MB that are tall enough
 // to occupy the SMs without a split, at up to 16 tokens.  Launching the further CTAs costs the pair up to 0.5 us, which a
-// shorter or a split stream does not give back.  us without / with it, r = 64, 8 tokens: 4096 -> 22016 21.2 / 19.5, 5120 -> 35840
-// 34.25 / 33.5; on the other side of the line 4096 -> 12288 13.93 / 14.04, 11008 -> 4096 13.53 / 13.55, and the four linears
-// of a block of width 2048 / 6400 32.3 / 33.1, 1280 / 4096 27.4 / 29.5; of 4096 / 11008 56.9 / 55.3, of 3584 / 9600 49.7 / 48.5.
+// shorter or a split stream does not give back.  us without / with it, r = 64, 8 tokens: 4096 -> 22016 21.1 / 19.7, 5120 -> 35840
+// 34.45 / 33.6, 4096 -> 16384 16.1 / 15.55, 2304 -> 16384 11.52 / 11.52; on the other side of the line 4096 -> 12288 13.93 / 14.04,
+// 11008 -> 4096 13.53 / 13.55, and the four linears of a block of width 2048 / 6400 32.3 / 33.1, 1280 / 4096 27.4 / 29.5.
+// The bytes it asks for hold up T itself.  A T of few SMs is in nobody's way; a T of wide ranks (32 SMs at r = 256) is when the forward has
+// more CTAs than find room beside it: at r = 256 with 1.5 CTAs per SM and fewer 1 token 3584 -> 19200 19.0 / 17.7, 4096 -> 24576
+// 23.7 / 22.5, 8 tokens 5120 -> 27648 29.6 / 29.1, with more of them 16 tokens 5120 -> 32768 35.1 / 35.2, 1 token 5120 -> 40960
+// 47.6 / 48.6 (r = 64: 47.0 / 44.75), the four linears of a block of width 5120 / 17920 101.9 / 102.2 (r = 64: 82.7 / 81.5).
 constexpr double kPairPrefetchFrom = 40e6;
 constexpr int kPairPrefetchRows = 16384;
 static WeightPrefetch pair_prefetch(const FwdAdapterPlan& plan, int ntok, const void* vals, const void* meta, int M, int K, int r,
@@ -844,8 +851,9 @@ static WeightPrefetch pair_prefetch(const FwdAdapterPlan& plan, int ntok, const 
         return skinny_split_count<n(), a(), b()>(ntok, M, K, r, info, 2);
     });
     if (splits == 0) return WeightPrefetch{};
-    // (clusters of 8 fill 120 of 148 SMs)
-    const int slices = M / kBlockM * splits, free_sms = info.sm_count * 120 / 148 - adapter_sms(plan.T, ntok, r, info.sm_count);
+    const int slices = M / kBlockM * splits, T_sms = adapter_sms(plan.T, ntok, r, info.sm_count);
+    if (8 * T_sms > info.sm_count && 2 * slices > 3 * info.sm_count) return WeightPrefetch{};
+    const int free_sms = cluster_sms(plan.T.splits, info.sm_count) - T_sms;
     const int blocks = std::max(std::min(slices, free_sms), 0) / plan.T.splits * plan.T.splits;
     return WeightPrefetch{static_cast<const uint8_t*>(vals), static_cast<const uint8_t*>(meta), K, splits, slices, blocks};
 }

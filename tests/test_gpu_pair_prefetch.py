@@ -1,5 +1,5 @@
 """Few tokens through tall weights with adapters: the T launch has further CTAs that ask L2 for the forward's weights.  Sizes on
-either side of the line (16384 rows, 40 MB of compressed weights), one and two CTAs per SM in the forward, T in one and in several
+either side of the line (16384 rows, 40 MB of compressed weights; at wide ranks no more than 1.5 slabs per SM), one and two CTAs per SM in the forward, T in one and in several
 column tiles, repeated calls behind the kernel that writes the activations.
 
 The reference is the fp64 product with T as written, on sampled features; outputs are rounded once (1.7e-3 relative on
@@ -21,6 +21,9 @@ pytestmark = pytest.mark.gpu
     (8, 2560, 16512, 256),       # 129 slabs, widest rank
     (3, 4096, 22016, 64),        # 172 slabs, two CTAs per SM
     (17, 2304, 16384, 16),       # a token more than the line
+    (5, 640, 65536, 32),         # T in clusters of four
+    (2, 2048, 28160, 256),       # widest rank, 220 slabs: as many as are served beside it
+    (2, 1536, 29696, 256),       # 232 slabs: more
 ])
 def test_forward_with_adapter(b, d_in, d_out, r):
     import torch
