@@ -1251,7 +1251,7 @@ namespace slope {
 constexpr int kCarrySplits = 8;            // partial sums per row block of dR^T / dL in the fused launch
 
 struct DwAdapterPlan {
-    bool fused;
+    bool fused, alternate_k;      // alternate_k: tiles in the order of the weight gradient alone
     int splits_r, splits_l;
 };
 
@@ -1259,8 +1259,8 @@ struct DwAdapterPlan {
 // provided no tile that carries adapter work lies among the halved items of the last wave (those run
 // at half width, too narrow to serve as the A operand of the dL product).  Everything else takes the
 // separate launches.
-static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_count) {
-    DwAdapterPlan plan{false, 1, 1};
+static DwAdapterPlan plan_dw_adapter(int b, int d_out, int d_in, int r, int sm_count) {
+    DwAdapterPlan plan{false, false, 1, 1};
     const int num_m = (d_out + 255) / 256, num_n = (d_in + 255) / 256, num_kb = (b + 63) / 64;
     if (r > 128 || num_m * num_n * 2 <= sm_count) return plan;
     plan.splits_r = num_n < kCarrySplits ? num_n : kCarrySplits;
@@ -1268,17 +1268,21 @@ static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_c
     if (plan.splits_r > num_kb) plan.splits_r = num_kb;
     if (plan.splits_l > num_kb) plan.splits_l = num_kb;
     const int num_pairs = sm_count / 2, num_tiles = num_m * num_n;
-    const bool turn = long_reduction(d_out, b, choose_dense_width(d_out, d_in, b, true, true, num_pairs));
+    plan.alternate_k = long_reduction(d_out, b, choose_dense_width(d_out, d_in, b, true, true, num_pairs));
     const int full = (num_tiles / num_pairs) * num_pairs, rem = num_tiles - full;
     if (rem > 0 && 2 * rem <= num_pairs) {
         for (int tile = full; tile < num_tiles; ++tile) {
             int m, n, pos;
-            raster_tile(tile, num_m, num_n, turn, m, n, pos);
+            raster_tile(tile, num_m, num_n, plan.alternate_k, m, n, pos);
             if (m < plan.splits_l || pos < plan.splits_r) return plan;
         }
     }
     plan.fused = true;
     return plan;
+}
+static DwAdapterPlan dw_adapter_plan(int b, int d_out, int d_in, int r, int sm_count) {
+    thread_local SizeMemo<DwAdapterPlan> memo;
+    return memo.get({b, d_out, d_in, r, sm_count, 0}, [&] { return plan_dw_adapter(b, d_out, d_in, r, sm_count); });
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -1320,7 +1324,7 @@ slope_status_t slope_linear_bwd_dw_adapter(const void* dY, const void* X, const 
     DwAdapterParams p = {};
     p.M = d_out; p.N = d_in; p.K = b; p.r = r;
     p.splits_r = plan.splits_r; p.splits_l = plan.splits_l;
-    p.alternate_k = long_reduction(d_out, b, choose_dense_width(d_out, d_in, b, true, true, info.sm_count / 2));   // as the weight gradient alone
+    p.alternate_k = plan.alternate_k;
     p.dWc = static_cast<uint16_t*>(dWc_vals);
     p.mask = static_cast<const uint8_t*>(mask1_bits);
     p.ws_r = static_cast<float*>(workspace);

@@ -54,6 +54,34 @@ def test_weight_gradient(b, d_in, d_out, r):
     layer.poll()
 
 
+def test_carriers_in_a_ragged_reversed_group():
+    """9 x 13 tiles, in one launch with the adapter gradients: the second group of tile rows is a single row, half empty, and runs
+    backwards, so that the first carrier of its dR is the half-empty last column tile."""
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    b, d_in, d_out, r = 8193, 3200, 2176, 64
+    gen = torch.Generator("cuda").manual_seed(68)
+    new = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+    nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+    X, dY, T, dT = new(b, d_in), new(b, d_out), new(b, r), new(b, r)
+    vals, meta, mask = B.alloc_compressed(d_out, d_in)
+    B.slope_prune_24(new(d_out, d_in), vals, meta, mask)
+    dWc, dWc2, dL, dR = nan(d_out, d_in // 2), nan(d_out, d_in // 2), nan(d_in, r), nan(r, d_out)
+    ws = torch.empty(B.slope_bwd_dw_adapter_workspace_bytes(b, d_out, d_in, r), dtype=torch.uint8, device="cuda")
+    ws.view(torch.float32).fill_(float("nan"))             # (a carrier that skips its share leaves this in the sums)
+    B.slope_linear_bwd_dw_masked(dY, X, mask, dWc)
+    launches = B.slope_launch_count()
+    B.slope_linear_bwd_dw_adapter(dY, X, T, dT, mask, dWc2, dL, dR, ws)
+    assert B.slope_launch_count() - launches == 2          # the fused one and the sum of its shares
+    assert B.slope_poll_status() == 0
+    assert torch.equal(dWc.view(torch.int16), dWc2.view(torch.int16))
+    g = lambda t: to_f64(B.bits_from_bf16(t))
+    assert parity_error(g(dR), g(T).T @ g(dY)) <= REL_TOL
+    assert parity_error(g(dL), g(X).T @ g(dT)) <= REL_TOL
+
+
 @pytest.mark.parametrize("b,d_in,d_out,r", [
     (5001, 13824, 2560, 64),     # 5 row tiles of 512, the weights of all of them in one group
     (4500, 11008, 3968, 0),      # 31 row blocks: one CTA of the last row tile has rows for one sub-tile only
