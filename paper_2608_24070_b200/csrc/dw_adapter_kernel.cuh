@@ -32,7 +32,7 @@ struct DwAdapterParams {
     int M, N, K;                  // d_out, d_in, tokens
     int r;                        // adapter rank, multiple of 16, <= 128
     int splits_r, splits_l;       // partial sums per dR^T row block / per dL row block
-    int alternate_k;              // 1: tiles and ends of the reduction in the order of dense_gemm_pair_kernel<LONG>
+    int alternate_k;              // 1: tiles and ends of the reduction in the order of dense_gemm_pair_kernel<LONG>, one tile after the other
     uint16_t* dWc;                // [M x N/2]
     const uint8_t* mask;          // [M x N/8]
     float* ws_r;                  // [splits_r][M][r]

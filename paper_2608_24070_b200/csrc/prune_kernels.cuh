@@ -259,8 +259,9 @@ __global__ void __launch_bounds__(256, 4) prune24_double_kernel(const uint4* __r
     // ---- first pass: the two groups of this thread's 8 columns, row by row; W becomes W^R in place, in the packed order, in
     //      which words of the second pass are pairs of columns j, j + 4 (four byte permutes per row less than back in natural
     //      order).  The masked words are pinned: merged into the second pass they cost 204 bytes of spills, 22 us
-    //      instead of 18 at 4096 x 4096.  us, natural / packed order: 4096 x 4096 16.4 / 16.1, 4096 x 11008 40.2 / 39.5,
-    //      13824 x 5120 62.5 / 61.4, 2048 x 2048 6.27 / 6.10.
+    //      instead of 18 at 4096 x 4096 (nvcc 12.9).  us under sustained load, natural / packed order: 1024 x 1024 3.84 / 3.68,
+    //      2048 x 2048 6.14 / 6.05, 4096 x 4096 16.42 / 16.18, 2048 x 13824 26.1 / 25.9, 4096 x 11008 40.6 / 40.0, 13824 x 5120
+    //      62.9 / 61.9, 9600 x 8192 69.5 / 68.6: 0.8 to 4 % on each of 17 matrices of 1 to 79 M weights.
     const uint32_t one = opaque_one();
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
@@ -335,16 +336,22 @@ __global__ void __launch_bounds__(256) meta_to_canonical_kernel(const uint16_t* 
 // "sparseAdd": out = beta * A + gamma * B on two compressed value arrays with one pattern
 // (fp32 arithmetic, one rounding to bf16).  Pure streaming: 16-byte vectors, grid-stride.
 // `out` may be A or B (every thread reads its vectors before it writes them), hence no __restrict__.
-// B, the weights in weight decay, is what the refresh of the transposed copy reads next: L2 is asked to keep it rather than
-// the gradient, and update_transposed_kernel begins with the rows that were read last.  us for the two calls, without /
-// with both: 13824 x 5120 61.9 / 60.3, 11008 x 4096 41.1 / 40.3, 4096 x 4096 18.05 / 17.9, 2048 x 2048 7.4 / 7.4.
+// B, the weights in weight decay, is read again by the refresh of the transposed copy: from kKeepAddend vectors on (KEEP) L2 is asked
+// to keep it rather than the gradient, and update_transposed_kernel begins with the rows that were read last.  us under sustained
+// load, without / with both: the two calls back to back 13824 x 5120 62.7 / 61.2, 11008 x 4096 41.5 / 40.7, 4096 x 4096 18.15 /
+// 17.99; with an Adam pass over states of its own between them 201.7 / 198.7, 167.0 / 164.4, 59.3 / 58.9, 11008 x 11008 336.7 / 336.0;
+// as SGD in place (out = B) 63.1 / 62.3, 42.4 / 41.6, 18.03 / 17.95, 4096 x 3584 16.90 / 16.79, 4096 x 2560 12.71 / 12.68, but
+// 4096 x 2048 11.67 / 11.72 and 2048 x 2048 7.34 / 7.36, where all of it stays in L2 unasked.  What follows does not pay for the lines that stay: this call and a forward of the layer, 500 tokens
+// 5120 -> 13824 87.4 / 87.2, 2048 tokens 4096 -> 4096 47.4 / 47.3; the call alone 32.3 / 32.2.
+constexpr size_t kKeepAddend = size_t(640) << 10;
+template <bool KEEP>
 __global__ void __launch_bounds__(256) sparse_add_kernel(const uint4* A, const uint4* B, float beta, float gamma,
                                                          size_t n_vec, uint4* out) {
     griddep_stream(8);
-    const uint64_t keep = l2_policy_evict_last();
+    const uint64_t keep = KEEP ? l2_policy_evict_last() : 0;
     for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < n_vec;
          idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
-        const uint4 a = ld_v4(A + idx), b = ld_hint_v4(B + idx, keep);
+        const uint4 a = ld_v4(A + idx), b = KEEP ? ld_hint_v4(B + idx, keep) : ld_v4(B + idx);
         const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
         uint32_t r[4];
 #pragma unroll

@@ -1351,7 +1351,7 @@ slope_status_t slope_sparse_add(const void* A_vals, const void* B_vals, float be
     DeviceInfo info;
     if (slope_status_t st = check_arch(info)) return st;
     const size_t n_vec = static_cast<size_t>(rows) * cols / 2 / 8;
-    return launch_stream(sparse_add_kernel, dim3(stream_grid(n_vec, info)), static_cast<cudaStream_t>(stream),
+    return launch_stream(n_vec >= kKeepAddend ? sparse_add_kernel<true> : sparse_add_kernel<false>, dim3(stream_grid(n_vec, info)), static_cast<cudaStream_t>(stream),
                          static_cast<const uint4*>(A_vals), static_cast<const uint4*>(B_vals), beta, gamma, n_vec,
                          static_cast<uint4*>(out_vals));
 }

@@ -48,6 +48,22 @@ def test_sparse_add(B, oracle, rows, cols):
     assert np.array_equal(B.bits_from_bf16(out), A)
 
 
+@pytest.mark.parametrize("rows,cols", [(2432, 4096), (2560, 4096)])        # on either side of the line that L2 is asked to keep B from
+def test_sparse_add_in_place(B, rows, cols):
+    """Over either operand, bit for bit what the call writes elsewhere."""
+    import torch
+
+    A, Bv = (B.bf16_from_bits(si.gaussian_bf16((rows, cols // 2), sigma, seed)) for sigma, seed in ((1.0, 55), (0.02, 56)))
+    out, over_A, over_B = torch.empty_like(A), A.clone(), Bv.clone()
+    B.slope_sparse_add(A, Bv, -0.125, 1.0, out)
+    B.slope_sparse_add(over_A, Bv, -0.125, 1.0, over_A)
+    B.slope_sparse_add(A, over_B, -0.125, 1.0, over_B)
+    assert B.slope_poll_status() == 0
+    bits = lambda t: t.view(torch.int16)
+    assert torch.equal(bits(out), bits(over_A)) and torch.equal(bits(out), bits(over_B))
+    assert torch.equal(out, (-0.125 * A.double() + Bv.double()).float().bfloat16())
+
+
 @pytest.mark.parametrize("d_out,d_in", [(512, 512), (384, 640), (1280, 128), (11008, 4096), (4096, 11008)])
 def test_update_sparse_matrix(B, oracle, d_out, d_in):
     import torch
