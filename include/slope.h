@@ -24,7 +24,9 @@
  *  - Device-side waits are bounded; a wait that runs out makes the kernel stop
  *    and record SLOPE_ERR_TIMEOUT in a sticky status word, read (and cleared)
  *    by slope_poll_status().
- *  - Same inputs on the same device give bit-identical outputs.
+ *  - Same inputs on the same device give bit-identical outputs.  Equal tokens of
+ *    one call have equal rows in Y, dX, T and dT, wherever in the batch they
+ *    stand.
  *
  * Compressed 2:4 format of a matrix A[rows x cols] pruned along its columns
  *  - values  [rows x cols/2] bf16: for each group of 4 consecutive columns the

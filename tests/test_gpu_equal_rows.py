@@ -28,6 +28,7 @@ def _assert_equal_rows(out):
     (4500, 11008, 3968, 0),      # 31 row blocks, 168 tiles
     (9000, 4096, 4096, 16),      # weights that stay in L2
     (700, 11008, 2048, 0),       # 256-row tiles
+    (128, 11008, 512, 64),       # the few-token kernel, its reduction split over clusters
 ])
 def test_sparse_products(b, k, m, r):
     import torch
@@ -48,6 +49,25 @@ def test_sparse_products(b, k, m, r):
     _assert_equal_rows(dX)
     if not r:
         assert torch.equal(Y, dX)      # without adapters the two calls are one product
+
+
+@pytest.mark.parametrize("b,d,r", [(300, 4096, 64), (4097, 2048, 256), (16384, 768, 16)])
+def test_adapter_products(b, d, r):
+    import torch
+    from paper_2608_24070_b200 import binding as B, build
+
+    build.build()
+    gen = torch.Generator("cuda").manual_seed(96)
+    L, R = (torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16) for shape in ((d, r), (r, d)))
+    X = _rows(b, d, 97)
+    T, dT = (torch.full((b, r), float("nan"), device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    B.slope_adapter_fwd_bwd(0, X, None, L, None, b, d, d, r, T=T)
+    ws = torch.empty(max(16, B.slope_adapter_workspace_bytes(b, d, d, r)), dtype=torch.uint8, device="cuda")
+    dL, dR = (torch.empty(shape, device="cuda", dtype=torch.bfloat16) for shape in ((d, r), (r, d)))
+    B.slope_adapter_fwd_bwd(1, X, X, L, R, b, d, d, r, T=T, dT=dT, dL=dL, dR=dR, workspace=ws)
+    assert B.slope_poll_status() == 0
+    _assert_equal_rows(T)
+    _assert_equal_rows(dT)
 
 
 @pytest.mark.parametrize("b,k,m,backward", [
