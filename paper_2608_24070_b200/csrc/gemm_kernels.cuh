@@ -651,8 +651,9 @@ sparse_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 //     215.5 / 209.7; forward 8192 tokens 5120 -> 4096 258.7 / 258.7, 5632 282.1 / 280.1, 7168 370.9 / 361.9;
 //   tile rows, 16384 tokens 8192 -> 1024, 1536, 1792: 217.2 / 216.5, 323.6 / 318.7, 373.0 / 363.4; but with six 12000 tokens
 //     7168 -> 1408 205.2 / 205.4, 8500 145.2 / 146.2, forward 1536 tokens 11008 -> 4096 115.2 / 116.0, 1792 138.5 / 136.7.
-// DRAM reads in MB, one tile after the other / alternating ends only / so: 16384 tokens 4096 x 4096 631 / 534 / 436, 4096 -> 11008
-// 2059 / 1554 / 1294, 11008 -> 4096 1698 / 1452 / 1231.  (32 k-blocks at a time instead of 16 took 1 to 2 % longer where rows are many.)
+// DRAM reads in MB, one tile after the other / alternating ends only / so (captures differ by up to a seventh from GPU to GPU): 16384 tokens
+// 4096 x 4096 631 / 534 / 430 to 440, 4096 -> 11008 2059 / 1554 / 1140 to 1300, 11008 -> 4096 1698 / 1452 / 1050 to 1230.  (32 k-blocks
+// at a time instead of 16: 1 to 2 % longer in wide layers.)
 constexpr int kRasterGroupM = 8;
 constexpr int kLongFrom = 5632, kLongTileRows = 7;
 constexpr int kInterleaveBlocks = 16;
